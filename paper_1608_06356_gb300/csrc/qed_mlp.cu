@@ -6,24 +6,28 @@
 //   k_mlp_grad   each CTA draws mini-batches of (ln chi, kappa) uniformly over
 //                the network's domain (Philox), takes the target ln delta from
 //                the FP64 inverse table (bicubic, FP64), and runs the forward
-//                pass and the hand-written backward pass in FP32 (activations
-//                of one mini-batch in shared memory); the CTA's gradient sum
-//                goes to its own row of a partial-gradient array;
+//                pass and the hand-written backward pass in FP32 as register-
+//                tiled products (activations of one mini-batch in shared
+//                memory); the CTA's gradient sum goes to its own row of a
+//                partial-gradient array;
 //   k_mlp_adam   sums the partial rows in a fixed order (deterministic), and
 //                applies one bias-corrected Adam step to the FP32 weights;
 //   k_mlp_pack   converts W2 and W3 to BF16 tensor-core fragments.
 // The loss is the mean squared error of z (ln delta minus its asymptote).
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 
 #include "qed_internal.h"
 #include "qed_mlp.cuh"
 
 namespace qed {
 
-constexpr int GRAD_B = 128;   // samples per mini-batch (one per two threads)
-constexpr int GRAD_THREADS = 256;
-constexpr int APAD = 65;      // padded row length of the activation arrays
+constexpr int GRAD_B = 128;            // samples per mini-batch
+constexpr int GRAD_MATH = 256;         // threads of the matrix work: 8 samples x 4 units each
+constexpr int GRAD_THREADS = GRAD_MATH + GRAD_B;  // and one thread per sample of the next mini-batch
+constexpr int ALD = GRAD_B + 4;        // row length of the activation arrays [unit][sample]
+constexpr int LOSS_ROWS = 8;           // optimiser steps whose losses are kept on the device
 
 struct GradArgs {
   const float *w;        // FP32 weights
@@ -41,229 +45,322 @@ struct GradArgs {
   float scale;           // dL/dz = scale * (z - t)
 };
 
+// Shared memory of the gradient kernel.  Activations are kept unit-major, so
+// that eight samples of a unit are two 16-byte loads; the weights twice, each
+// with the four units u, u + 16, u + 32, u + 48 of a thread side by side:
+// Wp[k][4 u' + q] = W[k][u' + 16 q] for the forward products and
+// WT[k][4 u' + q] = W[u' + 16 q][k] for the backward ones.
+struct GradSmem {
+  float Wp[2][64 * 64], WT[2][64 * 64];
+  float W1[128], b1[64], b2[64], b3[64], W4[64], b4[4];
+  float X[2][2][GRAD_B], T[2][GRAD_B];  // inputs and targets (then dL/dz), two mini-batches
+  float Zp[GRAD_B];                     // half-row output partials
+  float H1[64 * ALD], H2[64 * ALD], D2[64 * ALD], D3[64 * ALD];
+  double loss[GRAD_MATH / 32];
+};
+
+// C[8][4] += A[k][samples r0 .. r0+7] B[k][4 cg ..] over the 64 units k
+__device__ __forceinline__ void gemm_8x4(const float *A, const float *B, int r0, int cg, float (&acc)[8][4]) {
+#pragma unroll 4
+  for (int k = 0; k < 64; ++k) {
+    const float4 a0 = *reinterpret_cast<const float4 *>(A + k * ALD + r0);
+    const float4 a1 = *reinterpret_cast<const float4 *>(A + k * ALD + r0 + 4);
+    const float4 w = *reinterpret_cast<const float4 *>(B + k * 64 + 4 * cg);
+    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[i][q] = fmaf(av[i], wv[q], acc[i][q]);
+  }
+}
+
+// G[i][q] += the sum over the mini-batch, in sample order, of
+// H[jg + 16 i][s] D[kg + 16 q][s]
+__device__ __forceinline__ void outer_4x4(const float *H, const float *D, int jg, int kg, float (&G)[4][4]) {
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
+#pragma unroll 2
+  for (int r = 0; r < GRAD_B; r += 4) {
+    float4 h[4], d[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      h[q] = *reinterpret_cast<const float4 *>(H + (jg + 16 * q) * ALD + r);
+      d[q] = *reinterpret_cast<const float4 *>(D + (kg + 16 * q) * ALD + r);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        acc[i][q] = fmaf(h[i].w, d[q].w, fmaf(h[i].z, d[q].z, fmaf(h[i].y, d[q].y, fmaf(h[i].x, d[q].x, acc[i][q]))));
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) G[i][q] += acc[i][q];
+}
+
+// sum over the mini-batch, in sample order, of f[s] row[s] (f null: of row[s])
+__device__ __forceinline__ float sample_sum(const float *row, const float *f) {
+  float v = 0.f;
+#pragma unroll 4
+  for (int r = 0; r < GRAD_B; r += 4) {
+    const float4 a = *reinterpret_cast<const float4 *>(row + r);
+    const float4 b = f ? *reinterpret_cast<const float4 *>(f + r) : make_float4(1.f, 1.f, 1.f, 1.f);
+    v = fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, v))));
+  }
+  return v;
+}
+
+__device__ __forceinline__ void put8(float *row, const float (&v)[8]) {
+  *reinterpret_cast<float4 *>(row) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4 *>(row + 4) = make_float4(v[4], v[5], v[6], v[7]);
+}
+
+// SiLU and its derivative at a
 __device__ __forceinline__ float silu_f(float a) { return a / (1.f + __expf(-a)); }
 __device__ __forceinline__ float dsilu_f(float a) {
-  float s = 1.f / (1.f + __expf(-a));
+  const float s = 1.f / (1.f + __expf(-a));
   return s * (1.f + a * (1.f - s));
 }
 
-__global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(GradArgs A) {
-  extern __shared__ __align__(16) float sm[];
-  float *W = sm;                       // MLP_NP (+3 pad)
-  float *G = W + MLP_NP + 3;           // MLP_NP (+3 pad) gradient accumulator
-  float *A1 = G + MLP_NP + 3;          // [GRAD_B][APAD]
-  float *A2 = A1 + GRAD_B * APAD;
-  float *A3 = A2 + GRAD_B * APAD;
-  float *X = A3 + GRAD_B * APAD;       // [GRAD_B][2]
-  float *T = X + 2 * GRAD_B;           // targets, then dL/dz
-  float *Zp = T + GRAD_B;              // half-row output partials
-  __shared__ double s_loss[GRAD_THREADS / 32];
-  const int tid = threadIdx.x;
-  for (int k = tid; k < MLP_NP; k += blockDim.x) {
-    W[k] = A.w[k];
-    G[k] = 0.f;
+// the math threads' own barrier
+__device__ __forceinline__ void math_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(GRAD_MATH) : "memory"); }
+
+// all threads, reached from the two roles' own code
+__device__ __forceinline__ void block_sync() { asm volatile("bar.sync 0, %0;\n" ::"n"(GRAD_THREADS) : "memory"); }
+
+// Input and target of sample t of mini-batch bi.
+__device__ __forceinline__ void grad_input(const GradArgs &A, GradSmem &S, int bi, int t) {
+  const int64_t s = ((int64_t)bi * gridDim.x + blockIdx.x) * GRAD_B + t;
+  float x0 = 0.f, x1 = 0.f, tt = 0.f;
+  bool valid = true;
+  if (A.x) {
+    valid = s < A.n;
+    if (valid) { x0 = A.x[2 * s]; x1 = A.x[2 * s + 1]; tt = A.t[s]; }
+  } else {
+    U4 r = philox4x32_10(U4{(uint32_t)s, (uint32_t)(s >> 32), (uint32_t)A.step, 0x4D4C5031u},
+                         (uint32_t)A.seed, (uint32_t)(A.seed >> 32));
+    const double ul = ((double)r.x + 0.5) * 0x1p-32, uk = ((double)r.y + 0.5) * 0x1p-32;
+    // the training domain extends past the one the network serves, so
+    // that its edges are not the edges of the fit
+    const double l = (MLP_L_LO - MLP_TRAIN_DL) + (MLP_L_HI - MLP_L_LO + 2 * MLP_TRAIN_DL) * ul;
+    const double k = (MLP_K_LO - MLP_TRAIN_DK) + (MLP_K_HI - MLP_K_LO + 2 * MLP_TRAIN_DK) * uk;
+    const double Y = interp2(A.Y64, A.gl, l, A.gk, k);
+    const double sp = k > 30.0 ? k : log1p(exp(k));
+    x0 = (float)((l - MLP_LC) / MLP_LS);
+    x1 = (float)((k - MLP_KC) / MLP_KS);
+    tt = (float)(Y - (3.0 * k - 2.0 * sp));
   }
-  double loss = 0.0;
+  S.X[bi & 1][0][t] = x0;
+  S.X[bi & 1][1][t] = x1;
+  S.T[bi & 1][t] = valid ? tt : NAN;  // NaN marks a padding row (no gradient)
+}
+
+// One CTA per SM.  The eight math warps run the six 64-wide matrix products of
+// a mini-batch (two forward, two weight gradients, two backward) as register
+// tiles: 8 samples x 4 units a thread, 32 FMAs per three 16-byte shared loads;
+// the weight gradients stay in registers over the CTA's mini-batches.  The
+// four auxiliary warps meanwhile make the next mini-batch's targets, whose
+// FP64 arithmetic would otherwise stand alone, and the sums over samples of
+// W1, W4 and the biases.  Every sum is taken in the order of the units or the
+// samples, so the result does not depend on how the work is divided.
+__global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(GradArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  GradSmem &S = *reinterpret_cast<GradSmem *>(smem_raw);
+  const int tid = threadIdx.x;
+  for (int k = tid; k < 64 * 64; k += GRAD_THREADS) {
+    const int in = k >> 6, out = k & 63;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const float w = A.w[(l ? MLP_OFF_W3 : MLP_OFF_W2) + k];
+      S.Wp[l][in * 64 + 4 * (out & 15) + (out >> 4)] = w;
+      S.WT[l][out * 64 + 4 * (in & 15) + (in >> 4)] = w;
+    }
+  }
+  if (tid < 128) S.W1[tid] = A.w[MLP_OFF_W1 + tid];
+  if (tid < 64) {
+    S.b1[tid] = A.w[MLP_OFF_B1 + tid];
+    S.b2[tid] = A.w[MLP_OFF_B2 + tid];
+    S.b3[tid] = A.w[MLP_OFF_B3 + tid];
+    S.W4[tid] = A.w[MLP_OFF_W4 + tid];
+  }
+  if (tid == 0) S.b4[0] = A.w[MLP_OFF_B4];
   const int nb = A.x ? (int)((A.n + (int64_t)GRAD_B * gridDim.x - 1) / ((int64_t)GRAD_B * gridDim.x))
                      : A.batches_per_cta;
-  __syncthreads();
+  float *P = A.partial + (size_t)blockIdx.x * MLP_NP;
+  if (tid >= GRAD_MATH) {
+    // ---- auxiliary warps: the block barriers match the math warps' below
+    const int a = tid - GRAD_MATH, c = a & 63;
+    const bool lo = a < 64;
+    float gW4 = 0.f, gb4 = 0.f, gb3 = 0.f, gb2 = 0.f, gb1 = 0.f, gW1 = 0.f;
+    grad_input(A, S, 0, a);
+    block_sync();
+    for (int bi = 0; bi < nb; ++bi) {
+      const float *T = S.T[bi & 1], *X = S.X[bi & 1][lo ? 0 : 1];
+      block_sync();  // (H2 free)
+      block_sync();  // h3 in D3, dL/dz in T
+      if (lo) gW4 += sample_sum(S.D3 + c * ALD, T);
+      else if (a == 64) gb4 += sample_sum(T, nullptr);
+      block_sync();  // (D3 free)
+      block_sync();  // dA3 in D3
+      if (!lo) gb3 += sample_sum(S.D3 + c * ALD, nullptr);
+      if (bi + 1 < nb) grad_input(A, S, bi + 1, a);
+      block_sync();  // dA2 in D2
+      if (lo) gb2 += sample_sum(S.D2 + c * ALD, nullptr);
+      block_sync();  // dA1 in H2, the next inputs in X and T
+      if (lo) gb1 += sample_sum(S.H2 + c * ALD, nullptr);
+      gW1 += sample_sum(S.H2 + c * ALD, X);
+    }
+    P[MLP_OFF_W1 + a] = gW1;
+    if (lo) {
+      P[MLP_OFF_W4 + c] = gW4;
+      P[MLP_OFF_B2 + c] = gb2;
+      P[MLP_OFF_B1 + c] = gb1;
+    } else {
+      P[MLP_OFF_B3 + c] = gb3;
+      if (a == 64) P[MLP_OFF_B4] = gb4;
+    }
+    return;
+  }
+  // ---- math warps
+  const int r0 = (tid >> 4) * 8, cg = tid & 15, jg = tid >> 4;  // samples, units; weight-gradient rows
+  const int row = tid & (GRAD_B - 1), c0 = (tid / GRAD_B) * 32;  // output layer: sample, unit half
+  float G2[4][4], G3[4][4];
+  double loss = 0.0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) G2[i][q] = G3[i][q] = 0.f;
+  block_sync();
   for (int bi = 0; bi < nb; ++bi) {
-    const int64_t first = ((int64_t)bi * gridDim.x + blockIdx.x) * GRAD_B;
-    // ---- inputs and targets
-    if (tid < GRAD_B) {
-      float x0 = 0.f, x1 = 0.f, tt = 0.f;
-      bool valid = true;
-      if (A.x) {
-        const int64_t s = first + tid;
-        valid = s < A.n;
-        if (valid) { x0 = A.x[2 * s]; x1 = A.x[2 * s + 1]; tt = A.t[s]; }
-      } else {
-        U4 r = philox4x32_10(U4{(uint32_t)(first + tid), (uint32_t)((first + tid) >> 32),
-                                (uint32_t)A.step, 0x4D4C5031u},
-                             (uint32_t)A.seed, (uint32_t)(A.seed >> 32));
-        const double ul = ((double)r.x + 0.5) * 0x1p-32, uk = ((double)r.y + 0.5) * 0x1p-32;
-        // the training domain extends past the one the network serves, so
-        // that its edges are not the edges of the fit
-        const double l = (MLP_L_LO - MLP_TRAIN_DL) + (MLP_L_HI - MLP_L_LO + 2 * MLP_TRAIN_DL) * ul;
-        const double k = (MLP_K_LO - MLP_TRAIN_DK) + (MLP_K_HI - MLP_K_LO + 2 * MLP_TRAIN_DK) * uk;
-        const double Y = interp2(A.Y64, A.gl, l, A.gk, k);
-        const double sp = k > 30.0 ? k : log1p(exp(k));
-        x0 = (float)((l - MLP_LC) / MLP_LS);
-        x1 = (float)((k - MLP_KC) / MLP_KS);
-        tt = (float)(Y - (3.0 * k - 2.0 * sp));
-      }
-      X[2 * tid] = x0;
-      X[2 * tid + 1] = x1;
-      T[tid] = valid ? tt : NAN;  // NaN marks a padding row (no gradient)
+    const float *X0 = S.X[bi & 1][0] + r0, *X1 = S.X[bi & 1][1] + r0;
+    float *T = S.T[bi & 1];
+    // ---- forward: layer 1 on two inputs
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = cg + 16 * q;
+      float h[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) h[i] = silu_f(fmaf(X0[i], S.W1[c], fmaf(X1[i], S.W1[64 + c], S.b1[c])));
+      put8(S.H1 + c * ALD + r0, h);
     }
-    __syncthreads();
-    // ---- forward: A1 = X W1 + b1 ; thread -> (row = tid % 128, column half = tid / 128)
-    const int row = tid % GRAD_B, c0 = (tid / GRAD_B) * 32;
-    for (int c = c0; c < c0 + 32; ++c)
-      A1[row * APAD + c] = fmaf(X[2 * row], W[MLP_OFF_W1 + c],
-                                fmaf(X[2 * row + 1], W[MLP_OFF_W1 + 64 + c], W[MLP_OFF_B1 + c]));
-    __syncthreads();
-    {
-      float acc[32];
+    math_sync();
+    float acc[8][4];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = W[MLP_OFF_B2 + c0 + j];
-      for (int k = 0; k < 64; ++k) {
-        const float h = silu_f(A1[row * APAD + k]);
-        const float *wr = W + MLP_OFF_W2 + k * 64 + c0;
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = fmaf(h, wr[j], acc[j]);
+      for (int i = 0; i < 8; ++i) acc[i][q] = S.b2[cg + 16 * q];
+    gemm_8x4(S.H1, S.Wp[0], r0, cg, acc);
+    block_sync();  // H2 free (the sums of dA1 of the mini-batch before)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {  // layer 2's output and derivative
+      const int c = cg + 16 * q;
+      float h[8], d[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        h[i] = silu_f(acc[i][q]);
+        d[i] = dsilu_f(acc[i][q]);
       }
-#pragma unroll
-      for (int j = 0; j < 32; ++j) A2[row * APAD + c0 + j] = acc[j];
+      put8(S.H2 + c * ALD + r0, h);
+      put8(S.D2 + c * ALD + r0, d);
     }
-    __syncthreads();
-    {
-      float acc[32];
+    math_sync();
 #pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = W[MLP_OFF_B3 + c0 + j];
-      for (int k = 0; k < 64; ++k) {
-        const float h = silu_f(A2[row * APAD + k]);
-        const float *wr = W + MLP_OFF_W3 + k * 64 + c0;
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = fmaf(h, wr[j], acc[j]);
-      }
+      for (int i = 0; i < 8; ++i) acc[i][q] = S.b3[cg + 16 * q];
+    gemm_8x4(S.H2, S.Wp[1], r0, cg, acc);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) A3[row * APAD + c0 + j] = acc[j];
+    for (int q = 0; q < 4; ++q) {
+      float h[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) h[i] = silu_f(acc[i][q]);
+      put8(S.D3 + (cg + 16 * q) * ALD + r0, h);
     }
-    __syncthreads();
-    // ---- output and dL/dz (two threads per row: column halves combined in shared memory)
+    math_sync();
+    // output and dL/dz (two threads per sample, unit halves)
     {
       float part = 0.f;
-      for (int c = c0; c < c0 + 32; ++c) part = fmaf(silu_f(A3[row * APAD + c]), W[MLP_OFF_W4 + c], part);
-      if (tid >= GRAD_B) Zp[row] = part;
-      __syncthreads();
-      if (tid < GRAD_B) {
-        const float z = part + Zp[row] + W[MLP_OFF_B4];
-        const float tt = T[row];
+#pragma unroll 8
+      for (int c = c0; c < c0 + 32; ++c) part = fmaf(S.D3[c * ALD + row], S.W4[c], part);
+      if (c0) S.Zp[row] = part;
+      math_sync();
+      if (!c0) {
+        const float z = part + S.Zp[row] + S.b4[0], t = T[row];
         float dz = 0.f;
-        if (!isnan(tt)) {
-          const float r = z - tt;
+        if (!isnan(t)) {
+          const float r = z - t;
           loss += (double)r * r;
           dz = A.scale * r;
         }
         T[row] = dz;
       }
-      __syncthreads();
     }
-    // ---- backward
-    // W4, b4 (one thread per column, rows summed in order)
-    if (tid < 64) {
-      float gw = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) gw = fmaf(silu_f(A3[r * APAD + tid]), T[r], gw);
-      G[MLP_OFF_W4 + tid] += gw;
-    } else if (tid == 64) {
-      float gb = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) gb += T[r];
-      G[MLP_OFF_B4] += gb;
+    block_sync();  // h3 in D3, dL/dz in T
+    // ---- backward: dA3 = dL/dz W4 silu'(a3)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i][q] = T[r0 + i] * S.W4[cg + 16 * q] * dsilu_f(acc[i][q]);
+    block_sync();  // D3 free
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float d[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) d[i] = acc[i][q];
+      put8(S.D3 + (cg + 16 * q) * ALD + r0, d);
     }
-    __syncthreads();
-    // dA3 = dz * W4 * silu'(A3), in place
-    for (int c = c0; c < c0 + 32; ++c)
-      A3[row * APAD + c] = T[row] * W[MLP_OFF_W4 + c] * dsilu_f(A3[row * APAD + c]);
-    __syncthreads();
-    // gW3[j][k] = sum_r h2[r][j] dA3[r][k]; gb3[k] = sum_r dA3[r][k]
-    {
-      const int j = tid / 4, kb = (tid % 4) * 16;
-      float acc[16];
+    block_sync();  // dA3 in D3
+    outer_4x4(S.H2, S.D3, jg, cg, G3);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) acc[q] = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) {
-        const float h = silu_f(A2[r * APAD + j]);
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int q = 0; q < 16; ++q) acc[q] = fmaf(h, A3[r * APAD + kb + q], acc[q]);
-      }
+      for (int i = 0; i < 8; ++i) acc[i][q] = 0.f;
+    gemm_8x4(S.D3, S.WT[1], r0, cg, acc);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) G[MLP_OFF_W3 + j * 64 + kb + q] += acc[q];
+    for (int q = 0; q < 4; ++q) {
+      float *own = S.D2 + (cg + 16 * q) * ALD + r0;  // this thread's elements
+      float d[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) d[i] = acc[i][q] * own[i];
+      put8(own, d);
     }
-    if (tid < 64) {
-      float gb = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) gb += A3[r * APAD + tid];
-      G[MLP_OFF_B3 + tid] += gb;
+    block_sync();  // dA2 in D2
+    outer_4x4(S.H1, S.D2, jg, cg, G2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i][q] = 0.f;
+    gemm_8x4(S.D2, S.WT[0], r0, cg, acc);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = cg + 16 * q;
+      float d[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        d[i] = acc[i][q] * dsilu_f(fmaf(X0[i], S.W1[c], fmaf(X1[i], S.W1[64 + c], S.b1[c])));
+      put8(S.H2 + c * ALD + r0, d);
     }
-    __syncthreads();
-    // dH2 = dA3 W3^T ; dA2 = dH2 * silu'(A2) (in place)
-    {
-      float acc[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-      for (int k = 0; k < 64; ++k) {
-        const float d = A3[row * APAD + k];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = fmaf(d, W[MLP_OFF_W3 + (c0 + j) * 64 + k], acc[j]);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const int c = c0 + j;
-        A2[row * APAD + c] = acc[j] * dsilu_f(A2[row * APAD + c]);
-      }
-    }
-    __syncthreads();
-    // gW2, gb2 from h1 = silu(A1) and dA2
-    {
-      const int j = tid / 4, kb = (tid % 4) * 16;
-      float acc[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) acc[q] = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) {
-        const float h = silu_f(A1[r * APAD + j]);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) acc[q] = fmaf(h, A2[r * APAD + kb + q], acc[q]);
-      }
-#pragma unroll
-      for (int q = 0; q < 16; ++q) G[MLP_OFF_W2 + j * 64 + kb + q] += acc[q];
-    }
-    if (tid < 64) {
-      float gb = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) gb += A2[r * APAD + tid];
-      G[MLP_OFF_B2 + tid] += gb;
-    }
-    __syncthreads();
-    // dH1 = dA2 W2^T ; dA1 = dH1 * silu'(A1) (in place)
-    {
-      float acc[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-      for (int k = 0; k < 64; ++k) {
-        const float d = A2[row * APAD + k];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = fmaf(d, W[MLP_OFF_W2 + (c0 + j) * 64 + k], acc[j]);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const int c = c0 + j;
-        A1[row * APAD + c] = acc[j] * dsilu_f(A1[row * APAD + c]);
-      }
-    }
-    __syncthreads();
-    // gW1[i][k] = sum_r x[r][i] dA1[r][k] ; gb1[k] = sum_r dA1[r][k]
-    if (tid < 192) {
-      const int k = tid % 64, which = tid / 64;  // 0: W1 row 0, 1: W1 row 1, 2: b1
-      float acc = 0.f;
-      for (int r = 0; r < GRAD_B; ++r) {
-        const float d = A1[r * APAD + k];
-        const float f = which == 2 ? 1.f : X[2 * r + which];
-        acc = fmaf(f, d, acc);
-      }
-      if (which == 2) G[MLP_OFF_B1 + k] += acc;
-      else G[MLP_OFF_W1 + which * 64 + k] += acc;
-    }
-    __syncthreads();
+    block_sync();  // dA1 in H2
   }
-  for (int k = tid; k < MLP_NP; k += blockDim.x) A.partial[(size_t)blockIdx.x * MLP_NP + k] = G[k];
-  // loss of this CTA
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int o = (jg + 16 * i) * 64 + cg + 16 * q;
+      P[MLP_OFF_W2 + o] = G2[i][q];
+      P[MLP_OFF_W3 + o] = G3[i][q];
+    }
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-  if ((tid & 31) == 0) s_loss[tid >> 5] = loss;
-  __syncthreads();
+  if ((tid & 31) == 0) S.loss[tid >> 5] = loss;
+  math_sync();
   if (tid == 0) {
     double s = 0.0;
-    for (int w = 0; w < GRAD_THREADS / 32; ++w) s += s_loss[w];
+    for (int w = 0; w < GRAD_MATH / 32; ++w) s += S.loss[w];
     A.loss_sum[blockIdx.x] = s;
   }
 }
@@ -277,11 +374,22 @@ struct AdamArgs {
   int apply;
 };
 
-__global__ void k_mlp_adam(AdamArgs A) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+// One thread per parameter in CTAs of one warp, so that the rows' loads come
+// from every SM; the rows are added in order, ADAM_BATCH loads in flight.
+constexpr int ADAM_THREADS = 32, ADAM_BATCH = 16;
+constexpr int ADAM_BLOCKS = (MLP_NP + ADAM_THREADS - 1) / ADAM_THREADS;
+__global__ void __launch_bounds__(ADAM_THREADS) k_mlp_adam(AdamArgs A) {
+  const int k = blockIdx.x * ADAM_THREADS + threadIdx.x;
   if (k >= MLP_NP) return;
   float g = 0.f;
-  for (int p = 0; p < A.nparts; ++p) g += A.partial[(size_t)p * MLP_NP + k];  // fixed order
+#pragma unroll 2
+  for (int p = 0; p < A.nparts; p += ADAM_BATCH) {
+    float v[ADAM_BATCH];
+#pragma unroll
+    for (int q = 0; q < ADAM_BATCH; ++q) v[q] = p + q < A.nparts ? A.partial[(size_t)(p + q) * MLP_NP + k] : 0.f;
+#pragma unroll
+    for (int q = 0; q < ADAM_BATCH; ++q) g += v[q];
+  }
   if (A.grad_out) A.grad_out[k] = g;
   if (!A.apply) return;
   const float m = A.b1 * A.m[k] + (1.f - A.b1) * g;
@@ -311,15 +419,13 @@ __global__ void k_mlp_pack(const float *w, uint32_t *frag) {
   pack_split(W[(k0 + 8) * 64 + n], W[(k0 + 9) * 64 + n], F[o + 1], Fl[o + 1]);
 }
 
-static size_t grad_smem() {
-  return sizeof(float) * (2 * (MLP_NP + 3) + 3 * GRAD_B * APAD + 4 * GRAD_B);
-}
+static size_t grad_smem() { return sizeof(GradSmem); }
 
 int mlp_alloc(qed_ctx *c) {
   c->mlp_parts = c->num_sms;
   size_t bytes = sizeof(float) * MLP_NP * 4 + sizeof(uint32_t) * MLP_FRAG_WORDS +
                  sizeof(float) * MLP_SMEM_FLOATS + sizeof(float) * (size_t)MLP_NP * c->mlp_parts +
-                 sizeof(double) * c->mlp_parts;
+                 sizeof(double) * LOSS_ROWS * c->mlp_parts;
   if (cudaMalloc(&c->mlp_mem, bytes) != cudaSuccess) return QED_ERR_NOMEM;
   float *f = static_cast<float *>(c->mlp_mem);
   c->mlp_w = f;
@@ -430,7 +536,7 @@ extern "C" int qed_mlp_grad(qed_ctx *c, const float *x, const float *t, int64_t 
   a.nparts = c->mlp_parts;
   a.grad_out = grad;
   a.apply = 0;
-  k_mlp_adam<<<(MLP_NP + 255) / 256, 256, 0, st>>>(a);
+  k_mlp_adam<<<ADAM_BLOCKS, ADAM_THREADS, 0, st>>>(a);
   c->launches += 2;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && loss) {
@@ -468,34 +574,34 @@ extern "C" int qed_mlp_train(qed_ctx *c, int64_t n_samples, float lr, uint64_t s
   a.eps = 1e-8f;
   a.apply = 1;
   const float lr_min = lr * 0.01f;
-  double loss_tail = 0.0;
-  int64_t tail_n = 0;
+  const int64_t tail = steps < LOSS_ROWS ? steps : LOSS_ROWS;  // steps whose mean loss is returned
   for (int64_t s = 0; s < steps; ++s) {
     g.step = c->mlp_step + s;
+    g.loss_sum = c->mlp_loss + (s % LOSS_ROWS) * c->mlp_parts;
     k_mlp_grad<<<c->mlp_parts, GRAD_THREADS, grad_smem(), st>>>(g);
     const int64_t k = c->mlp_step + s + 1;  // Adam step count (from 1)
     a.lr = lr_min + 0.5f * (lr - lr_min) * (1.f + cosf(3.14159265f * (float)s / (float)steps));
     a.bc1 = 1.f - powf(a.b1, (float)k);
     a.bc2 = 1.f - powf(a.b2, (float)k);
-    k_mlp_adam<<<(MLP_NP + 255) / 256, 256, 0, st>>>(a);
+    k_mlp_adam<<<ADAM_BLOCKS, ADAM_THREADS, 0, st>>>(a);
     c->launches += 2;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(e, "qed_mlp_train");
-    if (s >= steps - 8) {  // mean loss of the last steps (synchronises only there)
-      double tmp[1024];
-      int np = c->mlp_parts < 1024 ? c->mlp_parts : 1024;
-      e = cudaMemcpyAsync(tmp, c->mlp_loss, sizeof(double) * np, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) return fail(e, "qed_mlp_train");
-      double sum = 0.0;
-      for (int p = 0; p < np; ++p) sum += tmp[p];
-      loss_tail += sum / (double)per_step;
-      tail_n += 1;
-    }
   }
   c->mlp_step += steps;
+  double *rows = (double *)malloc(sizeof(double) * LOSS_ROWS * c->mlp_parts);
+  if (!rows) return QED_ERR_NOMEM;
   cudaError_t e = pack(c, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(rows, c->mlp_loss, sizeof(double) * LOSS_ROWS * c->mlp_parts, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (final_loss) *final_loss = tail_n ? loss_tail / tail_n : 0.0;
+  double loss_tail = 0.0;
+  for (int64_t s = steps - tail; s < steps; ++s) {
+    double sum = 0.0;
+    for (int p = 0; p < c->mlp_parts; ++p) sum += rows[(s % LOSS_ROWS) * c->mlp_parts + p];
+    loss_tail += sum / (double)per_step;
+  }
+  free(rows);
+  if (final_loss && e == cudaSuccess) *final_loss = loss_tail / (double)tail;
   return fail(e, "qed_mlp_train");
 }
