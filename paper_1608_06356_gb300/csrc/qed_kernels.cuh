@@ -40,6 +40,26 @@ struct Out {
   ScanState scan;
 };
 
+// One node of the grid, 32 bytes: one 256-bit load where the grid is aligned
+// to its nodes, else two of 128 bits.  A node is one sector, so the wide load
+// halves the requests of a gather whose lanes touch different nodes.
+struct Node { float v[8]; };
+__device__ __forceinline__ Node load_node(const float *p, bool wide) {
+  Node n;
+  if (wide) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+        : "=f"(n.v[0]), "=f"(n.v[1]), "=f"(n.v[2]), "=f"(n.v[3]), "=f"(n.v[4]), "=f"(n.v[5]),
+          "=f"(n.v[6]), "=f"(n.v[7])
+        : "l"(p));
+  } else {
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+    const float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+    n.v[0] = a.x; n.v[1] = a.y; n.v[2] = a.z; n.v[3] = a.w;
+    n.v[4] = b.x; n.v[5] = b.y; n.v[6] = b.z; n.v[7] = b.w;
+  }
+  return n;
+}
+
 // CIC gather from grid[nz][ny][nx][8] (periodic).
 template <class Real>
 __device__ __forceinline__ void cic_gather(const Fld<Real> &f, Real x, Real y, Real z, Real E[3],
@@ -56,6 +76,7 @@ __device__ __forceinline__ void cic_gather(const Fld<Real> &f, Real x, Real y, R
   long long k1 = k0 + 1 == f.nz ? 0 : k0 + 1;
 #pragma unroll
   for (int c = 0; c < 3; ++c) { E[c] = (Real)0; B[c] = (Real)0; }
+  const bool wide = (reinterpret_cast<uintptr_t>(f.grid) & 31) == 0;
 #pragma unroll
   for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
@@ -64,10 +85,9 @@ __device__ __forceinline__ void cic_gather(const Fld<Real> &f, Real x, Real y, R
       for (int di = 0; di < 2; ++di) {
         Real w = (di ? wx : (Real)1 - wx) * (dj ? wy : (Real)1 - wy) * (dk ? wz : (Real)1 - wz);
         long long node = ((dk ? k1 : k0) * f.ny + (dj ? j1 : j0)) * f.nx + (di ? i1 : i0);
-        const float4 *pn = reinterpret_cast<const float4 *>(f.grid + 8 * node);
-        float4 a = __ldg(pn), b = __ldg(pn + 1);
-        E[0] += w * (Real)a.x; E[1] += w * (Real)a.y; E[2] += w * (Real)a.z;
-        B[0] += w * (Real)a.w; B[1] += w * (Real)b.x; B[2] += w * (Real)b.y;
+        const Node n = load_node(f.grid + 8 * node, wide);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) { E[c] += w * (Real)n.v[c]; B[c] += w * (Real)n.v[3 + c]; }
       }
 }
 

@@ -17,11 +17,12 @@
 // neighbours coming from planes that L2 still holds.  One step is four
 // passes -- B half-step, E step (which zeroes J behind it), B half-step, node
 // grid -- because each needs its neighbours' results of the one before.  The
-// deposit is one thread per particle, grid-stride over a persistent grid:
-// 8 CIC weights x 3 components at their staggered positions, reduced in L2
-// by atomics -- the two x-neighbours of each stencil row by one 16-byte
-// vector atomic where they share an aligned group of four floats (3 rows
-// in 4), so about 15 atomic operations per particle instead of 24.
+// deposit adds 8 CIC weights x 3 components per particle at their staggered
+// positions: few particles directly, one thread each, by atomics in L2 -- the
+// two x-neighbours of each stencil row by one 16-byte vector atomic where they
+// share an aligned group of four floats (3 rows in 4), so about 15 atomic
+// operations per particle instead of 24 -- and many by tiles of cells that
+// are summed on chip.
 #include <cmath>
 #include <cstdio>
 
@@ -192,31 +193,407 @@ __device__ __forceinline__ void spread(float *J, const DepArgs<Real> &A, Real fx
     }
 }
 
+// Velocity times dt-independent parts of one particle's deposit: reduced
+// coordinates (cells) of its mid-step position and the currents a v.  The
+// products are written with explicit fused operations so that every kernel
+// that calls this rounds alike.
+template <class Real> struct DepPoint { Real f[3], j[3]; };
+
+// 1 / sqrt(x), x >= 1: the fast reciprocal root and one Newton step (to the
+// last bit or so; the IEEE root and division are a third of the instructions
+// of a binning kernel, which issue bounds).  An infinite x gives NaN, as
+// inf * 0 would.
+__device__ __forceinline__ float dep_rsqrt(float x) {
+  const float y = rsqrtf(x);
+  return y * fmaf(-0.5f * x * y, y, 1.5f);
+}
+__device__ __forceinline__ double dep_rsqrt(double x) { return 1.0 / sqrt(x); }
+
 template <class Real>
-__global__ void __launch_bounds__(DEPOSIT_THREADS) k_pic_deposit(DepArgs<Real> A) {
+__device__ __forceinline__ bool dep_point(const DepArgs<Real> &A, int64_t p, DepPoint<Real> &d) {
+  const Real px = A.px[p], py = A.py[p], pz = A.pz[p];
+  const Real ig = dep_rsqrt(fma(pz, pz, fma(py, py, fma(px, px, (Real)1))));
+  const Real vx = px * ig, vy = py * ig, vz = pz * ig;
+  d.f[0] = (fma(-A.half_dt, vx, A.x[p]) - A.x0) * A.idx;
+  d.f[1] = (fma(-A.half_dt, vy, A.y[p]) - A.y0) * A.idy;
+  d.f[2] = (fma(-A.half_dt, vz, A.z[p]) - A.z0) * A.idz;
+  d.j[0] = vx; d.j[1] = vy; d.j[2] = vz;  // scaled by the caller
+  const Real lim = (Real)4.0e15;  // reduced coordinates beyond this are not finite cells
+  return fabs(d.f[0]) < lim && fabs(d.f[1]) < lim && fabs(d.f[2]) < lim;  // also false for NaN
+}
+
+template <class Real>
+__device__ __forceinline__ void dep_direct(const DepArgs<Real> &A, const DepPoint<Real> &d) {
+  spread(A.jx, A, d.f[0] - (Real)0.5, d.f[1], d.f[2], d.j[0]);
+  spread(A.jy, A, d.f[0], d.f[1] - (Real)0.5, d.f[2], d.j[1]);
+  spread(A.jz, A, d.f[0], d.f[1], d.f[2] - (Real)0.5, d.j[2]);
+}
+
+template <class Real> __device__ __forceinline__ int64_t dep_count(const DepArgs<Real> &A) {
   int64_t n = *A.d_n;
   if (A.d_lim && *A.d_lim < n) n = *A.d_lim;
-  if (n > A.cap) n = A.cap;
-  const Real lim = (Real)4.0e15;  // reduced coordinates beyond this are not finite cells
+  return n > A.cap ? A.cap : n;
+}
+
+// Segment of the records of one tile, or of one of `ways` parts of a tile: the
+// CTAs of a grid with few tiles spread their atomics over that many counters.
+// A sector each: neighbouring counters in one sector would share its queue.
+struct alignas(32) TileSeg { uint32_t cursor, end, start, pad[5]; };
+
+struct TileArgs {
+  TileSeg *seg;     // [ntiles * ways]
+  uint32_t *total;  // records allocated
+  uint32_t ntiles, ways, rec_cap;
+  uint32_t ntx, nty;
+  int64_t min_n, max_n;  // other numbers of particles are deposited directly
+};
+
+// Direct deposit: a particle's 24 contributions as atomics (launches too small
+// for the tiled path, and its particles without a record).
+template <class Real>
+__global__ void __launch_bounds__(DEPOSIT_THREADS) k_pic_deposit(DepArgs<Real> A, TileArgs T) {
+  const int64_t n = dep_count(A);
+  if (n >= T.min_n && n <= T.max_n) return;  // the tiled path's
   unsigned bad = 0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
-    const Real px = A.px[p], py = A.py[p], pz = A.pz[p];
-    const Real ig = (Real)1 / sqrt((Real)1 + px * px + py * py + pz * pz);
-    const Real vx = px * ig, vy = py * ig, vz = pz * ig;
-    const Real fx = (A.x[p] - A.half_dt * vx - A.x0) * A.idx;
-    const Real fy = (A.y[p] - A.half_dt * vy - A.y0) * A.idy;
-    const Real fz = (A.z[p] - A.half_dt * vz - A.z0) * A.idz;
-    if (!(fabs(fx) < lim && fabs(fy) < lim && fabs(fz) < lim)) {  // also false for NaN
+    DepPoint<Real> d;
+    if (!dep_point(A, p, d)) {
       bad = 1;
       continue;
     }
     const Real a = A.scale * A.w[p];
-    spread(A.jx, A, fx - (Real)0.5, fy, fz, a * vx);
-    spread(A.jy, A, fx, fy - (Real)0.5, fz, a * vy);
-    spread(A.jz, A, fx, fy, fz - (Real)0.5, a * vz);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d.j[c] *= a;
+    dep_direct(A, d);
   }
   if (bad) atomicOr(&A.cnt->status, (unsigned)QED_STATUS_NONFINITE);
+}
+
+// ---------------------------------------------------------------------------
+// Tiled deposit.  The direct deposit is bound by atomics in L2: 15 per
+// particle, on lines that a random particle order brings from HBM each time
+// once J is larger than L2.  Here the particles are first binned by tile of
+// 8 x 8 x 4 cells (count, segment allocation, scatter of 32-byte records -- one
+// 256-bit store each, which a scattered order takes at twice the rate of two of
+// 128 bits: 434 against 794 us for 16.8M), then a CTA sums a tile's currents on
+// chip: one thread per cell, the particles of a batch ordered by cell, 36 sums
+// in registers (3 x 2 x 2 positions per component around the cell), added up
+// in a shared (8+2) x (8+2) x (4+2) halo tile; only that tile goes to J, by
+// atomics that are contiguous along x.  16.8M particles: 256^3 cells in random
+// order 5.00 -> 1.34 ms (count 0.14, scatter 0.42, tiles 0.78: bound by the
+// scattered stores and by instruction issue in the tiles), 128^3 by cell 1.44
+// -> 0.59 ms (0.09, 0.24, 0.26).
+// ---------------------------------------------------------------------------
+constexpr int TLX = 8, TLY = 8, TLZ = 4, TL_CELLS = TLX * TLY * TLZ;
+constexpr int HLX = TLX + 2, HLY = TLY + 2, HLZ = TLZ + 2, HL_CELLS = HLX * HLY * HLZ;
+constexpr int TILE_THREADS = TL_CELLS;  // a thread per cell
+
+template <class Real> struct alignas(8 * sizeof(Real)) DepRec {
+  Real w[3], key, j[3], pad;  // offsets in the cell; cell of the tile (a small integer); a v
+};
+
+// A record is written and read by whole 32-byte sectors.
+__device__ __forceinline__ void put_rec(DepRec<float> *p, const DepRec<float> &r) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "f"(r.w[0]), "f"(r.w[1]),
+               "f"(r.w[2]), "f"(r.key), "f"(r.j[0]), "f"(r.j[1]), "f"(r.j[2]), "f"(r.pad)
+               : "memory");
+}
+__device__ __forceinline__ void put_rec(DepRec<double> *p, const DepRec<double> &r) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "d"(r.w[0]), "d"(r.w[1]), "d"(r.w[2]),
+               "d"(r.key)
+               : "memory");
+  asm volatile("st.global.v4.f64 [%0 + 32], {%1, %2, %3, %4};\n" ::"l"(p), "d"(r.j[0]), "d"(r.j[1]), "d"(r.j[2]),
+               "d"(r.pad)
+               : "memory");
+}
+__device__ __forceinline__ DepRec<float> get_rec(const DepRec<float> *p) {
+  DepRec<float> r;
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+               : "=f"(r.w[0]), "=f"(r.w[1]), "=f"(r.w[2]), "=f"(r.key), "=f"(r.j[0]), "=f"(r.j[1]), "=f"(r.j[2]),
+                 "=f"(r.pad)
+               : "l"(p));
+  return r;
+}
+__device__ __forceinline__ DepRec<double> get_rec(const DepRec<double> *p) {
+  DepRec<double> r;
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];\n"
+               : "=d"(r.w[0]), "=d"(r.w[1]), "=d"(r.w[2]), "=d"(r.key)
+               : "l"(p));
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4 + 32];\n"
+               : "=d"(r.j[0]), "=d"(r.j[1]), "=d"(r.j[2]), "=d"(r.pad)
+               : "l"(p));
+  return r;
+}
+
+// Periodic cell index of an integral reduced coordinate.
+template <class Real> __device__ __forceinline__ uint32_t dep_wrap(Real f, int n) {
+  if (f >= (Real)0 && f < (Real)n) return (uint32_t)f;
+  int64_t i = (int64_t)f % n;
+  return (uint32_t)(i < 0 ? i + n : i);
+}
+
+// Tile of a particle, its cell in the tile and its offsets in the cell.
+template <class Real>
+__device__ __forceinline__ uint32_t dep_tile(const DepArgs<Real> &A, const TileArgs &T,
+                                             const DepPoint<Real> &d, Real w[3], uint32_t &cell) {
+  const Real ix = floor(d.f[0]), iy = floor(d.f[1]), iz = floor(d.f[2]);
+  w[0] = d.f[0] - ix; w[1] = d.f[1] - iy; w[2] = d.f[2] - iz;
+  const uint32_t i = dep_wrap(ix, A.nx), j = dep_wrap(iy, A.ny), k = dep_wrap(iz, A.nz);
+  cell = ((k % TLZ) * TLY + j % TLY) * TLX + i % TLX;
+  return ((k / TLZ) * T.nty + j / TLY) * T.ntx + i / TLX;
+}
+
+constexpr uint32_t NO_TILE = 0xFFFFFFFFu;
+
+// Particles per tile (in T.end), one atomic per distinct tile of a warp: the
+// atomics of particles stored by cell would otherwise queue up on the counters
+// of a few tiles.
+template <class Real>
+__global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<Real> A, TileArgs T) {
+  const int64_t n = dep_count(A);
+  if (n < T.min_n || n > T.max_n) return;
+  const int lane = threadIdx.x & 31;
+  const uint32_t way = blockIdx.x & (T.ways - 1);
+  unsigned bad = 0;
+  // warp-uniform loop
+  for (int64_t b = (int64_t)blockIdx.x * DEPOSIT_THREADS + (threadIdx.x & ~31); b < n;
+       b += (int64_t)gridDim.x * DEPOSIT_THREADS) {
+    const int64_t p = b + lane;
+    uint32_t t = NO_TILE;
+    DepPoint<Real> d;
+    if (p < n) {
+      if (dep_point(A, p, d)) {
+        Real w[3];
+        uint32_t cell;
+        t = dep_tile(A, T, d, w, cell) * T.ways + way;
+      } else {
+        bad = 1;
+      }
+    }
+    const unsigned same = __match_any_sync(0xFFFFFFFFu, t);
+    if (t != NO_TILE && lane == __ffs(same) - 1) atomicAdd(&T.seg[t].end, (uint32_t)__popc(same));
+  }
+  if (bad) atomicOr(&A.cnt->status, (unsigned)QED_STATUS_NONFINITE);
+}
+
+// Record segments: any order of the tiles does, so a CTA takes room for its
+// segments with one atomic (the parts of a tile stay next to each other: ways
+// divides ALLOC_THREADS).
+constexpr int ALLOC_THREADS = 256;
+__global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(TileArgs T) {
+  __shared__ uint32_t sm[33];
+  __shared__ uint32_t s_base;
+  const uint32_t t = blockIdx.x * ALLOC_THREADS + threadIdx.x, nseg = T.ntiles * T.ways;
+  const uint32_t c = t < nseg ? T.seg[t].end : 0u;
+  const uint32_t ex = block_excl_scan(c, sm);
+  if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(T.total, sm[32]) : 0u;
+  __syncthreads();
+  if (t < nseg) {
+    T.seg[t].start = T.seg[t].cursor = s_base + ex;
+    T.seg[t].end = s_base + ex + c;
+  }
+}
+
+template <class Real>
+__global__ void __launch_bounds__(DEPOSIT_THREADS, sizeof(Real) == 4 ? 4 : 2)
+k_dep_scatter(DepArgs<Real> A, TileArgs T, DepRec<Real> *rec) {
+  const int64_t n = dep_count(A);
+  if (n < T.min_n || n > T.max_n) return;
+  const int lane = threadIdx.x & 31;
+  const uint32_t way = blockIdx.x & (T.ways - 1);  // the same CTA as in k_dep_count (equal grids)
+  for (int64_t b = (int64_t)blockIdx.x * DEPOSIT_THREADS + (threadIdx.x & ~31); b < n;
+       b += (int64_t)gridDim.x * DEPOSIT_THREADS) {
+    const int64_t p = b + lane;
+    uint32_t t = NO_TILE;
+    DepRec<Real> r;
+    bool direct = false;
+    if (p < n) {
+      const Real a = A.scale * A.w[p];
+      DepPoint<Real> d;
+      if (dep_point(A, p, d)) {
+        uint32_t cell;
+        t = dep_tile(A, T, d, r.w, cell) * T.ways + way;
+        r.key = (Real)cell;
+        r.pad = (Real)0;
+        direct = !isfinite(a);  // reaches its own eight nodes per component and no others
+#pragma unroll
+        for (int c = 0; c < 3; ++c) r.j[c] = direct ? (Real)0 : d.j[c] * a;
+      }
+    }
+    const unsigned same = __match_any_sync(0xFFFFFFFFu, t);
+    const int leader = __ffs(same) - 1;
+    uint32_t pos = 0;
+    if (t != NO_TILE && lane == leader) pos = atomicAdd(&T.seg[t].cursor, (uint32_t)__popc(same));
+    pos = __shfl_sync(0xFFFFFFFFu, pos, leader) + __popc(same & ((1u << lane) - 1u));
+    if (t != NO_TILE) {
+      if (pos < T.rec_cap) put_rec(rec + pos, r);
+      else direct = true;  // no room for its record
+    }
+    if (direct) {
+      const Real a = A.scale * A.w[p];
+      DepPoint<Real> d;
+      dep_point(A, p, d);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d.j[c] *= a;
+      dep_direct(A, d);
+    }
+  }
+}
+
+// weights at the half-integer positions cell - 1/2, + 1/2, + 3/2
+template <class Real> __device__ __forceinline__ void dep_half(Real w, Real s[3]) {
+  const bool lo = w < (Real)0.5;
+  const Real u = lo ? w + (Real)0.5 : w - (Real)0.5;
+  s[0] = lo ? (Real)1 - u : (Real)0;
+  s[1] = lo ? u : (Real)1 - u;
+  s[2] = lo ? (Real)0 : u;
+}
+
+// particles of a tile ordered by cell at a time (a warp's threads do as many
+// turns as its fullest cell, so the more at a time the better they are used)
+constexpr int DEP_BATCH = 2048;
+
+template <class Real>
+__global__ void __launch_bounds__(TILE_THREADS, sizeof(Real) == 4 ? 4 : 2)
+k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
+  constexpr int BATCH = DEP_BATCH, PER = BATCH / TILE_THREADS;
+  __shared__ uint16_t s_perm[BATCH];  // the batch's records by cell
+  __shared__ uint32_t s_cnt[TL_CELLS];
+  __shared__ uint32_t sm[33];
+  __shared__ float s_J[3][HL_CELLS];
+  __shared__ int64_t s_row[HLY * HLZ];  // first element of J's row of each halo row
+  const int64_t n = dep_count(A);
+  if (n < T.min_n || n > T.max_n) return;
+  const int c = threadIdx.x;
+  for (uint32_t t = blockIdx.x; t < T.ntiles; t += gridDim.x) {
+    const uint32_t beg = T.seg[t * T.ways].start;
+    uint32_t end = T.seg[t * T.ways + T.ways - 1].end;
+    if (end > T.rec_cap) end = T.rec_cap;
+    if (beg >= end) continue;
+    const int x0 = (int)(t % T.ntx * TLX) - 1;
+    if (c < HLY * HLZ) {
+      int y = ((int)(t / T.ntx % T.nty * TLY) - 1 + c % HLY) % A.ny;
+      int z = ((int)(t / (T.ntx * T.nty) * TLZ) - 1 + c / HLY) % A.nz;
+      if (y < 0) y += A.ny;
+      if (z < 0) z += A.nz;
+      s_row[c] = ((int64_t)z * A.ny + y) * A.nx;
+    }
+    Real jx[2][2][3], jy[2][3][2], jz[3][2][2];  // [z][y][x] around the cell
+#pragma unroll
+    for (int q = 0; q < 12; ++q) (&jx[0][0][0])[q] = (&jy[0][0][0])[q] = (&jz[0][0][0])[q] = (Real)0;
+    for (uint32_t b = beg; b < end; b += BATCH) {
+      const uint32_t m = end - b < BATCH ? end - b : BATCH;
+      s_cnt[c] = 0;
+      __syncthreads();
+      // a record's rank among its cell's, then its place in cell order
+      uint32_t place[PER];  // cell | rank << 8
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        if (q * TILE_THREADS >= m) break;
+        const uint32_t i = q * TILE_THREADS + threadIdx.x;
+        if (i < m) {
+          const uint32_t cell = (uint32_t)rec[b + i].key & (TL_CELLS - 1);
+          place[q] = cell | atomicAdd(&s_cnt[cell], 1u) << 8;
+        }
+      }
+      __syncthreads();
+      const uint32_t mine = s_cnt[c];
+      const uint32_t first = block_excl_scan(mine, sm);
+      s_cnt[c] = first;
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        if (q * TILE_THREADS >= m) break;
+        const uint32_t i = q * TILE_THREADS + threadIdx.x;
+        if (i < m) s_perm[s_cnt[place[q] & (TL_CELLS - 1)] + (place[q] >> 8)] = (uint16_t)i;
+      }
+      __syncthreads();
+      for (uint32_t i = first; i < first + mine; ++i) {
+        const DepRec<Real> r = get_rec(rec + b + s_perm[i]);
+        const Real wx = r.w[0], wy = r.w[1], wz = r.w[2];
+        const Real X[2] = {(Real)1 - wx, wx}, Y[2] = {(Real)1 - wy, wy}, Z[2] = {(Real)1 - wz, wz};
+        const Real ax = r.j[0], ay = r.j[1], az = r.j[2];
+        Real h[3];
+        dep_half(wx, h);
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+          for (int y = 0; y < 2; ++y) {
+            const Real f = ax * Y[y] * Z[z];
+#pragma unroll
+            for (int x = 0; x < 3; ++x) jx[z][y][x] += f * h[x];
+          }
+        dep_half(wy, h);
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const Real f = ay * X[x] * Z[z];
+#pragma unroll
+            for (int y = 0; y < 3; ++y) jy[z][y][x] += f * h[y];
+          }
+        dep_half(wz, h);
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const Real f = az * X[x] * Y[y];
+#pragma unroll
+            for (int z = 0; z < 3; ++z) jz[z][y][x] += f * h[z];
+          }
+      }
+      __syncthreads();
+    }
+    // the cells' sums into the halo tile.  Along x (8 consecutive lanes) by
+    // shuffles: a lane keeps what lies on its own column, the row's first and
+    // last lane also the columns beside the tile; then in rounds in which every
+    // thread adds at the same offset from its own cell, so that no two add to
+    // one place
+    for (int q = threadIdx.x; q < 3 * HL_CELLS; q += TILE_THREADS) (&s_J[0][0])[q] = 0.f;
+    const int lx = c % TLX, ly = c / TLX % TLY, lz = c / (TLX * TLY);
+    const bool first_x = lx == 0, last_x = lx == TLX - 1;
+    const int h0 = ((lz + 1) * HLY + ly + 1) * HLX + lx + 1;
+    auto up = [&](Real v) { const float r = __shfl_up_sync(0xFFFFFFFFu, (float)v, 1, TLX); return first_x ? 0.f : r; };
+    auto down = [&](Real v) { const float r = __shfl_down_sync(0xFFFFFFFFu, (float)v, 1, TLX); return last_x ? 0.f : r; };
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        __syncthreads();
+        if (s < 2) {
+          const int h = h0 + (u * HLY + s) * HLX;
+          const float v = (float)jx[u][s][1] + up(jx[u][s][2]) + down(jx[u][s][0]);
+          s_J[0][h] += v;
+          if (first_x) s_J[0][h - 1] += (float)jx[u][s][0];
+          if (last_x) s_J[0][h + 1] += (float)jx[u][s][2];
+        }
+        const int hy = h0 + (u * HLY + s - 1) * HLX, hz = h0 + ((s - 1) * HLY + u) * HLX;
+        const float vy = (float)jy[u][s][0] + up(jy[u][s][1]), vz = (float)jz[s][u][0] + up(jz[s][u][1]);
+        s_J[1][hy] += vy;
+        s_J[2][hz] += vz;
+        if (last_x) {
+          s_J[1][hy + 1] += (float)jy[u][s][1];
+          s_J[2][hz + 1] += (float)jz[s][u][1];
+        }
+      }
+    __syncthreads();
+    // to J: 16 lanes per halo row, 10 of them with a column
+    const int hx = threadIdx.x & 15;
+    int x = x0 + hx;
+    if (x < 0 || x >= A.nx) {
+      x %= A.nx;
+      if (x < 0) x += A.nx;
+    }
+    if (hx < HLX)
+      for (int r = threadIdx.x >> 4; r < 3 * HLY * HLZ; r += TILE_THREADS / 16) {
+        const float v = (&s_J[0][0])[r * HLX + hx];
+        if (v == 0.f) continue;
+        const int comp = r / (HLY * HLZ);
+        atomicAdd((comp == 0 ? A.jx : comp == 1 ? A.jy : A.jz) + s_row[r - comp * (HLY * HLZ)] + x, v);
+      }
+    __syncthreads();  // the shared arrays are the next tile's
+  }
 }
 
 bool yee_ok(const qed_yee *y) {
@@ -256,6 +633,57 @@ cudaError_t launch_fields(qed_ctx *c, const qed_yee *y, bool advance, cudaStream
   return cudaGetLastError();
 }
 
+// Persistent grid over `capacity` particles: no more CTAs than they need.
+template <class Kern>
+cudaError_t particle_grid(const qed_ctx *c, Kern kern, int64_t capacity, unsigned *blocks) {
+  int per_sm = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DEPOSIT_THREADS, 0);
+  if (e != cudaSuccess) return e;
+  const int64_t need = (capacity + DEPOSIT_THREADS - 1) / DEPOSIT_THREADS;
+  int64_t b = (int64_t)c->num_sms * (per_sm < 1 ? 1 : per_sm);
+  if (need < b) b = need;
+  *blocks = (unsigned)(b < 1 ? 1 : b);
+  return cudaSuccess;
+}
+
+// When the tiled path is taken.  The rule is on the number of particles on the
+// device; the host sees only capacities, so where the capacity allows the
+// tiled path both are launched and the kernels of the other return at once.
+// Measured, tiled / direct in us (stored by cell; random order):
+//   64^3 cells:  2^18 particles 28/22; 32/23    2^20 47/93; 65/83    2^23 372/941; 424/672
+//   128^3:       2^20 109/68; 117/79            2^22 213/297; 243/322
+//   180^3:       2^22 355/282; 384/331          2^23 484/539; 551/654
+//   81 x 39 x 167: 2^19 (one a cell), random 70/42
+// so two particles per cell and 2^18 pay for a tile's fixed work; where J (12
+// bytes a cell) no longer fits L2 half of one, as each direct deposit of a
+// random order then fetches its lines (256^3, 2^24 random: 1340/5000).  Few
+// tiles leave the chip idle (16^3, 2^18: 188/78) and a very full cell is one
+// thread's work (32^3 by cell: 128 a cell 739/696, 256 a cell 2057/1435).
+constexpr int64_t TILED_MIN_PARTICLES = 1 << 18, TILED_MIN_TILES = 128, TILED_MAX_PER_CELL = 64;
+constexpr int64_t L2_CELLS = 6 << 20;
+
+// The scratch is the step's: records in the staging area, segments in the
+// per-entry counts (both are free between steps, and calls that share a
+// context are ordered).
+template <class Real>
+cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<Real> &A, const TileArgs &T, cudaStream_t st) {
+  DepRec<Real> *rec = static_cast<DepRec<Real> *>(c->stage);
+  const uint32_t nseg = T.ntiles * T.ways;
+  unsigned count_blocks = 0, blocks = 0;
+  cudaError_t e = cudaMemsetAsync(T.seg, 0, sizeof(TileSeg) * ((size_t)nseg + 1), st);
+  if (e == cudaSuccess) e = particle_grid(c, k_dep_count<Real>, A.cap, &count_blocks);
+  if (e == cudaSuccess) e = particle_grid(c, k_dep_scatter<Real>, A.cap, &blocks);
+  if (e != cudaSuccess) return e;
+  if (count_blocks < blocks || T.ways > 1) blocks = count_blocks = count_blocks < blocks ? count_blocks : blocks;
+  k_dep_count<Real><<<count_blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
+  k_dep_alloc<<<(nseg + ALLOC_THREADS - 1) / ALLOC_THREADS, ALLOC_THREADS, 0, st>>>(T);
+  k_dep_scatter<Real><<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T, rec);
+  const uint32_t most = (uint32_t)c->num_sms * 32;
+  k_dep_tile<Real><<<T.ntiles < most ? T.ntiles : most, TILE_THREADS, 0, st>>>(A, T, rec);
+  c->launches += 4;
+  return cudaGetLastError();
+}
+
 template <class Real>
 cudaError_t launch_deposit(qed_ctx *c, const qed_species *s, const qed_yee *y, double weight_unit,
                            const int64_t *d_lim, cudaStream_t st) {
@@ -272,17 +700,32 @@ cudaError_t launch_deposit(qed_ctx *c, const qed_species *s, const qed_yee *y, d
   A.scale = (Real)((double)s->q * weight_unit / (y->dx * y->dy * y->dz));
   A.half_dt = (Real)(0.5 * c->cfg.dt);
   A.cnt = c->d_counters;
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pic_deposit<Real>,
-                                                                DEPOSIT_THREADS, 0);
+  TileArgs T;
+  T.ntx = (y->nx + TLX - 1) / TLX;
+  T.nty = (y->ny + TLY - 1) / TLY;
+  const int64_t cells = (int64_t)y->nx * y->ny * y->nz;
+  const int64_t ntiles = (int64_t)T.ntx * T.nty * ((y->nz + TLZ - 1) / TLZ);
+  T.ways = 1;
+  while (ntiles * T.ways < 4096 && T.ways < 64) T.ways *= 2;
+  T.min_n = cells > L2_CELLS ? cells / 2 : 2 * cells;
+  if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
+  T.max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
+  unsigned blocks = 0;
+  cudaError_t e = particle_grid(c, k_pic_deposit<Real>, s->capacity, &blocks);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  // no more CTAs than the capacity needs
-  const int64_t need = (s->capacity + DEPOSIT_THREADS - 1) / DEPOSIT_THREADS;
-  int64_t blocks = (int64_t)c->num_sms * per_sm;
-  if (need < blocks) blocks = need;
-  if (blocks < 1) blocks = 1;
-  k_pic_deposit<Real><<<(unsigned)blocks, DEPOSIT_THREADS, 0, st>>>(A);
+  if (T.max_n >= T.min_n && s->capacity >= T.min_n && s->capacity <= 0x7fffffff &&
+      8 * (ntiles * T.ways + 1) <= c->heavy_slots) {
+    T.ntiles = (uint32_t)ntiles;
+    T.seg = reinterpret_cast<TileSeg *>(c->sub_cnt);
+    T.total = &T.seg[ntiles * T.ways].end;
+    const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
+    T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
+    e = launch_deposit_tiled(c, A, T, st);
+    if (e != cudaSuccess) return e;
+  } else {
+    T.max_n = 0;  // all numbers directly
+  }
+  k_pic_deposit<Real><<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
   c->launches += 1;
   return cudaGetLastError();
 }
