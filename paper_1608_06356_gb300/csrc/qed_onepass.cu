@@ -11,7 +11,8 @@
 // depends on the scheduling of the warps), so the photon buffer is the same
 // set in another order.
 //
-// How the work is laid out, per warp of a persistent grid:
+// How the work is laid out, per warp of a persistent grid (one CTA of OP_WARPS
+// warps per SM, which share the rate tables in shared memory):
 //   streaming: each lane takes one particle of a 32-particle slice (the next
 //     slice's words are in flight into shared memory, cp.async), pushes it and
 //     computes chi.  The rate bound W <= w_j chi / gamma (w_j = alpha a_S
@@ -20,24 +21,19 @@
 //     settles most particles without the 2-D tables: if w_j chi Dt / gamma <=
 //     0.2 the particle has one sub-step, and if its first draw r1 is not
 //     below that bound it has no event -- it is finished (its pushed state
-//     written).  The others go
-//     to the warp's queue in shared memory (pushed momentum, fields, id,
-//     slot).
-//   heavy phase: when the queue holds 32 particles (a scheduling parameter,
-//     as are the lane counts below), the warp runs them with
-//     a per-warp scheduler of lane states -- idle; rate (chi and the exact
-//     rate, and N for a new particle; idle lanes are refilled from the queue
-//     at the start of such a round); scanning (Method I draws, four per
-//     iteration from two independent Philox calls, up to 8 per round, the
-//     round ending early when fewer than 8 lanes are still drawing); or pending (an
-//     event; the emitting lanes run together: xi, the recoil, the photon;
-//     then the rate again for the remaining sub-steps).  An
-//     emission round reserves slots for its photons with one atomic on the
-//     photon count and writes them there.  A round runs only when enough
-//     lanes are in its state (16 for an emission, 12 otherwise); when none can,
-//     the warp goes back to streaming and the chains still running are parked
-//     in shared memory, to be resumed (with new entries) by the next heavy
-//     phase.  After the last slice the queue is drained.
+//     written).  The others enter the warp's pool.
+//   pool: PCAP chains in shared memory, each in one of three states: rate due
+//     (chi and the exact rate; a new particle also gets N), scanning (Method I
+//     draws due), or event pending (xi, the recoil, the photon).  A round
+//     takes up to 32 chains of one state -- any lane runs any chain -- and
+//     files each under its next state; a chain that ends frees its entry.  The
+//     warp streams while the pool has room for a slice, and then runs the
+//     fullest state, so a round nearly always has 27 to 32 lanes at work,
+//     where a lane that keeps its own chain in registers waits for its
+//     neighbours' states (14 to 23 lanes).  After the last slice the pool is
+//     drained.
+//   photons: an emission round reserves slots for its photons with one atomic
+//     on the photon count and writes them there.
 //   learned sampler: an event of a one-sub-step lepton inside the network's
 //     domain ends its chain with a 16-byte record instead of an emission; the
 //     dense pass k_net_emit (below) finishes those emissions, 32 per warp.
@@ -55,14 +51,19 @@ namespace qed {
 
 namespace {
 
-// CTAs of 4 warps: with the per-warp shared memory below, 5 fit on an SM
-constexpr int OP_THREADS = 128;
-constexpr int OP_WARPS = OP_THREADS / 32;
-constexpr int QCAP = 64;       // queue entries per warp
-constexpr int QEXIT = QCAP - 32;  // a heavy phase may end once the queue holds at most this many
-constexpr int QF = 9;          // queue floats per entry: px py pz ex ey ez bx by bz
-constexpr int PF = 17;         // parked floats per lane
-constexpr int PU = 9;          // parked words per lane
+// one CTA per SM: its warps share the tables, and its shared memory is full
+constexpr int OP_WARPS = 20;
+constexpr int OP_THREADS = OP_WARPS * 32;
+constexpr int PCAP = 96;  // chains per warp's pool
+// words of a pool entry: the slot, the id, the momentum of a new particle and
+// then the unit direction, gamma, chi, the event threshold W Dt / N, kappa_min,
+// N (0: new), the sub-step (top bit: it has emitted), the word r2 of the
+// event and, unless the field is uniform, E and B
+enum { W_SLOT, W_ID0, W_ID1, W_VX, W_VY, W_VZ, W_G, W_CHI, W_THR, W_KMIN, W_N, W_K, W_R2, W_FIELDS };
+constexpr uint32_t EMITTED = 0x80000000u;
+template <int FM> __host__ __device__ constexpr int pool_words() { return FM == FM_UNIFORM ? W_FIELDS : W_FIELDS + 6; }
+// the states of a chain, and the list of free entries
+enum { L_RATE = 0, L_SCAN = 1, L_PEND = 2, L_FREE = 3, LISTS = 4 };
 
 struct OnePassArgs {
   Sp<float> sp[2];
@@ -81,33 +82,17 @@ struct OnePassArgs {
   float4 *net_rec;           // records of the deferred network emissions
   unsigned long long *net_n; // their count
   int64_t net_cap;
-  // chain scheduling (QED_SCHED_*): an emission round waits for emit_lanes
-  // lanes with an event, a rate or scanning round runs with at least
-  // round_lanes lanes, a scanning round draws scan_iters times four
-  // sub-steps per lane and ends early when fewer than scan_left lanes are
-  // still drawing; a heavy phase starts when the queue holds qtrig entries
-  // (qtrig - 1 + 32 <= QCAP)
-  int emit_lanes, round_lanes, scan_iters, scan_left, qtrig;
 };
 
-// dynamic shared memory: prefetch buffers, per-warp queues and park areas.
-// The rate tables are read through L1: only the queued particles evaluate the
-// exact rate.
-template <int FM> __host__ __device__ size_t onepass_layout(const OnePassArgs &a, size_t off[4]) {
-  size_t o = 0;
-  off[0] = o;  // prefetch: two buffers of [NV][OP_THREADS] words and [OP_THREADS] ids
-  o += 2 * OP_THREADS * ((size_t)stream_words<FM>() * sizeof(float) + sizeof(uint64_t));
-  off[1] = o;  // queues: slot [QCAP], floats [QF][QCAP], ids [QCAP] per warp
-  o += (size_t)OP_WARPS * QCAP * (4 + 4 * QF + 8);
-  off[2] = o;  // park: floats [PF][32], words [PU][32] per warp
-  o += (size_t)OP_WARPS * 32 * 4 * (PF + PU);
-  o = (o + 15) & ~(size_t)15;
-  off[3] = o;
-  return o;
+// Dynamic shared memory: per warp the prefetch words and ids of a slice, the
+// pool and its lists; then the rate and forward tables (TAB; tables that do not
+// fit are read through L1).
+template <int FM> __host__ __device__ constexpr size_t warp_smem() {
+  return 32 * ((size_t)stream_words<FM>() * 4 + 8) + (size_t)PCAP * (4 * pool_words<FM>() + LISTS);
 }
-
-// lane states of a chain
-enum { ST_IDLE = 0, ST_RATE = 1, ST_SCAN = 2, ST_PEND = 3, ST_DONE = 4 };
+template <int FM> size_t onepass_smem(const qed_ctx *c, bool tab) {
+  return OP_WARPS * warp_smem<FM>() + (tab ? sizeof(float) * (size_t)c->gl.n * (1 + c->gy.n) : 0);
+}
 
 // Learned-sampler emissions deferred to the dense pass: one record per
 // emission, 16 bytes -- the lepton's index (species in the top bit) and kappa
@@ -144,36 +129,36 @@ __device__ __forceinline__ int64_t substep_count_op(const Consts &C, float W, fl
   return (int64_t)nn;
 }
 
-// DEF: the default chain scheduling as compile-time constants (the runtime
-// values cost ~3.5% of the kernel's time); otherwise the values in A.
-template <int FM, int MODE, bool MLP, bool DEF>
-__global__ void __launch_bounds__(OP_THREADS, 5) k_lepton_onepass(OnePassArgs A) {
-  const int emit_lanes = DEF ? SCHED_DEF_EMIT_LANES : A.emit_lanes;
-  const int round_lanes = DEF ? SCHED_DEF_ROUND_LANES : A.round_lanes;
-  const int scan_iters = DEF ? (SCHED_DEF_SCAN_DRAWS + 3) / 4 : A.scan_iters;
-  const int scan_left = DEF ? SCHED_DEF_SCAN_LEFT : A.scan_left;
-  const int qtrig = DEF ? SCHED_DEF_QUEUE_TRIGGER : A.qtrig;
+// Method I on the sub-steps that a draw serves (2j and 2j + 1; a chain may
+// enter at the odd one): the next state, L_FREE at the end of the chain.
+__device__ __forceinline__ int draw_two(const U4 &r, float thr, int N, int &k, uint32_t &r2) {
+  if (!(k & 1)) {
+    if (thr > unif<float>(r.x)) { r2 = r.y; return L_PEND; }
+    if (++k >= N) return L_FREE;
+  }
+  if (thr > unif<float>(r.z)) { r2 = r.w; return L_PEND; }
+  return ++k >= N ? L_FREE : L_SCAN;
+}
+
+template <int FM, int MODE, bool MLP, bool TAB>
+__global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint32_t s_hist[64];
   __shared__ BlockTally bt;
   __shared__ long long s_meta[4];
   __shared__ unsigned long long s_deferred;
   constexpr int NV = stream_words<FM>();
-  const int64_t step_ = A.d_step ? *A.d_step : A.step;
-  size_t off[4];
-  onepass_layout<FM>(A, off);
-  const float *sR = A.T.R, *sF = A.T.F;
-  float *pf = reinterpret_cast<float *>(smem_raw + off[0]);
-  uint64_t *pf_id = reinterpret_cast<uint64_t *>(pf + 2 * NV * OP_THREADS);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;  // wid < OP_WARPS
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
-  unsigned char *qbase = smem_raw + off[1] + (size_t)wid * QCAP * (4 + 4 * QF + 8);
-  uint32_t *q_slot = reinterpret_cast<uint32_t *>(qbase);
-  float *q_f = reinterpret_cast<float *>(qbase + 4 * QCAP);
-  uint64_t *q_id = reinterpret_cast<uint64_t *>(qbase + 4 * QCAP + 4 * QF * QCAP);
-  unsigned char *pbase = smem_raw + off[2] + (size_t)wid * 32 * 4 * (PF + PU);
-  float *pk_f = reinterpret_cast<float *>(pbase);
-  uint32_t *pk_u = reinterpret_cast<uint32_t *>(pbase + 4 * PF * 32);
+  unsigned char *const mine = smem_raw + (size_t)wid * warp_smem<FM>();
+  uint64_t *const pf_id = reinterpret_cast<uint64_t *>(mine);                 // [32]
+  float *const pf = reinterpret_cast<float *>(mine + 256);                    // [NV][32]
+  uint32_t *const pool = reinterpret_cast<uint32_t *>(pf + NV * 32);          // [words][PCAP]
+  uint8_t *const list = reinterpret_cast<uint8_t *>(pool + pool_words<FM>() * PCAP);  // [LISTS][PCAP]
+  float *const tab = reinterpret_cast<float *>(smem_raw + OP_WARPS * warp_smem<FM>());
+  const float *const sR = TAB ? tab : A.T.R, *const sF = TAB ? tab + A.T.gl.n : A.T.F;
   block_tally_init(&bt);
+  if (threadIdx.x < 64) s_hist[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     s_meta[0] = *(volatile int64_t *)A.sp[0].d_n;
     s_meta[1] = A.nsp > 1 ? *(volatile int64_t *)A.sp[1].d_n : 0;
@@ -181,314 +166,110 @@ __global__ void __launch_bounds__(OP_THREADS, 5) k_lepton_onepass(OnePassArgs A)
     s_deferred = 0;
   }
   __syncthreads();
+  const int64_t step_ = A.d_step ? *A.d_step : A.step;
   const int64_t n0 = s_meta[0], n1 = s_meta[1];
   const uint32_t epoch = (uint32_t)s_meta[2];
   const int64_t T0 = (n0 + TILE - 1) / TILE, T1 = (n1 + TILE - 1) / TILE;
   const int64_t nslots = (T0 + T1) * TILE;
+  // consecutive slices go to different SMs
+  const int64_t stride = (int64_t)gridDim.x * OP_THREADS;
+  int64_t slot = ((int64_t)wid * gridDim.x + blockIdx.x) * 32 + lane;
+  if (TAB && (int64_t)blockIdx.x * 32 < nslots) {  // (a CTA without a slice needs no tables)
+    load_tables_smem(tab, A.T.R, A.T.gl.n);
+    load_tables_smem(tab + A.T.gl.n, A.T.F, A.T.gl.n * A.T.gy.n);
+  }
+  __syncthreads();
   const float inv_aS = A.C.f_inv_aS, dt = A.C.f_dt, wdt_max = A.C.f_wdt_max;
   Tally tl;
   tl.clear();
-  uint32_t deferred = 0;  // heavy particles taken by this lane
-  int qn = 0;             // queue length (warp-uniform)
-  unsigned parked = 0;    // lanes with a parked chain (warp-uniform)
+  uint32_t deferred = 0;  // new particles taken by this lane
 
   auto slot_index = [&](int64_t sl, int &si, int64_t &i) {
     const int64_t tile = sl / TILE;
     si = tile < T0 ? 0 : 1;
     i = (tile - (si ? T0 : 0)) * TILE + (sl % TILE);
   };
-
-  // ---- heavy phase: the queued particles' Method I chains ---------------
-  // Lane states: idle; rate (chi and the exact rate due: a new particle or a
-  // recoiled one); scan (drawing sub-steps); pend (an event, emission due).
-  auto heavy_phase = [&](bool final_drain) {
-    int st = ST_IDLE;
-    uint32_t hslot = 0, wy = 0, cnt = 0;
-    int N = 1, k = 0;
-    float px = 0.f, py = 0.f, pz = 1.f, g = 1.f, chi = 0.f, dts = 0.f, nx = 0.f, ny = 0.f, nz = 0.f;
-    float E[3] = {0.f, 0.f, 0.f}, B[3] = {0.f, 0.f, 0.f};
-    RateOut<float> ro{0.f, -1e30f, 0.f};
-    uint64_t pid = 0;
-    if (parked & (1u << lane)) {  // resume a parked chain
-      px = pk_f[0 * 32 + lane]; py = pk_f[1 * 32 + lane]; pz = pk_f[2 * 32 + lane];
-      g = pk_f[3 * 32 + lane]; chi = pk_f[4 * 32 + lane]; dts = pk_f[5 * 32 + lane];
-      ro.W = pk_f[6 * 32 + lane]; ro.kmin = pk_f[7 * 32 + lane]; ro.l = pk_f[8 * 32 + lane];
+  // ---- the pool's lists: entries of a state in any order (lengths warp-uniform)
+  int len[LISTS] = {0, 0, 0, PCAP};
+  for (int q = lane; q < PCAP; q += 32) list[L_FREE * PCAP + q] = (uint8_t)q;
+  __syncwarp();
+  auto word = [&](int w, int e) -> uint32_t & { return pool[w * PCAP + e]; };
+  auto real = [&](int w, int e) -> float & { return reinterpret_cast<float *>(pool)[w * PCAP + e]; };
+  // file entry e of each lane with state st (-1: none)
+  auto file = [&](int st, int e) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        E[c] = pk_f[(9 + c) * 32 + lane];
-        B[c] = pk_f[(12 + c) * 32 + lane];
-      }
-      st = (int)pk_u[0 * 32 + lane];
-      hslot = pk_u[1 * 32 + lane];
-      N = (int)pk_u[2 * 32 + lane];
-      k = (int)pk_u[3 * 32 + lane];
-      wy = pk_u[4 * 32 + lane];
-      cnt = pk_u[5 * 32 + lane];
-      pid = (uint64_t)pk_u[6 * 32 + lane] | ((uint64_t)pk_u[7 * 32 + lane] << 32);
-      nx = pk_f[15 * 32 + lane]; ny = pk_f[16 * 32 + lane];
-      nz = __uint_as_float(pk_u[8 * 32 + lane]);
-    }
-    parked = 0;
-    for (;;) {
-      const unsigned idle = __ballot_sync(0xFFFFFFFFu, st == ST_IDLE);
-      const unsigned rate = __ballot_sync(0xFFFFFFFFu, st == ST_RATE);
-      const unsigned scan = __ballot_sync(0xFFFFFFFFu, st == ST_SCAN);
-      const unsigned pend = __ballot_sync(0xFFFFFFFFu, st == ST_PEND);
-      const int ni = __popc(idle), nr = __popc(rate), ns = __popc(scan), np = __popc(pend);
-      // idle lanes are refilled from the queue at the start of a rate round
-      const int take = min(qn, ni);
-      // a round runs only with enough lanes in its state; otherwise the warp
-      // goes back to streaming (once the queue has room for another slice)
-      // and the chains wait, parked, for the next heavy phase -- except in
-      // the final drain, which runs whatever is left
-      int phase;
-      if (np >= emit_lanes) phase = ST_PEND;
-      else if (nr + take >= round_lanes) phase = ST_RATE;
-      else if (ns >= round_lanes) phase = ST_SCAN;
-      else if (!final_drain && qn <= QEXIT) break;
-      else if (nr + take) phase = ST_RATE;
-      else if (ns) phase = ST_SCAN;
-      else if (np) phase = ST_PEND;
-      else break;
-      if (phase == ST_RATE) {
-        // refill: idle lanes take queue entries from the top, in lane order
-        if (st == ST_IDLE) {
-          const int r = __popc(idle & lt_mask);
-          if (r < take) {
-            const int q = qn - 1 - r;
-            hslot = q_slot[q];
-            px = q_f[0 * QCAP + q]; py = q_f[1 * QCAP + q]; pz = q_f[2 * QCAP + q];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              E[c] = q_f[(3 + c) * QCAP + q];
-              B[c] = q_f[(6 + c) * QCAP + q];
-            }
-            pid = q_id[q];
-            gamma_dir(px, py, pz, g, nx, ny, nz);
-            k = 0;
-            cnt = 0;
-            st = ST_RATE;
-          }
-        }
-        qn -= take;
-        // chi (Eq. 2) and the exact rate; a new particle also gets N
-        if (st == ST_RATE) {
-          chi = chi_lepton(px, py, pz, g, E[0], E[1], E[2], B[0], B[1], B[2], inv_aS);
-          ro = photon_rate(sR, sF, A.T, A.C, chi, g, tl);
-          if (k == 0 && cnt == 0) {
-            N = (int)substep_count_op(A.C, ro.W, dt, wdt_max, tl.status);
-            tl.substeps += N;
-            dts = dt / (float)N;
-            deferred += 1;
-          }
-          st = ST_SCAN;
-        }
-      } else if (phase == ST_SCAN) {
-        // draws two sub-steps at a time (independent Philox chains run
-        // interleaved; the second is used only if the first has no event),
-        // for as long as enough lanes are still drawing: the others keep
-        // their state for a later round
-        const float thr = ro.W * dts;
-        const bool was_scan = st == ST_SCAN;
-        bool drawing = was_scan;
-        for (int it = 0; it < scan_iters; ++it) {
-          if (drawing) {
-            // sub-steps 2j .. 2j+3 from the draws j and j+1 (words 0-1 and
-            // 2-3 of each); a chain at an odd sub-step starts at 2j+1
-            const int64_t j = k >> 1;
-            const U4 ra = draw(A.C, pid, step_, j, STREAM_EMIT);
-            const U4 rb = draw(A.C, pid, step_, j + 1, STREAM_EMIT);
-            const uint32_t w1[4] = {ra.x, ra.z, rb.x, rb.z}, w2[4] = {ra.y, ra.w, rb.y, rb.w};
-            const int q0 = (int)(k & 1);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              if (q >= q0 && st == ST_SCAN) {
-                if (thr > unif<float>(w1[q])) { wy = w2[q]; st = ST_PEND; }
-                else if (++k >= N) { st = ST_DONE; }
-              }
-            }
-            drawing = st == ST_SCAN;
-          }
-          if (__popc(__ballot_sync(0xFFFFFFFFu, drawing)) < scan_left) break;
-        }
-        if (MLP) {
-          // an event of a one-sub-step particle inside the network's domain
-          // takes its xi from the learned sampler, in the dense pass that
-          // follows this kernel: a record here (one per such particle: at
-          // most n0 + n1, which the records hold), no photon yet (cnt = 0)
-          bool net = false;
-          float kap = 0.f;
-          if (was_scan && st == ST_PEND && N == 1) {
-            kap = photon_kappa(ro.kmin, unif<float>(wy), unif<float>(~wy));
-            const float lchi = chi > 0.f ? logf(chi) : MLP_L_LO - 1.f;
-            net = lchi >= MLP_L_LO && lchi <= MLP_L_HI && kap >= MLP_K_LO && kap <= MLP_K_HI;
-          }
-          const unsigned nm = __ballot_sync(0xFFFFFFFFu, net);
-          if (nm) {
-            const int leader = __ffs(nm) - 1;
-            unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(A.net_n, (unsigned long long)__popc(nm));
-            base = __shfl_sync(0xFFFFFFFFu, base, leader);
-            if (net) {
-              constexpr int RS = net_stride<FM>();
-              const unsigned long long r = base + __popc(nm & lt_mask);
-              if (r < (unsigned long long)(A.net_cap / RS)) {
-                int si;
-                int64_t i;
-                slot_index(hslot, si, i);
-                float4 *R = A.net_rec + RS * r;
-                R[0] = make_float4(__uint_as_float((uint32_t)i),
-                                   __uint_as_float((uint32_t)((uint64_t)i >> 32) | ((uint32_t)si << 31)),
-                                   kap, E[0]);
-                if (FM == FM_GRID) {
-                  R[1] = make_float4(E[1], E[2], B[0], B[1]);
-                  R[2] = make_float4(B[2], 0.f, 0.f, 0.f);
-                }
-              } else {  // only with counts beyond the species' capacities
-                tl.dropped += 1;
-                tl.status |= QED_STATUS_CAPACITY;
-              }
-              st = ST_DONE;
-            }
-          }
-        }
-      } else {
-        // emission by every lane with an event: kappa and ln delta from the
-        // inverse table (Eq. 7), xi, the recoil and the photon
-        const bool ev = st == ST_PEND;
-        const float kap = ev ? photon_kappa(ro.kmin, unif<float>(wy), unif<float>(~wy)) : 0.f;
-        float eph = 0.f, g2 = g;
-        if (ev) {
-          const float Y = photon_lndelta_table(A.T.Y, A.T, ro.l, kap, tl);
-          const XiOut<float> xo = xi_from_lndelta(chi, Y);
-          g2 = g * xo.omxi;
-          eph = g * xo.xi;
-          if (g2 < 1.f) { g2 = 1.f; eph = g - 1.f; }
-          const int b = spec_bin(A.C, eph);
-          const unsigned em = __activemask();
-          const unsigned same = __match_any_sync(em, b);
-          if (b >= 0 && lane == __ffs(same) - 1) atomicAdd(&bt.hist[b], (unsigned long long)__popc(same));
-        }
-        // photon slots: one atomic per emission round
-        const unsigned em = __ballot_sync(0xFFFFFFFFu, ev);
-        const int leader = __ffs(em) - 1;
-        unsigned long long base = 0;
-        if (lane == leader)
-          base = atomicAdd(reinterpret_cast<unsigned long long *>(A.ph.d_n), (unsigned long long)__popc(em));
-        base = __shfl_sync(0xFFFFFFFFu, base, leader < 0 ? 0 : leader);
-        if (ev) {
-          const int64_t pos = (int64_t)base + __popc(em & lt_mask);
-          if (pos >= A.ph.cap) {
-            tl.dropped += 1;
-            tl.status |= QED_STATUS_CAPACITY;
-          } else {
-            int si;
-            int64_t i;
-            slot_index(hslot, si, i);
-            const Sp<float> &S = A.sp[si];
-            const U4 cid = draw(A.C, pid, step_, k, STREAM_PHOTON_ID);
-            write_child(A.ph, pos, S.x[i], S.y[i], S.z[i], eph * nx, eph * ny, eph * nz, S.w[i],
-                        (uint64_t)cid.x | ((uint64_t)cid.y << 32), E, B, S.tag ? S.tag[i] : 0u);
-          }
-          ++cnt;
-          const float pm2 = sqrtf((g2 - 1.f) * (g2 + 1.f));
-          px = pm2 * nx; py = pm2 * ny; pz = pm2 * nz;
-          g = g2;
-          // the rate for the remaining sub-steps, or the end of the chain
-          st = ++k >= N ? ST_DONE : ST_RATE;
-        }
-      }
-      // the end of a chain: the recoiled momentum of a particle that emitted
-      if (st == ST_DONE) {
-        if (cnt > 0) {
-          int si;
-          int64_t i;
-          slot_index(hslot, si, i);
-          const Sp<float> &S = A.sp[si];
-          const float pm = sqrtf((g - 1.f) * (g + 1.f));
-          S.px[i] = pm * nx; S.py[i] = pm * ny; S.pz[i] = pm * nz;
-        }
-        tl.events += cnt;
-        st = ST_IDLE;
-      }
-    }
-    // park the chains still running
-    parked = __ballot_sync(0xFFFFFFFFu, st != ST_IDLE);
-    if (st != ST_IDLE) {
-      pk_f[0 * 32 + lane] = px; pk_f[1 * 32 + lane] = py; pk_f[2 * 32 + lane] = pz;
-      pk_f[3 * 32 + lane] = g; pk_f[4 * 32 + lane] = chi; pk_f[5 * 32 + lane] = dts;
-      pk_f[6 * 32 + lane] = ro.W; pk_f[7 * 32 + lane] = ro.kmin; pk_f[8 * 32 + lane] = ro.l;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        pk_f[(9 + c) * 32 + lane] = E[c];
-        pk_f[(12 + c) * 32 + lane] = B[c];
-      }
-      pk_f[15 * 32 + lane] = nx;
-      pk_f[16 * 32 + lane] = ny;
-      pk_u[0 * 32 + lane] = (uint32_t)st;
-      pk_u[1 * 32 + lane] = hslot;
-      pk_u[2 * 32 + lane] = (uint32_t)N;
-      pk_u[3 * 32 + lane] = (uint32_t)k;
-      pk_u[4 * 32 + lane] = wy;
-      pk_u[5 * 32 + lane] = cnt;
-      pk_u[6 * 32 + lane] = (uint32_t)pid;
-      pk_u[7 * 32 + lane] = (uint32_t)(pid >> 32);
-      pk_u[8 * 32 + lane] = __float_as_uint(nz);
+    for (int s = 0; s < LISTS; ++s) {
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, st == s);
+      if (st == s) list[s * PCAP + len[s] + __popc(m & lt_mask)] = (uint8_t)e;
+      len[s] += __popc(m);
     }
     __syncwarp();
   };
-
-  // ---- streaming over all leptons, with the heavy phase in between -------
-  // Each lane copies its next particle's words into shared memory with
-  // asynchronous copies (cp.async) while the current one computes.  (One-
-  // dimensional bulk copies of a warp's 128-byte slice of each array, issued
-  // by one lane and completed on an mbarrier, measured slower: 3.98 against
-  // 3.25 ms per step at 64M electrons.)
-  const int t = threadIdx.x;
-  auto prefetch = [&](int64_t sl, int b) {
+  auto fields_of = [&](int e, float E[3], float B[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      E[c] = FM == FM_UNIFORM ? A.f.e[c] : real(W_FIELDS + c, e);
+      B[c] = FM == FM_UNIFORM ? A.f.b[c] : real(W_FIELDS + 3 + c, e);
+    }
+  };
+  // the end of a chain that has emitted: the recoiled momentum
+  auto store_recoil = [&](uint32_t sl, float g, float nx, float ny, float nz) {
     int si;
     int64_t i;
     slot_index(sl, si, i);
     const Sp<float> &S = A.sp[si];
-    if (i >= (si ? n1 : n0)) return;
-    float *d = pf + (size_t)b * NV * OP_THREADS + t;
-    const float *src[12] = {S.x, S.y, S.z, S.px, S.py, S.pz, S.ex, S.ey, S.ez, S.bx, S.by, S.bz};
-#pragma unroll
-    for (int c = 0; c < NV; ++c) cp_async<4>(d + c * OP_THREADS, src[c] + i);
-    cp_async<8>(pf_id + b * OP_THREADS + t, S.id + i);
+    const float pm = sqrtf((g - 1.f) * (g + 1.f));
+    S.px[i] = pm * nx; S.py[i] = pm * ny; S.pz[i] = pm * nz;
   };
-  const int64_t stride = (int64_t)gridDim.x * OP_THREADS;
-  int buf = 0;
-  int64_t slot = blockIdx.x * (int64_t)OP_THREADS + threadIdx.x;
-  if (slot < nslots) prefetch(slot, 0);
+
+  // Each lane copies its next particle's words into its own words of shared
+  // memory (cp.async), as soon as it has read the current ones from there.
+  auto prefetch = [&](int64_t sl) {
+    int si;
+    int64_t i;
+    slot_index(sl, si, i);
+    const Sp<float> &S = A.sp[si];
+    if (i < (si ? n1 : n0)) {
+      const float *src[12] = {S.x, S.y, S.z, S.px, S.py, S.pz, S.ex, S.ey, S.ez, S.bx, S.by, S.bz};
+#pragma unroll
+      for (int c = 0; c < NV; ++c) cp_async<4>(pf + c * 32 + lane, src[c] + i);
+      cp_async<8>(pf_id + lane, S.id + i);
+    }
+  };
+  if (slot < nslots) prefetch(slot);
   cp_async_commit();
-  // nslots is a multiple of OP_THREADS: every lane of a warp runs the same
-  // iterations; the one call of the heavy phase keeps its code once
+
   for (;;) {
+    // nslots is a multiple of 32: every lane of a warp sees the same
     const bool streaming = slot < nslots;
-    if (streaming) {
-      if (slot + stride < nslots) prefetch(slot + stride, buf ^ 1);
-      cp_async_commit();
-      cp_async_wait<1>();
+    // the fullest state (ties to the later one, which is nearer its end)
+    int phase = L_RATE, most = len[L_RATE];
+    if (len[L_SCAN] >= most) { phase = L_SCAN; most = len[L_SCAN]; }
+    if (len[L_PEND] >= most) { phase = L_PEND; most = len[L_PEND]; }
+    if (streaming && most < 32 && len[L_FREE] >= 32) {
+      // ---- a slice of leptons
+      cp_async_wait<0>();
       int si;
       int64_t i;
       slot_index(slot, si, i);
       const Sp<float> &S = A.sp[si];
       bool heavy = false;
-      float px = 0.f, py = 0.f, pz = 0.f;
+      float x = pf[lane], y = pf[32 + lane], z = pf[64 + lane];
+      float px = pf[96 + lane], py = pf[128 + lane], pz = pf[160 + lane];
       float E[3] = {0.f, 0.f, 0.f}, B[3] = {0.f, 0.f, 0.f};
-      uint64_t pid = 0;
-      if (i < (si ? n1 : n0)) {
-        const float *v = pf + (size_t)buf * NV * OP_THREADS + t;
-        float x = v[0], y = v[OP_THREADS], z = v[2 * OP_THREADS];
-        px = v[3 * OP_THREADS]; py = v[4 * OP_THREADS]; pz = v[5 * OP_THREADS];
-        if (FM == FM_PER_PARTICLE) {
-          E[0] = v[6 * OP_THREADS]; E[1] = v[7 * OP_THREADS]; E[2] = v[8 * OP_THREADS];
-          B[0] = v[9 * OP_THREADS]; B[1] = v[10 * OP_THREADS]; B[2] = v[11 * OP_THREADS];
-        } else {
-          get_fields<float, FM>(S, A.f, i, x, y, z, E, B);
+      if (FM == FM_PER_PARTICLE) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          E[c] = pf[(6 + c) * 32 + lane];
+          B[c] = pf[(9 + c) * 32 + lane];
         }
-        pid = pf_id[buf * OP_THREADS + t];
+      }
+      const uint64_t pid = pf_id[lane];
+      const int64_t next = slot + stride;
+      if (next < nslots) prefetch(next);
+      cp_async_commit();
+      if (i < (si ? n1 : n0)) {
+        if (FM != FM_PER_PARTICLE) get_fields<float, FM>(S, A.f, i, x, y, z, E, B);
         float g;
         if (MODE != MODE_EMIT) {
           g = boris(px, py, pz, E, B, S.q, dt);
@@ -506,19 +287,17 @@ __global__ void __launch_bounds__(OP_THREADS, 5) k_lepton_onepass(OnePassArgs A)
           const float fj = (r_log(chi) - A.T.gl.x0) * A.T.gl.inv_h;
           const int j = fj >= 0.f ? (fj < (float)(A.T.gl.n - 1) ? (int)fj : A.T.gl.n - 1) : 0;
           const float wdt_up = r_div(__ldg(A.w_up_row + j) * dt * chi, g);
-          bool done = false;
+          heavy = true;
           if (wdt_up <= wdt_max) {
             const U4 r = draw(A.C, pid, step_, 0, STREAM_EMIT);
-            done = !(wdt_up > unif<float>(r.x));
+            heavy = wdt_up > unif<float>(r.x);
           }
-          if (done) {
+          if (!heavy) {
             tl.substeps += 1;
             if (chi > 0.f && (chi < A.chi_tab_lo || chi > A.chi_tab_hi)) {
               tl.domain += 1;
               tl.status |= QED_STATUS_DOMAIN;
             }
-          } else {
-            heavy = true;
           }
           if (MODE != MODE_EMIT) {
             S.x[i] = x; S.y[i] = y; S.z[i] = z;
@@ -526,30 +305,189 @@ __global__ void __launch_bounds__(OP_THREADS, 5) k_lepton_onepass(OnePassArgs A)
           }
         }
       }
+      // the deferred ones take free entries
       const unsigned hm = __ballot_sync(0xFFFFFFFFu, heavy);
       if (heavy) {
-        const int q = qn + __popc(hm & lt_mask);
-        q_slot[q] = (uint32_t)slot;
-        q_f[0 * QCAP + q] = px; q_f[1 * QCAP + q] = py; q_f[2 * QCAP + q] = pz;
+        const int r = __popc(hm & lt_mask);
+        const int e = list[L_FREE * PCAP + len[L_FREE] - 1 - r];
+        word(W_SLOT, e) = (uint32_t)slot;
+        word(W_ID0, e) = (uint32_t)pid;
+        word(W_ID1, e) = (uint32_t)(pid >> 32);
+        real(W_VX, e) = px; real(W_VY, e) = py; real(W_VZ, e) = pz;
+        word(W_N, e) = 0u;
+        word(W_K, e) = 0u;
+        if (FM != FM_UNIFORM) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          q_f[(3 + c) * QCAP + q] = E[c];
-          q_f[(6 + c) * QCAP + q] = B[c];
+          for (int c = 0; c < 3; ++c) {
+            real(W_FIELDS + c, e) = E[c];
+            real(W_FIELDS + 3 + c, e) = B[c];
+          }
         }
-        q_id[q] = pid;
+        list[L_RATE * PCAP + len[L_RATE] + r] = (uint8_t)e;
       }
-      qn += __popc(hm);
-      slot += stride;
-      buf ^= 1;
+      const int nh = __popc(hm);
+      len[L_FREE] -= nh;
+      len[L_RATE] += nh;
+      slot = next;
+      __syncwarp();  // the entries, and the pushed state written above, are visible to the warp
+      continue;
+    }
+    if (most == 0) break;  // (a pool with nothing to run has room, so nothing is left to stream)
+    const int take = min(most, 32);
+    const bool act = lane < take;
+    const int e = act ? list[phase * PCAP + most - 1 - lane] : 0;
+    int st = -1;
+    if (phase == L_RATE) {
+      len[L_RATE] -= take;
+      // ---- chi (Eq. 2) and the exact rate; a new particle also gets N; then
+      // the first draw
+      float kap = 0.f;
+      bool net = false;
+      float E[3], B[3];
+      if (act) {
+        fields_of(e, E, B);
+        float nx = real(W_VX, e), ny = real(W_VY, e), nz = real(W_VZ, e), px, py, pz, g;
+        int N = (int)word(W_N, e);
+        uint32_t kw = word(W_K, e);
+        const bool fresh = N == 0;
+        if (fresh) {
+          px = nx; py = ny; pz = nz;
+          gamma_dir(px, py, pz, g, nx, ny, nz);
+        } else {
+          g = real(W_G, e);
+          const float pm = sqrtf((g - 1.f) * (g + 1.f));
+          px = pm * nx; py = pm * ny; pz = pm * nz;
+        }
+        const float chi = chi_lepton(px, py, pz, g, E[0], E[1], E[2], B[0], B[1], B[2], inv_aS);
+        const RateOut<float> ro = photon_rate(sR, sF, A.T, A.C, chi, g, tl);
+        if (fresh) {
+          N = (int)substep_count_op(A.C, ro.W, dt, wdt_max, tl.status);
+          tl.substeps += N;
+          deferred += 1;
+          word(W_N, e) = (uint32_t)N;
+          real(W_VX, e) = nx; real(W_VY, e) = ny; real(W_VZ, e) = nz;
+          real(W_G, e) = g;
+        }
+        const float thr = ro.W * (dt / (float)N);
+        real(W_CHI, e) = chi;
+        real(W_THR, e) = thr;
+        real(W_KMIN, e) = ro.kmin;
+        int k = (int)(kw & ~EMITTED);
+        uint32_t r2 = 0;
+        const uint64_t pid = (uint64_t)word(W_ID0, e) | ((uint64_t)word(W_ID1, e) << 32);
+        st = draw_two(draw(A.C, pid, step_, k >> 1, STREAM_EMIT), thr, N, k, r2);
+        word(W_K, e) = (uint32_t)k | (kw & EMITTED);
+        word(W_R2, e) = r2;
+        if (st == L_FREE && (kw & EMITTED)) store_recoil(word(W_SLOT, e), g, nx, ny, nz);
+        if (MLP && st == L_PEND && N == 1) {
+          // an event of a one-sub-step particle inside the network's domain
+          // takes its xi from the learned sampler, in the dense pass that
+          // follows this kernel: a record here (one per such particle: at
+          // most n0 + n1, which the records hold), no photon yet
+          kap = photon_kappa(ro.kmin, unif<float>(r2), unif<float>(~r2));
+          const float lchi = chi > 0.f ? logf(chi) : MLP_L_LO - 1.f;
+          net = lchi >= MLP_L_LO && lchi <= MLP_L_HI && kap >= MLP_K_LO && kap <= MLP_K_HI;
+        }
+      }
+      if (MLP) {
+        const unsigned nm = __ballot_sync(0xFFFFFFFFu, net);
+        if (nm) {
+          const int leader = __ffs(nm) - 1;
+          unsigned long long base = 0;
+          if (lane == leader) base = atomicAdd(A.net_n, (unsigned long long)__popc(nm));
+          base = __shfl_sync(0xFFFFFFFFu, base, leader);
+          if (net) {
+            constexpr int RS = net_stride<FM>();
+            const unsigned long long r = base + __popc(nm & lt_mask);
+            if (r < (unsigned long long)(A.net_cap / RS)) {
+              int si;
+              int64_t i;
+              slot_index(word(W_SLOT, e), si, i);
+              float4 *R = A.net_rec + RS * r;
+              R[0] = make_float4(__uint_as_float((uint32_t)i),
+                                 __uint_as_float((uint32_t)((uint64_t)i >> 32) | ((uint32_t)si << 31)),
+                                 kap, E[0]);
+              if (FM == FM_GRID) {
+                R[1] = make_float4(E[1], E[2], B[0], B[1]);
+                R[2] = make_float4(B[2], 0.f, 0.f, 0.f);
+              }
+            } else {  // only with counts beyond the species' capacities
+              tl.dropped += 1;
+              tl.status |= QED_STATUS_CAPACITY;
+            }
+            st = L_FREE;
+          }
+        }
+      }
+    } else if (phase == L_SCAN) {
+      len[L_SCAN] -= take;
+      // ---- the next four sub-steps, from two independent draws
+      if (act) {
+        const uint64_t pid = (uint64_t)word(W_ID0, e) | ((uint64_t)word(W_ID1, e) << 32);
+        const uint32_t kw = word(W_K, e);
+        const int N = (int)word(W_N, e);
+        const float thr = real(W_THR, e);
+        int k = (int)(kw & ~EMITTED);
+        uint32_t r2 = 0;
+        const U4 ra = draw(A.C, pid, step_, k >> 1, STREAM_EMIT);
+        const U4 rb = draw(A.C, pid, step_, (k >> 1) + 1, STREAM_EMIT);
+        st = draw_two(ra, thr, N, k, r2);
+        if (st == L_SCAN) st = draw_two(rb, thr, N, k, r2);
+        word(W_K, e) = (uint32_t)k | (kw & EMITTED);
+        word(W_R2, e) = r2;
+        if (st == L_FREE && (kw & EMITTED))
+          store_recoil(word(W_SLOT, e), real(W_G, e), real(W_VX, e), real(W_VY, e), real(W_VZ, e));
+      }
     } else {
-      cp_async_wait<0>();
+      len[L_PEND] -= take;
+      // ---- emission: kappa and ln delta from the inverse table (Eq. 7), xi,
+      // the recoil and the photon, whose slots come from one atomic
+      unsigned long long base = 0;
+      if (lane == 0)
+        base = atomicAdd(reinterpret_cast<unsigned long long *>(A.ph.d_n), (unsigned long long)take);
+      base = __shfl_sync(0xFFFFFFFFu, base, 0);
+      if (act) {
+        const float chi = real(W_CHI, e), g = real(W_G, e);
+        const uint32_t r2 = word(W_R2, e), kw = word(W_K, e);
+        const float kap = photon_kappa(real(W_KMIN, e), unif<float>(r2), unif<float>(~r2));
+        float l = r_log(chi);  // (clamped as in photon_rate)
+        l = l < A.T.gl.lo ? A.T.gl.lo : l > A.T.gl.hi ? A.T.gl.hi : l;
+        const XiOut<float> xo = xi_from_lndelta(chi, photon_lndelta_table(A.T.Y, A.T, l, kap, tl));
+        float g2 = g * xo.omxi, eph = g * xo.xi;
+        if (g2 < 1.f) { g2 = 1.f; eph = g - 1.f; }
+        const int b = spec_bin(A.C, eph);
+        if (b >= 0) atomicAdd(&s_hist[b], 1u);
+        const float nx = real(W_VX, e), ny = real(W_VY, e), nz = real(W_VZ, e);
+        const uint32_t sl = word(W_SLOT, e);
+        int k = (int)(kw & ~EMITTED);
+        const int64_t pos = (int64_t)base + lane;
+        if (pos >= A.ph.cap) {
+          tl.dropped += 1;
+          tl.status |= QED_STATUS_CAPACITY;
+        } else {
+          int si;
+          int64_t i;
+          slot_index(sl, si, i);
+          const Sp<float> &S = A.sp[si];
+          const uint64_t pid = (uint64_t)word(W_ID0, e) | ((uint64_t)word(W_ID1, e) << 32);
+          const U4 cid = draw(A.C, pid, step_, k, STREAM_PHOTON_ID);
+          float E[3], B[3];
+          fields_of(e, E, B);
+          write_child(A.ph, pos, S.x[i], S.y[i], S.z[i], eph * nx, eph * ny, eph * nz, S.w[i],
+                      (uint64_t)cid.x | ((uint64_t)cid.y << 32), E, B, S.tag ? S.tag[i] : 0u);
+        }
+        tl.events += 1;
+        // the rate for the remaining sub-steps, or the end of the chain
+        st = ++k >= (int)word(W_N, e) ? L_FREE : L_RATE;
+        real(W_G, e) = g2;
+        word(W_K, e) = (uint32_t)k | EMITTED;
+        if (st == L_FREE) store_recoil(sl, g2, nx, ny, nz);
+      }
     }
-    if (qn >= qtrig || !streaming) {
-      __syncwarp();  // queue entries and the pushed state written above are visible to the warp
-      heavy_phase(!streaming);
-    }
-    if (!streaming) break;
+    __syncwarp();
+    file(st, e);
   }
+  cp_async_wait<0>();
 
   tally_flush(&bt, tl);
   {
@@ -558,6 +496,8 @@ __global__ void __launch_bounds__(OP_THREADS, 5) k_lepton_onepass(OnePassArgs A)
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
     if (lane == 0 && d) atomicAdd(&s_deferred, (unsigned long long)d);
   }
+  __syncthreads();
+  if (threadIdx.x < 64) bt.hist[threadIdx.x] = s_hist[threadIdx.x];
   __syncthreads();
   block_tally_commit(&bt, A.o.cnt, 0);
   if (threadIdx.x == 0) {
@@ -744,18 +684,17 @@ cudaError_t launch_net_emit(qed_ctx *c, const OnePassArgs &a, int fm, cudaStream
 
 template <int FM, int MODE, bool MLP>
 cudaError_t launch_onepass_t(qed_ctx *c, const OnePassArgs &a, cudaStream_t st) {
-  size_t off[4];
-  const size_t sm = onepass_layout<FM>(a, off);
-  bool dflt = true;
-  for (int k = 0; k < QED_SCHED_PARAMS; ++k) dflt = dflt && sched_param(c, k) == sched_default(k);
-  auto kern = dflt ? k_lepton_onepass<FM, MODE, MLP, true> : k_lepton_onepass<FM, MODE, MLP, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  int max_smem = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, OP_THREADS, sm);
+  // the tables of the default density (30 KB) fit; a denser grid is read through L1
+  constexpr size_t STATIC_SMEM = 2048;  // more than the kernel's static arrays
+  const bool tab = onepass_smem<FM>(c, true) + STATIC_SMEM <= (size_t)max_smem;
+  const size_t sm = onepass_smem<FM>(c, tab);
+  auto kern = tab ? k_lepton_onepass<FM, MODE, MLP, true> : k_lepton_onepass<FM, MODE, MLP, false>;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_STREAM);
-  kern<<<c->num_sms * per_sm, OP_THREADS, sm, st>>>(a);
+  kern<<<c->num_sms, OP_THREADS, sm, st>>>(a);
   c->launches += 1;
   return cudaGetLastError();
 }
@@ -794,11 +733,6 @@ cudaError_t launch_lepton_onepass(qed_ctx *c, const qed_species *s0, const qed_s
   a.net_rec = c->net_rec;
   a.net_n = c->net_n;
   a.net_cap = c->net_cap;
-  a.emit_lanes = sched_param(c, QED_SCHED_EMIT_LANES);
-  a.round_lanes = sched_param(c, QED_SCHED_ROUND_LANES);
-  a.scan_iters = (sched_param(c, QED_SCHED_SCAN_DRAWS) + 3) / 4;
-  a.scan_left = sched_param(c, QED_SCHED_SCAN_LEFT);
-  a.qtrig = min(sched_param(c, QED_SCHED_QUEUE_TRIGGER), QCAP - 31);
   const bool mlp = c->cfg.sampler == QED_SAMPLER_MLP && c->mlp_ready && c->net_rec;
   cudaError_t e;
   if (mode == MODE_EMIT)
