@@ -387,11 +387,10 @@ int qed_autotune(qed_ctx *ctx, const qed_species *e, const qed_species *p, const
                  qed_stream_t stream);
 
 /* Launch tuning by kernel group.  Every step kernel is a persistent launch of
- * a fixed block size (256 threads; the single-pass lepton kernel 128) whose
- * grid is the number of SMs times a number of CTAs per SM; that number, up to
- * what fits, is chosen per group of kernels:
- *   QED_TUNE_STREAM   lepton streaming: k_lepton_stream, the single-pass
- *                     lepton kernel, the push-only pass
+ * a fixed block size (256 threads) whose grid is the number of SMs times a
+ * number of CTAs per SM; that number, up to what fits, is chosen per group of
+ * kernels (the single-pass lepton kernel is one CTA of 640 threads per SM):
+ *   QED_TUNE_STREAM   lepton streaming: k_lepton_stream, the push-only pass
  *   QED_TUNE_CHAINS   the ordered path's Method I chains (counting, replay)
  *   QED_TUNE_ORDER    the ordered path's lists, scans and writing pass
  *   QED_TUNE_PHOTON   photon streaming and pair passes
@@ -400,22 +399,20 @@ int qed_autotune(qed_ctx *ctx, const qed_species *e, const qed_species *p, const
 enum { QED_TUNE_STREAM = 0, QED_TUNE_CHAINS = 1, QED_TUNE_ORDER = 2, QED_TUNE_PHOTON = 3,
        QED_TUNE_COMPACT = 4, QED_TUNE_GROUPS = 5, QED_TUNE_MAX_FACTOR = 8 };
 
-/* Scheduling of the Method I chains of the deferred leptons, run a warp at a
- * time with lanes in states (idle, rate, scanning, event pending) and one
- * state per round (the single-pass kernel's heavy phase, and the ordered
- * counting pass).  0 = the default, in brackets:
+/* Scheduling of the Method I chains of the ordered counting pass, run a warp at
+ * a time with lanes in states (idle, scanning, event pending) and one state
+ * per round.  0 = the default, in brackets:
  *   QED_SCHED_EMIT_LANES     an emission round waits for this many lanes with
- *                            an event, 1..32 [16] (both paths)
- *   QED_SCHED_ROUND_LANES    a rate or scanning round of the single pass runs
- *                            with at least this many lanes, 1..32 [12]
+ *                            an event, 1..32 [16]
+ *   QED_SCHED_ROUND_LANES    1..32 [12], without effect
  *   QED_SCHED_SCAN_DRAWS     Method I sub-steps drawn per lane per scanning
- *                            round, 2..16, even [8] (both paths; the single
- *                            pass draws four at a time)
- *   QED_SCHED_SCAN_LEFT      a scanning round of the single pass ends when
- *                            fewer lanes are still drawing, 1..32 [8]
- *   QED_SCHED_QUEUE_TRIGGER  queued deferred leptons that start a heavy phase
- *                            of the single pass, 1..33 [32]
- * The results (particles, photons, counters) do not depend on them. */
+ *                            round, 2..16, even [8]
+ *   QED_SCHED_SCAN_LEFT      1..32 [8], without effect
+ *   QED_SCHED_QUEUE_TRIGGER  1..33 [32], without effect
+ * The single-pass kernel keeps its chains in a pool per warp and always runs
+ * the state with most chains, so nothing is left to tune there; the values
+ * without effect belonged to its earlier scheduler and are still checked and
+ * kept.  The results (particles, photons, counters) do not depend on them. */
 enum { QED_SCHED_EMIT_LANES = 0, QED_SCHED_ROUND_LANES = 1, QED_SCHED_SCAN_DRAWS = 2,
        QED_SCHED_SCAN_LEFT = 3, QED_SCHED_QUEUE_TRIGGER = 4, QED_SCHED_PARAMS = 5,
        QED_SCHED_MAX_CANDIDATES = 6 };

@@ -12,7 +12,7 @@
 // set in another order.
 //
 // How the work is laid out, per warp of a persistent grid (one CTA of OP_WARPS
-// warps per SM, which share the rate tables in shared memory):
+// warps per SM):
 //   streaming: each lane takes one particle of a 32-particle slice (the next
 //     slice's words are in flight into shared memory, cp.async), pushes it and
 //     computes chi.  The rate bound W <= w_j chi / gamma (w_j = alpha a_S
@@ -27,11 +27,11 @@
 //     draws due), or event pending (xi, the recoil, the photon).  A round
 //     takes up to 32 chains of one state -- any lane runs any chain -- and
 //     files each under its next state; a chain that ends frees its entry.  The
-//     warp streams while the pool has room for a slice, and then runs the
-//     fullest state, so a round nearly always has 27 to 32 lanes at work,
-//     where a lane that keeps its own chain in registers waits for its
-//     neighbours' states (14 to 23 lanes).  After the last slice the pool is
-//     drained.
+//     warp streams while the pool has room for a slice, and otherwise runs the
+//     fullest state (19 chains at least then), where a lane that keeps its own
+//     chain in registers waits for its neighbours' states: 26 of 32 lanes
+//     active over the whole kernel instead of 22.  After the last slice the
+//     pool is drained.
 //   photons: an emission round reserves slots for its photons with one atomic
 //     on the photon count and writes them there.
 //   learned sampler: an event of a one-sub-step lepton inside the network's
@@ -41,6 +41,19 @@
 // particle is read once and its slot written once or twice (the pushed state,
 // then the recoiled momentum of one that emitted, shortly after, while the
 // line is still in L2).
+//
+// What bounds it: instruction issue, 62% of the slots of 20 warps an SM (the
+// rest is the latency of dependent arithmetic); DRAM moves little more than the
+// algorithmic bytes.  The 64M-electron ensemble: 2.93 -> 2.04 ms per launch
+// (2.18 -> 3.13 TB/s algorithmic), at 16M 735 -> 544 us, of which streaming
+// alone 239 (198 at the copy rate).  Steps and choices measured at 16M: chains in
+// a pool (20 warps of 96 entries, tables in shared memory) 647; fewer entries
+// leave more L1 to the inverse table and fewer lanes to a round (80: 601, 72:
+// 629, 64: 682), and the tables are as fast through L1, which leaves room for 88
+// entries: 594; 16 warps of 120 entries 692, 24 of 80 entries (80 registers)
+// 630; E and B left in global memory for larger pools 651; the parent's words
+// and the photon slots requested before the inverse look-up 563; slices by
+// 16-byte copies past L1 544.
 #include <cstdio>
 
 #include "qed_internal.h"
@@ -51,19 +64,24 @@ namespace qed {
 
 namespace {
 
-// one CTA per SM: its warps share the tables, and its shared memory is full
+// one CTA per SM; 20 warps leave 96 registers to a thread
 constexpr int OP_WARPS = 20;
 constexpr int OP_THREADS = OP_WARPS * 32;
-constexpr int PCAP = 96;  // chains per warp's pool
+constexpr int PCAP = 88;  // chains per warp's pool
 // words of a pool entry: the slot, the id, the momentum of a new particle and
-// then the unit direction, gamma, chi, the event threshold W Dt / N, kappa_min,
-// N (0: new), the sub-step (top bit: it has emitted), the word r2 of the
-// event and, unless the field is uniform, E and B
-enum { W_SLOT, W_ID0, W_ID1, W_VX, W_VY, W_VZ, W_G, W_CHI, W_THR, W_KMIN, W_N, W_K, W_R2, W_FIELDS };
+// then the unit direction, gamma, chi, the event threshold W Dt / N (of a
+// pending event its word r2), kappa_min, N (0: new), the sub-step (top bit: it
+// has emitted) and, unless the field is uniform, E and B
+enum { W_SLOT, W_ID0, W_ID1, W_VX, W_VY, W_VZ, W_G, W_CHI, W_THR, W_KMIN, W_N, W_K, W_FIELDS, W_R2 = W_THR };
 constexpr uint32_t EMITTED = 0x80000000u;
 template <int FM> __host__ __device__ constexpr int pool_words() { return FM == FM_UNIFORM ? W_FIELDS : W_FIELDS + 6; }
-// the states of a chain, and the list of free entries
-enum { L_RATE = 0, L_SCAN = 1, L_PEND = 2, L_FREE = 3, LISTS = 4 };
+// The states of a chain, and the free entries.  An entry is in one list, so two
+// lists share an array of PCAP bytes from its two ends: rate (up) and scan
+// (down), pending (up) and free (down).
+enum { L_RATE = 0, L_SCAN = 1, L_PEND = 2, L_FREE = 3, LIST_ARRAYS = 2 };
+__device__ __forceinline__ constexpr int list_at(int l, int k) {
+  return (l >> 1) * PCAP + ((l & 1) ? PCAP - 1 - k : k);
+}
 
 struct OnePassArgs {
   Sp<float> sp[2];
@@ -82,17 +100,17 @@ struct OnePassArgs {
   float4 *net_rec;           // records of the deferred network emissions
   unsigned long long *net_n; // their count
   int64_t net_cap;
+  bool aligned16;  // every array a slice is read from starts on a 16-byte boundary
 };
 
-// Dynamic shared memory: per warp the prefetch words and ids of a slice, the
-// pool and its lists; then the rate and forward tables (TAB; tables that do not
-// fit are read through L1).
+// Dynamic shared memory per warp: the prefetch words and ids of a slice, the
+// pool and its lists.  The tables are read through L1.
 template <int FM> __host__ __device__ constexpr size_t warp_smem() {
-  return 32 * ((size_t)stream_words<FM>() * 4 + 8) + (size_t)PCAP * (4 * pool_words<FM>() + LISTS);
+  return 32 * ((size_t)stream_words<FM>() * 4 + 8) + (size_t)PCAP * (4 * pool_words<FM>() + LIST_ARRAYS);
 }
-template <int FM> size_t onepass_smem(const qed_ctx *c, bool tab) {
-  return OP_WARPS * warp_smem<FM>() + (tab ? sizeof(float) * (size_t)c->gl.n * (1 + c->gy.n) : 0);
-}
+
+static_assert(warp_smem<0>() % 16 == 0 && warp_smem<1>() % 16 == 0 && warp_smem<2>() % 16 == 0,
+              "a warp's shared memory starts on a 16-byte boundary (cp.async)");
 
 // Learned-sampler emissions deferred to the dense pass: one record per
 // emission, 16 bytes -- the lepton's index (species in the top bit) and kappa
@@ -140,13 +158,14 @@ __device__ __forceinline__ int draw_two(const U4 &r, float thr, int N, int &k, u
   return ++k >= N ? L_FREE : L_SCAN;
 }
 
-template <int FM, int MODE, bool MLP, bool TAB>
+template <int FM, int MODE, bool MLP>
 __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t s_hist[64];
   __shared__ BlockTally bt;
   __shared__ long long s_meta[4];
   __shared__ unsigned long long s_deferred;
+  __shared__ unsigned long long s_src[2][13];  // the arrays a slice is read from
   constexpr int NV = stream_words<FM>();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -154,9 +173,7 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
   uint64_t *const pf_id = reinterpret_cast<uint64_t *>(mine);                 // [32]
   float *const pf = reinterpret_cast<float *>(mine + 256);                    // [NV][32]
   uint32_t *const pool = reinterpret_cast<uint32_t *>(pf + NV * 32);          // [words][PCAP]
-  uint8_t *const list = reinterpret_cast<uint8_t *>(pool + pool_words<FM>() * PCAP);  // [LISTS][PCAP]
-  float *const tab = reinterpret_cast<float *>(smem_raw + OP_WARPS * warp_smem<FM>());
-  const float *const sR = TAB ? tab : A.T.R, *const sF = TAB ? tab + A.T.gl.n : A.T.F;
+  uint8_t *const list = reinterpret_cast<uint8_t *>(pool + pool_words<FM>() * PCAP);  // [LIST_ARRAYS][PCAP]
   block_tally_init(&bt);
   if (threadIdx.x < 64) s_hist[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
@@ -164,46 +181,44 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
     s_meta[1] = A.nsp > 1 ? *(volatile int64_t *)A.sp[1].d_n : 0;
     s_meta[2] = (long long)A.o.scan.sync[2];
     s_deferred = 0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const Sp<float> &S = A.sp[k];
+      const void *src[13] = {S.x, S.y, S.z, S.px, S.py, S.pz, S.ex, S.ey, S.ez, S.bx, S.by, S.bz, S.id};
+#pragma unroll
+      for (int c = 0; c < 13; ++c) s_src[k][c] = reinterpret_cast<unsigned long long>(src[c]);
+    }
   }
   __syncthreads();
   const int64_t step_ = A.d_step ? *A.d_step : A.step;
-  const int64_t n0 = s_meta[0], n1 = s_meta[1];
+  // slots fit 32 bits: a species holds at most 2^30 - 4096 particles
+  const uint32_t n0 = (uint32_t)s_meta[0], n1 = (uint32_t)s_meta[1];
   const uint32_t epoch = (uint32_t)s_meta[2];
-  const int64_t T0 = (n0 + TILE - 1) / TILE, T1 = (n1 + TILE - 1) / TILE;
-  const int64_t nslots = (T0 + T1) * TILE;
+  const uint32_t slots0 = (n0 + TILE - 1) / TILE * TILE, nslots = slots0 + (n1 + TILE - 1) / TILE * TILE;
   // consecutive slices go to different SMs
-  const int64_t stride = (int64_t)gridDim.x * OP_THREADS;
-  int64_t slot = ((int64_t)wid * gridDim.x + blockIdx.x) * 32 + lane;
-  if (TAB && (int64_t)blockIdx.x * 32 < nslots) {  // (a CTA without a slice needs no tables)
-    load_tables_smem(tab, A.T.R, A.T.gl.n);
-    load_tables_smem(tab + A.T.gl.n, A.T.F, A.T.gl.n * A.T.gy.n);
-  }
-  __syncthreads();
+  const uint32_t stride = gridDim.x * OP_THREADS;
+  uint32_t slot = (wid * gridDim.x + blockIdx.x) * 32 + lane;
   const float inv_aS = A.C.f_inv_aS, dt = A.C.f_dt, wdt_max = A.C.f_wdt_max;
   Tally tl;
   tl.clear();
   uint32_t deferred = 0;  // new particles taken by this lane
 
-  auto slot_index = [&](int64_t sl, int &si, int64_t &i) {
-    const int64_t tile = sl / TILE;
-    si = tile < T0 ? 0 : 1;
-    i = (tile - (si ? T0 : 0)) * TILE + (sl % TILE);
+  // species and index of a slot (species 1 starts at a tile of its own)
+  auto slot_index = [&](uint32_t sl, int &si, uint32_t &i) {
+    si = sl < slots0 ? 0 : 1;
+    i = si ? sl - slots0 : sl;
   };
   // ---- the pool's lists: entries of a state in any order (lengths warp-uniform)
-  int len[LISTS] = {0, 0, 0, PCAP};
-  for (int q = lane; q < PCAP; q += 32) list[L_FREE * PCAP + q] = (uint8_t)q;
+  int len[4] = {0, 0, 0, PCAP};
+  for (int q = lane; q < PCAP; q += 32) list[list_at(L_FREE, q)] = (uint8_t)q;
   __syncwarp();
   auto word = [&](int w, int e) -> uint32_t & { return pool[w * PCAP + e]; };
   auto real = [&](int w, int e) -> float & { return reinterpret_cast<float *>(pool)[w * PCAP + e]; };
-  // file entry e of each lane with state st (-1: none)
-  auto file = [&](int st, int e) {
-#pragma unroll
-    for (int s = 0; s < LISTS; ++s) {
-      const unsigned m = __ballot_sync(0xFFFFFFFFu, st == s);
-      if (st == s) list[s * PCAP + len[s] + __popc(m & lt_mask)] = (uint8_t)e;
-      len[s] += __popc(m);
-    }
-    __syncwarp();
+  // file entry e of each lane whose next state is s
+  auto file = [&](int s, bool in, int e) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+    if (in) list[list_at(s, len[s] + __popc(m & lt_mask))] = (uint8_t)e;
+    len[s] += __popc(m);
   };
   auto fields_of = [&](int e, float E[3], float B[3]) {
 #pragma unroll
@@ -215,29 +230,60 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
   // the end of a chain that has emitted: the recoiled momentum
   auto store_recoil = [&](uint32_t sl, float g, float nx, float ny, float nz) {
     int si;
-    int64_t i;
+    uint32_t i;
     slot_index(sl, si, i);
     const Sp<float> &S = A.sp[si];
     const float pm = sqrtf((g - 1.f) * (g + 1.f));
     S.px[i] = pm * nx; S.py[i] = pm * ny; S.pz[i] = pm * nz;
   };
 
-  // Each lane copies its next particle's words into its own words of shared
-  // memory (cp.async), as soon as it has read the current ones from there.
-  auto prefetch = [&](int64_t sl) {
-    int si;
-    int64_t i;
-    slot_index(sl, si, i);
-    const Sp<float> &S = A.sp[si];
-    if (i < (si ? n1 : n0)) {
-      const float *src[12] = {S.x, S.y, S.z, S.px, S.py, S.pz, S.ex, S.ey, S.ez, S.bx, S.by, S.bz};
+  // The next slice's words are copied into shared memory (cp.async) as soon as
+  // the current ones have been read from there: 16 bytes per lane and copy
+  // where the arrays are aligned (a slice is 8 such pieces of each float array
+  // and 16 of the ids; past L1, which the tables need), else each lane its
+  // own particle's words.
+  constexpr int PIECES = (NV * 8 + 31) / 32;  // 16-byte pieces of a slice per lane
+  const float *piece[PIECES];
+  const uint64_t *piece_id = nullptr;
+  int piece_si = -1;
+  auto prefetch = [&](uint32_t sl) {
+    const int si = sl < slots0 ? 0 : 1;
+    const uint32_t i = si ? sl - slots0 : sl, n = si ? n1 : n0, q0 = i - lane;
+    if (A.aligned16) {
+      if (si != piece_si) {  // this lane's pieces of the species' arrays
+        piece_si = si;
 #pragma unroll
-      for (int c = 0; c < NV; ++c) cp_async<4>(pf + c * 32 + lane, src[c] + i);
-      cp_async<8>(pf_id + lane, S.id + i);
+        for (int t = 0; t < PIECES; ++t) {
+          const int q = t * 32 + lane;
+          piece[t] = reinterpret_cast<const float *>(s_src[si][q < NV * 8 ? q >> 3 : 0]) + (q & 7) * 4;
+        }
+        piece_id = reinterpret_cast<const uint64_t *>(s_src[si][12]) + 2 * (lane & 15);
+      }
+      if (q0 + 32 <= n) {
+#pragma unroll
+        for (int t = 0; t < PIECES; ++t)
+          if (t * 32 + lane < NV * 8) cp_async16(pf + (t * 32 + lane) * 4, piece[t] + q0, 16);
+        if (lane < 16) cp_async16(pf_id + 2 * lane, piece_id + q0, 16);
+      } else if (q0 < n) {  // the species' last slice
+        const int left = (int)(n - q0), p = (lane & 7) * 4;
+#pragma unroll
+        for (int t = 0; t < PIECES; ++t)
+          if (t * 32 + lane < NV * 8 && p < left)
+            cp_async16(pf + (t * 32 + lane) * 4, piece[t] + q0, min(left - p, 4) * 4);
+        if (lane < 16 && 2 * lane < left) cp_async16(pf_id + 2 * lane, piece_id + q0, min(left - 2 * lane, 2) * 8);
+      }
+    } else if (i < n) {
+#pragma unroll
+      for (int c = 0; c < NV; ++c) cp_async<4>(pf + c * 32 + lane, reinterpret_cast<const float *>(s_src[si][c]) + i);
+      cp_async<8>(pf_id + lane, reinterpret_cast<const uint64_t *>(s_src[si][12]) + i);
     }
+    cp_async_commit();
+  };
+  auto store_pushed = [&](const Sp<float> &S, uint32_t i, float x, float y, float z, float px, float py, float pz) {
+    S.x[i] = x; S.y[i] = y; S.z[i] = z;
+    S.px[i] = px; S.py[i] = py; S.pz[i] = pz;
   };
   if (slot < nslots) prefetch(slot);
-  cp_async_commit();
 
   for (;;) {
     // nslots is a multiple of 32: every lane of a warp sees the same
@@ -249,10 +295,10 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
     if (streaming && most < 32 && len[L_FREE] >= 32) {
       // ---- a slice of leptons
       cp_async_wait<0>();
+      __syncwarp();
       int si;
-      int64_t i;
+      uint32_t i;
       slot_index(slot, si, i);
-      const Sp<float> &S = A.sp[si];
       bool heavy = false;
       float x = pf[lane], y = pf[32 + lane], z = pf[64 + lane];
       float px = pf[96 + lane], py = pf[128 + lane], pz = pf[160 + lane];
@@ -265,14 +311,14 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
         }
       }
       const uint64_t pid = pf_id[lane];
-      const int64_t next = slot + stride;
+      const uint32_t next = slot + stride;
+      __syncwarp();  // the words are read by all lanes
       if (next < nslots) prefetch(next);
-      cp_async_commit();
       if (i < (si ? n1 : n0)) {
-        if (FM != FM_PER_PARTICLE) get_fields<float, FM>(S, A.f, i, x, y, z, E, B);
+        if (FM != FM_PER_PARTICLE) get_fields<float, FM>(A.sp[0], A.f, i, x, y, z, E, B);
         float g;
         if (MODE != MODE_EMIT) {
-          g = boris(px, py, pz, E, B, S.q, dt);
+          g = boris(px, py, pz, E, B, si ? A.sp[1].q : A.sp[0].q, dt);
           const float ig = r_div(dt, g);
           x += px * ig; y += py * ig; z += pz * ig;
         } else {
@@ -300,8 +346,8 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
             }
           }
           if (MODE != MODE_EMIT) {
-            S.x[i] = x; S.y[i] = y; S.z[i] = z;
-            S.px[i] = px; S.py[i] = py; S.pz[i] = pz;
+            if (si == 0) store_pushed(A.sp[0], i, x, y, z, px, py, pz);
+            else store_pushed(A.sp[1], i, x, y, z, px, py, pz);
           }
         }
       }
@@ -309,8 +355,8 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
       const unsigned hm = __ballot_sync(0xFFFFFFFFu, heavy);
       if (heavy) {
         const int r = __popc(hm & lt_mask);
-        const int e = list[L_FREE * PCAP + len[L_FREE] - 1 - r];
-        word(W_SLOT, e) = (uint32_t)slot;
+        const int e = list[list_at(L_FREE, len[L_FREE] - 1 - r)];
+        word(W_SLOT, e) = slot;
         word(W_ID0, e) = (uint32_t)pid;
         word(W_ID1, e) = (uint32_t)(pid >> 32);
         real(W_VX, e) = px; real(W_VY, e) = py; real(W_VZ, e) = pz;
@@ -323,7 +369,7 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
             real(W_FIELDS + 3 + c, e) = B[c];
           }
         }
-        list[L_RATE * PCAP + len[L_RATE] + r] = (uint8_t)e;
+        list[list_at(L_RATE, len[L_RATE] + r)] = (uint8_t)e;
       }
       const int nh = __popc(hm);
       len[L_FREE] -= nh;
@@ -335,7 +381,8 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
     if (most == 0) break;  // (a pool with nothing to run has room, so nothing is left to stream)
     const int take = min(most, 32);
     const bool act = lane < take;
-    const int e = act ? list[phase * PCAP + most - 1 - lane] : 0;
+    const int e = act ? list[list_at(phase, most - 1 - lane)] : 0;
+    __syncwarp();  // the entries are taken before others are filed
     int st = -1;
     if (phase == L_RATE) {
       len[L_RATE] -= take;
@@ -359,7 +406,7 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
           px = pm * nx; py = pm * ny; pz = pm * nz;
         }
         const float chi = chi_lepton(px, py, pz, g, E[0], E[1], E[2], B[0], B[1], B[2], inv_aS);
-        const RateOut<float> ro = photon_rate(sR, sF, A.T, A.C, chi, g, tl);
+        const RateOut<float> ro = photon_rate(A.T.R, A.T.F, A.T, A.C, chi, g, tl);
         if (fresh) {
           N = (int)substep_count_op(A.C, ro.W, dt, wdt_max, tl.status);
           tl.substeps += N;
@@ -377,7 +424,7 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
         const uint64_t pid = (uint64_t)word(W_ID0, e) | ((uint64_t)word(W_ID1, e) << 32);
         st = draw_two(draw(A.C, pid, step_, k >> 1, STREAM_EMIT), thr, N, k, r2);
         word(W_K, e) = (uint32_t)k | (kw & EMITTED);
-        word(W_R2, e) = r2;
+        if (st == L_PEND) word(W_R2, e) = r2;
         if (st == L_FREE && (kw & EMITTED)) store_recoil(word(W_SLOT, e), g, nx, ny, nz);
         if (MLP && st == L_PEND && N == 1) {
           // an event of a one-sub-step particle inside the network's domain
@@ -401,12 +448,10 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
             const unsigned long long r = base + __popc(nm & lt_mask);
             if (r < (unsigned long long)(A.net_cap / RS)) {
               int si;
-              int64_t i;
+              uint32_t i;
               slot_index(word(W_SLOT, e), si, i);
               float4 *R = A.net_rec + RS * r;
-              R[0] = make_float4(__uint_as_float((uint32_t)i),
-                                 __uint_as_float((uint32_t)((uint64_t)i >> 32) | ((uint32_t)si << 31)),
-                                 kap, E[0]);
+              R[0] = make_float4(__uint_as_float(i), __uint_as_float((uint32_t)si << 31), kap, E[0]);
               if (FM == FM_GRID) {
                 R[1] = make_float4(E[1], E[2], B[0], B[1]);
                 R[2] = make_float4(B[2], 0.f, 0.f, 0.f);
@@ -434,7 +479,7 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
         st = draw_two(ra, thr, N, k, r2);
         if (st == L_SCAN) st = draw_two(rb, thr, N, k, r2);
         word(W_K, e) = (uint32_t)k | (kw & EMITTED);
-        word(W_R2, e) = r2;
+        if (st == L_PEND) word(W_R2, e) = r2;
         if (st == L_FREE && (kw & EMITTED))
           store_recoil(word(W_SLOT, e), real(W_G, e), real(W_VX, e), real(W_VY, e), real(W_VZ, e));
       }
@@ -445,36 +490,43 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
       unsigned long long base = 0;
       if (lane == 0)
         base = atomicAdd(reinterpret_cast<unsigned long long *>(A.ph.d_n), (unsigned long long)take);
-      base = __shfl_sync(0xFFFFFFFFu, base, 0);
-      if (act) {
+      float x = 0.f, y = 0.f, z = 0.f, w = 0.f, eph = 0.f, g2 = 1.f;
+      uint32_t sl = 0, tag = 0;
+      if (act) {  // (the parent's words and the slots are on their way during the look-up)
+        sl = word(W_SLOT, e);
+        int si;
+        uint32_t i;
+        slot_index(sl, si, i);
+        const Sp<float> &S = A.sp[si];
+        x = S.x[i]; y = S.y[i]; z = S.z[i]; w = S.w[i];
+        if (S.tag) tag = S.tag[i];
         const float chi = real(W_CHI, e), g = real(W_G, e);
-        const uint32_t r2 = word(W_R2, e), kw = word(W_K, e);
+        const uint32_t r2 = word(W_R2, e);
         const float kap = photon_kappa(real(W_KMIN, e), unif<float>(r2), unif<float>(~r2));
         float l = r_log(chi);  // (clamped as in photon_rate)
         l = l < A.T.gl.lo ? A.T.gl.lo : l > A.T.gl.hi ? A.T.gl.hi : l;
         const XiOut<float> xo = xi_from_lndelta(chi, photon_lndelta_table(A.T.Y, A.T, l, kap, tl));
-        float g2 = g * xo.omxi, eph = g * xo.xi;
+        g2 = g * xo.omxi;
+        eph = g * xo.xi;
         if (g2 < 1.f) { g2 = 1.f; eph = g - 1.f; }
         const int b = spec_bin(A.C, eph);
         if (b >= 0) atomicAdd(&s_hist[b], 1u);
+      }
+      base = __shfl_sync(0xFFFFFFFFu, base, 0);
+      if (act) {
         const float nx = real(W_VX, e), ny = real(W_VY, e), nz = real(W_VZ, e);
-        const uint32_t sl = word(W_SLOT, e);
-        int k = (int)(kw & ~EMITTED);
+        int k = (int)(word(W_K, e) & ~EMITTED);
         const int64_t pos = (int64_t)base + lane;
         if (pos >= A.ph.cap) {
           tl.dropped += 1;
           tl.status |= QED_STATUS_CAPACITY;
         } else {
-          int si;
-          int64_t i;
-          slot_index(sl, si, i);
-          const Sp<float> &S = A.sp[si];
           const uint64_t pid = (uint64_t)word(W_ID0, e) | ((uint64_t)word(W_ID1, e) << 32);
           const U4 cid = draw(A.C, pid, step_, k, STREAM_PHOTON_ID);
           float E[3], B[3];
           fields_of(e, E, B);
-          write_child(A.ph, pos, S.x[i], S.y[i], S.z[i], eph * nx, eph * ny, eph * nz, S.w[i],
-                      (uint64_t)cid.x | ((uint64_t)cid.y << 32), E, B, S.tag ? S.tag[i] : 0u);
+          write_child(A.ph, pos, x, y, z, eph * nx, eph * ny, eph * nz, w,
+                      (uint64_t)cid.x | ((uint64_t)cid.y << 32), E, B, tag);
         }
         tl.events += 1;
         // the rate for the remaining sub-steps, or the end of the chain
@@ -484,8 +536,14 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
         if (st == L_FREE) store_recoil(sl, g2, nx, ny, nz);
       }
     }
+    if (phase == L_PEND) {
+      file(L_RATE, st == L_RATE, e);
+    } else {
+      file(L_SCAN, st == L_SCAN, e);
+      file(L_PEND, st == L_PEND, e);
+    }
+    file(L_FREE, st == L_FREE, e);
     __syncwarp();
-    file(st, e);
   }
   cp_async_wait<0>();
 
@@ -682,17 +740,22 @@ cudaError_t launch_net_emit(qed_ctx *c, const OnePassArgs &a, int fm, cudaStream
   return launch_net_emit_t<FM_GRID>(c, n, st);
 }
 
+template <int FM> bool slices_aligned(const OnePassArgs &a) {
+  uintptr_t all = 0;
+  for (int k = 0; k < a.nsp; ++k) {
+    const Sp<float> &S = a.sp[k];
+    const void *src[13] = {S.id, S.x, S.y, S.z, S.px, S.py, S.pz, S.ex, S.ey, S.ez, S.bx, S.by, S.bz};
+    for (int c = 0; c <= stream_words<FM>(); ++c) all |= reinterpret_cast<uintptr_t>(src[c]);
+  }
+  return (all & 15) == 0;
+}
+
 template <int FM, int MODE, bool MLP>
-cudaError_t launch_onepass_t(qed_ctx *c, const OnePassArgs &a, cudaStream_t st) {
-  int max_smem = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-  if (e != cudaSuccess) return e;
-  // the tables of the default density (30 KB) fit; a denser grid is read through L1
-  constexpr size_t STATIC_SMEM = 2048;  // more than the kernel's static arrays
-  const bool tab = onepass_smem<FM>(c, true) + STATIC_SMEM <= (size_t)max_smem;
-  const size_t sm = onepass_smem<FM>(c, tab);
-  auto kern = tab ? k_lepton_onepass<FM, MODE, MLP, true> : k_lepton_onepass<FM, MODE, MLP, false>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+cudaError_t launch_onepass_t(qed_ctx *c, OnePassArgs a, cudaStream_t st) {
+  a.aligned16 = slices_aligned<FM>(a);
+  const size_t sm = OP_WARPS * warp_smem<FM>();
+  auto kern = k_lepton_onepass<FM, MODE, MLP>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   kern<<<c->num_sms, OP_THREADS, sm, st>>>(a);
   c->launches += 1;
