@@ -85,7 +85,7 @@ static void free_ctx(qed_ctx *c) {
                   c->P32, c->Yp32, c->tile_state, c->sync, c->snap, c->pic_n, c->d_counters,
                   c->heavy_flags, c->heavy_list, c->heavy_n, c->cls_chunk_cnt,
                   c->cls_chunk_off, c->cls_off, c->sub_cnt, c->sub_gf, c->rec_e,
-                  c->rec_k, c->sub_meta, c->fill_meta, c->replay_n, c->stage, c->stage_tag,
+                  c->rec_k, c->sub_meta, c->fill_meta, c->ord_n, c->replay_n, c->stage, c->stage_tag,
                   c->stage_idx, c->stage_n, c->probe_state,
                   c->mlp_mem, c->w_up_row, c->net_rec, c->net_n};
   for (void *p : ptrs)
@@ -286,6 +286,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
       cudaMalloc(&c->stage_n, sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->sub_meta, 4 * sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&c->fill_meta, 2 * sizeof(int64_t)) != cudaSuccess ||
+      cudaMalloc(&c->ord_n, 4 * sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->replay_n, sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->probe_state, 2 * sizeof(unsigned long long)) != cudaSuccess) {
     free_ctx(c);
@@ -295,6 +296,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   if (e == cudaSuccess) e = cudaMemsetAsync(c->sync, 0, sizeof(unsigned int) * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->snap, 0, sizeof(int64_t) * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counters, 0, sizeof(qed_counters), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->ord_n, 0, 4 * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->stage_n, 0, sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->probe_state, 0, 2 * sizeof(unsigned long long), st);
   if (e != cudaSuccess) { free_ctx(c); return cuda_fail(e, "memset"); }

@@ -812,8 +812,10 @@ __global__ void __launch_bounds__(TILE) k_sub_scan(SubScanArgs A) {
 // emission chains -- same draws, same tables -- and write their photons and
 // final momenta.  It is separate so that the common case carries neither the
 // tables nor the chain's registers, and dense, so that the rare long replays
-// share warps.
-template <class Real, int FM, int MODE>
+// share warps.  BY_SLOT: the list is of slots, leptons of the single pass
+// whose momentum (with grid fields also position) is stored as before the
+// step, and sub_cnt is per slot.
+template <class Real, int FM, int MODE, bool BY_SLOT>
 __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) {
   const int64_t step_ = A.d_step ? *A.d_step : A.step;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -832,7 +834,7 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
   block_tally_init(&bt);
   if (threadIdx.x == 0) {
     s_meta[0] = *(volatile int64_t *)A.sp[0].d_n;
-    s_meta[1] = A.cls_off[NCLS];
+    s_meta[1] = BY_SLOT ? 0 : A.cls_off[NCLS];
     s_meta[2] = A.sub_meta[0];  // photons of all entries
     s_meta[3] = A.sub_meta[1];  // photon count before them
   }
@@ -850,19 +852,26 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
     const int64_t h = (int64_t)A.replay_list[q];
     // sub_cnt holds the exclusive prefix of the counts now
     const uint32_t off = A.sub_cnt[h];
-    const uint32_t cnt = (h + 1 < nh ? A.sub_cnt[h + 1] : total) - off;
-    const int32_t e = A.heavy_list[h];
+    // (by slot: all that the chain emits; the single pass counted the dropped)
+    const uint32_t cnt = BY_SLOT ? 0xFFFFFFFFu : (h + 1 < nh ? A.sub_cnt[h + 1] : total) - off;
+    const int32_t e = BY_SLOT ? -(int32_t)h - 1 : A.heavy_list[h];
     const int64_t out0 = nph + (int64_t)off;
     Entry<Real> P;
     load_entry<Real, FM, MODE>(A, e, T0, dt, P);
+    if (BY_SLOT && MODE != MODE_EMIT && FM != FM_GRID) {  // its stored position is the pushed one already
+      const Sp<Real> &S = A.sp[P.si];
+      P.x = S.x[P.i]; P.y = S.y[P.i]; P.z = S.z[P.i];
+    }
     Real nx, ny, nz;
     unit_dir(P, nx, ny, nz);
     Real g = P.g;
     auto put = [&](uint32_t j, Real eph, int64_t kk) {
       const int64_t out = out0 + j;
       if (out >= A.ph.cap) {
-        tl.dropped += 1;
-        tl.status |= QED_STATUS_CAPACITY;
+        if (!BY_SLOT) {
+          tl.dropped += 1;
+          tl.status |= QED_STATUS_CAPACITY;
+        }
         return;
       }
       U4 cid = draw(A.C, P.id, step_, kk, STREAM_PHOTON_ID);
@@ -891,7 +900,7 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
       chi = chi_lepton(pm2 * nx, pm2 * ny, pm2 * nz, g, E[0], E[1], E[2], B[0], B[1], B[2], inv_aS);
       ro = photon_rate(sR, sF, A.T, A.C, chi, g, dummy);
     }
-    if (j != cnt) {  // the replay disagreed with the count: zero-energy photons fill the slots
+    if (!BY_SLOT && j != cnt) {  // the replay disagreed with the count: zero-energy photons fill the slots
       tl.status |= QED_STATUS_REPLAY;
       for (; j < cnt; ++j) put(j, (Real)0, 0);
     }
@@ -2153,7 +2162,7 @@ static cudaError_t launch_lepton_t(qed_ctx *c, const LeptonArgs<Real> &a, cudaSt
   if (e == cudaSuccess) e = prof_mark(c, 4, st);
   if (e == cudaSuccess) e = launch_plain_kernel<Real>(c, k_substep_write_coop<Real, FM, MODE>, a, st);
   if (e == cudaSuccess)
-    e = launch_tables_kernel<Real>(c, k_substep_replay<Real, FM, MODE>, a, false, QED_TUNE_CHAINS, st);
+    e = launch_tables_kernel<Real>(c, k_substep_replay<Real, FM, MODE, false>, a, false, QED_TUNE_CHAINS, st);
   if (e == cudaSuccess) e = prof_mark(c, 5, st);
   return e;
 }
@@ -2167,19 +2176,37 @@ static cudaError_t launch_lepton_m(qed_ctx *c, const LeptonArgs<Real> &a, int fm
 
 cudaError_t launch_lepton_onepass(qed_ctx *c, const qed_species *s0, const qed_species *s1,
                                   const qed_species *ph, const qed_fields *f, int64_t step,
-                                  int mode, cudaStream_t st);
+                                  int mode, bool ordered, cudaStream_t st);
+
+// The replay of a single pass with ordered appends (the leptons whose records
+// found no room: more photons in the step than max_particles).
+template <int MODE>
+static cudaError_t launch_replay_by_slot(qed_ctx *c, const LeptonArgs<float> &a, int fm, cudaStream_t st) {
+  if (fm == QED_FIELDS_UNIFORM)
+    return launch_tables_kernel<float>(c, k_substep_replay<float, FM_UNIFORM, MODE, true>, a, false, QED_TUNE_CHAINS, st);
+  if (fm == QED_FIELDS_PER_PARTICLE)
+    return launch_tables_kernel<float>(c, k_substep_replay<float, FM_PER_PARTICLE, MODE, true>, a, false, QED_TUNE_CHAINS, st);
+  return launch_tables_kernel<float>(c, k_substep_replay<float, FM_GRID, MODE, true>, a, false, QED_TUNE_CHAINS, st);
+}
 
 template <class Real>
 cudaError_t launch_lepton(qed_ctx *c, const qed_species *s0, const qed_species *s1,
                           const qed_species *ph, const qed_fields *f, int64_t step, int mode,
                           cudaStream_t st) {
-  if (sizeof(Real) == 4 && mode != MODE_PUSH && c->cfg.append_order == QED_APPEND_ANY &&
-      c->cfg.generator == QED_GEN_METHOD_I) {
+  // FP32 contexts under Method I take the single pass; with ordered appends the
+  // learned sampler keeps the multi-pass path
+  const bool ordered = c->cfg.append_order == QED_APPEND_ORDERED;
+  const bool single = sizeof(Real) == 4 && mode != MODE_PUSH && c->cfg.generator == QED_GEN_METHOD_I &&
+                      !(ordered && c->cfg.sampler == QED_SAMPLER_MLP && c->mlp_ready);
+  if (single) {
     // marks: 1 after the single-pass kernel (recorded by it), 2..5 after the
-    // learned sampler's dense pass, if any
-    cudaError_t e = launch_lepton_onepass(c, s0, s1, ph, f, step, mode, st);
-    for (int k = 2; k <= 5 && e == cudaSuccess; ++k) e = prof_mark(c, k, st);
-    return e;
+    // learned sampler's dense pass or the ordered writes, if any
+    cudaError_t e = launch_lepton_onepass(c, s0, s1, ph, f, step, mode, ordered, st);
+    if (!ordered) {
+      for (int k = 2; k <= 5 && e == cudaSuccess; ++k) e = prof_mark(c, k, st);
+      return e;
+    }
+    if (e != cudaSuccess) return e;
   }
   LeptonArgs<Real> a{};
   a.sp[0] = to_sp<Real>(s0);
@@ -2214,6 +2241,15 @@ cudaError_t launch_lepton(qed_ctx *c, const qed_species *s0, const qed_species *
   a.emit_lanes = sched_param(c, QED_SCHED_EMIT_LANES);
   a.scan_draws = sched_param(c, QED_SCHED_SCAN_DRAWS);
   a.d_step = c->use_dstep ? c->d_step : nullptr;
+  if constexpr (sizeof(Real) == 4) {
+    if (single) {
+      a.replay_n = c->ord_n + 3;
+      cudaError_t e = mode == MODE_EMIT ? launch_replay_by_slot<MODE_EMIT>(c, a, f->mode, st)
+                                        : launch_replay_by_slot<MODE_FUSED>(c, a, f->mode, st);
+      for (int k = 2; k <= 5 && e == cudaSuccess; ++k) e = prof_mark(c, k, st);
+      return e;
+    }
+  }
   if (mode == MODE_PUSH) return launch_lepton_m<Real, MODE_PUSH>(c, a, f->mode, st);
   if (mode == MODE_EMIT) return launch_lepton_m<Real, MODE_EMIT>(c, a, f->mode, st);
   return launch_lepton_m<Real, MODE_FUSED>(c, a, f->mode, st);
