@@ -60,6 +60,14 @@ __device__ __forceinline__ Node load_node(const float *p, bool wide) {
   return n;
 }
 
+// Periodic index of an integral reduced coordinate: a particle in the box needs
+// no remainder (three 64-bit ones are a third of a grid step's instructions).
+template <class Real> __device__ __forceinline__ int wrap_cell(Real f, int n) {
+  if (f >= (Real)0 && f < (Real)n) return (int)f;
+  long long i = (long long)f % n;
+  return (int)(i < 0 ? i + n : i);
+}
+
 // CIC gather from grid[nz][ny][nx][8] (periodic).
 template <class Real>
 __device__ __forceinline__ void cic_gather(const Fld<Real> &f, Real x, Real y, Real z, Real E[3],
@@ -67,28 +75,26 @@ __device__ __forceinline__ void cic_gather(const Fld<Real> &f, Real x, Real y, R
   Real fx = (x - f.x0) * f.idx, fy = (y - f.y0) * f.idy, fz = (z - f.z0) * f.idz;
   Real ix = m_floor(fx), iy = m_floor(fy), iz = m_floor(fz);
   Real wx = fx - ix, wy = fy - iy, wz = fz - iz;
-  long long i0 = (long long)ix, j0 = (long long)iy, k0 = (long long)iz;
-  i0 %= f.nx; if (i0 < 0) i0 += f.nx;
-  j0 %= f.ny; if (j0 < 0) j0 += f.ny;
-  k0 %= f.nz; if (k0 < 0) k0 += f.nz;
-  long long i1 = i0 + 1 == f.nx ? 0 : i0 + 1;
-  long long j1 = j0 + 1 == f.ny ? 0 : j0 + 1;
-  long long k1 = k0 + 1 == f.nz ? 0 : k0 + 1;
+  const int i0 = wrap_cell(ix, f.nx), j0 = wrap_cell(iy, f.ny), k0 = wrap_cell(iz, f.nz);
+  const int i1 = i0 + 1 == f.nx ? 0 : i0 + 1;
+  const int j1 = j0 + 1 == f.ny ? 0 : j0 + 1;
+  const int k1 = k0 + 1 == f.nz ? 0 : k0 + 1;
 #pragma unroll
   for (int c = 0; c < 3; ++c) { E[c] = (Real)0; B[c] = (Real)0; }
   const bool wide = (reinterpret_cast<uintptr_t>(f.grid) & 31) == 0;
 #pragma unroll
   for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
-    for (int dj = 0; dj < 2; ++dj)
+    for (int dj = 0; dj < 2; ++dj) {
+      const float *row = f.grid + 8 * (((long long)(dk ? k1 : k0) * f.ny + (dj ? j1 : j0)) * f.nx);
 #pragma unroll
       for (int di = 0; di < 2; ++di) {
         Real w = (di ? wx : (Real)1 - wx) * (dj ? wy : (Real)1 - wy) * (dk ? wz : (Real)1 - wz);
-        long long node = ((dk ? k1 : k0) * f.ny + (dj ? j1 : j0)) * f.nx + (di ? i1 : i0);
-        const Node n = load_node(f.grid + 8 * node, wide);
+        const Node n = load_node(row + 8 * (long long)(di ? i1 : i0), wide);
 #pragma unroll
         for (int c = 0; c < 3; ++c) { E[c] += w * (Real)n.v[c]; B[c] += w * (Real)n.v[3 + c]; }
       }
+    }
 }
 
 // Relativistic Boris push; returns gamma after the push.

@@ -79,6 +79,13 @@ template <class Real> struct LeptonArgs {
 };
 
 
+// First slot of a thread: consecutive slices of 32 go to different CTAs, so that
+// a small species is spread over the SMs (FP64 runs at 2 FMAs per clock and SM:
+// 10^4 electrons in 40 CTAs of 256 took 26 us, over all SMs 11).
+__device__ __forceinline__ int64_t spread_slot() {
+  return ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+}
+
 // ---------------------------------------------------------------------------
 // Push-only pass (qed_gather_push): field gather, Boris push and position
 // update of every lepton; no emission, so no ordering is needed.
@@ -94,8 +101,7 @@ __global__ void __launch_bounds__(TILE) k_lepton_push(LeptonArgs<Real> A) {
   const int64_t n0 = s_meta[0], n1 = s_meta[1];
   const Real dt = sel<Real>(A.C.dt, A.C.f_dt);
   uint32_t status = 0;
-  for (int64_t g = blockIdx.x * (int64_t)TILE + threadIdx.x; g < n0 + n1;
-       g += (int64_t)gridDim.x * TILE) {
+  for (int64_t g = spread_slot(); g < n0 + n1; g += (int64_t)gridDim.x * TILE) {
     const int si = g < n0 ? 0 : 1;
     const Sp<Real> &S = A.sp[si];
     const int64_t i = si ? g - n0 : g;
@@ -176,7 +182,7 @@ __global__ void __launch_bounds__(TILE, sizeof(Real) == 4 ? 3 : 2) k_lepton_stre
   };
   const int64_t stride = (int64_t)gridDim.x * TILE;
   int buf = 0;
-  int64_t slot = blockIdx.x * (int64_t)TILE + threadIdx.x;
+  int64_t slot = spread_slot();
   if (slot < nslots) prefetch(slot, 0);
   cp_async_commit();
   // nslots is a multiple of TILE: every lane of a warp runs the same iterations
@@ -327,7 +333,7 @@ constexpr int REC = SUB_REC;
 // Work scheduling of the counting pass: a lane is idle (no particle), scanning
 // (drawing sub-steps) or pending (an event found, its emission not yet done).
 enum { LS_IDLE = 0, LS_SCAN = 1, LS_PEND = 2 };
-constexpr int CNT_CHUNK = 64;       // entries per queue chunk of a warp
+constexpr int CNT_CHUNK = 64, CNT_CHUNK_MIN = 16;  // entries per queue chunk of a warp
 // An emission round waits for A.emit_lanes lanes with an event, a refill
 // round for CNT_MIN_INIT idle lanes; a scanning round draws A.scan_draws
 // sub-steps per lane.
@@ -462,12 +468,15 @@ __global__ void __launch_bounds__(TILE, sizeof(Real) == 4 && !MLP ? 3 : 2) k_sub
   const int64_t rc = A.rec_cap;
   Tally tl;
   tl.clear();
-  // This warp's queue: chunks w, w + W, w + 2W, ... of CNT_CHUNK entries,
-  // counted from the end of the list (the heaviest classes first).
+  // This warp's queue: chunks w, w + W, w + 2W, ... of `chunk` entries, counted
+  // from the end of the list (the heaviest classes first).  The first chunks
+  // go to different CTAs, and a short list is cut into smaller ones, so that
+  // its chains run on all SMs (250 FP64 entries: 62 us on one SM).
   const int64_t W = (int64_t)gridDim.x * (TILE / 32);
-  const int64_t w = blockIdx.x * (int64_t)(TILE / 32) + (threadIdx.x >> 5);
-  const int64_t nchunks = (nh + CNT_CHUNK - 1) / CNT_CHUNK;
-  const int64_t qend = w < nchunks ? ((nchunks - 1 - w) / W + 1) * CNT_CHUNK : 0;
+  const int64_t w = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const int chunk = nh >= W * CNT_CHUNK ? CNT_CHUNK : CNT_CHUNK_MIN;
+  const int64_t nchunks = (nh + chunk - 1) / chunk;
+  const int64_t qend = w < nchunks ? ((nchunks - 1 - w) / W + 1) * chunk : 0;
   int64_t next = 0;  // queue position (warp-uniform)
   // lane state
   int state = LS_IDLE;
@@ -510,7 +519,7 @@ __global__ void __launch_bounds__(TILE, sizeof(Real) == 4 && !MLP ? 3 : 2) k_sub
       // refill: the idle lanes take the next queue positions, in lane order
       if (state == LS_IDLE) {
         const int64_t q = next + __popc(idle & lt_mask);
-        const int64_t hr = q < qend ? (w + (q / CNT_CHUNK) * W) * CNT_CHUNK + (q % CNT_CHUNK) : nh;
+        const int64_t hr = q < qend ? (w + (q / chunk) * W) * chunk + (q % chunk) : nh;
         if (hr < nh) {
           h = nh - 1 - hr;
           Entry<Real> P;
