@@ -156,14 +156,13 @@ class Species:
         return out
 
     def struct(self) -> B.qed_species:
-        s = B.qed_species()
-        for k in STATE + FIELD_NAMES + ("id", "alive", "tag", "od_p", "od_r"):
-            t = getattr(self, k)
-            setattr(s, k, t.data_ptr() if t is not None and t.numel() else None)
-        s.d_n = self.n.data_ptr()
-        s.capacity = self.capacity
-        s.q = self.q
-        return s
+        # positional, in the order of qed_species: set one attribute at a time it
+        # took longer than the launches of a small step
+        n = self.x.numel()
+        p = [t.data_ptr() if n and t is not None else None
+             for t in (self.x, self.y, self.z, self.px, self.py, self.pz, self.w, self.id, self.alive,
+                       self.ex, self.ey, self.ez, self.bx, self.by, self.bz, self.tag, self.od_p, self.od_r)]
+        return B.qed_species(*p[:15], self.n.data_ptr(), n, self.q, 0, *p[15:])
 
 
 class Fields:

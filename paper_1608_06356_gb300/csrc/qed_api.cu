@@ -83,9 +83,9 @@ static void free_ctx(qed_ctx *c) {
   free_host_step(c);
   void *ptrs[] = {c->R64, c->F64, c->Y64, c->P64, c->Yp64, c->R32, c->F32, c->Y32,
                   c->P32, c->Yp32, c->tile_state, c->sync, c->snap, c->pic_n, c->d_counters,
-                  c->heavy_flags, c->heavy_list, c->heavy_n, c->cls_chunk_cnt,
+                  c->heavy_flags, c->heavy_list, c->pair_n, c->pair_sum, c->cls_chunk_cnt,
                   c->cls_chunk_off, c->cls_off, c->sub_cnt, c->sub_gf, c->rec_e,
-                  c->rec_k, c->sub_meta, c->fill_meta, c->ord_n, c->replay_n, c->stage, c->stage_tag,
+                  c->rec_k, c->sub_meta, c->fill_meta, c->ord_n, c->compact_n, c->replay_n, c->stage, c->stage_tag,
                   c->stage_idx, c->stage_n, c->probe_state,
                   c->mlp_mem, c->w_up_row, c->net_rec, c->net_n};
   for (void *p : ptrs)
@@ -260,11 +260,11 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   c->cls_chunks = c->heavy_slots / CLS_CHUNK_FLAGS + 1;
   // emission records for the first max_particles / 4 entries of the sub-step
   // list; later entries (and particles with more than SUB_REC photons) replay
-  c->rec_cap = cfg->max_particles / 4 > 4096 ? cfg->max_particles / 4 : 4096;
+  c->rec_cap = cfg->max_particles / 4 > 4096 ? cfg->max_particles / 4 + 1 : 4096;
   const size_t rsize = f64 ? sizeof(double) : sizeof(float);
   // staging records for the leptons the streaming pass defers (a record is
   // 16 words); past stage_cap a deferred particle is gathered from its arrays
-  c->stage_cap = cfg->max_particles / 2 > 65536 ? cfg->max_particles / 2 : 65536;
+  c->stage_cap = cfg->max_particles / 2 > 65536 ? cfg->max_particles / 2 + 1 : 65536;
   if (cudaMalloc(&c->tile_state, sizeof(unsigned long long) * c->max_tiles) != cudaSuccess ||
       cudaMalloc(&c->sync, sizeof(unsigned int) * 4) != cudaSuccess ||
       cudaMalloc(&c->snap, sizeof(int64_t) * 4) != cudaSuccess ||
@@ -272,7 +272,8 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
       cudaMalloc(&c->d_counters, sizeof(qed_counters)) != cudaSuccess ||
       cudaMalloc(&c->heavy_flags, (size_t)c->heavy_slots + 4096) != cudaSuccess ||
       cudaMalloc(&c->heavy_list, sizeof(int) * (size_t)c->heavy_slots) != cudaSuccess ||
-      cudaMalloc(&c->heavy_n, sizeof(int64_t)) != cudaSuccess ||
+      cudaMalloc(&c->pair_n, 2 * sizeof(unsigned int)) != cudaSuccess ||
+      cudaMalloc(&c->pair_sum, sizeof(uint32_t) * (size_t)c->cls_chunks) != cudaSuccess ||
       cudaMalloc(&c->cls_chunk_cnt, sizeof(unsigned long long) * (size_t)c->cls_chunks) != cudaSuccess ||
       cudaMalloc(&c->cls_chunk_off, sizeof(uint32_t) * 5 * (size_t)c->cls_chunks) != cudaSuccess ||
       cudaMalloc(&c->cls_off, sizeof(int64_t) * 8) != cudaSuccess ||
@@ -285,8 +286,9 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
       cudaMalloc(&c->stage_idx, sizeof(int32_t) * (size_t)c->heavy_slots) != cudaSuccess ||
       cudaMalloc(&c->stage_n, sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->sub_meta, 4 * sizeof(int64_t)) != cudaSuccess ||
-      cudaMalloc(&c->fill_meta, 2 * sizeof(int64_t)) != cudaSuccess ||
+      cudaMalloc(&c->fill_meta, 3 * sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&c->ord_n, 4 * sizeof(unsigned int)) != cudaSuccess ||
+      cudaMalloc(&c->compact_n, 3 * sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->replay_n, sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->probe_state, 2 * sizeof(unsigned long long)) != cudaSuccess) {
     free_ctx(c);
@@ -296,6 +298,9 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   if (e == cudaSuccess) e = cudaMemsetAsync(c->sync, 0, sizeof(unsigned int) * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->snap, 0, sizeof(int64_t) * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counters, 0, sizeof(qed_counters), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->pair_n, 0, 2 * sizeof(unsigned int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->pair_sum, 0, sizeof(uint32_t) * (size_t)c->cls_chunks, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->compact_n, 0, 3 * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ord_n, 0, 4 * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->stage_n, 0, sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->probe_state, 0, 2 * sizeof(unsigned long long), st);

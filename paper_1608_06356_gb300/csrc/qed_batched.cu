@@ -12,23 +12,24 @@ __global__ void k_step_advance(int64_t *d_step) { *d_step += 1; }
 
 __global__ void k_step_set(int64_t *d_step, int64_t v) { *d_step = v; }
 
-// Alive photons per tag (run index).
+// Alive photons per tag (run index).  32-bit counts in shared memory: photons
+// of a run lie together, and an SM adds a warp's 32-bit counts on one address
+// at full rate, 64-bit ones one by one.
 __global__ void k_tag_count(const uint8_t *alive, const uint32_t *tag, const int64_t *d_n,
                             int n_runs, int64_t *out) {
-  extern __shared__ unsigned long long s_cnt[];
-  for (int r = threadIdx.x; r < n_runs; r += blockDim.x) s_cnt[r] = 0ull;
+  extern __shared__ unsigned int s_cnt[];
+  for (int r = threadIdx.x; r < n_runs; r += blockDim.x) s_cnt[r] = 0u;
   __syncthreads();
   const int64_t n = *d_n;
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    if (alive[i]) {
-      uint32_t t = tag[i];
-      if (t < (uint32_t)n_runs) atomicAdd(&s_cnt[t], 1ull);
-    }
+    const uint32_t t = tag[i];
+    if (alive[i] && t < (uint32_t)n_runs) atomicAdd(&s_cnt[t], 1u);
   }
   __syncthreads();
   for (int r = threadIdx.x; r < n_runs; r += blockDim.x)
-    if (s_cnt[r]) atomicAdd(reinterpret_cast<unsigned long long *>(&out[r]), s_cnt[r]);
+    if (s_cnt[r]) atomicAdd(reinterpret_cast<unsigned long long *>(&out[r]), (unsigned long long)s_cnt[r]);
 }
 
 }  // namespace qed
@@ -122,7 +123,7 @@ extern "C" int qed_run_batched(qed_ctx *c, const qed_species *e, const qed_speci
   if (d_run_photons) {
     err = cudaMemsetAsync(d_run_photons, 0, sizeof(int64_t) * n_runs, st);
     if (err == cudaSuccess) {
-      k_tag_count<<<c->num_sms * 2, 256, sizeof(unsigned long long) * n_runs, st>>>(
+      k_tag_count<<<c->num_sms * 4, 256, sizeof(unsigned int) * n_runs, st>>>(
           g->alive, g->tag, g->d_n, n_runs, d_run_photons);
       err = cudaGetLastError();
     }

@@ -26,7 +26,6 @@ struct qed_ctx {
   int64_t heavy_slots;   // block-tile slots of both lepton species
   uint8_t *heavy_flags;  // [heavy_slots] streaming-pass class flags
   int *heavy_list;       // [heavy_slots] ordered deferred slots
-  int64_t *heavy_n;      // length of heavy_list (photon pass)
   // class list of the streaming lepton pass: per-chunk packed counts and
   // per-class offsets, class starts
   unsigned long long *cls_chunk_cnt;  // [cls_chunks]
@@ -39,8 +38,11 @@ struct qed_ctx {
   void *rec_e;        // Real [SUB_REC][rec_cap]
   uint32_t *rec_k;    // [SUB_REC][rec_cap]
   int64_t rec_cap;
-  int64_t *sub_meta;  // [4] appends of the emission (or pair) entries, counts before them
-  int64_t *fill_meta; // [2] count before and after a hole-filling compaction
+  int64_t *sub_meta;  // [4] photons of the emission entries, counts before them (or before the pairs)
+  int64_t *fill_meta; // [3] count before and after a hole-filling compaction, holes
+  unsigned int *compact_n; // [3] stable compaction: tiles taken, CTAs done, waits that ran out
+  unsigned int *pair_n;    // [2] pairs of the photon stage: records, those being written
+  uint32_t *pair_sum;      // [cls_chunks] pairs per chunk of photons (zero between steps)
   unsigned int *ord_n;     // [4] ordered appends of the single pass: records and replays asked for, of the pass being written
   unsigned int *replay_n;  // entries the writing pass leaves to its replay launch
   unsigned long long *probe_state;  // [2] look-back words of qed_test_wait_expiry (tile 0 never published)

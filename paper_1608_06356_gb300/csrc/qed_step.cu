@@ -1,22 +1,22 @@
-// qed_step.cu -- the per-macroparticle QED Monte Carlo step on sm_103a.
+// qed_step.cu -- the per-macroparticle QED Monte Carlo step on sm_103a: the push,
+// the multi-pass lepton step (FP64 contexts, Methods II and III, the learned
+// sampler with ordered appends; the others take the single pass of
+// qed_onepass.cu), compaction, the isolated sampler and the parity hooks.  The
+// photons' stage is qed_photon.cu's.
 //
-// What is computed per particle:
-//   leptons: field gather (uniform / per-particle / CIC) -> Boris push ->
-//            chi_e (Eq. 2) -> W_rad from the tables (Eq. 1 with the xi_min
-//            cut) -> N = max(1, ceil(W Dt / 0.2)) sub-steps -> Method I events
-//            with Philox draws -> xi from Eq. (7) -> recoil; photons appended.
-//   photons: ballistic push -> chi_ph (Eq. 3) -> W_pair (Eq. 6) -> Method I ->
-//            pair split xi (Eq. 6) -> e-/e+ appended, photon marked dead.
-// How the lepton step is laid out: a streaming pass reads every particle once
-// (coalesced), pushes it and decides with a cheap upper bound of the rate
-// whether it surely has N = 1 and no event; those (most) are finished there.
-// The rest are staged as 64-byte records, ordered by a class list (binned by
-// N so that lanes of a warp do similar work), and run through a counting
-// pass, a scan and a writing pass that append their photons in list order.
-// Photons: a streaming pass, then an ordered pass over the flagged ones.
-// Appends keep a deterministic order (and sub-step order within a particle);
-// ordered passes scan within the block and across tiles by a single-pass
-// decoupled look-back, so slot = count at launch + global prefix.
+// What is computed per lepton: field gather (uniform / per-particle / CIC) ->
+// Boris push -> chi_e (Eq. 2) -> W_rad from the tables (Eq. 1 with the xi_min
+// cut) -> N = max(1, ceil(W Dt / 0.2)) sub-steps -> Method I events with Philox
+// draws -> xi from Eq. (7) -> recoil; photons appended.
+// How the multi-pass step is laid out: a streaming pass reads every particle
+// once (coalesced), pushes it and evaluates the rate and the first draw; those
+// with one sub-step and no event (most) are finished there.  The rest are
+// staged as 64-byte records, ordered by a class list (binned by N so that
+// lanes of a warp do similar work), and run through a counting pass, a scan
+// and a writing pass that append their photons in list order.  Appends keep a
+// deterministic order (and sub-step order within a particle); the scan works
+// within the block and across tiles by a single-pass decoupled look-back, so
+// slot = count at launch + global prefix.
 // Particle state is structure-of-arrays; loads and stores of a tile are
 // coalesced 4-byte (FP32) or 8-byte (FP64) accesses.
 #include <cstdio>
@@ -56,7 +56,6 @@ template <class Real> struct LeptonArgs {
   int64_t step;
   uint8_t *heavy_flags;     // [streaming-pass slot] class flag (0 = finished)
   const int *heavy_list;    // class list: staging record or -(slot + 1), class-major
-  const int64_t *heavy_n;   // length of heavy_list
   const int64_t *d_step;    // if set, the step index is read here (graph replay)
   const int64_t *cls_off;   // class list: class c occupies [cls_off[c-1], cls_off[c])
   Stage<Real> *stage;       // pushed state of the flagged leptons (streaming pass)
@@ -744,9 +743,9 @@ struct SubScanArgs {
   uint32_t *cnt;
   unsigned int *replay_n;  // reset here for the writing pass
   const int64_t *n_entries;
-  int64_t *sub_meta;       // [0] total, [1] count of out1 before, [2] count of out2 before
-  int64_t *out1_n, *out2_n;  // species counts to advance by the total (out2 optional)
-  int64_t out1_cap, out2_cap;
+  int64_t *sub_meta;       // [0] total, [1] photon count before
+  int64_t *out_n;          // the photon count, advanced by the total
+  int64_t out_cap;
   Out o;
 };
 constexpr int SCAN_ITEMS = 16;
@@ -756,12 +755,11 @@ __global__ void __launch_bounds__(TILE) k_sub_scan(SubScanArgs A) {
   __shared__ long long s_meta[6];
   if (threadIdx.x == 0) {
     s_meta[2] = *(volatile const int64_t *)A.n_entries;
-    s_meta[3] = *(volatile int64_t *)A.out1_n;
+    s_meta[3] = *(volatile int64_t *)A.out_n;
     s_meta[4] = (long long)A.o.scan.sync[2];
-    s_meta[5] = A.out2_n ? *(volatile int64_t *)A.out2_n : 0;
   }
   __syncthreads();
-  const int64_t nh = s_meta[2], nph = s_meta[3], n2 = s_meta[5];
+  const int64_t nh = s_meta[2], nph = s_meta[3];
   const uint32_t epoch = (uint32_t)s_meta[4];
   const int64_t per_tile = (int64_t)TILE * SCAN_ITEMS;
   const int64_t ntiles = (nh + per_tile - 1) / per_tile;
@@ -771,7 +769,6 @@ __global__ void __launch_bounds__(TILE) k_sub_scan(SubScanArgs A) {
     if (ntiles == 0) {
       A.sub_meta[0] = 0;
       A.sub_meta[1] = nph;
-      A.sub_meta[2] = n2;
     }
   }
   for (;;) {
@@ -798,9 +795,7 @@ __global__ void __launch_bounds__(TILE) k_sub_scan(SubScanArgs A) {
           const int64_t tot = (int64_t)pre + agg;
           A.sub_meta[0] = tot;
           A.sub_meta[1] = nph;
-          A.sub_meta[2] = n2;
-          *A.out1_n = nph + tot < A.out1_cap ? nph + tot : A.out1_cap;
-          if (A.out2_n) *A.out2_n = n2 + tot < A.out2_cap ? n2 + tot : A.out2_cap;
+          *A.out_n = nph + tot < A.out_cap ? nph + tot : A.out_cap;
         }
       }
     }
@@ -918,79 +913,6 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
   tally_flush(&bt, tl);
   __syncthreads();
   block_tally_commit(&bt, A.o.cnt, 0);
-}
-
-// ---------------------------------------------------------------------------
-// Ordered list of the deferred (heavy) particles: stable compaction of the
-// streaming pass's flags, one flag per slot (tile * TILE + lane).
-// ---------------------------------------------------------------------------
-struct HeavyListArgs {
-  const uint8_t *flags;
-  uint8_t want;  // flag value to collect
-  const int32_t *stage_idx;  // if set: list the staging record (or -(slot + 1))
-  int *list;
-  int64_t *count;
-  const int64_t *n0, *n1;  // species counts (size the streaming pass's slot range)
-  Out o;
-};
-
-constexpr int LIST_ITEMS = 16;  // flags per thread (one 16-byte load)
-
-__global__ void __launch_bounds__(TILE) k_heavy_list(HeavyListArgs A) {
-  __shared__ uint32_t scan_sm[33];
-  __shared__ long long s_meta[8];
-  if (threadIdx.x == 0) {
-    int64_t n0 = *(volatile const int64_t *)A.n0;
-    int64_t n1 = A.n1 ? *(volatile const int64_t *)A.n1 : 0;
-    s_meta[2] = ((n0 + TILE - 1) / TILE + (n1 + TILE - 1) / TILE) * TILE;  // flag slots
-    s_meta[5] = (long long)A.o.scan.sync[2];
-  }
-  __syncthreads();
-  const int64_t nslots = s_meta[2];
-  const int64_t per_tile = (int64_t)TILE * LIST_ITEMS;
-  const int64_t ntiles = (nslots + per_tile - 1) / per_tile;
-  const uint32_t epoch = (uint32_t)s_meta[5];
-  uint32_t status = 0;
-  if (ntiles == 0 && blockIdx.x == 0 && threadIdx.x == 0) *A.count = 0;
-  for (;;) {
-    if (threadIdx.x == 0) s_meta[0] = (long long)atomicAdd(&A.o.scan.sync[0], 1u);
-    __syncthreads();
-    const int64_t t = s_meta[0];
-    __syncthreads();
-    if (t >= ntiles) break;
-    const int64_t first = t * per_tile + (int64_t)threadIdx.x * LIST_ITEMS;
-    uint4 raw = make_uint4(0, 0, 0, 0);
-    if (first < nslots) raw = *reinterpret_cast<const uint4 *>(A.flags + first);
-    const uint8_t *fl = reinterpret_cast<const uint8_t *>(&raw);
-    uint32_t mask = 0;
-#pragma unroll
-    for (int j = 0; j < LIST_ITEMS; ++j)
-      if (fl[j] == A.want && first + j < nslots) mask |= 1u << j;
-    uint32_t cnt = __popc(mask);
-    uint32_t excl = block_excl_scan(cnt, scan_sm);
-    uint32_t agg = scan_sm[32];
-    if (threadIdx.x < 32) {
-      uint32_t pre = lookback_warp(A.o.scan, t, epoch, agg, status);
-      if (threadIdx.x == 0) {
-        s_meta[1] = pre;
-        if (t == ntiles - 1) *A.count = (int64_t)pre + agg;
-      }
-    }
-    __syncthreads();
-    int64_t out = s_meta[1] + excl;
-    while (mask) {
-      int j = __ffs(mask) - 1;
-      mask &= mask - 1;
-      int v = (int)(first + j);
-      if (A.stage_idx) {
-        const int32_t sidx = A.stage_idx[first + j];
-        v = sidx >= 0 ? sidx : -v - 1;
-      }
-      A.list[out++] = v;
-    }
-  }
-  if (threadIdx.x == 0 && status) atomicOr(&A.o.cnt->status, status);
-  launch_epilogue(A.o.scan, epoch);
 }
 
 // ---------------------------------------------------------------------------
@@ -1190,431 +1112,223 @@ __global__ void __launch_bounds__(TILE) k_cls_scatter(ClassListArgs A) {
 }
 
 // ---------------------------------------------------------------------------
-// Photon kernel: push + Breit-Wheeler pairs
+// Stable in-place compaction of dead particles (alive == 0): the live particles
+// of every tile are counted (from the flags alone), the counts scanned, and the
+// tiles moved.  A moving tile reads its particles into registers, publishes
+// that, waits until the tiles whose range it writes to -- at most two, which
+// lie before it by the particles dead so far -- have published too, and writes:
+// no word is overwritten before it has been read.  Tiles are taken in order, so
+// the ones waited for are under way.  The wait is bounded.  (8.4M photons of 61
+// bytes, one in ten dead: 268 us with the positions from a look-back, which
+// had each tile wait for the sums of all before it, one 2048-particle tile of
+// 1024 threads in flight per SM; COMPACT_US this way, 135 at the copy rate.)
 // ---------------------------------------------------------------------------
-template <class Real> struct PhotonArgs {
-  Sp<Real> ph, el, po;
-  const int64_t *n_active;  // photons [0, *n_active) are processed
-  Fld<Real> f;
-  Consts C;
-  Tables<Real> T;
-  Out o;
-  int64_t step;
-  uint8_t *flags;       // streaming pass: 1 = redo in the ordered pass
-  const int *list;      // ordered pass: staging record (>= 0) or -(index + 1)
-  Stage<Real> *stage;   // pushed state of the flagged photons (streaming pass)
-  uint32_t *stage_tag;
-  int32_t *stage_idx;   // [index] staging record of a flagged photon, -1 if not staged
-  unsigned int *stage_n;
-  int64_t stage_cap;
-  const int64_t *list_n;
-  const int64_t *d_step;  // if set, the step index is read here (graph replay)
-  uint32_t *sub_cnt;      // pairs per list entry, then their exclusive prefix
-  const int64_t *sub_meta;  // [0] pairs in all, [1] electrons before, [2] positrons before
-  Real *rec_e;            // [0][h] gamma_e, [1][h] gamma_p of entry h's pair (h < rec_cap)
-  uint32_t *rec_k;        // [h] its sub-step
-  int64_t rec_cap;
-};
-
-// ---------------------------------------------------------------------------
-// Streaming photon pass: ballistic push, chi_ph, pair rate and the first
-// Method I draw, with no block-wide synchronisation.  Photons with one
-// sub-step and no event are finished here; the rest are flagged and redone
-// by the pair passes over the list (k_pair_count, k_pair_write).
-// ---------------------------------------------------------------------------
-template <class Real, int FM>
-__global__ void __launch_bounds__(TILE, sizeof(Real) == 4 ? 4 : 2) k_photon_stream(PhotonArgs<Real> A) {
-  const int64_t step_ = A.d_step ? *A.d_step : A.step;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Real *sP = reinterpret_cast<Real *>(smem_raw);
-  __shared__ long long s_meta[2];
-  __shared__ BlockTally bt;
-  load_tables_smem(sP, A.T.P, A.T.glp.n);
-  block_tally_init(&bt);
-  if (threadIdx.x == 0) s_meta[0] = *(volatile const int64_t *)A.n_active;
-  __syncthreads();
-  const int64_t n = s_meta[0];
-  const int64_t nslots = (n + TILE - 1) / TILE * TILE;
-  const Real inv_aS = sel<Real>(A.C.inv_aS, A.C.f_inv_aS);
-  const Real dt = sel<Real>(A.C.dt, A.C.f_dt), wdt_max = sel<Real>(A.C.wdt_max, A.C.f_wdt_max);
-  const int lane = threadIdx.x & 31;
-  uint32_t batch_base = 0, batch_used = STAGE_BATCH;  // this warp's staging batch
-  Tally tl;
-  tl.clear();
-  // nslots is a multiple of TILE: every lane of a warp runs the same iterations
-  for (int64_t i = blockIdx.x * (int64_t)TILE + threadIdx.x; i < nslots;
-       i += (int64_t)gridDim.x * TILE) {
-    uint8_t flag = 0;
-    Real x = 0, y = 0, z = 0, px = 0, py = 0, pz = 0;
-    Real E[3] = {0, 0, 0}, B[3] = {0, 0, 0};
-    uint64_t pid = 0;
-    if (i < n && A.ph.alive[i]) {
-      x = A.ph.x[i]; y = A.ph.y[i]; z = A.ph.z[i];
-      px = A.ph.px[i]; py = A.ph.py[i]; pz = A.ph.pz[i];
-      get_fields<Real, FM>(A.ph, A.f, i, x, y, z, E, B);
-      Real k = m_sqrt(px * px + py * py + pz * pz);
-      Real chi = chi_photon(px, py, pz, E[0], E[1], E[2], B[0], B[1], B[2], inv_aS);
-      Tally t0;
-      t0.clear();
-      RateOut<Real> ro = pair_rate(sP, A.T, A.C, chi, k, t0);
-      Real wdt = ro.W * dt;
-      if (wdt > wdt_max) {
-        flag = 1;
-        pid = A.ph.id[i];
-      } else if (ro.W > (Real)0) {  // (most soft photons have W = 0: no id read)
-        pid = A.ph.id[i];
-        U4 r = draw(A.C, pid, step_, 0, STREAM_PAIR);
-        if (wdt > unif<Real>(r.x)) flag = 1;
-      }
-      if (k > (Real)0) {
-        Real ik = dt / k;
-        x += px * ik; y += py * ik; z += pz * ik;
-      }
-      if (!flag) {
-        tl.substeps += 1;
-        tl.status |= t0.status;
-        tl.domain += t0.domain;
-        if (k > (Real)0) { A.ph.x[i] = x; A.ph.y[i] = y; A.ph.z[i] = z; }
-      }
-    }
-    A.flags[i] = flag;
-    // stage the flagged photons (warp-collective)
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, flag != 0);
-    if (m) {
-      const uint32_t cm = __popc(m);
-      if (batch_used + cm > STAGE_BATCH) {
-        uint32_t nb = 0;
-        if (lane == 0) nb = atomicAdd(A.stage_n, STAGE_BATCH);
-        batch_base = __shfl_sync(0xFFFFFFFFu, nb, 0);
-        batch_used = 0;
-      }
-      if (flag) {
-        const uint64_t pos = (uint64_t)batch_base + batch_used + __popc(m & ((1u << lane) - 1u));
-        int32_t sidx = -1;
-        if (pos < (uint64_t)A.stage_cap) {
-          sidx = (int32_t)pos;
-          Stage<Real> r;
-          r.p[0] = px; r.p[1] = py; r.p[2] = pz;
-          r.e[0] = E[0]; r.e[1] = E[1]; r.e[2] = E[2];
-          r.b[0] = B[0]; r.b[1] = B[1]; r.b[2] = B[2];
-          r.id_lo = (uint32_t)pid; r.id_hi = (uint32_t)(pid >> 32);
-          r.w = A.ph.w[i];
-          r.x[0] = x; r.x[1] = y; r.x[2] = z;
-          r.slot = (uint32_t)i;
-          const uint4 *src = reinterpret_cast<const uint4 *>(&r);
-          uint4 *dst = reinterpret_cast<uint4 *>(A.stage + pos);
-#pragma unroll
-          for (int q = 0; q < (int)(sizeof(Stage<Real>) / 16); ++q) dst[q] = src[q];
-          if (A.ph.tag) A.stage_tag[pos] = A.ph.tag[i];
-          // the pushed position does not depend on the pair decision
-          A.ph.x[i] = x; A.ph.y[i] = y; A.ph.z[i] = z;
-        }
-        A.stage_idx[i] = sidx;
-      }
-      batch_used += cm;
-    }
-  }
-  tally_flush(&bt, tl);
-  __syncthreads();
-  block_tally_commit(&bt, A.o.cnt, 1);
-}
-
-// ---------------------------------------------------------------------------
-// Pair passes over the list of flagged photons (list order = photon index
-// order), split like the lepton emission passes: a counting pass with no
-// ordering (the photon's Method I chain: at most one pair, after which the
-// photon is dead), the in-place scan of the counts, and a writing pass that
-// appends the e-/e+ of each pair at its scanned slot.
-// ---------------------------------------------------------------------------
-template <class Real> struct PhotonEntry {
-  Real x, y, z, px, py, pz, k, w;
-  Real E[3], B[3];
-  uint64_t id;
-  uint32_t tag;
-  int64_t i;  // photon index
-};
-
-// List entry e >= 0: staging record e (pushed position already stored);
-// e < 0: photon -e-1, which the counting pass (COUNT) pushes and stores and
-// the writing pass reads back already pushed.
-template <class Real, int FM, bool COUNT>
-__device__ __forceinline__ void load_photon(const PhotonArgs<Real> &A, int32_t e, Real dt,
-                                            PhotonEntry<Real> &P) {
-  if (e >= 0) {
-    Stage<Real> r;
-    const uint4 *src = reinterpret_cast<const uint4 *>(A.stage + e);
-    uint4 *dst = reinterpret_cast<uint4 *>(&r);
-#pragma unroll
-    for (int q = 0; q < (int)(sizeof(Stage<Real>) / 16); ++q) dst[q] = src[q];
-    P.px = r.p[0]; P.py = r.p[1]; P.pz = r.p[2];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) { P.E[c] = r.e[c]; P.B[c] = r.b[c]; }
-    P.id = (uint64_t)r.id_lo | ((uint64_t)r.id_hi << 32);
-    P.w = r.w;
-    P.x = r.x[0]; P.y = r.x[1]; P.z = r.x[2];
-    P.i = r.slot;
-    P.tag = A.ph.tag ? A.stage_tag[e] : 0u;
-    P.k = m_sqrt(P.px * P.px + P.py * P.py + P.pz * P.pz);
-    return;
-  }
-  const int64_t i = -(int64_t)e - 1;
-  P.i = i;
-  P.x = A.ph.x[i]; P.y = A.ph.y[i]; P.z = A.ph.z[i];
-  P.px = A.ph.px[i]; P.py = A.ph.py[i]; P.pz = A.ph.pz[i];
-  P.w = A.ph.w[i];
-  P.id = A.ph.id[i];
-  P.tag = A.ph.tag ? A.ph.tag[i] : 0u;
-  get_fields<Real, FM>(A.ph, A.f, i, P.x, P.y, P.z, P.E, P.B);  // at the position before the push
-  P.k = m_sqrt(P.px * P.px + P.py * P.py + P.pz * P.pz);
-  if (COUNT && P.k > (Real)0) {
-    Real ik = dt / P.k;
-    P.x += P.px * ik; P.y += P.py * ik; P.z += P.pz * ik;
-    A.ph.x[i] = P.x; A.ph.y[i] = P.y; A.ph.z[i] = P.z;
-  }
-}
-
-// Method I for one photon (Eqs. 3, 6): 1 and the pair's (gamma_e, gamma_p,
-// sub-step) on an event, else 0.
-template <class Real>
-__device__ __forceinline__ uint32_t pair_chain(const PhotonArgs<Real> &A, const Real *sP,
-                                               const PhotonEntry<Real> &P, int64_t step_, Real dt,
-                                               Tally &tl, int64_t &N, Real &ge, Real &gp,
-                                               int64_t &ks) {
-  const Real inv_aS = sel<Real>(A.C.inv_aS, A.C.f_inv_aS);
-  const Real wdt_max = sel<Real>(A.C.wdt_max, A.C.f_wdt_max);
-  Real chi = chi_photon(P.px, P.py, P.pz, P.E[0], P.E[1], P.E[2], P.B[0], P.B[1], P.B[2], inv_aS);
-  RateOut<Real> ro = pair_rate(sP, A.T, A.C, chi, P.k, tl);
-  N = 1;
-  const Real wdt = ro.W * dt;
-  if (wdt > wdt_max) {
-    Real nn = m_ceil(wdt / wdt_max);
-    if (nn > (Real)A.C.max_substeps) { nn = (Real)A.C.max_substeps; tl.status |= QED_STATUS_SUBSTEPS; }
-    N = (int64_t)nn;
-  }
-  const Real dts = dt / (Real)N;
-  for (int64_t s = 0; s < N; ++s) {
-    U4 r = draw(A.C, P.id, step_, s, STREAM_PAIR);
-    if (!(ro.W * dts > unif<Real>(r.x))) continue;
-    XiOut<Real> xo = pair_xi(A.T.Yp, A.T, ro.l, unif<Real>(r.y), unif<Real>(~r.y));
-    ge = xo.xi * P.k;
-    gp = xo.omxi * P.k;
-    if (ge < (Real)1) { ge = (Real)1; gp = P.k - (Real)1; }
-    if (gp < (Real)1) { gp = (Real)1; ge = P.k - (Real)1; }
-    ks = s;
-    return 1u;
-  }
-  return 0u;
-}
-
-template <class Real, int FM>
-__global__ void __launch_bounds__(TILE) k_pair_count(PhotonArgs<Real> A) {
-  const int64_t step_ = A.d_step ? *A.d_step : A.step;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Real *sP = reinterpret_cast<Real *>(smem_raw);
-  __shared__ long long s_meta[1];
-  __shared__ BlockTally bt;
-  load_tables_smem(sP, A.T.P, A.T.glp.n);
-  block_tally_init(&bt);
-  if (threadIdx.x == 0) s_meta[0] = *(volatile const int64_t *)A.list_n;
-  __syncthreads();
-  const int64_t nl = s_meta[0];
-  const Real dt = sel<Real>(A.C.dt, A.C.f_dt);
-  const int64_t rc = A.rec_cap;
-  Tally tl;
-  tl.clear();
-  for (int64_t h = blockIdx.x * (int64_t)TILE + threadIdx.x; h < nl; h += (int64_t)gridDim.x * TILE) {
-    PhotonEntry<Real> P;
-    load_photon<Real, FM, true>(A, A.list[h], dt, P);
-    int64_t N = 1, ks = 0;
-    Real ge = 0, gp = 0;
-    const uint32_t cnt = pair_chain(A, sP, P, step_, dt, tl, N, ge, gp, ks);
-    tl.substeps += N;
-    tl.events += cnt;
-    A.sub_cnt[h] = cnt;
-    if (cnt) {
-      A.ph.alive[P.i] = 0;
-      if (h < rc) {
-        A.rec_e[h] = ge;
-        A.rec_e[rc + h] = gp;
-        A.rec_k[h] = (uint32_t)ks;
-      }
-    }
-  }
-  tally_flush(&bt, tl);
-  __syncthreads();
-  block_tally_commit(&bt, A.o.cnt, 1);
-}
-
-template <class Real, int FM>
-__global__ void __launch_bounds__(TILE) k_pair_write(PhotonArgs<Real> A) {
-  const int64_t step_ = A.d_step ? *A.d_step : A.step;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Real *sP = reinterpret_cast<Real *>(smem_raw);
-  __shared__ long long s_meta[4];
-  __shared__ BlockTally bt;
-  load_tables_smem(sP, A.T.P, A.T.glp.n);  // for entries past the record capacity
-  block_tally_init(&bt);
-  if (threadIdx.x == 0) {
-    s_meta[0] = *(volatile const int64_t *)A.list_n;
-    s_meta[1] = A.sub_meta[0];  // pairs of all entries
-    s_meta[2] = A.sub_meta[1];  // electron count before them
-    s_meta[3] = A.sub_meta[2];  // positron count before them
-  }
-  __syncthreads();
-  const int64_t nl = s_meta[0];
-  const uint32_t total = (uint32_t)s_meta[1];
-  const int64_t ne = s_meta[2], np = s_meta[3];
-  const Real dt = sel<Real>(A.C.dt, A.C.f_dt);
-  const int64_t rc = A.rec_cap;
-  Tally tl;
-  tl.clear();
-  for (int64_t h = blockIdx.x * (int64_t)TILE + threadIdx.x; h < nl; h += (int64_t)gridDim.x * TILE) {
-    const uint32_t off = A.sub_cnt[h];  // exclusive prefix of the counts now
-    const uint32_t cnt = (h + 1 < nl ? A.sub_cnt[h + 1] : total) - off;
-    if (!cnt) continue;
-    PhotonEntry<Real> P;
-    load_photon<Real, FM, false>(A, A.list[h], dt, P);
-    Real ge = 0, gp = 0;
-    int64_t ks = 0;
-    if (h < rc) {
-      ge = A.rec_e[h];
-      gp = A.rec_e[rc + h];
-      ks = A.rec_k[h];
-    } else {  // past the record capacity: redo the chain (same draws, same table)
-      Tally dummy;
-      dummy.clear();
-      int64_t N = 1;
-      if (!pair_chain(A, sP, P, step_, dt, dummy, N, ge, gp, ks)) {
-        tl.status |= QED_STATUS_REPLAY;  // should not happen: write a pair at rest
-        ge = gp = (Real)1;
-      }
-    }
-    const Real ik = (Real)1 / P.k;
-    const Real nx = P.px * ik, ny = P.py * ik, nz = P.pz * ik;
-    const U4 cid = draw(A.C, P.id, step_, ks, STREAM_PAIR_ID);
-    const Real pe = m_sqrt((ge - (Real)1) * (ge + (Real)1));
-    const Real pp = m_sqrt((gp - (Real)1) * (gp + (Real)1));
-    if (ne + off < A.el.cap)
-      write_child(A.el, ne + off, P.x, P.y, P.z, pe * nx, pe * ny, pe * nz, P.w,
-                  (uint64_t)cid.x | ((uint64_t)cid.y << 32), P.E, P.B, P.tag);
-    else { tl.dropped += 1; tl.status |= QED_STATUS_CAPACITY; }
-    if (np + off < A.po.cap)
-      write_child(A.po, np + off, P.x, P.y, P.z, pp * nx, pp * ny, pp * nz, P.w,
-                  (uint64_t)cid.z | ((uint64_t)cid.w << 32), P.E, P.B, P.tag);
-    else { tl.dropped += 1; tl.status |= QED_STATUS_CAPACITY; }
-  }
-  tally_flush(&bt, tl);
-  __syncthreads();
-  block_tally_commit(&bt, A.o.cnt, 1);
-}
-
-// ---------------------------------------------------------------------------
-// Stable in-place compaction of dead particles (alive == 0).  Every tile loads
-// its particles into registers before it publishes its count, and a tile
-// writes only below the end of its own range, after every earlier tile has
-// published -- so no data is overwritten before it has been read.
-// ---------------------------------------------------------------------------
-// Compaction tiles are COMPACT_ITEMS x 1024 particles (1024-thread CTAs, item k
-// of thread i is particle k * 1024 + i of the tile, so every load and store is
-// coalesced).  Tiles this large matter: a tile learns its prefix from the tile
-// states of its predecessors, a warp-wide window of 32 per round trip, so the
-// pass advances about 32 tiles per L2 round trip whatever the bandwidth.
-constexpr int COMPACT_TILE = 1024;
+constexpr int COMPACT_THREADS = 256;
 template <class Real> __host__ __device__ constexpr int compact_items() { return sizeof(Real) == 4 ? 2 : 1; }
+template <class Real> __host__ __device__ constexpr int compact_tile() { return COMPACT_THREADS * compact_items<Real>(); }
 
 template <class Real> struct CompactArgs {
   Sp<Real> s;
-  Out o;
+  uint32_t *off;        // [tile] live particles, then its first one's destination
+  uint32_t *read;       // [tile] 1: the tile's particles are in registers
+  uint32_t *total;      // live particles
+  unsigned int *ticket; // [0] tiles taken, [1] CTAs done, [2] waits that ran out (zero between calls)
+  qed_counters *cnt;
 };
 
+// nonzero bytes of a word
+__device__ __forceinline__ uint32_t live_bytes(uint32_t w) { return (uint32_t)__popc(__vsetne4(w, 0u)); }
+
+// A warp per tile.
 template <class Real>
-__global__ void __launch_bounds__(COMPACT_TILE) k_compact(CompactArgs<Real> A) {
-  constexpr int CI = compact_items<Real>();
-  constexpr int64_t TP = (int64_t)CI * COMPACT_TILE;  // particles per tile
-  __shared__ uint32_t scan_sm[33];
-  __shared__ long long s_meta[8];
-  if (threadIdx.x == 0) {
-    s_meta[2] = *(volatile int64_t *)A.s.d_n;
-    s_meta[5] = (long long)A.o.scan.sync[2];
+__global__ void __launch_bounds__(TILE) k_compact_count(CompactArgs<Real> A) {
+  constexpr int TP = compact_tile<Real>(), PER = TP / 32;  // flags per lane: 16 or 8
+  const int64_t n = *(volatile int64_t *)A.s.d_n;
+  const int64_t ntiles = (n + TP - 1) / TP;
+  const int lane = threadIdx.x & 31;
+  const bool aligned = (reinterpret_cast<uintptr_t>(A.s.alive) & 15) == 0;
+  for (int64_t t = ((int64_t)blockIdx.x * TILE + threadIdx.x) >> 5; t < ntiles;
+       t += ((int64_t)gridDim.x * TILE) >> 5) {
+    const int64_t first = t * TP + lane * PER;
+    uint32_t c = 0;
+    if (aligned && first + PER <= n) {
+      const uint2 *p = reinterpret_cast<const uint2 *>(A.s.alive + first);
+#pragma unroll
+      for (int q = 0; q < PER / 8; ++q) c += live_bytes(p[q].x) + live_bytes(p[q].y);
+    } else {
+      for (int j = 0; j < PER; ++j) c += first + j < n && A.s.alive[first + j] ? 1u : 0u;
+    }
+    c = __reduce_add_sync(0xFFFFFFFFu, c);
+    if (lane == 0) {
+      A.off[t] = c;
+      A.read[t] = 0u;
+    }
   }
-  __syncthreads();
-  const int64_t n = s_meta[2];
-  const uint32_t epoch = (uint32_t)s_meta[5];
+}
+
+// One CTA: exclusive scan of the tiles' counts.
+__global__ void __launch_bounds__(CLS_SCAN_THREADS) k_compact_scan(uint32_t *off, uint32_t *total, const int64_t *d_n,
+                                                                   int tile) {
+  constexpr int ITEMS = 8;
+  __shared__ uint32_t sm[33];
+  const int64_t ntiles = (*(volatile const int64_t *)d_n + tile - 1) / tile;
+  uint32_t carry = 0;
+  for (int64_t r0 = 0; r0 < ntiles; r0 += CLS_SCAN_THREADS * ITEMS) {
+    const int64_t c0 = r0 + (int64_t)threadIdx.x * ITEMS;
+    uint32_t v[ITEMS], t = 0;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      v[j] = c0 + j < ntiles ? off[c0 + j] : 0u;
+      t += v[j];
+    }
+    uint32_t run = carry + block_excl_scan(t, sm);
+    carry += sm[32];
+    __syncthreads();  // sm[32] is read
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      if (c0 + j < ntiles) off[c0 + j] = run;
+      run += v[j];
+    }
+  }
+  if (threadIdx.x == 0) *total = carry;
+}
+
+__device__ __forceinline__ uint32_t word_hash(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ uint32_t word_hash(double v) { return (uint32_t)__double2loint(v) ^ (uint32_t)__double2hiint(v); }
+
+template <class Real>
+__global__ void __launch_bounds__(COMPACT_THREADS, sizeof(Real) == 4 ? 4 : 3) k_compact_move(CompactArgs<Real> A) {
+  constexpr int CI = compact_items<Real>(), TP = compact_tile<Real>(), WARPS = COMPACT_THREADS / 32;
+  __shared__ uint32_t s_warp[CI][WARPS];
+  __shared__ uint32_t s_tile, s_off, s_end, s_go;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t n = *(volatile int64_t *)A.s.d_n;
   const int64_t ntiles = (n + TP - 1) / TP;
   const bool fields = A.s.ex != nullptr;
-  uint32_t status = 0;
+  bool gave_up = false;
+  // (thread 0) tile t's place, for all after the next barrier
+  auto put_tile = [&](uint32_t t) {
+    s_tile = t;
+    if (t < ntiles) {
+      s_off = A.off[t];
+      s_end = t + 1 < ntiles ? A.off[t + 1] : *A.total;
+    }
+  };
+  if (threadIdx.x == 0) put_tile(atomicAdd(&A.ticket[0], 1u));
+  __syncthreads();
   for (;;) {
-    if (threadIdx.x == 0) s_meta[0] = (long long)atomicAdd(&A.o.scan.sync[0], 1u);
-    __syncthreads();
-    const int64_t t = s_meta[0];
-    __syncthreads();
+    const int64_t t = s_tile;
     if (t >= ntiles) break;
-    uint32_t keep[CI];
-    Real v[CI][13];
-    uint64_t id[CI];
-    uint32_t tg[CI];
+    const uint32_t off = s_off, cnt = s_end - off;
+    // the next tile's ticket is taken now: a CTA waits only for tiles before its
+    // own, and those before the next one it holds never wait for it, so the
+    // first tile not done can always go on
+    uint32_t next = 0;
+    if (threadIdx.x == 0) next = atomicAdd(&A.ticket[0], 1u);
+    const bool whole = cnt == (uint32_t)(t + 1 < ntiles ? TP : n - t * TP);
+    // a tile that stays where it is moves nothing, and none writes into it
+    const bool stays = (int64_t)off == t * TP && whole;
+    if (!stays) {
+      bool keep[CI];
+      Real v[CI][13];
+      uint64_t id[CI];
+      uint32_t tg[CI], h = 0;
 #pragma unroll
-    for (int k = 0; k < CI; ++k) {
-      const int64_t i = t * TP + k * COMPACT_TILE + threadIdx.x;
-      keep[k] = 0;
-      id[k] = 0;
-      tg[k] = 0;
-      if (i < n && A.s.alive[i]) {
-        keep[k] = 1;
-        if (A.s.tag) tg[k] = A.s.tag[i];
-        v[k][0] = A.s.x[i]; v[k][1] = A.s.y[i]; v[k][2] = A.s.z[i];
-        v[k][3] = A.s.px[i]; v[k][4] = A.s.py[i]; v[k][5] = A.s.pz[i]; v[k][6] = A.s.w[i];
-        id[k] = A.s.id[i];
-        if (fields) {
-          v[k][7] = A.s.ex[i]; v[k][8] = A.s.ey[i]; v[k][9] = A.s.ez[i];
-          v[k][10] = A.s.bx[i]; v[k][11] = A.s.by[i]; v[k][12] = A.s.bz[i];
+      for (int k = 0; k < CI; ++k) {  // (the words do not wait for the flag)
+        const int64_t i = t * TP + k * COMPACT_THREADS + threadIdx.x;
+        keep[k] = false;
+        id[k] = 0;
+        tg[k] = 0;
+#pragma unroll
+        for (int q = 0; q < 13; ++q) v[k][q] = (Real)0;
+        if (i < n) {
+          keep[k] = A.s.alive[i];
+          v[k][0] = A.s.x[i]; v[k][1] = A.s.y[i]; v[k][2] = A.s.z[i];
+          v[k][3] = A.s.px[i]; v[k][4] = A.s.py[i]; v[k][5] = A.s.pz[i]; v[k][6] = A.s.w[i];
+          id[k] = A.s.id[i];
+          if (A.s.tag) tg[k] = A.s.tag[i];
+          if (fields) {
+            v[k][7] = A.s.ex[i]; v[k][8] = A.s.ey[i]; v[k][9] = A.s.ez[i];
+            v[k][10] = A.s.bx[i]; v[k][11] = A.s.by[i]; v[k][12] = A.s.bz[i];
+          }
         }
       }
-    }
-    // destination of item k within the tile: the items of the earlier stripes,
-    // then this stripe's prefix
-    uint32_t excl[CI];
-    uint32_t agg = 0;
 #pragma unroll
-    for (int k = 0; k < CI; ++k) {
-      if (k > 0) __syncthreads();  // scan_sm is reused
-      excl[k] = agg + block_excl_scan(keep[k], scan_sm);
-      agg += scan_sm[32];
-    }
-    if (threadIdx.x < 32) {
-      uint32_t st_tile = 0;
-      uint32_t pre = lookback_warp(A.o.scan, t, epoch, agg, st_tile);
-      // any lane of the walk may have given up (warp 0 runs converged here)
-      const bool gave_up = __any_sync(0xFFFFFFFFu, (st_tile & QED_STATUS_TIMEOUT) != 0);
-      status |= st_tile;
+      for (int k = 0; k < CI; ++k) {
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, keep[k]);
+        if (lane == 0) s_warp[k][wid] = __popc(m);
+        // a use of every word, so that all have arrived at the barrier
+        h ^= (uint32_t)id[k] ^ (uint32_t)(id[k] >> 32) ^ tg[k];
+#pragma unroll
+        for (int q = 0; q < 13; ++q) h ^= word_hash(v[k][q]);
+      }
+      __syncthreads_or((int)h);
       if (threadIdx.x == 0) {
-        s_meta[1] = pre;
-        // a look-back that gave up has no valid prefix: this tile writes
-        // nothing (an in-place write could land on particles an earlier tile
-        // has not read yet); the result is flagged QED_STATUS_TIMEOUT
-        s_meta[3] = gave_up ? 1 : 0;
-        if (t == ntiles - 1 && !s_meta[3]) *A.s.d_n = (int64_t)pre + agg;
+        __threadfence();
+        *(volatile uint32_t *)&A.read[t] = 1u;
+        uint32_t go = 1;
+        if (cnt)
+          for (int64_t s = off / TP; s <= (int64_t)((off + cnt - 1) / TP) && s < t; ++s) {
+            // (a tile that stays has published nothing, and nothing is written to it)
+            long long spins = 0;
+            while (*(volatile uint32_t *)&A.read[s] == 0u)
+              if (++spins > LOOKBACK_SPIN_LIMIT) {
+                go = 0;
+                break;
+              }
+          }
+        __threadfence();
+        s_go = go;
+        put_tile(next);
       }
-    }
-    __syncthreads();
-    const bool skip = s_meta[3] != 0;
+      __syncthreads();
+      if (s_go) {
+        uint32_t before = off;
 #pragma unroll
-    for (int k = 0; k < CI; ++k) {
-      if (!keep[k] || skip) continue;
-      const int64_t d = s_meta[1] + excl[k];
-      A.s.x[d] = v[k][0]; A.s.y[d] = v[k][1]; A.s.z[d] = v[k][2];
-      A.s.px[d] = v[k][3]; A.s.py[d] = v[k][4]; A.s.pz[d] = v[k][5]; A.s.w[d] = v[k][6];
-      A.s.id[d] = id[k];
-      A.s.alive[d] = 1;
-      if (A.s.tag) A.s.tag[d] = tg[k];
-      if (fields) {
-        A.s.ex[d] = v[k][7]; A.s.ey[d] = v[k][8]; A.s.ez[d] = v[k][9];
-        A.s.bx[d] = v[k][10]; A.s.by[d] = v[k][11]; A.s.bz[d] = v[k][12];
+        for (int k = 0; k < CI; ++k) {
+          uint32_t base = before;
+#pragma unroll
+          for (int w = 0; w < WARPS; ++w) {
+            if (w < wid) base += s_warp[k][w];
+            before += s_warp[k][w];
+          }
+          const unsigned m = __ballot_sync(0xFFFFFFFFu, keep[k]);
+          if (!keep[k]) continue;
+          const int64_t d = base + __popc(m & ((1u << lane) - 1u));
+          A.s.x[d] = v[k][0]; A.s.y[d] = v[k][1]; A.s.z[d] = v[k][2];
+          A.s.px[d] = v[k][3]; A.s.py[d] = v[k][4]; A.s.pz[d] = v[k][5]; A.s.w[d] = v[k][6];
+          A.s.id[d] = id[k];
+          A.s.alive[d] = 1;
+          if (A.s.tag) A.s.tag[d] = tg[k];
+          if (fields) {
+            A.s.ex[d] = v[k][7]; A.s.ey[d] = v[k][8]; A.s.ez[d] = v[k][9];
+            A.s.bx[d] = v[k][10]; A.s.by[d] = v[k][11]; A.s.bz[d] = v[k][12];
+          }
+        }
+      } else {
+        gave_up = true;
       }
+      __syncthreads();  // s_warp and s_go are read
+    } else {
+      __syncthreads();  // the tile's place is read
+      if (threadIdx.x == 0) put_tile(next);
+      __syncthreads();
     }
   }
-  if (threadIdx.x == 0 && status) atomicOr(&A.o.cnt->status, status);
-  launch_epilogue(A.o.scan, epoch);
+  // the last CTA publishes the count -- unless a tile gave up, and so wrote
+  // nothing -- and leaves the counters at zero
+  if (threadIdx.x == 0) {
+    if (gave_up) {
+      atomicOr(&A.cnt->status, (unsigned)QED_STATUS_TIMEOUT);
+      atomicAdd(&A.ticket[2], 1u);
+    }
+    __threadfence();
+    if (atomicAdd(&A.ticket[1], 1u) == gridDim.x - 1) {
+      __threadfence();
+      if (*(volatile unsigned *)&A.ticket[2] == 0u) *A.s.d_n = *A.total;
+      A.ticket[0] = A.ticket[1] = A.ticket[2] = 0u;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1632,8 +1346,8 @@ template <class Real> struct FillArgs {
   Sp<Real> s;
   unsigned long long *chunk_alive;  // [chunks]
   uint32_t *chunk_off;              // [chunks][NCLS]: [0] holes before, [1] tails before
-  int64_t *meta;                    // [0] n, [1] a
-  int *holes;                       // hole slots in index order
+  int64_t *meta;                    // [0] n, [1] a, [2] holes (as many as tails)
+  int *holes, *tails;               // their slots in index order
 };
 
 // live flags of this thread's 8 slots of chunk c (bit j: slot first + j)
@@ -1641,6 +1355,13 @@ __device__ __forceinline__ uint32_t fill_bits(const uint8_t *alive, int64_t c, i
                                               int64_t &first) {
   first = c * FILL_CHUNK + (int64_t)threadIdx.x * FILL_ITEMS;
   uint32_t bits = 0;
+  if (first + FILL_ITEMS <= n && (reinterpret_cast<uintptr_t>(alive) & 7) == 0) {
+    const uint2 w = *reinterpret_cast<const uint2 *>(alive + first);
+#pragma unroll
+    for (int j = 0; j < FILL_ITEMS; ++j)
+      if ((j < 4 ? w.x >> 8 * j : w.y >> 8 * (j - 4)) & 0xFFu) bits |= 1u << j;
+    return bits;
+  }
 #pragma unroll
   for (int j = 0; j < FILL_ITEMS; ++j)
     if (first + j < n && alive[first + j]) bits |= 1u << j;
@@ -1734,61 +1455,71 @@ __global__ void __launch_bounds__(CLS_SCAN_THREADS) k_fill_scan(const uint8_t *a
     carry_h += (int64_t)(uint32_t)tt;
     carry_t += (int64_t)(uint32_t)(tt >> 32);
   }
+  if (threadIdx.x == 0) A.meta[2] = carry_h;
 }
 
+// The holes' and the tails' slots.  (A chunk is below a, above it, or the one
+// that a lies in.)
 template <class Real>
 __global__ void __launch_bounds__(TILE) k_fill_holes(FillArgs<Real> A) {
   __shared__ uint32_t scan_sm[33];
   const int64_t n = A.meta[0], a = A.meta[1];
-  const int64_t nchunks = (a + FILL_CHUNK - 1) / FILL_CHUNK;  // chunks with slots below a
+  if (A.meta[2] == 0) return;
+  const int64_t nchunks = (n + FILL_CHUNK - 1) / FILL_CHUNK;
   for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
     int64_t first;
-    uint32_t bits = fill_bits(A.s.alive, c, n, first);
-    uint32_t hole = 0;
+    const uint32_t bits = fill_bits(A.s.alive, c, n, first);
+    uint32_t hole = 0, tail = 0;
 #pragma unroll
-    for (int j = 0; j < FILL_ITEMS; ++j)
+    for (int j = 0; j < FILL_ITEMS; ++j) {
       if (first + j < a && !(bits & (1u << j))) hole |= 1u << j;
-    uint32_t k = A.chunk_off[c * NCLS + 0] + block_excl_scan(__popc(hole), scan_sm);
+      if (first + j >= a && (bits & (1u << j))) tail |= 1u << j;
+    }
+    // (at most 2048 of each: two counts in a word)
+    const uint32_t ex = block_excl_scan(__popc(hole) | (uint32_t)__popc(tail) << 16, scan_sm);
+    uint32_t k = A.chunk_off[c * NCLS + 0] + (ex & 0xFFFFu);
     __syncthreads();
     while (hole) {
       const int j = __ffs(hole) - 1;
       hole &= hole - 1;
       A.holes[k++] = (int)(first + j);
     }
-  }
-}
-
-template <class Real>
-__global__ void __launch_bounds__(TILE) k_fill_move(FillArgs<Real> A) {
-  __shared__ uint32_t scan_sm[33];
-  const int64_t n = A.meta[0], a = A.meta[1];
-  const int64_t c_lo = a / FILL_CHUNK, nchunks = (n + FILL_CHUNK - 1) / FILL_CHUNK;
-  const Sp<Real> &S = A.s;
-  const bool fields = S.ex != nullptr;
-  for (int64_t c = c_lo + blockIdx.x; c < nchunks; c += gridDim.x) {
-    int64_t first;
-    const uint32_t bits = fill_bits(S.alive, c, n, first);
-    uint32_t tail = 0;
-#pragma unroll
-    for (int j = 0; j < FILL_ITEMS; ++j)
-      if (first + j >= a && (bits & (1u << j))) tail |= 1u << j;
-    uint32_t k = A.chunk_off[c * NCLS + 1] + block_excl_scan(__popc(tail), scan_sm);
-    __syncthreads();
+    k = A.chunk_off[c * NCLS + 1] + (ex >> 16);
     while (tail) {
       const int j = __ffs(tail) - 1;
       tail &= tail - 1;
-      const int64_t i = first + j, d = A.holes[k++];
-      S.x[d] = S.x[i]; S.y[d] = S.y[i]; S.z[d] = S.z[i];
-      S.px[d] = S.px[i]; S.py[d] = S.py[i]; S.pz[d] = S.pz[i];
-      S.w[d] = S.w[i];
-      S.id[d] = S.id[i];
-      if (S.tag) S.tag[d] = S.tag[i];
-      if (fields) {
-        S.ex[d] = S.ex[i]; S.ey[d] = S.ey[i]; S.ez[d] = S.ez[i];
-        S.bx[d] = S.bx[i]; S.by[d] = S.by[i]; S.bz[d] = S.bz[i];
-      }
-      S.alive[d] = 1;
+      A.tails[k++] = (int)(first + j);
     }
+  }
+}
+
+// A particle per thread: all its words are read before any is written (2000
+// moves of 15 arrays: 22 us with each chunk's threads moving their own tails
+// word by word, 5 this way).
+template <class Real>
+__global__ void __launch_bounds__(TILE) k_fill_move(FillArgs<Real> A) {
+  const int64_t m = A.meta[2];
+  const Sp<Real> &S = A.s;
+  const bool fields = S.ex != nullptr;
+  for (int64_t k = blockIdx.x * (int64_t)TILE + threadIdx.x; k < m; k += (int64_t)gridDim.x * TILE) {
+    const int64_t i = A.tails[k], d = A.holes[k];
+    const Real v[7] = {S.x[i], S.y[i], S.z[i], S.px[i], S.py[i], S.pz[i], S.w[i]};
+    const uint64_t id = S.id[i];
+    const uint32_t tag = S.tag ? S.tag[i] : 0u;
+    Real f[6] = {0, 0, 0, 0, 0, 0};
+    if (fields) {
+      f[0] = S.ex[i]; f[1] = S.ey[i]; f[2] = S.ez[i];
+      f[3] = S.bx[i]; f[4] = S.by[i]; f[5] = S.bz[i];
+    }
+    S.x[d] = v[0]; S.y[d] = v[1]; S.z[d] = v[2];
+    S.px[d] = v[3]; S.py[d] = v[4]; S.pz[d] = v[5]; S.w[d] = v[6];
+    S.id[d] = id;
+    if (S.tag) S.tag[d] = tag;
+    if (fields) {
+      S.ex[d] = f[0]; S.ey[d] = f[1]; S.ez[d] = f[2];
+      S.bx[d] = f[3]; S.by[d] = f[4]; S.bz[d] = f[5];
+    }
+    S.alive[d] = 1;
   }
 }
 
@@ -2037,27 +1768,6 @@ template <class Real> size_t lepton_smem(const qed_ctx *c) {
   return sizeof(Real) * ((size_t)c->gl.n + (size_t)c->gl.n * c->gy.n);
 }
 
-static cudaError_t launch_flag_list(qed_ctx *c, const uint8_t *flags, uint8_t want, const int64_t *n0,
-                                    const int64_t *n1, const Out &o, const int32_t *stage_idx,
-                                    cudaStream_t st) {
-  HeavyListArgs h{};
-  h.flags = flags;
-  h.want = want;
-  h.stage_idx = stage_idx;
-  h.list = c->heavy_list;
-  h.count = c->heavy_n;
-  h.n0 = n0;
-  h.n1 = n1;
-  h.o = o;
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_heavy_list, TILE, 0);
-  if (e != cudaSuccess) return e;
-  per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_ORDER);
-  k_heavy_list<<<c->num_sms * per_sm, TILE, 0, st>>>(h);
-  c->launches += 1;
-  return cudaGetLastError();
-}
-
 template <class Real, int FM>
 static cudaError_t launch_push(qed_ctx *c, const LeptonArgs<Real> &a, cudaStream_t st) {
   int per_sm = 0;
@@ -2126,18 +1836,15 @@ static cudaError_t launch_class_lists(qed_ctx *c, const int64_t *n0, const int64
   return cudaGetLastError();
 }
 
-static cudaError_t launch_sub_scan(qed_ctx *c, const int64_t *n_entries, int64_t *out1_n,
-                                   int64_t out1_cap, int64_t *out2_n, int64_t out2_cap,
+static cudaError_t launch_sub_scan(qed_ctx *c, const int64_t *n_entries, int64_t *out_n, int64_t out_cap,
                                    cudaStream_t st) {
   SubScanArgs a{};
   a.cnt = c->sub_cnt;
   a.replay_n = c->replay_n;
   a.n_entries = n_entries;
   a.sub_meta = c->sub_meta;
-  a.out1_n = out1_n;
-  a.out1_cap = out1_cap;
-  a.out2_n = out2_n;
-  a.out2_cap = out2_cap;
+  a.out_n = out_n;
+  a.out_cap = out_cap;
   a.o = out_of(c);
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sub_scan, TILE, 0);
@@ -2167,7 +1874,7 @@ static cudaError_t launch_lepton_t(qed_ctx *c, const LeptonArgs<Real> &a, cudaSt
             : launch_tables_kernel<Real>(c, k_substep_count<Real, FM, MODE, false>, a, false,
                                          QED_TUNE_CHAINS, st);
   if (e == cudaSuccess) e = prof_mark(c, 3, st);
-  if (e == cudaSuccess) e = launch_sub_scan(c, c->cls_off + NCLS, a.ph.d_n, a.ph.cap, nullptr, 0, st);
+  if (e == cudaSuccess) e = launch_sub_scan(c, c->cls_off + NCLS, a.ph.d_n, a.ph.cap, st);
   if (e == cudaSuccess) e = prof_mark(c, 4, st);
   if (e == cudaSuccess) e = launch_plain_kernel<Real>(c, k_substep_write_coop<Real, FM, MODE>, a, st);
   if (e == cudaSuccess)
@@ -2229,7 +1936,6 @@ cudaError_t launch_lepton(qed_ctx *c, const qed_species *s0, const qed_species *
   a.step = step;
   a.heavy_flags = c->heavy_flags;
   a.heavy_list = c->heavy_list;
-  a.heavy_n = c->heavy_n;
   a.cls_off = c->cls_off;
   a.sub_cnt = c->sub_cnt;
   a.sub_gf = static_cast<Real *>(c->sub_gf);
@@ -2264,82 +1970,27 @@ cudaError_t launch_lepton(qed_ctx *c, const qed_species *s0, const qed_species *
   return launch_lepton_m<Real, MODE_FUSED>(c, a, f->mode, st);
 }
 
-template <class Real, int FM>
-static cudaError_t launch_photon_t(qed_ctx *c, const PhotonArgs<Real> &a, cudaStream_t st) {
-  size_t sm = sizeof(Real) * (size_t)c->glp.n;
-  int per_sm = 0;
-  cudaError_t e = cudaMemsetAsync(a.stage_n, 0, sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_photon_stream<Real, FM>, TILE, sm);
-  if (e != cudaSuccess) return e;
-  per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_PHOTON);
-  k_photon_stream<Real, FM><<<c->num_sms * per_sm, TILE, sm, st>>>(a);
-  c->launches += 1;
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = prof_mark(c, 6, st);
-  if (e == cudaSuccess) e = launch_flag_list(c, a.flags, 1, a.n_active, nullptr, a.o, a.stage_idx, st);
-  if (e != cudaSuccess) return e;
-  // pairs: counting pass, scan (advances both lepton counts), writing pass
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair_count<Real, FM>, TILE, sm);
-  if (e != cudaSuccess) return e;
-  per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_PHOTON);
-  k_pair_count<Real, FM><<<c->num_sms * per_sm, TILE, sm, st>>>(a);
-  c->launches += 1;
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_sub_scan(c, a.list_n, a.el.d_n, a.el.cap, a.po.d_n, a.po.cap, st);
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair_write<Real, FM>, TILE, sm);
-  if (e != cudaSuccess) return e;
-  per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_PHOTON);
-  k_pair_write<Real, FM><<<c->num_sms * per_sm, TILE, sm, st>>>(a);
-  c->launches += 1;
-  return cudaGetLastError();
-}
-
-template <class Real>
-cudaError_t launch_photon(qed_ctx *c, const qed_species *g, const qed_species *e,
-                          const qed_species *p, const int64_t *n_active, const qed_fields *f,
-                          int64_t step, cudaStream_t st) {
-  PhotonArgs<Real> a{};
-  a.ph = to_sp<Real>(g);
-  a.el = to_sp<Real>(e);
-  a.po = to_sp<Real>(p);
-  a.n_active = n_active;
-  a.f = to_fld<Real>(f);
-  a.C = consts_of(c);
-  a.T = tables_of<Real>(c);
-  a.o = out_of(c);
-  a.step = step;
-  a.flags = c->heavy_flags;
-  a.list = c->heavy_list;
-  a.list_n = c->heavy_n;
-  a.stage = static_cast<Stage<Real> *>(c->stage);
-  a.stage_tag = c->stage_tag;
-  a.stage_idx = c->stage_idx;
-  a.stage_n = c->stage_n;
-  a.stage_cap = c->stage_cap;
-  a.sub_cnt = c->sub_cnt;
-  a.sub_meta = c->sub_meta;
-  a.rec_e = static_cast<Real *>(c->rec_e);
-  a.rec_k = c->rec_k;
-  a.rec_cap = c->rec_cap;
-  a.d_step = c->use_dstep ? c->d_step : nullptr;
-  if (f->mode == QED_FIELDS_UNIFORM) return launch_photon_t<Real, FM_UNIFORM>(c, a, st);
-  if (f->mode == QED_FIELDS_PER_PARTICLE) return launch_photon_t<Real, FM_PER_PARTICLE>(c, a, st);
-  return launch_photon_t<Real, FM_GRID>(c, a, st);
-}
-
 template <class Real>
 cudaError_t launch_compact(qed_ctx *c, const qed_species *s, cudaStream_t st) {
   CompactArgs<Real> a{};
+  constexpr int TP = compact_tile<Real>();
+  const int64_t tiles = (s->capacity + TP - 1) / TP;
   a.s = to_sp<Real>(s);
-  a.o = out_of(c);
+  a.off = c->sub_cnt;  // (scratch of the step, one word per slot)
+  a.read = c->sub_cnt + tiles;
+  a.total = c->sub_cnt + 2 * tiles;
+  a.ticket = c->compact_n;
+  a.cnt = c->d_counters;
+  const int64_t count_need = (tiles * 32 + TILE - 1) / TILE, count_most = (int64_t)c->num_sms * 8;
+  k_compact_count<Real><<<(unsigned)(count_need < 1 ? 1 : count_need < count_most ? count_need : count_most), TILE, 0, st>>>(a);
+  k_compact_scan<<<1, CLS_SCAN_THREADS, 0, st>>>(a.off, a.total, s->d_n, TP);
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_compact<Real>, COMPACT_TILE, 0);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_compact_move<Real>, COMPACT_THREADS, 0);
   if (e != cudaSuccess) return e;
   per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_COMPACT);
-  k_compact<Real><<<c->num_sms * per_sm, COMPACT_TILE, 0, st>>>(a);
-  c->launches += 1;
+  const int64_t most = (int64_t)c->num_sms * per_sm;
+  k_compact_move<Real><<<(unsigned)(tiles < 1 ? 1 : tiles < most ? tiles : most), COMPACT_THREADS, 0, st>>>(a);
+  c->launches += 3;
   return cudaGetLastError();
 }
 
@@ -2351,6 +2002,7 @@ cudaError_t launch_compact_fill(qed_ctx *c, const qed_species *s, cudaStream_t s
   a.chunk_off = c->cls_chunk_off;
   a.meta = c->fill_meta;
   a.holes = c->heavy_list;
+  a.tails = c->stage_idx;
   FillArgs<float> af{};  // the scan reads only the shared scratch
   af.chunk_alive = a.chunk_alive;
   af.chunk_off = a.chunk_off;
@@ -2358,7 +2010,9 @@ cudaError_t launch_compact_fill(qed_ctx *c, const qed_species *s, cudaStream_t s
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fill_count<Real>, TILE, 0);
   if (e != cudaSuccess) return e;
-  const int grid = c->num_sms * (per_sm > 0 ? per_sm : 1);
+  // no more CTAs than the capacity has chunks
+  const int64_t chunks = (s->capacity + FILL_CHUNK - 1) / FILL_CHUNK, most = (int64_t)c->num_sms * (per_sm > 0 ? per_sm : 1);
+  const unsigned grid = (unsigned)(chunks < 1 ? 1 : chunks < most ? chunks : most);
   k_fill_count<Real><<<grid, TILE, 0, st>>>(a);
   k_fill_scan<<<1, CLS_SCAN_THREADS, 0, st>>>(s->alive, s->d_n, af);
   k_fill_holes<Real><<<grid, TILE, 0, st>>>(a);
@@ -2468,12 +2122,6 @@ template cudaError_t launch_lepton<float>(qed_ctx *, const qed_species *, const 
 template cudaError_t launch_lepton<double>(qed_ctx *, const qed_species *, const qed_species *,
                                            const qed_species *, const qed_fields *, int64_t, int,
                                            cudaStream_t);
-template cudaError_t launch_photon<float>(qed_ctx *, const qed_species *, const qed_species *,
-                                          const qed_species *, const int64_t *, const qed_fields *,
-                                          int64_t, cudaStream_t);
-template cudaError_t launch_photon<double>(qed_ctx *, const qed_species *, const qed_species *,
-                                           const qed_species *, const int64_t *, const qed_fields *,
-                                           int64_t, cudaStream_t);
 template cudaError_t launch_compact<float>(qed_ctx *, const qed_species *, cudaStream_t);
 template cudaError_t launch_compact<double>(qed_ctx *, const qed_species *, cudaStream_t);
 template cudaError_t launch_compact_fill<float>(qed_ctx *, const qed_species *, cudaStream_t);
