@@ -288,7 +288,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
       cudaMalloc(&c->sub_meta, 4 * sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&c->fill_meta, 3 * sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&c->ord_n, 4 * sizeof(unsigned int)) != cudaSuccess ||
-      cudaMalloc(&c->compact_n, 3 * sizeof(unsigned int)) != cudaSuccess ||
+      cudaMalloc(&c->compact_n, COMPACT_WORDS * sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->replay_n, sizeof(unsigned int)) != cudaSuccess ||
       cudaMalloc(&c->probe_state, 2 * sizeof(unsigned long long)) != cudaSuccess) {
     free_ctx(c);
@@ -300,7 +300,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counters, 0, sizeof(qed_counters), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->pair_n, 0, 2 * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->pair_sum, 0, sizeof(uint32_t) * (size_t)c->cls_chunks, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->compact_n, 0, 3 * sizeof(unsigned int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->compact_n, 0, COMPACT_WORDS * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ord_n, 0, 4 * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->stage_n, 0, sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->probe_state, 0, 2 * sizeof(unsigned long long), st);

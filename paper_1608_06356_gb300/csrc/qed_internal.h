@@ -40,7 +40,7 @@ struct qed_ctx {
   int64_t rec_cap;
   int64_t *sub_meta;  // [4] photons of the emission entries, counts before them (or before the pairs)
   int64_t *fill_meta; // [3] count before and after a hole-filling compaction, holes
-  unsigned int *compact_n; // [3] stable compaction: tiles taken, CTAs done, waits that ran out
+  unsigned int *compact_n; // [COMPACT_WORDS] stable compaction: tiles taken, CTAs done, waits that ran out, counting CTAs done; its single launch
   unsigned int *pair_n;    // [2] pairs of the photon stage: records, those being written
   uint32_t *pair_sum;      // [cls_chunks] pairs per chunk of photons (zero between steps)
   unsigned int *ord_n;     // [4] ordered appends of the single pass: records and replays asked for, of the pass being written
@@ -148,6 +148,8 @@ inline cudaError_t prof_mark(qed_ctx *c, int k, cudaStream_t st) {
   return c->prof_cur ? cudaEventRecord(c->prof_cur[k], st) : cudaSuccess;
 }
 constexpr int TILE = 256;  // particles per tile = threads per block in the step kernels
+constexpr int COMPACT_ONE = 1024;  // most tiles of the stable compaction's single launch
+constexpr int COMPACT_WORDS = 5 + COMPACT_ONE + COMPACT_ONE / 32;
 constexpr int SUB_REC = 8; // emission records kept per particle by the sub-step counting pass
 constexpr int CLS_CHUNK_FLAGS = 2048;  // flags per chunk of the class-list passes
 }  // namespace qed

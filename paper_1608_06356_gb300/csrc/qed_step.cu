@@ -1114,14 +1114,17 @@ __global__ void __launch_bounds__(TILE) k_cls_scatter(ClassListArgs A) {
 // ---------------------------------------------------------------------------
 // Stable in-place compaction of dead particles (alive == 0): the live particles
 // of every tile are counted (from the flags alone), the counts scanned, and the
-// tiles moved.  A moving tile reads its particles into registers, publishes
-// that, waits until the tiles whose range it writes to -- at most two, which
-// lie before it by the particles dead so far -- have published too, and writes:
-// no word is overwritten before it has been read.  Tiles are taken in order, so
-// the ones waited for are under way.  The wait is bounded.  (8.4M photons of 61
-// bytes, one in ten dead: 268 us with the positions from a look-back, which
+// tiles moved.  The warps of a moving tile read its particles into registers and
+// publish that; the tile then waits until the tiles whose range it writes to --
+// at most two, which lie before it by the particles dead so far -- have published
+// too, and writes: no word is overwritten before it has been read.  Tiles are
+// taken in order, so the ones waited for are under way, and have mostly published
+// by the time this tile's own words arrive.  The wait is bounded.  (8.4M photons
+// of 61 bytes, one in ten dead: 268 us with the positions from a look-back, which
 // had each tile wait for the sums of all before it, one 2048-particle tile of
-// 1024 threads in flight per SM; COMPACT_US this way, 135 at the copy rate.)
+// 1024 threads in flight per SM; 198 with counts and a scan of their own launch,
+// and the CTA's barrier before it published; 185 this way, 135 at the copy
+// rate.  900,000: 31 -> 28 us.)
 // ---------------------------------------------------------------------------
 constexpr int COMPACT_THREADS = 256;
 template <class Real> __host__ __device__ constexpr int compact_items() { return sizeof(Real) == 4 ? 2 : 1; }
@@ -1130,25 +1133,42 @@ template <class Real> __host__ __device__ constexpr int compact_tile() { return 
 template <class Real> struct CompactArgs {
   Sp<Real> s;
   uint32_t *off;        // [tile] live particles, then its first one's destination
-  uint32_t *read;       // [tile] 1: the tile's particles are in registers
+  uint32_t *read;       // [tile] warps whose part of the tile is in registers
   uint32_t *total;      // live particles
-  unsigned int *ticket; // [0] tiles taken, [1] CTAs done, [2] waits that ran out (zero between calls)
+  uint32_t *one;        // [COMPACT_ONE] the single launch: live particles + 1 (zero between calls)
+  uint32_t *group;      // [COMPACT_ONE / 32] live particles and, from bit 20, tiles of 32 (zero between calls)
+  unsigned int *ticket; // [0] tiles taken, [1] CTAs done, [2] waits that ran out, [3] counting CTAs done (zero between calls)
   qed_counters *cnt;
 };
 
 // nonzero bytes of a word
 __device__ __forceinline__ uint32_t live_bytes(uint32_t w) { return (uint32_t)__popc(__vsetne4(w, 0u)); }
 
-// A warp per tile.
+// Eight words at a 32-byte boundary.
+__device__ __forceinline__ void load8(uint32_t (&v)[8], const uint32_t *p) {
+  asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "l"(p) : "memory");
+}
+__device__ __forceinline__ void store8(uint32_t *p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+
+// The tiles' counts, a warp per tile; the CTA that finishes last scans them, 8
+// tiles per thread by one load of 32 bytes (16M photons, 31250 tiles: 29 us with
+// a launch of its own for the scan and a word per load, 13 this way).
 template <class Real>
-__global__ void __launch_bounds__(TILE) k_compact_count(CompactArgs<Real> A) {
+__global__ void __launch_bounds__(CLS_SCAN_THREADS) k_compact_count(CompactArgs<Real> A) {
   constexpr int TP = compact_tile<Real>(), PER = TP / 32;  // flags per lane: 16 or 8
+  __shared__ uint32_t sm[33];
+  __shared__ bool s_last;
   const int64_t n = *(volatile int64_t *)A.s.d_n;
   const int64_t ntiles = (n + TP - 1) / TP;
   const int lane = threadIdx.x & 31;
   const bool aligned = (reinterpret_cast<uintptr_t>(A.s.alive) & 15) == 0;
-  for (int64_t t = ((int64_t)blockIdx.x * TILE + threadIdx.x) >> 5; t < ntiles;
-       t += ((int64_t)gridDim.x * TILE) >> 5) {
+  for (int64_t t = ((int64_t)blockIdx.x * CLS_SCAN_THREADS + threadIdx.x) >> 5; t < ntiles;
+       t += ((int64_t)gridDim.x * CLS_SCAN_THREADS) >> 5) {
     const int64_t first = t * TP + lane * PER;
     uint32_t c = 0;
     if (aligned && first + PER <= n) {
@@ -1164,156 +1184,276 @@ __global__ void __launch_bounds__(TILE) k_compact_count(CompactArgs<Real> A) {
       A.read[t] = 0u;
     }
   }
-}
-
-// One CTA: exclusive scan of the tiles' counts.
-__global__ void __launch_bounds__(CLS_SCAN_THREADS) k_compact_scan(uint32_t *off, uint32_t *total, const int64_t *d_n,
-                                                                   int tile) {
-  constexpr int ITEMS = 8;
-  __shared__ uint32_t sm[33];
-  const int64_t ntiles = (*(volatile const int64_t *)d_n + tile - 1) / tile;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(&A.ticket[3], 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last) return;
   uint32_t carry = 0;
-  for (int64_t r0 = 0; r0 < ntiles; r0 += CLS_SCAN_THREADS * ITEMS) {
-    const int64_t c0 = r0 + (int64_t)threadIdx.x * ITEMS;
-    uint32_t v[ITEMS], t = 0;
+  for (int64_t r0 = 0; r0 < ntiles; r0 += CLS_SCAN_THREADS * 8) {
+    const int64_t c0 = r0 + (int64_t)threadIdx.x * 8;
+    uint32_t v[8], t = 0;
+    if (c0 + 8 <= ntiles) {
+      load8(v, A.off + c0);
+    } else {
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      v[j] = c0 + j < ntiles ? off[c0 + j] : 0u;
-      t += v[j];
+      for (int j = 0; j < 8; ++j) v[j] = c0 + j < ntiles ? A.off[c0 + j] : 0u;
     }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) t += v[j];
     uint32_t run = carry + block_excl_scan(t, sm);
     carry += sm[32];
     __syncthreads();  // sm[32] is read
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      if (c0 + j < ntiles) off[c0 + j] = run;
-      run += v[j];
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t q = v[j];
+      v[j] = run;
+      run += q;
+    }
+    if (c0 + 8 <= ntiles) {
+      store8(A.off + c0, v);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (c0 + j < ntiles) A.off[c0 + j] = v[j];
     }
   }
-  if (threadIdx.x == 0) *total = carry;
+  if (threadIdx.x == 0) {
+    *A.total = carry;
+    A.ticket[3] = 0u;
+  }
 }
 
 __device__ __forceinline__ uint32_t word_hash(float v) { return __float_as_uint(v); }
 __device__ __forceinline__ uint32_t word_hash(double v) { return (uint32_t)__double2loint(v) ^ (uint32_t)__double2hiint(v); }
 
+// What a thread holds of a tile.
+template <class Real> struct CompactPart {
+  static constexpr int CI = compact_items<Real>();
+  bool keep[CI];
+  Real v[CI][13];
+  uint64_t id[CI];
+  uint32_t tg[CI];
+};
+
+template <class Real>
+__device__ __forceinline__ void compact_load(const Sp<Real> &S, int64_t t, int64_t n, CompactPart<Real> &r) {
+  const bool fields = S.ex != nullptr;
+#pragma unroll
+  for (int k = 0; k < r.CI; ++k) {  // (the words do not wait for the flag)
+    const int64_t i = t * compact_tile<Real>() + k * COMPACT_THREADS + threadIdx.x;
+    r.keep[k] = false;
+    r.id[k] = 0;
+    r.tg[k] = 0;
+#pragma unroll
+    for (int q = 0; q < 13; ++q) r.v[k][q] = (Real)0;
+    if (i < n) {
+      r.keep[k] = S.alive[i];
+      r.v[k][0] = S.x[i]; r.v[k][1] = S.y[i]; r.v[k][2] = S.z[i];
+      r.v[k][3] = S.px[i]; r.v[k][4] = S.py[i]; r.v[k][5] = S.pz[i]; r.v[k][6] = S.w[i];
+      r.id[k] = S.id[i];
+      if (S.tag) r.tg[k] = S.tag[i];
+      if (fields) {
+        r.v[k][7] = S.ex[i]; r.v[k][8] = S.ey[i]; r.v[k][9] = S.ez[i];
+        r.v[k][10] = S.bx[i]; r.v[k][11] = S.by[i]; r.v[k][12] = S.bz[i];
+      }
+    }
+  }
+}
+
+// The warp's live particles of each item into s_warp; the value is a use of
+// every word, which therefore have arrived where it is known.
+template <class Real>
+__device__ __forceinline__ uint32_t compact_arrived(const CompactPart<Real> &r,
+                                                    uint32_t (*s_warp)[COMPACT_THREADS / 32]) {
+  uint32_t h = 0;
+#pragma unroll
+  for (int k = 0; k < r.CI; ++k) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, r.keep[k]);
+    if ((threadIdx.x & 31) == 0) s_warp[k][threadIdx.x >> 5] = __popc(m);
+    h ^= (uint32_t)r.id[k] ^ (uint32_t)(r.id[k] >> 32) ^ r.tg[k];
+#pragma unroll
+    for (int q = 0; q < 13; ++q) h ^= word_hash(r.v[k][q]);
+  }
+  return h;
+}
+
+// The live particles to their places from `off` on.
+template <class Real>
+__device__ __forceinline__ void compact_store(const Sp<Real> &S, const CompactPart<Real> &r, uint32_t off,
+                                              const uint32_t (*s_warp)[COMPACT_THREADS / 32]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool fields = S.ex != nullptr;
+  uint32_t before = off;
+#pragma unroll
+  for (int k = 0; k < r.CI; ++k) {
+    uint32_t base = before;
+#pragma unroll
+    for (int w = 0; w < COMPACT_THREADS / 32; ++w) {
+      if (w < wid) base += s_warp[k][w];
+      before += s_warp[k][w];
+    }
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, r.keep[k]);
+    if (!r.keep[k]) continue;
+    const int64_t d = base + __popc(m & ((1u << lane) - 1u));
+    S.x[d] = r.v[k][0]; S.y[d] = r.v[k][1]; S.z[d] = r.v[k][2];
+    S.px[d] = r.v[k][3]; S.py[d] = r.v[k][4]; S.pz[d] = r.v[k][5]; S.w[d] = r.v[k][6];
+    S.id[d] = r.id[k];
+    S.alive[d] = 1;
+    if (S.tag) S.tag[d] = r.tg[k];
+    if (fields) {
+      S.ex[d] = r.v[k][7]; S.ey[d] = r.v[k][8]; S.ez[d] = r.v[k][9];
+      S.bx[d] = r.v[k][10]; S.by[d] = r.v[k][11]; S.bz[d] = r.v[k][12];
+    }
+  }
+}
+
+// Up to COMPACT_ONE tiles, one per CTA, in one launch: every tile publishes its
+// live particles once its words have arrived, for itself and for its group of
+// 32 tiles, and one warp adds up those of the groups and tiles before it, whose
+// words have then been read as well.  (24,000 FP32 photons: kernel 10 us with the
+// look-back, 12 and a launch gap in two launches, 7 this way; 200,000: 13, 15,
+// 11; 524,288, the most: 23, 22, 22.  All 256 threads polling the tiles before
+// it took 20 for 200,000.)
+template <class Real>
+__global__ void __launch_bounds__(COMPACT_THREADS, sizeof(Real) == 4 ? 4 : 3) k_compact_small(CompactArgs<Real> A) {
+  constexpr int CI = compact_items<Real>(), TP = compact_tile<Real>(), WARPS = COMPACT_THREADS / 32;
+  __shared__ uint32_t s_warp[CI][WARPS], s_off, s_tile;
+  const int64_t n = *(volatile int64_t *)A.s.d_n;
+  const int64_t ntiles = (n + TP - 1) / TP;
+  if (threadIdx.x == 0) s_tile = atomicAdd(&A.ticket[0], 1u);
+  __syncthreads();
+  const int64_t t = s_tile;
+  bool gave_up = false;
+  if (t < ntiles) {
+    CompactPart<Real> r;
+    compact_load(A.s, t, n, r);
+    __syncthreads_or((int)compact_arrived(r, s_warp));
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int k = 0; k < CI; ++k)
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) cnt += s_warp[k][w];
+    if (threadIdx.x < 32) {
+      const int lane = threadIdx.x, g = (int)t >> 5;
+      if (lane == 0) {
+        __threadfence();
+        *(volatile uint32_t *)&A.one[t] = cnt + 1;
+        atomicAdd(&A.group[g], (1u << 20) + cnt);
+      }
+      uint32_t a = lane < g ? 0u : 32u << 20, o = lane < (t & 31) ? 0u : 1u;
+      long long spins = 0;
+      while (a >> 20 != 32u || o == 0u) {
+        if (lane < g) a = *(volatile uint32_t *)&A.group[lane];
+        if (lane < (t & 31)) o = *(volatile uint32_t *)&A.one[(t & ~(int64_t)31) + lane];
+        if (++spins > LOOKBACK_SPIN_LIMIT) {
+          gave_up = true;
+          break;
+        }
+      }
+      __threadfence();
+      const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, (a & 0xFFFFFu) + o - 1u);
+      if (lane == 0) s_off = sum;
+    }
+    gave_up = __syncthreads_or(gave_up) != 0;
+    const uint32_t off = s_off;
+    if (!gave_up && (off != t * TP || cnt != (t + 1 < ntiles ? TP : n - t * TP))) compact_store(A.s, r, off, s_warp);
+    if (t == ntiles - 1 && threadIdx.x == 0) *A.total = off + cnt;
+  }
+  __syncthreads();
+  // the last CTA publishes the count, unless a tile gave up, and leaves zeros
+  if (threadIdx.x == 0) {
+    if (gave_up) {
+      atomicOr(&A.cnt->status, (unsigned)QED_STATUS_TIMEOUT);
+      atomicAdd(&A.ticket[2], 1u);
+    }
+    __threadfence();
+    s_tile = atomicAdd(&A.ticket[1], 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_tile) return;
+  for (int64_t s = threadIdx.x; s < ntiles; s += COMPACT_THREADS) A.one[s] = 0u;
+  if (threadIdx.x < COMPACT_ONE / 32) A.group[threadIdx.x] = 0u;
+  if (threadIdx.x == 0) {
+    if (ntiles > 0 && *(volatile unsigned *)&A.ticket[2] == 0u) *A.s.d_n = *(volatile uint32_t *)A.total;
+    A.ticket[0] = A.ticket[1] = A.ticket[2] = 0u;
+  }
+}
+
 template <class Real>
 __global__ void __launch_bounds__(COMPACT_THREADS, sizeof(Real) == 4 ? 4 : 3) k_compact_move(CompactArgs<Real> A) {
   constexpr int CI = compact_items<Real>(), TP = compact_tile<Real>(), WARPS = COMPACT_THREADS / 32;
-  __shared__ uint32_t s_warp[CI][WARPS];
-  __shared__ uint32_t s_tile, s_off, s_end, s_go;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ uint32_t s_warp[2][CI][WARPS];  // (what a tile leaves here alternates between two places)
+  __shared__ uint32_t s_tile[2], s_off[2], s_end[2], s_go[2];
+  const int lane = threadIdx.x & 31;
   const int64_t n = *(volatile int64_t *)A.s.d_n;
   const int64_t ntiles = (n + TP - 1) / TP;
-  const bool fields = A.s.ex != nullptr;
   bool gave_up = false;
-  // (thread 0) tile t's place, for all after the next barrier
-  auto put_tile = [&](uint32_t t) {
-    s_tile = t;
+  // (thread 0) takes a tile
+  auto take = [&](int p) {
+    const uint32_t t = atomicAdd(&A.ticket[0], 1u);
+    s_tile[p] = t;
     if (t < ntiles) {
-      s_off = A.off[t];
-      s_end = t + 1 < ntiles ? A.off[t + 1] : *A.total;
+      s_off[p] = A.off[t];
+      s_end[p] = t + 1 < ntiles ? A.off[t + 1] : *A.total;
     }
   };
-  if (threadIdx.x == 0) put_tile(atomicAdd(&A.ticket[0], 1u));
+  if (threadIdx.x == 0) take(0);
   __syncthreads();
-  for (;;) {
-    const int64_t t = s_tile;
+  for (int p = 0;; p ^= 1) {
+    const int64_t t = s_tile[p];
     if (t >= ntiles) break;
-    const uint32_t off = s_off, cnt = s_end - off;
-    // the next tile's ticket is taken now: a CTA waits only for tiles before its
-    // own, and those before the next one it holds never wait for it, so the
-    // first tile not done can always go on
-    uint32_t next = 0;
-    if (threadIdx.x == 0) next = atomicAdd(&A.ticket[0], 1u);
+    const uint32_t off = s_off[p], cnt = s_end[p] - off;
     const bool whole = cnt == (uint32_t)(t + 1 < ntiles ? TP : n - t * TP);
-    // a tile that stays where it is moves nothing, and none writes into it
-    const bool stays = (int64_t)off == t * TP && whole;
-    if (!stays) {
-      bool keep[CI];
-      Real v[CI][13];
-      uint64_t id[CI];
-      uint32_t tg[CI], h = 0;
-#pragma unroll
-      for (int k = 0; k < CI; ++k) {  // (the words do not wait for the flag)
-        const int64_t i = t * TP + k * COMPACT_THREADS + threadIdx.x;
-        keep[k] = false;
-        id[k] = 0;
-        tg[k] = 0;
-#pragma unroll
-        for (int q = 0; q < 13; ++q) v[k][q] = (Real)0;
-        if (i < n) {
-          keep[k] = A.s.alive[i];
-          v[k][0] = A.s.x[i]; v[k][1] = A.s.y[i]; v[k][2] = A.s.z[i];
-          v[k][3] = A.s.px[i]; v[k][4] = A.s.py[i]; v[k][5] = A.s.pz[i]; v[k][6] = A.s.w[i];
-          id[k] = A.s.id[i];
-          if (A.s.tag) tg[k] = A.s.tag[i];
-          if (fields) {
-            v[k][7] = A.s.ex[i]; v[k][8] = A.s.ey[i]; v[k][9] = A.s.ez[i];
-            v[k][10] = A.s.bx[i]; v[k][11] = A.s.by[i]; v[k][12] = A.s.bz[i];
-          }
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < CI; ++k) {
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, keep[k]);
-        if (lane == 0) s_warp[k][wid] = __popc(m);
-        // a use of every word, so that all have arrived at the barrier
-        h ^= (uint32_t)id[k] ^ (uint32_t)(id[k] >> 32) ^ tg[k];
-#pragma unroll
-        for (int q = 0; q < 13; ++q) h ^= word_hash(v[k][q]);
-      }
-      __syncthreads_or((int)h);
-      if (threadIdx.x == 0) {
-        __threadfence();
-        *(volatile uint32_t *)&A.read[t] = 1u;
-        uint32_t go = 1;
-        if (cnt)
-          for (int64_t s = off / TP; s <= (int64_t)((off + cnt - 1) / TP) && s < t; ++s) {
-            // (a tile that stays has published nothing, and nothing is written to it)
-            long long spins = 0;
-            while (*(volatile uint32_t *)&A.read[s] == 0u)
-              if (++spins > LOOKBACK_SPIN_LIMIT) {
-                go = 0;
-                break;
-              }
-          }
-        __threadfence();
-        s_go = go;
-        put_tile(next);
-      }
+    if ((int64_t)off == t * TP && whole) {
+      // a tile that stays where it is moves nothing, and none writes into it
+      if (threadIdx.x == 0) take(p ^ 1);
       __syncthreads();
-      if (s_go) {
-        uint32_t before = off;
-#pragma unroll
-        for (int k = 0; k < CI; ++k) {
-          uint32_t base = before;
-#pragma unroll
-          for (int w = 0; w < WARPS; ++w) {
-            if (w < wid) base += s_warp[k][w];
-            before += s_warp[k][w];
-          }
-          const unsigned m = __ballot_sync(0xFFFFFFFFu, keep[k]);
-          if (!keep[k]) continue;
-          const int64_t d = base + __popc(m & ((1u << lane) - 1u));
-          A.s.x[d] = v[k][0]; A.s.y[d] = v[k][1]; A.s.z[d] = v[k][2];
-          A.s.px[d] = v[k][3]; A.s.py[d] = v[k][4]; A.s.pz[d] = v[k][5]; A.s.w[d] = v[k][6];
-          A.s.id[d] = id[k];
-          A.s.alive[d] = 1;
-          if (A.s.tag) A.s.tag[d] = tg[k];
-          if (fields) {
-            A.s.ex[d] = v[k][7]; A.s.ey[d] = v[k][8]; A.s.ez[d] = v[k][9];
-            A.s.bx[d] = v[k][10]; A.s.by[d] = v[k][11]; A.s.bz[d] = v[k][12];
-          }
-        }
-      } else {
-        gave_up = true;
-      }
-      __syncthreads();  // s_warp and s_go are read
-    } else {
-      __syncthreads();  // the tile's place is read
-      if (threadIdx.x == 0) put_tile(next);
-      __syncthreads();
+      continue;
     }
+    CompactPart<Real> r;
+    compact_load(A.s, t, n, r);
+    // (thread 0, while its words are on their way) the tiles before this one
+    // that it writes to: at most two
+    const int64_t s0 = off / TP, s1 = cnt ? (int64_t)((off + cnt - 1) / TP) : -1;
+    uint32_t f0 = WARPS, f1 = WARPS;
+    if (threadIdx.x == 0) {
+      if (s0 <= s1 && s0 < t) f0 = *(volatile uint32_t *)&A.read[s0];
+      if (s0 < s1 && s1 < t) f1 = *(volatile uint32_t *)&A.read[s1];
+    }
+    // the warp publishes when its words have arrived
+    const uint32_t h = __reduce_or_sync(0xFFFFFFFFu, compact_arrived(r, s_warp[p]));
+    if (lane == 0) {
+      __threadfence();
+      asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(A.read + t), "r"(1u), "r"(h) : "memory");
+    }
+    if (threadIdx.x == 0) {
+      // a CTA waits with no other tile in hand, after publishing its own, and
+      // only for tiles before it
+      uint32_t go = 1;
+      for (int64_t s = s0; s <= s1 && s < t; ++s) {
+        uint32_t f = s == s0 ? f0 : f1;
+        long long spins = 0;
+        while (f != WARPS && (f = *(volatile uint32_t *)&A.read[s]) != WARPS)
+          if (++spins > LOOKBACK_SPIN_LIMIT) {
+            go = 0;
+            break;
+          }
+      }
+      __threadfence();
+      s_go[p] = go;
+      take(p ^ 1);
+    }
+    __syncthreads();
+    if (!s_go[p]) {
+      gave_up = true;
+      continue;
+    }
+    compact_store(A.s, r, off, s_warp[p]);
   }
   // the last CTA publishes the count -- unless a tile gave up, and so wrote
   // nothing -- and leaves the counters at zero
@@ -1980,17 +2120,25 @@ cudaError_t launch_compact(qed_ctx *c, const qed_species *s, cudaStream_t st) {
   a.read = c->sub_cnt + tiles;
   a.total = c->sub_cnt + 2 * tiles;
   a.ticket = c->compact_n;
+  a.one = c->compact_n + 4;
   a.cnt = c->d_counters;
-  const int64_t count_need = (tiles * 32 + TILE - 1) / TILE, count_most = (int64_t)c->num_sms * 8;
-  k_compact_count<Real><<<(unsigned)(count_need < 1 ? 1 : count_need < count_most ? count_need : count_most), TILE, 0, st>>>(a);
-  k_compact_scan<<<1, CLS_SCAN_THREADS, 0, st>>>(a.off, a.total, s->d_n, TP);
+  if (tiles <= COMPACT_ONE) {
+    a.group = a.one + COMPACT_ONE;
+    a.total = a.group + COMPACT_ONE / 32;
+    k_compact_small<Real><<<(unsigned)(tiles < 1 ? 1 : tiles), COMPACT_THREADS, 0, st>>>(a);
+    c->launches += 1;
+    return cudaGetLastError();
+  }
+  const int64_t count_need = (tiles * 32 + CLS_SCAN_THREADS - 1) / CLS_SCAN_THREADS, count_most = (int64_t)c->num_sms * 2;
+  k_compact_count<Real><<<(unsigned)(count_need < 1 ? 1 : count_need < count_most ? count_need : count_most),
+                          CLS_SCAN_THREADS, 0, st>>>(a);
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_compact_move<Real>, COMPACT_THREADS, 0);
   if (e != cudaSuccess) return e;
   per_sm = persistent_blocks_per_sm(c, per_sm, QED_TUNE_COMPACT);
   const int64_t most = (int64_t)c->num_sms * per_sm;
   k_compact_move<Real><<<(unsigned)(tiles < 1 ? 1 : tiles < most ? tiles : most), COMPACT_THREADS, 0, st>>>(a);
-  c->launches += 3;
+  c->launches += 2;
   return cudaGetLastError();
 }
 
