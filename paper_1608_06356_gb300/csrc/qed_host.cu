@@ -7,16 +7,18 @@
 // previous chunk has been copied out), stepped on the caller's stream -- the
 // same launches as qed_step_fused's lepton stage, appending photons to the
 // device photon species -- and its positions and momenta copied back on the
-// output stream.  The photons a chunk appended go to the host mirror of the
-// photon species on the output stream too: by a copy kernel that reads the
-// chunk's range on the device and writes through host-mapped pointers, so
-// that every chunk is queued at once and the host waits only at the end (or,
-// for mirror memory the device cannot map, by copies whose ranges the host
-// reads after each chunk).  Particle ids key the random
+// output stream, together with the photons the chunk appended for the host
+// mirror of the photon species.  Both ways a copy kernel works through
+// host-mapped pointers; the photons' range is read on the device, so that
+// every chunk is queued at once and the host waits only at the end.  Memory the
+// device cannot map goes by copies per array, the photons' after the host has
+// read their range.  Particle ids key the random
 // streams, so chunking changes no result, only the order of the photons
 // (chunks in order; within a chunk as the lepton step appends them).
 #include <cstdio>
 #include <cstring>
+
+#include <cuda.h>
 
 #include "qed_internal.h"
 
@@ -38,48 +40,119 @@ int cuda_fail(cudaError_t e, const char *what) {
 __global__ void k_set_count(int64_t *d_n, int64_t v) { *d_n = v; }
 __global__ void k_mark_count(int64_t *dst, const int64_t *src) { *dst = *src; }
 
-// Copy of the photons appended by one chunk, [*lo, *hi) clamped to the
-// capacity, from the device photon species to its host mirror through
-// host-mapped pointers: the range is read on the device, so no host round
-// trip is needed between the chunks.
-constexpr int MAX_PARRAYS = 16;
-struct PhotonCopy {
-  const char *src[MAX_PARRAYS];
-  char *dst[MAX_PARRAYS];
-  int esz[MAX_PARRAYS];
-  int wide[MAX_PARRAYS];  // 16: both bases 16-byte aligned; 4: 4-byte aligned; else bytes
-  int np;
+// One chunk's arrays between host memory and the GPU, copied by the SMs through
+// host-mapped pointers: arrays [0, nl) over n elements, and arrays [nl, na)
+// over the photons a chunk appended, [*lo, *hi) clamped to the capacity -- a
+// range read on the device, so no host round trip is needed between chunks.
+//
+// The host link bounds the host step.  A copy engine takes one array at a time
+// and idles between them: 120 copies of 2 MB ran at 173 GB/s in, and at 146
+// with the copies out beside them (58); a launch per chunk each way gives 211
+// alone, 197 beside 79.  4M leptons in 8 chunks: 2012 -> 1570 us, 1195 of them
+// the link's for what comes in.
+// The copies must run beside the lepton kernel, which leaves 4096 registers of
+// an SM: a CTA is 128 threads of at most 32 registers (units of 8 KB, round
+// robin over the arrays, 64 bytes in flight per thread), and it asks for the
+// shared memory carve-out the lepton kernel needs -- an SM changes its carve-out
+// only when it is empty, so with the default the lepton kernel waited for the
+// copies to end (1860 us).  One CTA per SM in: with half as many, 1700.  A
+// quarter of the SMs out, so that what goes out takes its share of the link over
+// the whole of the next chunk: half of them 1750, a twelfth 1830.
+constexpr int MAX_LANES = 17;     // of a lepton species
+constexpr int MAX_PARRAYS = 16;   // of a photon species
+constexpr int MAX_COPY = MAX_LANES + MAX_PARRAYS;
+constexpr int COPY_THREADS = 128, COPY_UNIT = 4 * COPY_THREADS;  // 16-byte words per unit
+struct CopyArgs {
+  const char *src[MAX_COPY];
+  char *dst[MAX_COPY];
+  int esz[MAX_COPY];
+  int wide[MAX_COPY];  // 16: both bases 16-byte aligned; 4: 4-byte aligned; else bytes
+  int nl, na;
+  int64_t n;
   const int64_t *lo, *hi;
   int64_t cap;
+  int64_t *set_n;  // where n is left as the chunk's count, or null
 };
 
-__global__ void __launch_bounds__(256) k_copy_photons(PhotonCopy A) {
+// Array between offsets b0 and b1 of its bytes: bytes or 4-byte words up to a
+// 16-byte boundary, units of 16-byte words, and the rest.  base = units handed
+// out so far.
+__device__ __forceinline__ void copy_array(const char *src, char *dst, int esz, int wide, int64_t b0,
+                                           int64_t b1, int64_t &base) {
+  const int64_t t0 = (int64_t)blockIdx.x * COPY_THREADS + threadIdx.x;
+  const int64_t nt = (int64_t)gridDim.x * COPY_THREADS;
+  if (b1 <= b0) return;
+  if (esz % 4 || wide < 4) {  // alive flags, or unaligned bases
+    for (int64_t q = b0 + t0; q < b1; q += nt) dst[q] = src[q];
+    return;
+  }
+  const uint32_t *s4 = reinterpret_cast<const uint32_t *>(src);
+  uint32_t *d4 = reinterpret_cast<uint32_t *>(dst);
+  const int64_t m0 = (b0 + 15) & ~(int64_t)15, m1 = b1 & ~(int64_t)15;
+  if (m0 >= m1 || wide < 16) {
+    for (int64_t q = b0 / 4 + t0; q < b1 / 4; q += nt) d4[q] = s4[q];
+    return;
+  }
+  if (t0 < 3) {  // at most three words on either side
+    if (b0 / 4 + t0 < m0 / 4) d4[b0 / 4 + t0] = s4[b0 / 4 + t0];
+    if (m1 / 4 + t0 < b1 / 4) d4[m1 / 4 + t0] = s4[m1 / 4 + t0];
+  }
+  const uint4 *s = reinterpret_cast<const uint4 *>(src + m0);
+  uint4 *d = reinterpret_cast<uint4 *>(dst + m0);
+  const int64_t nw = (m1 - m0) / 16, nu = (nw + COPY_UNIT - 1) / COPY_UNIT;
+  const int grid = (int)gridDim.x, r = (int)(base % grid);
+  for (int64_t u = (int)blockIdx.x >= r ? blockIdx.x - r : blockIdx.x - r + grid; u < nu; u += grid) {
+    const int64_t w = u * COPY_UNIT + threadIdx.x;
+    uint4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (w + k * COPY_THREADS < nw) v[k] = s[w + k * COPY_THREADS];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (w + k * COPY_THREADS < nw) d[w + k * COPY_THREADS] = v[k];
+  }
+  base += nu;
+}
+
+__global__ void __launch_bounds__(COPY_THREADS, 16) k_copy_chunk(const __grid_constant__ CopyArgs A) {
+  if (A.set_n && blockIdx.x == 0 && threadIdx.x == 0) *A.set_n = A.n;
+  int64_t base = 0;
+  for (int a = 0; a < A.nl; ++a)
+    copy_array(A.src[a], A.dst[a], A.esz[a], A.wide[a], 0, A.n * A.esz[a], base);
+  if (A.na == A.nl) return;
   int64_t lo = *A.lo, hi = *A.hi;
   lo = lo < A.cap ? lo : A.cap;
   hi = hi < A.cap ? hi : A.cap;
-  if (hi <= lo) return;
-  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nt = (int64_t)gridDim.x * blockDim.x;
-  for (int a = 0; a < A.np; ++a) {
-    const int64_t b0 = lo * A.esz[a], b1 = hi * A.esz[a];
-    if (A.esz[a] % 4 || A.wide[a] < 4) {  // bytes (alive flags, or unaligned bases)
-      for (int64_t q = b0 + t0; q < b1; q += nt) A.dst[a][q] = A.src[a][q];
-      continue;
-    }
-    // 4-byte words up to a 16-byte boundary, 16-byte words, 4-byte words after
-    const int64_t m0 = (b0 + 15) & ~(int64_t)15, m1 = b1 & ~(int64_t)15;
-    if (m0 >= m1 || A.wide[a] < 16) {
-      for (int64_t q = b0 / 4 + t0; q < b1 / 4; q += nt)
-        reinterpret_cast<uint32_t *>(A.dst[a])[q] = reinterpret_cast<const uint32_t *>(A.src[a])[q];
-      continue;
-    }
-    for (int64_t q = b0 / 4 + t0; q < m0 / 4; q += nt)
-      reinterpret_cast<uint32_t *>(A.dst[a])[q] = reinterpret_cast<const uint32_t *>(A.src[a])[q];
-    for (int64_t q = m0 / 16 + t0; q < m1 / 16; q += nt)
-      reinterpret_cast<uint4 *>(A.dst[a])[q] = reinterpret_cast<const uint4 *>(A.src[a])[q];
-    for (int64_t q = m1 / 4 + t0; q < b1 / 4; q += nt)
-      reinterpret_cast<uint32_t *>(A.dst[a])[q] = reinterpret_cast<const uint32_t *>(A.src[a])[q];
-  }
+  for (int a = A.nl; a < A.na; ++a)
+    copy_array(A.src[a], A.dst[a], A.esz[a], A.wide[a], lo * A.esz[a], hi * A.esz[a], base);
+}
+
+int width_of(const void *a, const void *b) {
+  const uintptr_t al = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
+  return al % 16 == 0 ? 16 : al % 4 == 0 ? 4 : 1;
+}
+
+// The device pointer of `bytes` bytes of host memory that the device can map
+// (page-locked memory allocated by the CUDA runtime is), or null: the whole
+// range must lie in one allocation or registration.
+char *map_host(void *h, size_t bytes) {
+  static const auto query = [] {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess)
+      fn = nullptr;
+    return reinterpret_cast<CUresult (*)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr)>(fn);
+  }();
+  CUpointer_attribute what[3] = {CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  CUdeviceptr d = 0, start = 0;
+  size_t size = 0;
+  void *out[3] = {&d, &start, &size};
+  // (what is not known of a pointer reads as zero)
+  if (!query || query(3, what, out, reinterpret_cast<CUdeviceptr>(h)) != CUDA_SUCCESS || !d) return nullptr;
+  if (d < start || d - start > size || size - (d - start) < bytes) return nullptr;
+  return reinterpret_cast<char *>(d);
 }
 
 // One array of the lepton species as the host step moves it: host pointer,
@@ -97,7 +170,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // The arrays of a lepton species, in staging order; *per_buf = staging bytes
 // of one buffer for `chunk` leptons.
-int lanes_of(const qed_species *s, size_t real, int64_t chunk, Lane out[16], size_t *per_buf) {
+int lanes_of(const qed_species *s, size_t real, int64_t chunk, Lane out[MAX_LANES], size_t *per_buf) {
   int n = 0;
   size_t off = 0;
   auto add = [&](void *p, size_t esz, bool back) {
@@ -210,7 +283,7 @@ int lepton_step_host(qed_ctx *c, const qed_species *lh, const qed_species *g,
   const size_t real = f64 ? sizeof(double) : sizeof(float);
   const int64_t n = *lh->d_n;
   if (n < 0 || n > lh->capacity) return QED_ERR_ARG;
-  Lane L[16];
+  Lane L[MAX_LANES];
   size_t per_buf = 0;
   const int nl = lanes_of(lh, real, chunk, L, &per_buf);
   void *pdev[16], *phost[16];
@@ -222,32 +295,38 @@ int lepton_step_host(qed_ctx *c, const qed_species *lh, const qed_species *g,
     return QED_ERR_UNSUPPORTED;
   int rc = ensure_host_step(c, per_buf);
   if (rc != QED_OK) return rc;
-  // The photons go to the host mirror by a copy kernel writing through
-  // host-mapped pointers when every mirror array is mapped (page-locked
-  // memory allocated by the CUDA runtime is); otherwise by copies whose
-  // ranges the host reads after each chunk.
-  PhotonCopy pc{};
+  // The arrays are copied by k_copy_chunk where the device can map them all:
+  // the leptons if they are 16-byte aligned too (a chunk is rounded to a
+  // multiple of four leptons to keep them so), else by a copy per array; the
+  // photons else by copies whose ranges the host reads after each chunk.
+  if (chunk > 4) chunk &= ~(int64_t)3;
+  char *lmap[MAX_LANES];
+  bool lmapped = true;
+  for (int a = 0; a < nl && lmapped; ++a) {
+    lmap[a] = map_host(L[a].host, (size_t)n * L[a].esz);
+    lmapped = lmap[a] && width_of(lmap[a], L[a].host) == 16;
+  }
+  if (n > chunk && chunk % 4) lmapped = false;
+  CopyArgs pc{};
   bool mapped = gh != nullptr && np > 0;
   for (int a = 0; a < np && mapped; ++a) {
-    void *dp = nullptr;
-    if (cudaHostGetDevicePointer(&dp, phost[a], 0) != cudaSuccess) {
-      mapped = false;
-      cudaGetLastError();  // clear the error of the query
-      break;
-    }
+    char *dp = map_host(phost[a], (size_t)g->capacity * pesz[a]);
+    mapped = dp != nullptr;
     pc.src[a] = static_cast<const char *>(pdev[a]);
-    pc.dst[a] = static_cast<char *>(dp);
+    pc.dst[a] = dp;
     pc.esz[a] = (int)pesz[a];
-    const uintptr_t al = reinterpret_cast<uintptr_t>(pdev[a]) | reinterpret_cast<uintptr_t>(dp);
-    pc.wide[a] = al % 16 == 0 ? 16 : al % 4 == 0 ? 4 : 1;
+    pc.wide[a] = width_of(pdev[a], dp);
   }
-  pc.np = np;
+  pc.na = mapped ? np : 0;
   pc.cap = g->capacity;
+  const int in_blocks = c->num_sms, out_blocks = (c->num_sms + 3) / 4;
   constexpr int R = NBUF + 1;  // device ring of photon counts after each chunk
   int64_t *ring = c->hs_dn + NBUF;
   cudaEvent_t *in_done = c->hs_ev, *comp_done = c->hs_ev + NBUF, *out_done = c->hs_ev + 2 * NBUF;
   int64_t *cnt = c->hs_cnt;  // [0, NBUF): photon count after chunk k (slot k % NBUF); [NBUF]: at start
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k_copy_chunk, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                       cudaSharedmemCarveoutMaxShared);
+  if (e != cudaSuccess) return cuda_fail(e, "qed_lepton_step_host");
   int64_t m_done = 0;  // (host-read ranges) photons already on the host mirror
   if (mapped) {
     k_mark_count<<<1, 1, 0, st>>>(ring, g->d_n);
@@ -281,13 +360,29 @@ int lepton_step_host(qed_ctx *c, const qed_species *lh, const qed_species *g,
     char *base = static_cast<char *>(c->hs_mem) + (size_t)b * c->hs_per_buf;
     // in: once the buffer's previous chunk has been copied out
     if (k >= NBUF) e = cudaStreamWaitEvent(c->hs_in, out_done[b], 0);
-    for (int a = 0; a < nl && e == cudaSuccess; ++a)
-      e = cudaMemcpyAsync(base + L[a].off, L[a].host + (size_t)off * L[a].esz, (size_t)nk * L[a].esz,
-                          cudaMemcpyHostToDevice, c->hs_in);
-    if (e == cudaSuccess) {
-      k_set_count<<<1, 1, 0, c->hs_in>>>(c->hs_dn + b, nk);
+    if (e == cudaSuccess && lmapped) {
+      CopyArgs in{};
+      for (int a = 0; a < nl; ++a) {
+        in.src[a] = lmap[a] + (size_t)off * L[a].esz;
+        in.dst[a] = base + L[a].off;
+        in.esz[a] = (int)L[a].esz;
+        in.wide[a] = 16;
+      }
+      in.nl = in.na = nl;
+      in.n = nk;
+      in.set_n = c->hs_dn + b;
+      k_copy_chunk<<<in_blocks, COPY_THREADS, 0, c->hs_in>>>(in);
       c->launches += 1;
       e = cudaGetLastError();
+    } else {
+      for (int a = 0; a < nl && e == cudaSuccess; ++a)
+        e = cudaMemcpyAsync(base + L[a].off, L[a].host + (size_t)off * L[a].esz,
+                            (size_t)nk * L[a].esz, cudaMemcpyHostToDevice, c->hs_in);
+      if (e == cudaSuccess) {
+        k_set_count<<<1, 1, 0, c->hs_in>>>(c->hs_dn + b, nk);
+        c->launches += 1;
+        e = cudaGetLastError();
+      }
     }
     if (e == cudaSuccess) e = cudaEventRecord(in_done[b], c->hs_in);
     // step on the caller's stream, then the photon count after it
@@ -308,16 +403,29 @@ int lepton_step_host(qed_ctx *c, const qed_species *lh, const qed_species *g,
     // out: the updated positions and momenta (and event-generator state), and
     // with mapped mirrors the chunk's photons
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->hs_out, comp_done[b], 0);
-    for (int a = 0; a < nl && e == cudaSuccess; ++a)
-      if (L[a].back)
-        e = cudaMemcpyAsync(L[a].host + (size_t)off * L[a].esz, base + L[a].off, (size_t)nk * L[a].esz,
-                            cudaMemcpyDeviceToHost, c->hs_out);
-    if (e == cudaSuccess && mapped) {
+    if (!lmapped)
+      for (int a = 0; a < nl && e == cudaSuccess; ++a)
+        if (L[a].back)
+          e = cudaMemcpyAsync(L[a].host + (size_t)off * L[a].esz, base + L[a].off,
+                              (size_t)nk * L[a].esz, cudaMemcpyDeviceToHost, c->hs_out);
+    if (e == cudaSuccess && (lmapped || mapped)) {
+      CopyArgs out{};
+      int m = 0;
+      auto add = [&](const char *src, char *dst, int esz, int wide) {
+        out.src[m] = src; out.dst[m] = dst; out.esz[m] = esz; out.wide[m] = wide; ++m;
+      };
+      for (int a = 0; a < nl && lmapped; ++a)
+        if (L[a].back) add(base + L[a].off, lmap[a] + (size_t)off * L[a].esz, (int)L[a].esz, 16);
+      out.nl = m;
+      for (int a = 0; a < pc.na; ++a) add(pc.src[a], pc.dst[a], pc.esz[a], pc.wide[a]);
+      out.na = m;
+      out.n = nk;
       // ring slot k % R is rewritten only by chunk k + NBUF, whose input copy
       // waits for this buffer's out_done (recorded after this copy)
-      pc.lo = ring + k % R;
-      pc.hi = ring + (k + 1) % R;
-      k_copy_photons<<<2 * c->num_sms, 256, 0, c->hs_out>>>(pc);
+      out.lo = ring + k % R;
+      out.hi = ring + (k + 1) % R;
+      out.cap = pc.cap;
+      k_copy_chunk<<<out_blocks, COPY_THREADS, 0, c->hs_out>>>(out);
       c->launches += 1;
       e = cudaGetLastError();
     }
