@@ -57,7 +57,7 @@ LEPTON_ONEPASS_TRAFFIC_64M = 6.59e9
 # the photon buffer holds 1.6x that
 PHOTONS_PER_ELECTRON_CAP = 0.3
 # the lepton step runs in a single pass, appending photons in no particular
-# order (the same photons as the ordered multi-pass path, bit for bit)
+# order (the same photons as with ordered appends, bit for bit)
 APPEND_ORDER = 1
 QED_STATUS_CAPACITY = 1
 QED_STATUS_ERRORS = 1 | 4 | 8 | 32  # capacity, non-finite, timeout, replay
@@ -282,8 +282,8 @@ def lepton_roofline(r, n, steps, peak, peak_kind, mlp=False):
     """Roofline of the lepton step (the per-lepton unit whose algorithmic
     bytes are 84 B + 61 B per emitted photon), timed by CUDA events that the
     library records on the launching stream: the single-pass kernel (and,
-    with the learned sampler, its dense pass), or the ordered path's five
-    phases (streaming pass, class list, counting pass, scan, writing pass)."""
+    with the learned sampler, its dense pass), or with ordered appends the
+    single pass (the first phase) and its ordering passes."""
     import paper_1608_06356_gb300.api as A
     phases, nprof = r["phases"], max(r["nprof"], 1)
     lep_ms = sum(phases[k] for k in A.PROF_PHASES[:5]) / nprof
@@ -294,8 +294,7 @@ def lepton_roofline(r, n, steps, peak, peak_kind, mlp=False):
     return {"bound": "hbm",
             "kernel": (("lepton step: k_lepton_onepass + k_net_emit (the learned sampler's dense pass)"
                         if mlp else "lepton step: k_lepton_onepass") if APPEND_ORDER else
-                       "lepton step: k_lepton_stream + k_cls_count/scan/scatter + k_substep_count + "
-                       "k_sub_scan + k_substep_write_coop + k_substep_replay"),
+                       "lepton step: k_lepton_onepass + k_ord_scan/offsets/index/write + k_substep_replay"),
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "peak_source": f"{peak_kind} HBM copy (MEASURED_PEAKS.json hbm_gbs)",
             "traffic": (LEPTON_ONEPASS_TRAFFIC_64M if APPEND_ORDER and not mlp and n == N_PART else None),

@@ -202,11 +202,10 @@ int qed_pair(qed_ctx *ctx, const qed_species *photons, const qed_species *electr
              const qed_species *positrons, const qed_fields *f, int64_t step,
              qed_stream_t stream);
 
-/* Stable in-place removal of dead particles (alive == 0).  If a look-back
- * wait runs out (QED_STATUS_TIMEOUT), the tile that gave up writes nothing
- * and the count is left unchanged when it is the last tile: the species is
- * then not compacted (particles may be duplicated or stale) and must not be
- * used as the result. */
+/* Stable in-place removal of dead particles (alive == 0).  If a tile's wait for
+ * the tiles before it runs out (QED_STATUS_TIMEOUT), it writes nothing and the
+ * count is left unchanged: the species is then not compacted (particles may be
+ * duplicated or stale) and must not be used as the result. */
 int qed_compact(qed_ctx *ctx, const qed_species *s, qed_stream_t stream);
 
 /* Removal of dead particles that moves only as many particles as died.  With
