@@ -43,8 +43,7 @@ def test_lost_records_are_replayed(api, W, mode, ne, npos, dt):  # noqa: F811
         F = api.Fields.per_particle() if fields else api.Fields.uniform((0.0, 50.0, 0.0), (0.0, 0.0, 9000.0))
     a, b = {k: v[:ne] for k, v in st.items()}, {k: v[ne:] for k, v in st.items()}
     cap_g = 1 << 16
-    # (grid: the leptons' stage only; a second step has photons, whose pass on a
-    # grid depends on max_particles where its own records run out)
+    # (grid: the leptons' stage only)
     steps = 1 if mode == "grid" else 2
     small = _step(api, 1 << 16, a, b, cap_g, F, fields, dt, steps)
     large = _step(api, 1 << 22, a, b, cap_g, F, fields, dt, steps)
