@@ -49,7 +49,7 @@ __global__ void k_mark_count(int64_t *dst, const int64_t *src) { *dst = *src; }
 // and idles between them: 120 copies of 2 MB ran at 173 GB/s in, and at 146
 // with the copies out beside them (58); a launch per chunk each way gives 211
 // alone, 197 beside 79.  4M leptons in 8 chunks: 2012 -> 1570 us, 1195 of them
-// the link's for what comes in.
+// the link's for what comes in; 64M in 16, where a copy is 16 MB: 22.8 -> 20.8 ms.
 // The copies must run beside the lepton kernel, which leaves 4096 registers of
 // an SM: a CTA is 128 threads of at most 32 registers (units of 8 KB, round
 // robin over the arrays, 64 bytes in flight per thread), and it asks for the
@@ -74,28 +74,28 @@ struct CopyArgs {
   int64_t *set_n;  // where n is left as the chunk's count, or null
 };
 
-// Array between offsets b0 and b1 of its bytes: bytes or 4-byte words up to a
-// 16-byte boundary, units of 16-byte words, and the rest.  base = units handed
-// out so far.
+// Array between offsets b0 and b1 of its bytes: bytes up to a 16-byte boundary,
+// units of 16-byte words, and the rest (by words or bytes if the bases are not so
+// aligned).  base = units handed out so far.
 __device__ __forceinline__ void copy_array(const char *src, char *dst, int esz, int wide, int64_t b0,
                                            int64_t b1, int64_t &base) {
   const int64_t t0 = (int64_t)blockIdx.x * COPY_THREADS + threadIdx.x;
   const int64_t nt = (int64_t)gridDim.x * COPY_THREADS;
   if (b1 <= b0) return;
-  if (esz % 4 || wide < 4) {  // alive flags, or unaligned bases
-    for (int64_t q = b0 + t0; q < b1; q += nt) dst[q] = src[q];
-    return;
-  }
-  const uint32_t *s4 = reinterpret_cast<const uint32_t *>(src);
-  uint32_t *d4 = reinterpret_cast<uint32_t *>(dst);
   const int64_t m0 = (b0 + 15) & ~(int64_t)15, m1 = b1 & ~(int64_t)15;
   if (m0 >= m1 || wide < 16) {
-    for (int64_t q = b0 / 4 + t0; q < b1 / 4; q += nt) d4[q] = s4[q];
+    if (esz % 4 || wide < 4) {
+      for (int64_t q = b0 + t0; q < b1; q += nt) dst[q] = src[q];
+    } else {
+      const uint32_t *s4 = reinterpret_cast<const uint32_t *>(src);
+      uint32_t *d4 = reinterpret_cast<uint32_t *>(dst);
+      for (int64_t q = b0 / 4 + t0; q < b1 / 4; q += nt) d4[q] = s4[q];
+    }
     return;
   }
-  if (t0 < 3) {  // at most three words on either side
-    if (b0 / 4 + t0 < m0 / 4) d4[b0 / 4 + t0] = s4[b0 / 4 + t0];
-    if (m1 / 4 + t0 < b1 / 4) d4[m1 / 4 + t0] = s4[m1 / 4 + t0];
+  if (t0 < 15) {  // at most 15 bytes on either side
+    if (b0 + t0 < m0) dst[b0 + t0] = src[b0 + t0];
+    if (m1 + t0 < b1) dst[m1 + t0] = src[m1 + t0];
   }
   const uint4 *s = reinterpret_cast<const uint4 *>(src + m0);
   uint4 *d = reinterpret_cast<uint4 *>(dst + m0);
@@ -319,7 +319,7 @@ int lepton_step_host(qed_ctx *c, const qed_species *lh, const qed_species *g,
   }
   pc.na = mapped ? np : 0;
   pc.cap = g->capacity;
-  const int in_blocks = c->num_sms, out_blocks = (c->num_sms + 3) / 4;
+  const int in_blocks = c->num_sms, out_blocks = lmapped ? (c->num_sms + 3) / 4 : 4 * c->num_sms;
   constexpr int R = NBUF + 1;  // device ring of photon counts after each chunk
   int64_t *ring = c->hs_dn + NBUF;
   cudaEvent_t *in_done = c->hs_ev, *comp_done = c->hs_ev + NBUF, *out_done = c->hs_ev + 2 * NBUF;
