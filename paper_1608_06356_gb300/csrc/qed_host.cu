@@ -48,16 +48,17 @@ __global__ void k_mark_count(int64_t *dst, const int64_t *src) { *dst = *src; }
 // The host link bounds the host step.  A copy engine takes one array at a time
 // and idles between them: 120 copies of 2 MB ran at 173 GB/s in, and at 146
 // with the copies out beside them (58); a launch per chunk each way gives 211
-// alone, 197 beside 79.  4M leptons in 8 chunks: 2012 -> 1570 us, 1195 of them
-// the link's for what comes in; 64M in 16, where a copy is 16 MB: 22.8 -> 20.8 ms.
+// alone, 197 beside 79.  4M leptons in 8 chunks: 2012 -> 1660 us, 1195 of them
+// the link's for what comes in; 64M in 16, where a copy is 16 MB: 23.85 -> 23.2 ms.
 // The copies must run beside the lepton kernel, which leaves 4096 registers of
 // an SM: a CTA is 128 threads of at most 32 registers (units of 8 KB, round
 // robin over the arrays, 64 bytes in flight per thread), and it asks for the
 // shared memory carve-out the lepton kernel needs -- an SM changes its carve-out
 // only when it is empty, so with the default the lepton kernel waited for the
-// copies to end (1860 us).  One CTA per SM in: with half as many, 1700.  A
-// quarter of the SMs out, so that what goes out takes its share of the link over
-// the whole of the next chunk: half of them 1750, a twelfth 1830.
+// copies to end (1860 us).  One CTA per SM in: with half as many, 1700.  Three
+// in eight of the SMs out, so that what goes out takes its share of the link over
+// the whole of the next chunk: a quarter 1580 us for the 4M but 25.1 ms for the
+// 64M, half of them 24.4 ms.
 constexpr int MAX_LANES = 17;     // of a lepton species
 constexpr int MAX_PARRAYS = 16;   // of a photon species
 constexpr int MAX_COPY = MAX_LANES + MAX_PARRAYS;
@@ -319,7 +320,7 @@ int lepton_step_host(qed_ctx *c, const qed_species *lh, const qed_species *g,
   }
   pc.na = mapped ? np : 0;
   pc.cap = g->capacity;
-  const int in_blocks = c->num_sms, out_blocks = lmapped ? (c->num_sms + 3) / 4 : 4 * c->num_sms;
+  const int in_blocks = c->num_sms, out_blocks = lmapped ? (c->num_sms * 3 + 7) / 8 : 4 * c->num_sms;
   constexpr int R = NBUF + 1;  // device ring of photon counts after each chunk
   int64_t *ring = c->hs_dn + NBUF;
   cudaEvent_t *in_done = c->hs_ev, *comp_done = c->hs_ev + NBUF, *out_done = c->hs_ev + 2 * NBUF;
