@@ -258,13 +258,13 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   // of the two lepton species
   c->heavy_slots = ((cfg->max_particles + TILE - 1) / TILE * 2 + 2) * TILE;
   c->cls_chunks = c->heavy_slots / CLS_CHUNK_FLAGS + 1;
-  // emission records for the first max_particles / 4 entries of the sub-step
-  // list; later entries (and particles with more than SUB_REC photons) replay
-  c->rec_cap = cfg->max_particles / 4 > 4096 ? cfg->max_particles / 4 + 1 : 4096;
+  // emission records for the first quarter of the entries of the sub-step list;
+  // later entries (and particles with more than SUB_REC photons) replay
+  c->rec_cap = rec_entries(cfg->max_particles);
   const size_t rsize = f64 ? sizeof(double) : sizeof(float);
   // staging records for the leptons the streaming pass defers (a record is
   // 16 words); past stage_cap a deferred particle is gathered from its arrays
-  c->stage_cap = cfg->max_particles / 2 > 65536 ? cfg->max_particles / 2 + 1 : 65536;
+  c->stage_cap = stage_records(cfg->max_particles);
   if (cudaMalloc(&c->tile_state, sizeof(unsigned long long) * c->max_tiles) != cudaSuccess ||
       cudaMalloc(&c->sync, sizeof(unsigned int) * 4) != cudaSuccess ||
       cudaMalloc(&c->snap, sizeof(int64_t) * 4) != cudaSuccess ||

@@ -6,6 +6,7 @@
 
 #include "qed.h"
 #include "qed_device.cuh"
+#include "qed_scratch.h"
 
 struct qed_ctx {
   qed_config cfg;
@@ -150,6 +151,5 @@ inline cudaError_t prof_mark(qed_ctx *c, int k, cudaStream_t st) {
 constexpr int TILE = 256;  // particles per tile = threads per block in the step kernels
 constexpr int COMPACT_ONE = 1024;  // most tiles of the stable compaction's single launch
 constexpr int COMPACT_WORDS = 5 + COMPACT_ONE + COMPACT_ONE / 32;
-constexpr int SUB_REC = 8; // emission records kept per particle by the sub-step counting pass
 constexpr int CLS_CHUNK_FLAGS = 2048;  // flags per chunk of the class-list passes
 }  // namespace qed

@@ -56,7 +56,7 @@ template <class Real> struct PhotonArgs {
   const int64_t *d_step;  // if set, the step index is read here (graph replay)
   uint32_t *mask;         // [photon / 32] bits of the photons that convert
   uint32_t *sum, *off;    // [chunk] pairs (zero between steps), then the first pair's position
-  uint2 *rec_i;           // [record] photon, sub-step
+  uint2 *rec_i;           // [record] photon, sub-step (records for every photon: holds_pairs)
   Real *rec;              // [record][8] gamma_e, gamma_p, E, B (E, B with grid fields)
   unsigned int *n;        // [0] records, [1] those of the pass being written
   int64_t *meta;          // [1], [2] electron and positron counts before
@@ -67,6 +67,13 @@ template <class Real, int FM> size_t photon_smem(const qed_ctx *c) {
   return PH_WARPS * PH_POOL * (sizeof(PoolEntry<Real, FM>) + 2) + sizeof(Real) * (size_t)c->glp.n;
 }
 
+// Photons of the pass: never more than the species holds, so never more pairs
+// than there are records.
+__device__ __forceinline__ int64_t photons_of(const int64_t *n_active, int64_t cap) {
+  const int64_t n = *(volatile const int64_t *)n_active;
+  return n < cap ? n : cap;
+}
+
 template <class Real, int FM>
 __global__ void __launch_bounds__(PH_THREADS, sizeof(Real) == 4 ? 4 : 2) k_photon_stream(PhotonArgs<Real> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -74,7 +81,7 @@ __global__ void __launch_bounds__(PH_THREADS, sizeof(Real) == 4 ? 4 : 2) k_photo
   uint8_t *const s_list = reinterpret_cast<uint8_t *>(s_pool + PH_WARPS * PH_POOL);
   Real *const sP = reinterpret_cast<Real *>(s_list + PH_WARPS * 2 * PH_POOL);
   __shared__ BlockTally bt;
-  const int64_t n = *(volatile const int64_t *)A.n_active;
+  const int64_t n = photons_of(A.n_active, A.ph.cap);
   const int64_t nslices = (n + 31) / 32;
   if (blockIdx.x >= nslices) return;  // (slice w of warp wid is wid * gridDim + blockIdx, so none here)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -250,6 +257,7 @@ __global__ void __launch_bounds__(PH_THREADS, sizeof(Real) == 4 ? 4 : 2) k_photo
 constexpr int PSCAN_THREADS = 1024, PSCAN_CHUNKS = 4;
 struct PairScanArgs {
   const int64_t *n_active;
+  int64_t ph_cap;
   uint32_t *sum, *off;
   unsigned int *n;
   int64_t *el_n, *po_n, *meta;
@@ -261,7 +269,7 @@ __global__ void __launch_bounds__(PSCAN_THREADS) k_pair_scan(PairScanArgs A) {
   const unsigned pairs = *(volatile unsigned *)A.n;
   if (threadIdx.x == 0) A.n[1] = pairs;
   if (pairs == 0) return;
-  const int64_t nchunks = (*(volatile const int64_t *)A.n_active + CHUNK - 1) / CHUNK;
+  const int64_t nchunks = (photons_of(A.n_active, A.ph_cap) + CHUNK - 1) / CHUNK;
   uint32_t carry = 0;
   for (int64_t r0 = 0; r0 < nchunks; r0 += PSCAN_THREADS * PSCAN_CHUNKS) {
     const int64_t c0 = r0 + (int64_t)threadIdx.x * PSCAN_CHUNKS;
@@ -369,7 +377,7 @@ cudaError_t launch_photon_t(qed_ctx *c, const PhotonArgs<Real> &a, cudaStream_t 
   e = cudaGetLastError();
   if (e == cudaSuccess) e = prof_mark(c, 6, st);
   if (e != cudaSuccess) return e;
-  PairScanArgs s{a.n_active, a.sum, a.off, a.n, a.el.d_n, a.po.d_n, a.meta, a.el.cap, a.po.cap, a.cnt};
+  PairScanArgs s{a.n_active, a.ph.cap, a.sum, a.off, a.n, a.el.d_n, a.po.d_n, a.meta, a.el.cap, a.po.cap, a.cnt};
   k_pair_scan<<<1, PSCAN_THREADS, 0, st>>>(s);
   k_pair_write<Real, FM><<<grid, PH_THREADS, 0, st>>>(a);
   c->launches += 2;
