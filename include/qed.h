@@ -332,6 +332,13 @@ int qed_last_device_status(qed_ctx *ctx, uint32_t *bits, int64_t *dropped);
  * QED_ERR_TIMEOUT) and clear it with qed_reset_counters. */
 int qed_test_wait_expiry(qed_ctx *ctx, qed_stream_t stream);
 
+/* Failure-detection check of the replays: with ordered appends, a single-pass
+ * lepton step whose photon records run out redoes the leptons concerned from
+ * their stored state (QED_STATUS_REPLAY).  Those replays of later calls take the
+ * photon emission rate times `factor` (>= 0; 1 = as it is), so that they disagree
+ * with the photon counts of the step.  Steps without replays do not change. */
+int qed_test_replay_rate(qed_ctx *ctx, double factor);
+
 /* ---- learned inverse CDF (surrogate for the tabulated inverse of Eq. 7) --
  * A 2 -> 64 -> 64 -> 64 -> 1 SiLU network maps x0 = (ln chi + 1.1512925)/5.7564627,
  * x1 = (kappa + 3.25)/6.75 to z; ln delta = z + 3 kappa - 2 ln(1 + e^kappa), where

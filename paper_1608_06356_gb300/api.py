@@ -393,6 +393,11 @@ def qed_test_wait_expiry(ctx: Context, stream=None) -> None:
     B.check(B.lib().qed_test_wait_expiry(ctx.handle, _stream(stream)), "qed_test_wait_expiry")
 
 
+def qed_test_replay_rate(ctx: Context, factor: float) -> None:
+    """Let the replays of ordered appends disagree with their step (1: off)."""
+    B.check(B.lib().qed_test_replay_rate(ctx.handle, float(factor)), "qed_test_replay_rate")
+
+
 def qed_profile_begin(ctx: Context, max_steps: int) -> None:
     B.check(B.lib().qed_profile_begin(ctx.handle, int(max_steps)), "qed_profile_begin")
 

@@ -261,6 +261,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   // emission records for the first quarter of the entries of the sub-step list;
   // later entries (and particles with more than SUB_REC photons) replay
   c->rec_cap = rec_entries(cfg->max_particles);
+  c->replay_rate = 1.0;
   const size_t rsize = f64 ? sizeof(double) : sizeof(float);
   // staging records for the leptons the streaming pass defers (a record is
   // 16 words); past stage_cap a deferred particle is gathered from its arrays
@@ -572,6 +573,12 @@ extern "C" int qed_test_wait_expiry(qed_ctx *c, qed_stream_t stream) {
   k_wait_expiry<<<1, 32, 0, (cudaStream_t)stream>>>(c->probe_state, c->d_counters);
   c->launches += 1;
   return cuda_fail(cudaGetLastError(), "qed_test_wait_expiry");
+}
+
+extern "C" int qed_test_replay_rate(qed_ctx *c, double factor) {
+  if (!c || !(factor >= 0.0) || !std::isfinite(factor)) return QED_ERR_ARG;
+  c->replay_rate = factor;
+  return QED_OK;
 }
 
 extern "C" int qed_last_device_status(qed_ctx *c, uint32_t *bits, int64_t *dropped) {

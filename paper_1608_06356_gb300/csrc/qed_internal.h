@@ -46,6 +46,7 @@ struct qed_ctx {
   uint32_t *pair_sum;      // [cls_chunks] pairs per chunk of photons (zero between steps)
   unsigned int *ord_n;     // [4] ordered appends of the single pass: records and replays asked for, of the pass being written
   unsigned int *replay_n;  // entries the writing pass leaves to its replay launch
+  double replay_rate;      // photon rate of the ordered single pass's replays, as a multiple (1; qed_test_replay_rate)
   unsigned long long *probe_state;  // [2] look-back words of qed_test_wait_expiry (tile 0 never published)
   // staging records of the flagged leptons (streaming pass -> later passes)
   void *stage;          // Stage<Real> [stage_cap] (64 B FP32, 128 B FP64)

@@ -116,6 +116,7 @@ struct OrdArgs {
   uint32_t *idx;     // [position] its record
   unsigned int *n;   // [0] records asked for, [1] leptons to replay, [2], [3] of the pass being written
   int32_t *replay;   // slots of the leptons whose records found no room
+  uint32_t *replay_cnt;  // their photons
 };
 constexpr uint8_t FLAG_REPLAY = 0x80;
 
@@ -291,7 +292,9 @@ __global__ void __launch_bounds__(OP_THREADS, 1) k_lepton_onepass(OnePassArgs A)
         A.ord.cnt[sl] = cnt;
         atomicAdd(&A.ord.sum[sl / CLS_CHUNK_FLAGS * NCLS + cls[e] - 1], cnt);
         if (kw & LOST) {
-          A.ord.replay[atomicAdd(&A.ord.n[1], 1u)] = (int32_t)sl;
+          const unsigned r = atomicAdd(&A.ord.n[1], 1u);
+          A.ord.replay[r] = (int32_t)sl;
+          A.ord.replay_cnt[r] = cnt;
           return;
         }
       }
@@ -1169,6 +1172,7 @@ cudaError_t launch_lepton_onepass(qed_ctx *c, const qed_species *s0, const qed_s
     a.ord.idx = reinterpret_cast<uint32_t *>(c->heavy_list);
     a.ord.n = c->ord_n;
     a.ord.replay = c->stage_idx;
+    a.ord.replay_cnt = c->rec_k;
     // the chunks of the slots that the capacities allow
     const int64_t tiles = (s0->capacity + TILE - 1) / TILE + (s1 ? (s1->capacity + TILE - 1) / TILE : 0);
     const int64_t chunks = (tiles * TILE + CLS_CHUNK_FLAGS - 1) / CLS_CHUNK_FLAGS;

@@ -12,7 +12,9 @@ constexpr int SUB_REC = 8;  // emission records kept per particle by the sub-ste
 // rec_entries entries) and staging records (16 Reals each).  The photon stage
 // keeps a record per pair in the same memory -- two words of rec_k and eight
 // Reals of the stage -- and every photon may convert in one step, so both must
-// hold max_particles pairs, whatever the rounding of the divisions.
+// hold max_particles pairs, whatever the rounding of the divisions.  (The ordered
+// single pass keeps the photon count of every lepton to replay, 2 max_particles
+// words at most, in rec_k too: the same size.)
 constexpr int64_t rec_entries(int64_t max_particles) {
   const int64_t r = max_particles / 4 + 1;
   return r > 4096 ? r : 4096;

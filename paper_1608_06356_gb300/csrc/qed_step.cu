@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(TILE) k_sub_scan(SubScanArgs A) {
 // tables nor the chain's registers, and dense, so that the rare long replays
 // share warps.  BY_SLOT: the list is of slots, leptons of the single pass
 // whose momentum (with grid fields also position) is stored as before the
-// step, and sub_cnt is per slot.
+// step; sub_cnt is per slot then, and rec_k holds the photons of every list entry.
 template <class Real, int FM, int MODE, bool BY_SLOT>
 __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) {
   const int64_t step_ = A.d_step ? *A.d_step : A.step;
@@ -856,8 +856,8 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
     const int64_t h = (int64_t)A.replay_list[q];
     // sub_cnt holds the exclusive prefix of the counts now
     const uint32_t off = A.sub_cnt[h];
-    // (by slot: all that the chain emits; the single pass counted the dropped)
-    const uint32_t cnt = BY_SLOT ? 0xFFFFFFFFu : (h + 1 < nh ? A.sub_cnt[h + 1] : total) - off;
+    // the photons the lepton has places for (by slot: as the single pass counted them)
+    const uint32_t cnt = BY_SLOT ? A.rec_k[q] : (h + 1 < nh ? A.sub_cnt[h + 1] : total) - off;
     const int32_t e = BY_SLOT ? -(int32_t)h - 1 : A.heavy_list[h];
     const int64_t out0 = nph + (int64_t)off;
     Entry<Real> P;
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
     auto put = [&](uint32_t j, Real eph, int64_t kk) {
       const int64_t out = out0 + j;
       if (out >= A.ph.cap) {
-        if (!BY_SLOT) {
+        if (!BY_SLOT) {  // (by slot: the scan counted them)
           tl.dropped += 1;
           tl.status |= QED_STATUS_CAPACITY;
         }
@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(TILE, 2) k_substep_replay(LeptonArgs<Real> A) 
       chi = chi_lepton(pm2 * nx, pm2 * ny, pm2 * nz, g, E[0], E[1], E[2], B[0], B[1], B[2], inv_aS);
       ro = photon_rate(sR, sF, A.T, A.C, chi, g, dummy);
     }
-    if (!BY_SLOT && j != cnt) {  // the replay disagreed with the count: zero-energy photons fill the slots
+    if (j != cnt) {  // the replay disagreed with the count: zero-energy photons fill the slots
       tl.status |= QED_STATUS_REPLAY;
       for (; j < cnt; ++j) put(j, (Real)0, 0);
     }
@@ -2034,8 +2034,10 @@ cudaError_t launch_lepton_onepass(qed_ctx *c, const qed_species *s0, const qed_s
                                   const qed_species *ph, const qed_fields *f, int64_t step,
                                   int mode, bool ordered, cudaStream_t st);
 
-// The replay of a single pass with ordered appends (the leptons whose records
-// found no room: more photons in the step than max_particles).
+// The replay of a single pass with ordered appends: the leptons whose records
+// found no room.  16 stage_cap floats hold the records, so they run out past
+// max_particles / 2 photons in a step, or max_particles / 3 where the photons take
+// fields of their own.
 template <int MODE>
 static cudaError_t launch_replay_by_slot(qed_ctx *c, const LeptonArgs<float> &a, int fm, cudaStream_t st) {
   if (fm == QED_FIELDS_UNIFORM)
@@ -2099,6 +2101,7 @@ cudaError_t launch_lepton(qed_ctx *c, const qed_species *s0, const qed_species *
   if constexpr (sizeof(Real) == 4) {
     if (single) {
       a.replay_n = c->ord_n + 3;
+      a.C.f_alpha_aS *= (float)c->replay_rate;
       cudaError_t e = mode == MODE_EMIT ? launch_replay_by_slot<MODE_EMIT>(c, a, f->mode, st)
                                         : launch_replay_by_slot<MODE_FUSED>(c, a, f->mode, st);
       for (int k = 2; k <= 5 && e == cudaSuccess; ++k) e = prof_mark(c, k, st);
