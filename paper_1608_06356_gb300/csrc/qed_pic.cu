@@ -339,61 +339,42 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_pic_deposit(DepArgs<Real> A
 // atomics that are contiguous along x.  16.8M particles: 256^3 cells in random
 // order 5.00 -> 1.34 ms (count 0.14, scatter 0.42, tiles 0.78: bound by the
 // scattered stores and by instruction issue in the tiles), 128^3 by cell 1.44
-// -> 0.59 ms (0.09, 0.24, 0.26).
+// -> 0.59 ms (0.09, 0.24, 0.26).  FP32 contexts only.
 // ---------------------------------------------------------------------------
 constexpr int TLX = 8, TLY = 8, TLZ = 4, TL_CELLS = TLX * TLY * TLZ;
 constexpr int HLX = TLX + 2, HLY = TLY + 2, HLZ = TLZ + 2, HL_CELLS = HLX * HLY * HLZ;
 constexpr int TILE_THREADS = TL_CELLS;  // a thread per cell
 
-template <class Real> struct alignas(8 * sizeof(Real)) DepRec {
-  Real w[3], key, j[3], pad;  // offsets in the cell; cell of the tile (a small integer); a v
+struct alignas(32) DepRec {
+  float w[3], key, j[3], pad;  // offsets in the cell; cell of the tile (a small integer); a v
 };
 
-// A record is written and read by whole 32-byte sectors.
-__device__ __forceinline__ void put_rec(DepRec<float> *p, const DepRec<float> &r) {
+// A record is written and read by one 32-byte sector.
+__device__ __forceinline__ void put_rec(DepRec *p, const DepRec &r) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "f"(r.w[0]), "f"(r.w[1]),
                "f"(r.w[2]), "f"(r.key), "f"(r.j[0]), "f"(r.j[1]), "f"(r.j[2]), "f"(r.pad)
                : "memory");
 }
-__device__ __forceinline__ void put_rec(DepRec<double> *p, const DepRec<double> &r) {
-  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "d"(r.w[0]), "d"(r.w[1]), "d"(r.w[2]),
-               "d"(r.key)
-               : "memory");
-  asm volatile("st.global.v4.f64 [%0 + 32], {%1, %2, %3, %4};\n" ::"l"(p), "d"(r.j[0]), "d"(r.j[1]), "d"(r.j[2]),
-               "d"(r.pad)
-               : "memory");
-}
-__device__ __forceinline__ DepRec<float> get_rec(const DepRec<float> *p) {
-  DepRec<float> r;
+__device__ __forceinline__ DepRec get_rec(const DepRec *p) {
+  DepRec r;
   asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
                : "=f"(r.w[0]), "=f"(r.w[1]), "=f"(r.w[2]), "=f"(r.key), "=f"(r.j[0]), "=f"(r.j[1]), "=f"(r.j[2]),
                  "=f"(r.pad)
                : "l"(p));
   return r;
 }
-__device__ __forceinline__ DepRec<double> get_rec(const DepRec<double> *p) {
-  DepRec<double> r;
-  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];\n"
-               : "=d"(r.w[0]), "=d"(r.w[1]), "=d"(r.w[2]), "=d"(r.key)
-               : "l"(p));
-  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4 + 32];\n"
-               : "=d"(r.j[0]), "=d"(r.j[1]), "=d"(r.j[2]), "=d"(r.pad)
-               : "l"(p));
-  return r;
-}
 
 // Periodic cell index of an integral reduced coordinate.
-template <class Real> __device__ __forceinline__ uint32_t dep_wrap(Real f, int n) {
-  if (f >= (Real)0 && f < (Real)n) return (uint32_t)f;
+__device__ __forceinline__ uint32_t dep_wrap(float f, int n) {
+  if (f >= 0.f && f < (float)n) return (uint32_t)f;
   int64_t i = (int64_t)f % n;
   return (uint32_t)(i < 0 ? i + n : i);
 }
 
 // Tile of a particle, its cell in the tile and its offsets in the cell.
-template <class Real>
-__device__ __forceinline__ uint32_t dep_tile(const DepArgs<Real> &A, const TileArgs &T,
-                                             const DepPoint<Real> &d, Real w[3], uint32_t &cell) {
-  const Real ix = floor(d.f[0]), iy = floor(d.f[1]), iz = floor(d.f[2]);
+__device__ __forceinline__ uint32_t dep_tile(const DepArgs<float> &A, const TileArgs &T,
+                                             const DepPoint<float> &d, float w[3], uint32_t &cell) {
+  const float ix = floor(d.f[0]), iy = floor(d.f[1]), iz = floor(d.f[2]);
   w[0] = d.f[0] - ix; w[1] = d.f[1] - iy; w[2] = d.f[2] - iz;
   const uint32_t i = dep_wrap(ix, A.nx), j = dep_wrap(iy, A.ny), k = dep_wrap(iz, A.nz);
   cell = ((k % TLZ) * TLY + j % TLY) * TLX + i % TLX;
@@ -405,8 +386,7 @@ constexpr uint32_t NO_TILE = 0xFFFFFFFFu;
 // Particles per tile (in T.end), one atomic per distinct tile of a warp: the
 // atomics of particles stored by cell would otherwise queue up on the counters
 // of a few tiles.
-template <class Real>
-__global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<Real> A, TileArgs T) {
+__global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A, TileArgs T) {
   const int64_t n = dep_count(A);
   if (n < T.min_n || n > T.max_n) return;
   const int lane = threadIdx.x & 31;
@@ -417,10 +397,10 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<Real> A, 
        b += (int64_t)gridDim.x * DEPOSIT_THREADS) {
     const int64_t p = b + lane;
     uint32_t t = NO_TILE;
-    DepPoint<Real> d;
+    DepPoint<float> d;
     if (p < n) {
       if (dep_point(A, p, d)) {
-        Real w[3];
+        float w[3];
         uint32_t cell;
         t = dep_tile(A, T, d, w, cell) * T.ways + way;
       } else {
@@ -451,9 +431,8 @@ __global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(TileArgs T) {
   }
 }
 
-template <class Real>
-__global__ void __launch_bounds__(DEPOSIT_THREADS, sizeof(Real) == 4 ? 4 : 2)
-k_dep_scatter(DepArgs<Real> A, TileArgs T, DepRec<Real> *rec) {
+__global__ void __launch_bounds__(DEPOSIT_THREADS, 4)
+k_dep_scatter(DepArgs<float> A, TileArgs T, DepRec *rec) {
   const int64_t n = dep_count(A);
   if (n < T.min_n || n > T.max_n) return;
   const int lane = threadIdx.x & 31;
@@ -462,19 +441,19 @@ k_dep_scatter(DepArgs<Real> A, TileArgs T, DepRec<Real> *rec) {
        b += (int64_t)gridDim.x * DEPOSIT_THREADS) {
     const int64_t p = b + lane;
     uint32_t t = NO_TILE;
-    DepRec<Real> r;
+    DepRec r;
     bool direct = false;
     if (p < n) {
-      const Real a = A.scale * A.w[p];
-      DepPoint<Real> d;
+      const float a = A.scale * A.w[p];
+      DepPoint<float> d;
       if (dep_point(A, p, d)) {
         uint32_t cell;
         t = dep_tile(A, T, d, r.w, cell) * T.ways + way;
-        r.key = (Real)cell;
-        r.pad = (Real)0;
+        r.key = (float)cell;
+        r.pad = 0.f;
         direct = !isfinite(a);  // reaches its own eight nodes per component and no others
 #pragma unroll
-        for (int c = 0; c < 3; ++c) r.j[c] = direct ? (Real)0 : d.j[c] * a;
+        for (int c = 0; c < 3; ++c) r.j[c] = direct ? 0.f : d.j[c] * a;
       }
     }
     const unsigned same = __match_any_sync(0xFFFFFFFFu, t);
@@ -487,8 +466,8 @@ k_dep_scatter(DepArgs<Real> A, TileArgs T, DepRec<Real> *rec) {
       else direct = true;  // no room for its record
     }
     if (direct) {
-      const Real a = A.scale * A.w[p];
-      DepPoint<Real> d;
+      const float a = A.scale * A.w[p];
+      DepPoint<float> d;
       dep_point(A, p, d);
 #pragma unroll
       for (int c = 0; c < 3; ++c) d.j[c] *= a;
@@ -498,21 +477,20 @@ k_dep_scatter(DepArgs<Real> A, TileArgs T, DepRec<Real> *rec) {
 }
 
 // weights at the half-integer positions cell - 1/2, + 1/2, + 3/2
-template <class Real> __device__ __forceinline__ void dep_half(Real w, Real s[3]) {
-  const bool lo = w < (Real)0.5;
-  const Real u = lo ? w + (Real)0.5 : w - (Real)0.5;
-  s[0] = lo ? (Real)1 - u : (Real)0;
-  s[1] = lo ? u : (Real)1 - u;
-  s[2] = lo ? (Real)0 : u;
+__device__ __forceinline__ void dep_half(float w, float s[3]) {
+  const bool lo = w < 0.5f;
+  const float u = lo ? w + 0.5f : w - 0.5f;
+  s[0] = lo ? 1.f - u : 0.f;
+  s[1] = lo ? u : 1.f - u;
+  s[2] = lo ? 0.f : u;
 }
 
 // particles of a tile ordered by cell at a time (a warp's threads do as many
 // turns as its fullest cell, so the more at a time the better they are used)
 constexpr int DEP_BATCH = 2048;
 
-template <class Real>
-__global__ void __launch_bounds__(TILE_THREADS, sizeof(Real) == 4 ? 4 : 2)
-k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
+__global__ void __launch_bounds__(TILE_THREADS, 4)
+k_dep_tile(DepArgs<float> A, TileArgs T, const DepRec *rec) {
   constexpr int BATCH = DEP_BATCH, PER = BATCH / TILE_THREADS;
   __shared__ uint16_t s_perm[BATCH];  // the batch's records by cell
   __shared__ uint32_t s_cnt[TL_CELLS];
@@ -535,9 +513,9 @@ k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
       if (z < 0) z += A.nz;
       s_row[c] = ((int64_t)z * A.ny + y) * A.nx;
     }
-    Real jx[2][2][3], jy[2][3][2], jz[3][2][2];  // [z][y][x] around the cell
+    float jx[2][2][3], jy[2][3][2], jz[3][2][2];  // [z][y][x] around the cell
 #pragma unroll
-    for (int q = 0; q < 12; ++q) (&jx[0][0][0])[q] = (&jy[0][0][0])[q] = (&jz[0][0][0])[q] = (Real)0;
+    for (int q = 0; q < 12; ++q) (&jx[0][0][0])[q] = (&jy[0][0][0])[q] = (&jz[0][0][0])[q] = 0.f;
     for (uint32_t b = beg; b < end; b += BATCH) {
       const uint32_t m = end - b < BATCH ? end - b : BATCH;
       s_cnt[c] = 0;
@@ -566,17 +544,17 @@ k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
       }
       __syncthreads();
       for (uint32_t i = first; i < first + mine; ++i) {
-        const DepRec<Real> r = get_rec(rec + b + s_perm[i]);
-        const Real wx = r.w[0], wy = r.w[1], wz = r.w[2];
-        const Real X[2] = {(Real)1 - wx, wx}, Y[2] = {(Real)1 - wy, wy}, Z[2] = {(Real)1 - wz, wz};
-        const Real ax = r.j[0], ay = r.j[1], az = r.j[2];
-        Real h[3];
+        const DepRec r = get_rec(rec + b + s_perm[i]);
+        const float wx = r.w[0], wy = r.w[1], wz = r.w[2];
+        const float X[2] = {1.f - wx, wx}, Y[2] = {1.f - wy, wy}, Z[2] = {1.f - wz, wz};
+        const float ax = r.j[0], ay = r.j[1], az = r.j[2];
+        float h[3];
         dep_half(wx, h);
 #pragma unroll
         for (int z = 0; z < 2; ++z)
 #pragma unroll
           for (int y = 0; y < 2; ++y) {
-            const Real f = ax * Y[y] * Z[z];
+            const float f = ax * Y[y] * Z[z];
 #pragma unroll
             for (int x = 0; x < 3; ++x) jx[z][y][x] += f * h[x];
           }
@@ -585,7 +563,7 @@ k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
         for (int z = 0; z < 2; ++z)
 #pragma unroll
           for (int x = 0; x < 2; ++x) {
-            const Real f = ay * X[x] * Z[z];
+            const float f = ay * X[x] * Z[z];
 #pragma unroll
             for (int y = 0; y < 3; ++y) jy[z][y][x] += f * h[y];
           }
@@ -594,7 +572,7 @@ k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
         for (int y = 0; y < 2; ++y)
 #pragma unroll
           for (int x = 0; x < 2; ++x) {
-            const Real f = az * X[x] * Y[y];
+            const float f = az * X[x] * Y[y];
 #pragma unroll
             for (int z = 0; z < 3; ++z) jz[z][y][x] += f * h[z];
           }
@@ -610,8 +588,8 @@ k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
     const int lx = c % TLX, ly = c / TLX % TLY, lz = c / (TLX * TLY);
     const bool first_x = lx == 0, last_x = lx == TLX - 1;
     const int h0 = ((lz + 1) * HLY + ly + 1) * HLX + lx + 1;
-    auto up = [&](Real v) { const float r = __shfl_up_sync(0xFFFFFFFFu, (float)v, 1, TLX); return first_x ? 0.f : r; };
-    auto down = [&](Real v) { const float r = __shfl_down_sync(0xFFFFFFFFu, (float)v, 1, TLX); return last_x ? 0.f : r; };
+    auto up = [&](float v) { const float r = __shfl_up_sync(0xFFFFFFFFu, v, 1, TLX); return first_x ? 0.f : r; };
+    auto down = [&](float v) { const float r = __shfl_down_sync(0xFFFFFFFFu, v, 1, TLX); return last_x ? 0.f : r; };
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -619,18 +597,18 @@ k_dep_tile(DepArgs<Real> A, TileArgs T, const DepRec<Real> *rec) {
         __syncthreads();
         if (s < 2) {
           const int h = h0 + (u * HLY + s) * HLX;
-          const float v = (float)jx[u][s][1] + up(jx[u][s][2]) + down(jx[u][s][0]);
+          const float v = jx[u][s][1] + up(jx[u][s][2]) + down(jx[u][s][0]);
           s_J[0][h] += v;
-          if (first_x) s_J[0][h - 1] += (float)jx[u][s][0];
-          if (last_x) s_J[0][h + 1] += (float)jx[u][s][2];
+          if (first_x) s_J[0][h - 1] += jx[u][s][0];
+          if (last_x) s_J[0][h + 1] += jx[u][s][2];
         }
         const int hy = h0 + (u * HLY + s - 1) * HLX, hz = h0 + ((s - 1) * HLY + u) * HLX;
-        const float vy = (float)jy[u][s][0] + up(jy[u][s][1]), vz = (float)jz[s][u][0] + up(jz[s][u][1]);
+        const float vy = jy[u][s][0] + up(jy[u][s][1]), vz = jz[s][u][0] + up(jz[s][u][1]);
         s_J[1][hy] += vy;
         s_J[2][hz] += vz;
         if (last_x) {
-          s_J[1][hy + 1] += (float)jy[u][s][1];
-          s_J[2][hz + 1] += (float)jz[s][u][1];
+          s_J[1][hy + 1] += jy[u][s][1];
+          s_J[2][hz + 1] += jz[s][u][1];
         }
       }
     __syncthreads();
@@ -720,27 +698,46 @@ cudaError_t particle_grid(const qed_ctx *c, Kern kern, int64_t capacity, unsigne
 // random order then fetches its lines (256^3, 2^24 random: 1340/5000).  Few
 // tiles leave the chip idle (16^3, 2^18: 188/78) and a very full cell is one
 // thread's work (32^3 by cell: 128 a cell 739/696, 256 a cell 2057/1435).
+// FP64 contexts deposit directly: GB300 adds and multiplies doubles at a small
+// fraction of its float rate, and a tile is that work (128^3, 2^22 random: 1093 us
+// directly, 2369 by tiles; 64^3, 2^19: 161, 352).
 constexpr int64_t TILED_MIN_PARTICLES = 1 << 18, TILED_MIN_TILES = 128, TILED_MAX_PER_CELL = 64;
 constexpr int64_t L2_CELLS = 6 << 20;
 
-// The scratch is the step's: records in the staging area, segments in the
-// per-entry counts (both are free between steps, and calls that share a
-// context are ordered).
-template <class Real>
-cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<Real> &A, const TileArgs &T, cudaStream_t st) {
-  DepRec<Real> *rec = static_cast<DepRec<Real> *>(c->stage);
+// The tiled path's launches, where the capacities allow it.  The scratch is the
+// step's: records in the staging area, segments in the per-entry counts (both
+// are free between steps, and calls that share a context are ordered).
+cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_yee *y, TileArgs &T, cudaStream_t st) {
+  T.ntx = (y->nx + TLX - 1) / TLX;
+  T.nty = (y->ny + TLY - 1) / TLY;
+  const int64_t cells = (int64_t)y->nx * y->ny * y->nz;
+  const int64_t ntiles = (int64_t)T.ntx * T.nty * ((y->nz + TLZ - 1) / TLZ);
+  T.ways = 1;
+  while (ntiles * T.ways < 4096 && T.ways < 64) T.ways *= 2;
+  T.min_n = cells > L2_CELLS ? cells / 2 : 2 * cells;
+  if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
+  const int64_t max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
+  if (max_n < T.min_n || A.cap < T.min_n || A.cap > 0x7fffffff || 8 * (ntiles * T.ways + 1) > c->heavy_slots)
+    return cudaSuccess;
+  T.max_n = max_n;
+  T.ntiles = (uint32_t)ntiles;
+  T.seg = reinterpret_cast<TileSeg *>(c->sub_cnt);
+  T.total = &T.seg[ntiles * T.ways].end;
+  const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
+  T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
+  DepRec *rec = static_cast<DepRec *>(c->stage);
   const uint32_t nseg = T.ntiles * T.ways;
   unsigned count_blocks = 0, blocks = 0;
   cudaError_t e = cudaMemsetAsync(T.seg, 0, sizeof(TileSeg) * ((size_t)nseg + 1), st);
-  if (e == cudaSuccess) e = particle_grid(c, k_dep_count<Real>, A.cap, &count_blocks);
-  if (e == cudaSuccess) e = particle_grid(c, k_dep_scatter<Real>, A.cap, &blocks);
+  if (e == cudaSuccess) e = particle_grid(c, k_dep_count, A.cap, &count_blocks);
+  if (e == cudaSuccess) e = particle_grid(c, k_dep_scatter, A.cap, &blocks);
   if (e != cudaSuccess) return e;
   if (count_blocks < blocks || T.ways > 1) blocks = count_blocks = count_blocks < blocks ? count_blocks : blocks;
-  k_dep_count<Real><<<count_blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
+  k_dep_count<<<count_blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
   k_dep_alloc<<<(nseg + ALLOC_THREADS - 1) / ALLOC_THREADS, ALLOC_THREADS, 0, st>>>(T);
-  k_dep_scatter<Real><<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T, rec);
+  k_dep_scatter<<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T, rec);
   const uint32_t most = (uint32_t)c->num_sms * 32;
-  k_dep_tile<Real><<<T.ntiles < most ? T.ntiles : most, TILE_THREADS, 0, st>>>(A, T, rec);
+  k_dep_tile<<<T.ntiles < most ? T.ntiles : most, TILE_THREADS, 0, st>>>(A, T, rec);
   c->launches += 4;
   return cudaGetLastError();
 }
@@ -761,30 +758,14 @@ cudaError_t launch_deposit(qed_ctx *c, const qed_species *s, const qed_yee *y, d
   A.scale = (Real)((double)s->q * weight_unit / (y->dx * y->dy * y->dz));
   A.half_dt = (Real)(0.5 * c->cfg.dt);
   A.cnt = c->d_counters;
-  TileArgs T;
-  T.ntx = (y->nx + TLX - 1) / TLX;
-  T.nty = (y->ny + TLY - 1) / TLY;
-  const int64_t cells = (int64_t)y->nx * y->ny * y->nz;
-  const int64_t ntiles = (int64_t)T.ntx * T.nty * ((y->nz + TLZ - 1) / TLZ);
-  T.ways = 1;
-  while (ntiles * T.ways < 4096 && T.ways < 64) T.ways *= 2;
-  T.min_n = cells > L2_CELLS ? cells / 2 : 2 * cells;
-  if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
-  T.max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
+  TileArgs T{};
+  T.max_n = -1;  // all numbers directly
   unsigned blocks = 0;
   cudaError_t e = particle_grid(c, k_pic_deposit<Real>, s->capacity, &blocks);
   if (e != cudaSuccess) return e;
-  if (T.max_n >= T.min_n && s->capacity >= T.min_n && s->capacity <= 0x7fffffff &&
-      8 * (ntiles * T.ways + 1) <= c->heavy_slots) {
-    T.ntiles = (uint32_t)ntiles;
-    T.seg = reinterpret_cast<TileSeg *>(c->sub_cnt);
-    T.total = &T.seg[ntiles * T.ways].end;
-    const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
-    T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
-    e = launch_deposit_tiled(c, A, T, st);
+  if constexpr (sizeof(Real) == 4) {
+    e = launch_deposit_tiled(c, A, y, T, st);
     if (e != cudaSuccess) return e;
-  } else {
-    T.max_n = 0;  // all numbers directly
   }
   k_pic_deposit<Real><<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
   c->launches += 1;
