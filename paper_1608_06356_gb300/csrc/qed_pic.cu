@@ -297,9 +297,12 @@ template <class Real> __device__ __forceinline__ int64_t dep_count(const DepArgs
 struct alignas(32) TileSeg { uint32_t cursor, end, start, pad[5]; };
 
 struct TileArgs {
-  TileSeg *seg;     // [ntiles * ways]
-  uint32_t *total;  // records allocated
+  TileSeg *seg;       // [ntiles * ways]
+  uint32_t *total;    // records allocated
+  uint32_t *n_parts;  // parts of tiles with records
+  uint4 *part;        // [ntiles + rec_cap / DEP_PART_MIN] them: tile, first record, last + 1, batches with heavy cells
   uint32_t ntiles, ways, rec_cap;
+  uint32_t most_ctas;  // CTAs of k_dep_tile that fill the chip twice
   uint32_t ntx, nty;
   int64_t min_n, max_n;  // other numbers of particles are deposited directly
 };
@@ -381,7 +384,17 @@ __device__ __forceinline__ uint32_t dep_tile(const DepArgs<float> &A, const Tile
   return ((k / TLZ) * T.nty + j / TLY) * T.ntx + i / TLX;
 }
 
+// Part of its tile's segment that a particle is counted in: a CTA's particles
+// share one, the CTAs running at a time spread over all.
+__device__ __forceinline__ uint32_t dep_way(const TileArgs &T, int64_t p) {
+  return (uint32_t)(p / DEPOSIT_THREADS) & (T.ways - 1);
+}
+
 constexpr uint32_t NO_TILE = 0xFFFFFFFFu;
+// Most records of a tile that one CTA sums; fewer where they would not fill the
+// chip twice over.  The CTAs take the parts from a list: with the tiles' own
+// numbers and a stride a sheet's tiles all fell to one CTA in 32.
+constexpr uint32_t DEP_PART = 8192, DEP_PART_MIN = 2048;
 
 // Particles per tile (in T.end), one atomic per distinct tile of a warp: the
 // atomics of particles stored by cell would otherwise queue up on the counters
@@ -390,7 +403,6 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A,
   const int64_t n = dep_count(A);
   if (n < T.min_n || n > T.max_n) return;
   const int lane = threadIdx.x & 31;
-  const uint32_t way = blockIdx.x & (T.ways - 1);
   unsigned bad = 0;
   // warp-uniform loop
   for (int64_t b = (int64_t)blockIdx.x * DEPOSIT_THREADS + (threadIdx.x & ~31); b < n;
@@ -402,7 +414,7 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A,
       if (dep_point(A, p, d)) {
         float w[3];
         uint32_t cell;
-        t = dep_tile(A, T, d, w, cell) * T.ways + way;
+        t = dep_tile(A, T, d, w, cell) * T.ways + dep_way(T, p);
       } else {
         bad = 1;
       }
@@ -417,18 +429,38 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A,
 // segments with one atomic (the parts of a tile stay next to each other: ways
 // divides ALLOC_THREADS).
 constexpr int ALLOC_THREADS = 256;
-__global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(TileArgs T) {
-  __shared__ uint32_t sm[33];
+__global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(DepArgs<float> A, TileArgs T) {
+  __shared__ uint32_t sm[33], s_start[ALLOC_THREADS];
   __shared__ uint32_t s_base;
   const uint32_t t = blockIdx.x * ALLOC_THREADS + threadIdx.x, nseg = T.ntiles * T.ways;
   const uint32_t c = t < nseg ? T.seg[t].end : 0u;
   const uint32_t ex = block_excl_scan(c, sm);
   if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(T.total, sm[32]) : 0u;
   __syncthreads();
+  s_start[threadIdx.x] = s_base + ex;
   if (t < nseg) {
     T.seg[t].start = T.seg[t].cursor = s_base + ex;
     T.seg[t].end = s_base + ex + c;
   }
+  __syncthreads();
+  // the tiles with records, in parts of (nearly) equal numbers
+  uint32_t beg = 0, len = 0;
+  if (t < nseg && t % T.ways == T.ways - 1) {
+    beg = s_start[threadIdx.x - (T.ways - 1)];
+    uint32_t end = s_base + ex + c;
+    if (end > T.rec_cap) end = T.rec_cap;
+    len = end > beg ? end - beg : 0;
+  }
+  const uint32_t fill = (uint32_t)dep_count(A) / T.most_ctas;
+  const uint32_t most = fill < DEP_PART_MIN ? DEP_PART_MIN : fill > DEP_PART ? DEP_PART : fill;
+  const uint32_t k = len <= most ? len > 0 : (len + most - 1) / most;
+  const uint32_t at = block_excl_scan(k, sm);
+  if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(T.n_parts, sm[32]) : 0u;
+  __syncthreads();
+  if (k == 1) T.part[s_base + at] = make_uint4(t / T.ways, beg, beg + len, 0u);
+  for (uint32_t q = 0; k > 1 && q < k; ++q)
+    T.part[s_base + at + q] = make_uint4(t / T.ways, beg + (uint32_t)((uint64_t)len * q / k),
+                                         beg + (uint32_t)((uint64_t)len * (q + 1) / k), 0u);
 }
 
 __global__ void __launch_bounds__(DEPOSIT_THREADS, 4)
@@ -436,7 +468,6 @@ k_dep_scatter(DepArgs<float> A, TileArgs T, DepRec *rec) {
   const int64_t n = dep_count(A);
   if (n < T.min_n || n > T.max_n) return;
   const int lane = threadIdx.x & 31;
-  const uint32_t way = blockIdx.x & (T.ways - 1);  // the same CTA as in k_dep_count (equal grids)
   for (int64_t b = (int64_t)blockIdx.x * DEPOSIT_THREADS + (threadIdx.x & ~31); b < n;
        b += (int64_t)gridDim.x * DEPOSIT_THREADS) {
     const int64_t p = b + lane;
@@ -448,7 +479,7 @@ k_dep_scatter(DepArgs<float> A, TileArgs T, DepRec *rec) {
       DepPoint<float> d;
       if (dep_point(A, p, d)) {
         uint32_t cell;
-        t = dep_tile(A, T, d, r.w, cell) * T.ways + way;
+        t = dep_tile(A, T, d, r.w, cell) * T.ways + dep_way(T, p);
         r.key = (float)cell;
         r.pad = 0.f;
         direct = !isfinite(a);  // reaches its own eight nodes per component and no others
@@ -485,148 +516,272 @@ __device__ __forceinline__ void dep_half(float w, float s[3]) {
   s[2] = lo ? 0.f : u;
 }
 
+// The sums of one cell's particles over the positions around it, [z][y][x] of
+// each component: 12 of jx (2 x 2 x 3), of jy (2 x 3 x 2) and of jz (3 x 2 x 2).
+template <int COMP> __device__ __forceinline__ void cell_add(const DepRec &r, float (&v)[12]) {
+  const float wx = r.w[0], wy = r.w[1], wz = r.w[2];
+  const float X[2] = {1.f - wx, wx}, Y[2] = {1.f - wy, wy}, Z[2] = {1.f - wz, wz};
+  float h[3];
+  dep_half(COMP == 0 ? wx : COMP == 1 ? wy : wz, h);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const float f = COMP == 0 ? r.j[0] * Y[b] * Z[a] : COMP == 1 ? r.j[1] * X[b] * Z[a] : r.j[2] * X[b] * Y[a];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v[COMP == 0 ? (a * 2 + b) * 3 + k : COMP == 1 ? (a * 3 + k) * 2 + b : (k * 2 + a) * 2 + b] += f * h[k];
+    }
+}
+struct CellSums {
+  float vx[12], vy[12], vz[12];
+  __device__ __forceinline__ float x(int z, int y, int i) const { return vx[(z * 2 + y) * 3 + i]; }
+  __device__ __forceinline__ float y(int z, int j, int i) const { return vy[(z * 3 + j) * 2 + i]; }
+  __device__ __forceinline__ float z(int k, int y, int i) const { return vz[(k * 2 + y) * 2 + i]; }
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int q = 0; q < 12; ++q) vx[q] = vy[q] = vz[q] = 0.f;
+  }
+  __device__ __forceinline__ void add(const DepRec &r) {
+    cell_add<0>(r, vx);
+    cell_add<1>(r, vy);
+    cell_add<2>(r, vz);
+  }
+};
+
+// Place of a tile's cell in its halo tile.
+__device__ __forceinline__ int cell_place(int c) {
+  return ((c / (TLX * TLY) + 1) * HLY + c / TLX % TLY + 1) * HLX + c % TLX + 1;
+}
+// One component of a heavy cell's chunk by eight lanes, added to the halo tile J
+// around the cell: lane by lane, then over the lanes by an exchange in which a
+// lane keeps half of its sums at a time and is left with three.
+template <int COMP>
+__device__ __forceinline__ void chunk_add(const DepRec *rec, const uint16_t *perm, uint32_t len, float *J) {
+  const int l = threadIdx.x & 7;
+  float v[12] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (uint32_t i = l; i < len; i += 8) cell_add<COMP>(get_rec(rec + perm[i]), v);
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const float send = l & 4 ? v[i] : v[i + 6];
+    v[i] = (l & 4 ? v[i + 6] : v[i]) + __shfl_xor_sync(0xFFFFFFFFu, send, 4);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float send = l & 2 ? v[i] : v[i + 3];
+    v[i] = (l & 2 ? v[i + 3] : v[i]) + __shfl_xor_sync(0xFFFFFFFFu, send, 2);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) v[i] += __shfl_xor_sync(0xFFFFFFFFu, v[i], 1);
+  // sums 3 (l / 2) .. + 2: the even lane adds the first and the last, the odd one the second
+  auto add = [&](int q, float a) {
+    const int x = COMP == 0 ? q % 3 - 1 : q % 2;
+    const int y = COMP == 0 ? q / 3 % 2 : COMP == 1 ? q / 2 % 3 - 1 : q / 2 % 2;
+    const int z = COMP == 2 ? q / 4 - 1 : q / 6;
+    atomicAdd(J + COMP * HL_CELLS + (z * HLY + y) * HLX + x, a);
+  };
+  if (len) {
+    const int q = 3 * (l >> 2) * 2 + 3 * (l >> 1 & 1);
+    add(q + (l & 1), l & 1 ? v[1] : v[0]);
+    if (!(l & 1)) add(q + 2, v[2]);
+  }
+}
+
 // particles of a tile ordered by cell at a time (a warp's threads do as many
 // turns as its fullest cell, so the more at a time the better they are used)
 constexpr int DEP_BATCH = 2048;
+// A cell with more particles of a batch (8 a cell in a full batch of a uniform
+// plasma) is left to a second pass, which sums it by eight lanes per DEP_CHUNK
+// particles: one thread's turns would hold up the CTA.  16.8M particles, 256^3
+// cells, ms directly / all cells by threads / this way: half of them in one cell
+// 19 / 1095 / 1.9, in a ball of 8 cells' deviation 1.5 / 3.2 / 1.2, a sheet of one
+// cell 1.2 / 2.8 / 1.1, of two 1.1 / 1.9 / 1.2.  (A second pass, and not a branch of
+// the first: with the sums of both live the registers spill, uniform plasma 5%.
+// Chunks by whole warps: 10-30% slower; DEP_HEAVY 16 and 24 within 3%.)
+constexpr int DEP_HEAVY = 32, DEP_CHUNK = 64;
+constexpr int DEP_CHUNKS = DEP_BATCH / (DEP_HEAVY + 1) + DEP_BATCH / DEP_CHUNK + 1;  // most of a batch
+static_assert(DEP_BATCH <= 1 << 11 && DEP_CHUNK <= 1 << 8 && TL_CELLS <= 1 << 8, "a chunk in one word");
+
+// The chunks of a batch's heavy cells, eight lanes each (warp-uniform loop).
+__device__ __forceinline__ void dep_chunks(const DepRec *rec, const uint16_t *perm, const uint32_t *chunk, uint32_t nchunks,
+                                           float *J) {
+  for (uint32_t q0 = threadIdx.x >> 5 << 2; q0 < nchunks; q0 += TILE_THREADS / 8) {
+    const uint32_t q = q0 + (threadIdx.x >> 3 & 3), w = q < nchunks ? chunk[q] : 0u;
+    const uint32_t len = q < nchunks ? (w >> 19) + 1 : 0u;
+    const uint16_t *p = perm + (w >> 8 & 2047u);
+    float *const base = J + cell_place((int)(w & 255u));
+    chunk_add<0>(rec, p, len, base);
+    chunk_add<1>(rec, p, len, base);
+    chunk_add<2>(rec, p, len, base);
+  }
+}
+
+struct TileSmem {
+  uint16_t perm[DEP_BATCH];  // the batch's records by cell
+  uint32_t cnt[TL_CELLS];
+  uint32_t scan[33];
+  uint32_t heavy, light;     // whether any batch has heavy cells, and the part others
+  uint32_t chunk[DEP_CHUNKS], nchunks;  // chunks of heavy cells: cell, first, length - 1
+  float J[3][HL_CELLS];
+  int64_t row[HLY * HLZ];  // first element of J's row of each halo row
+};
+
+// The halo tile's rows of J, and the tile's zeros.
+__device__ __forceinline__ void dep_begin(const DepArgs<float> &A, const TileArgs &T, uint32_t t, TileSmem &s) {
+  const int c = threadIdx.x;
+  if (c < HLY * HLZ) {
+    int y = ((int)(t / T.ntx % T.nty * TLY) - 1 + c % HLY) % A.ny;
+    int z = ((int)(t / (T.ntx * T.nty) * TLZ) - 1 + c / HLY) % A.nz;
+    if (y < 0) y += A.ny;
+    if (z < 0) z += A.nz;
+    s.row[c] = ((int64_t)z * A.ny + y) * A.nx;
+  }
+  for (int q = threadIdx.x; q < 3 * HL_CELLS; q += TILE_THREADS) (&s.J[0][0])[q] = 0.f;
+}
+
+// The halo tile to J: 16 lanes per row, 10 of them with a column.
+__device__ __forceinline__ void dep_end(const DepArgs<float> &A, const TileArgs &T, uint32_t t, TileSmem &s) {
+  __syncthreads();
+  const int hx = threadIdx.x & 15;
+  int x = (int)(t % T.ntx * TLX) - 1 + hx;
+  if (x < 0 || x >= A.nx) {
+    x %= A.nx;
+    if (x < 0) x += A.nx;
+  }
+  if (hx < HLX)
+    for (int r = threadIdx.x >> 4; r < 3 * HLY * HLZ; r += TILE_THREADS / 16) {
+      const float v = (&s.J[0][0])[r * HLX + hx];
+      if (v == 0.f) continue;
+      const int comp = r / (HLY * HLZ);
+      atomicAdd((comp == 0 ? A.jx : comp == 1 ? A.jy : A.jz) + s.row[r - comp * (HLY * HLZ)] + x, v);
+    }
+  __syncthreads();  // the shared arrays are the next part's
+}
+
+// The order by cell of a batch of m records; the CTA's thread c gets cell c's
+// records, `mine` of them from the return value on, and whether any cell has more
+// than DEP_HEAVY.
+__device__ __forceinline__ uint32_t dep_sort(const DepRec *rec, uint32_t m, TileSmem &s, uint32_t &mine, bool &heavy) {
+  constexpr int PER = DEP_BATCH / TILE_THREADS;
+  s.cnt[threadIdx.x] = 0;
+  __syncthreads();
+  // a record's rank among its cell's, then its place in cell order
+  uint32_t place[PER];  // cell | rank << 8
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    if (q * TILE_THREADS >= m) break;
+    const uint32_t i = q * TILE_THREADS + threadIdx.x;
+    if (i < m) {
+      const uint32_t cell = (uint32_t)rec[i].key & (TL_CELLS - 1);
+      place[q] = cell | atomicAdd(&s.cnt[cell], 1u) << 8;
+    }
+  }
+  __syncthreads();
+  mine = s.cnt[threadIdx.x];
+  const uint32_t first = block_excl_scan(mine, s.scan);
+  s.cnt[threadIdx.x] = first;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    if (q * TILE_THREADS >= m) break;
+    const uint32_t i = q * TILE_THREADS + threadIdx.x;
+    if (i < m) s.perm[s.cnt[place[q] & (TL_CELLS - 1)] + (place[q] >> 8)] = (uint16_t)i;
+  }
+  heavy = __syncthreads_or(mine > DEP_HEAVY) != 0;
+  return first;
+}
 
 __global__ void __launch_bounds__(TILE_THREADS, 4)
 k_dep_tile(DepArgs<float> A, TileArgs T, const DepRec *rec) {
-  constexpr int BATCH = DEP_BATCH, PER = BATCH / TILE_THREADS;
-  __shared__ uint16_t s_perm[BATCH];  // the batch's records by cell
-  __shared__ uint32_t s_cnt[TL_CELLS];
-  __shared__ uint32_t sm[33];
-  __shared__ float s_J[3][HL_CELLS];
-  __shared__ int64_t s_row[HLY * HLZ];  // first element of J's row of each halo row
+  __shared__ TileSmem s;
   const int64_t n = dep_count(A);
   if (n < T.min_n || n > T.max_n) return;
   const int c = threadIdx.x;
-  for (uint32_t t = blockIdx.x; t < T.ntiles; t += gridDim.x) {
-    const uint32_t beg = T.seg[t * T.ways].start;
-    uint32_t end = T.seg[t * T.ways + T.ways - 1].end;
-    if (end > T.rec_cap) end = T.rec_cap;
-    if (beg >= end) continue;
-    const int x0 = (int)(t % T.ntx * TLX) - 1;
-    if (c < HLY * HLZ) {
-      int y = ((int)(t / T.ntx % T.nty * TLY) - 1 + c % HLY) % A.ny;
-      int z = ((int)(t / (T.ntx * T.nty) * TLZ) - 1 + c / HLY) % A.nz;
-      if (y < 0) y += A.ny;
-      if (z < 0) z += A.nz;
-      s_row[c] = ((int64_t)z * A.ny + y) * A.nx;
-    }
-    float jx[2][2][3], jy[2][3][2], jz[3][2][2];  // [z][y][x] around the cell
-#pragma unroll
-    for (int q = 0; q < 12; ++q) (&jx[0][0][0])[q] = (&jy[0][0][0])[q] = (&jz[0][0][0])[q] = 0.f;
-    for (uint32_t b = beg; b < end; b += BATCH) {
-      const uint32_t m = end - b < BATCH ? end - b : BATCH;
-      s_cnt[c] = 0;
-      __syncthreads();
-      // a record's rank among its cell's, then its place in cell order
-      uint32_t place[PER];  // cell | rank << 8
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        if (q * TILE_THREADS >= m) break;
-        const uint32_t i = q * TILE_THREADS + threadIdx.x;
-        if (i < m) {
-          const uint32_t cell = (uint32_t)rec[b + i].key & (TL_CELLS - 1);
-          place[q] = cell | atomicAdd(&s_cnt[cell], 1u) << 8;
+  // (little is kept over the sums: 36 of the 64 registers are theirs)
+  const volatile uint32_t *const parts = T.n_parts;
+  if (c == 0) s.heavy = 0;
+  for (uint32_t part = blockIdx.x; part < *parts; part += gridDim.x) {
+    dep_begin(A, T, T.part[part].x, s);
+    if (c == 0) s.light = 0;  // (set after the sort's barriers)
+    CellSums S;
+    S.clear();
+    const uint32_t end = T.part[part].z;
+    for (uint32_t b = T.part[part].y; b < end; b += DEP_BATCH) {
+      uint32_t mine;
+      bool heavy;
+      const uint32_t first = dep_sort(rec + b, end - b < DEP_BATCH ? end - b : DEP_BATCH, s, mine, heavy);
+      if (heavy) {
+        if (c == 0) {
+          s.heavy = 1;
+          T.part[part].w |= 1u << (b - T.part[part].y) / DEP_BATCH;
         }
+        if (mine > DEP_HEAVY) mine = 0;
+        else if (mine) s.light = 1;
+      } else if (c == 0) {
+        s.light = 1;
       }
-      __syncthreads();
-      const uint32_t mine = s_cnt[c];
-      const uint32_t first = block_excl_scan(mine, sm);
-      s_cnt[c] = first;
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        if (q * TILE_THREADS >= m) break;
-        const uint32_t i = q * TILE_THREADS + threadIdx.x;
-        if (i < m) s_perm[s_cnt[place[q] & (TL_CELLS - 1)] + (place[q] >> 8)] = (uint16_t)i;
-      }
-      __syncthreads();
-      for (uint32_t i = first; i < first + mine; ++i) {
-        const DepRec r = get_rec(rec + b + s_perm[i]);
-        const float wx = r.w[0], wy = r.w[1], wz = r.w[2];
-        const float X[2] = {1.f - wx, wx}, Y[2] = {1.f - wy, wy}, Z[2] = {1.f - wz, wz};
-        const float ax = r.j[0], ay = r.j[1], az = r.j[2];
-        float h[3];
-        dep_half(wx, h);
-#pragma unroll
-        for (int z = 0; z < 2; ++z)
-#pragma unroll
-          for (int y = 0; y < 2; ++y) {
-            const float f = ax * Y[y] * Z[z];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) jx[z][y][x] += f * h[x];
-          }
-        dep_half(wy, h);
-#pragma unroll
-        for (int z = 0; z < 2; ++z)
-#pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            const float f = ay * X[x] * Z[z];
-#pragma unroll
-            for (int y = 0; y < 3; ++y) jy[z][y][x] += f * h[y];
-          }
-        dep_half(wz, h);
-#pragma unroll
-        for (int y = 0; y < 2; ++y)
-#pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            const float f = az * X[x] * Y[y];
-#pragma unroll
-            for (int z = 0; z < 3; ++z) jz[z][y][x] += f * h[z];
-          }
-      }
+      for (uint32_t i = first; i < first + mine; ++i) S.add(get_rec(rec + b + s.perm[i]));
       __syncthreads();
     }
+    if (!s.light) continue;
     // the cells' sums into the halo tile.  Along x (8 consecutive lanes) by
     // shuffles: a lane keeps what lies on its own column, the row's first and
     // last lane also the columns beside the tile; then in rounds in which every
     // thread adds at the same offset from its own cell, so that no two add to
     // one place
-    for (int q = threadIdx.x; q < 3 * HL_CELLS; q += TILE_THREADS) (&s_J[0][0])[q] = 0.f;
-    const int lx = c % TLX, ly = c / TLX % TLY, lz = c / (TLX * TLY);
+    const int lx = c % TLX, h0 = cell_place(c);
     const bool first_x = lx == 0, last_x = lx == TLX - 1;
-    const int h0 = ((lz + 1) * HLY + ly + 1) * HLX + lx + 1;
     auto up = [&](float v) { const float r = __shfl_up_sync(0xFFFFFFFFu, v, 1, TLX); return first_x ? 0.f : r; };
     auto down = [&](float v) { const float r = __shfl_down_sync(0xFFFFFFFFu, v, 1, TLX); return last_x ? 0.f : r; };
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int s = 0; s < 3; ++s) {
+      for (int w = 0; w < 3; ++w) {
         __syncthreads();
-        if (s < 2) {
-          const int h = h0 + (u * HLY + s) * HLX;
-          const float v = jx[u][s][1] + up(jx[u][s][2]) + down(jx[u][s][0]);
-          s_J[0][h] += v;
-          if (first_x) s_J[0][h - 1] += jx[u][s][0];
-          if (last_x) s_J[0][h + 1] += jx[u][s][2];
+        if (w < 2) {
+          const int h = h0 + (u * HLY + w) * HLX;
+          const float v = S.x(u, w, 1) + up(S.x(u, w, 2)) + down(S.x(u, w, 0));
+          s.J[0][h] += v;
+          if (first_x) s.J[0][h - 1] += S.x(u, w, 0);
+          if (last_x) s.J[0][h + 1] += S.x(u, w, 2);
         }
-        const int hy = h0 + (u * HLY + s - 1) * HLX, hz = h0 + ((s - 1) * HLY + u) * HLX;
-        const float vy = jy[u][s][0] + up(jy[u][s][1]), vz = jz[s][u][0] + up(jz[s][u][1]);
-        s_J[1][hy] += vy;
-        s_J[2][hz] += vz;
+        const int hy = h0 + (u * HLY + w - 1) * HLX, hz = h0 + ((w - 1) * HLY + u) * HLX;
+        const float vy = S.y(u, w, 0) + up(S.y(u, w, 1)), vz = S.z(w, u, 0) + up(S.z(w, u, 1));
+        s.J[1][hy] += vy;
+        s.J[2][hz] += vz;
         if (last_x) {
-          s_J[1][hy + 1] += jy[u][s][1];
-          s_J[2][hz + 1] += jz[s][u][1];
+          s.J[1][hy + 1] += S.y(u, w, 1);
+          s.J[2][hz + 1] += S.z(w, u, 1);
         }
       }
-    __syncthreads();
-    // to J: 16 lanes per halo row, 10 of them with a column
-    const int hx = threadIdx.x & 15;
-    int x = x0 + hx;
-    if (x < 0 || x >= A.nx) {
-      x %= A.nx;
-      if (x < 0) x += A.nx;
-    }
-    if (hx < HLX)
-      for (int r = threadIdx.x >> 4; r < 3 * HLY * HLZ; r += TILE_THREADS / 16) {
-        const float v = (&s_J[0][0])[r * HLX + hx];
-        if (v == 0.f) continue;
-        const int comp = r / (HLY * HLZ);
-        atomicAdd((comp == 0 ? A.jx : comp == 1 ? A.jy : A.jz) + s_row[r - comp * (HLY * HLZ)] + x, v);
+    dep_end(A, T, T.part[part].x, s);
+  }
+  __syncthreads();  // (a CTA without parts)
+  if (!s.heavy) return;
+  // the heavy cells of this CTA's parts, their batches sorted again (apart from
+  // the threads' sums, which fill the registers)
+  for (uint32_t part = blockIdx.x; part < *parts; part += gridDim.x) {
+    const uint4 range = T.part[part];
+    if (range.w == 0) continue;
+    dep_begin(A, T, range.x, s);
+    for (uint32_t h = range.w; h; h &= h - 1) {
+      const uint32_t b = range.y + (__ffs(h) - 1) * DEP_BATCH;
+      if (c == 0) s.nchunks = 0;
+      uint32_t mine;
+      bool heavy;
+      const uint32_t first = dep_sort(rec + b, range.z - b < DEP_BATCH ? range.z - b : DEP_BATCH, s, mine, heavy);
+      if (mine > DEP_HEAVY) {
+        const uint32_t k = (mine + DEP_CHUNK - 1) / DEP_CHUNK, at = atomicAdd(&s.nchunks, k);
+        for (uint32_t q = 0; q < k; ++q) {
+          const uint32_t left = mine - q * DEP_CHUNK, len = left < DEP_CHUNK ? left : DEP_CHUNK;
+          s.chunk[at + q] = (uint32_t)c | (first + q * DEP_CHUNK) << 8 | (len - 1) << 19;
+        }
       }
-    __syncthreads();  // the shared arrays are the next tile's
+      __syncthreads();
+      dep_chunks(rec + b, s.perm, s.chunk, s.nchunks, &s.J[0][0]);
+      __syncthreads();
+    }
+    dep_end(A, T, range.x, s);
   }
 }
 
@@ -703,6 +858,9 @@ cudaError_t particle_grid(const qed_ctx *c, Kern kern, int64_t capacity, unsigne
 // directly, 2369 by tiles; 64^3, 2^19: 161, 352).
 constexpr int64_t TILED_MIN_PARTICLES = 1 << 18, TILED_MIN_TILES = 128, TILED_MAX_PER_CELL = 64;
 constexpr int64_t L2_CELLS = 6 << 20;
+// counters of a grid with few tiles: a ball of particles queues on few of them
+// (128^3, 2^22: 470 us with 4096, 370 with 16384; uniform 288, 281)
+constexpr int64_t DEP_SEGMENTS = 16384;
 
 // The tiled path's launches, where the capacities allow it.  The scratch is the
 // step's: records in the staging area, segments in the per-entry counts (both
@@ -713,18 +871,21 @@ cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_
   const int64_t cells = (int64_t)y->nx * y->ny * y->nz;
   const int64_t ntiles = (int64_t)T.ntx * T.nty * ((y->nz + TLZ - 1) / TLZ);
   T.ways = 1;
-  while (ntiles * T.ways < 4096 && T.ways < 64) T.ways *= 2;
+  while (ntiles * T.ways < DEP_SEGMENTS && T.ways < 64) T.ways *= 2;
   T.min_n = cells > L2_CELLS ? cells / 2 : 2 * cells;
   if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
   const int64_t max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
-  if (max_n < T.min_n || A.cap < T.min_n || A.cap > 0x7fffffff || 8 * (ntiles * T.ways + 1) > c->heavy_slots)
-    return cudaSuccess;
+  const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
+  T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
+  T.most_ctas = (uint32_t)c->num_sms * 8;
+  const int64_t scratch = 8 * (ntiles * T.ways + 1) + 4 * (ntiles + T.rec_cap / DEP_PART_MIN);
+  if (max_n < T.min_n || A.cap < T.min_n || A.cap > 0x7fffffff || scratch > c->heavy_slots) return cudaSuccess;
   T.max_n = max_n;
   T.ntiles = (uint32_t)ntiles;
   T.seg = reinterpret_cast<TileSeg *>(c->sub_cnt);
   T.total = &T.seg[ntiles * T.ways].end;
-  const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
-  T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
+  T.n_parts = &T.seg[ntiles * T.ways].cursor;
+  T.part = reinterpret_cast<uint4 *>(T.seg + ntiles * T.ways + 1);
   DepRec *rec = static_cast<DepRec *>(c->stage);
   const uint32_t nseg = T.ntiles * T.ways;
   unsigned count_blocks = 0, blocks = 0;
@@ -732,12 +893,11 @@ cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_
   if (e == cudaSuccess) e = particle_grid(c, k_dep_count, A.cap, &count_blocks);
   if (e == cudaSuccess) e = particle_grid(c, k_dep_scatter, A.cap, &blocks);
   if (e != cudaSuccess) return e;
-  if (count_blocks < blocks || T.ways > 1) blocks = count_blocks = count_blocks < blocks ? count_blocks : blocks;
   k_dep_count<<<count_blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
-  k_dep_alloc<<<(nseg + ALLOC_THREADS - 1) / ALLOC_THREADS, ALLOC_THREADS, 0, st>>>(T);
+  k_dep_alloc<<<(nseg + ALLOC_THREADS - 1) / ALLOC_THREADS, ALLOC_THREADS, 0, st>>>(A, T);
   k_dep_scatter<<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T, rec);
-  const uint32_t most = (uint32_t)c->num_sms * 32;
-  k_dep_tile<<<T.ntiles < most ? T.ntiles : most, TILE_THREADS, 0, st>>>(A, T, rec);
+  const uint32_t most = (uint32_t)c->num_sms * 32, need = T.ntiles + T.rec_cap / DEP_PART_MIN;
+  k_dep_tile<<<need < most ? need : most, TILE_THREADS, 0, st>>>(A, T, rec);
   c->launches += 4;
   return cudaGetLastError();
 }

@@ -34,3 +34,31 @@ def test_fp64_deposits_directly(api):
     api.qed_pic_deposit(ctx, e, y, 1.0)
     torch.cuda.synchronize()
     assert ctx.launches - before == 1
+
+
+def _time(fn, n=5):
+    ms = []
+    for _ in range(n + 2):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        a.record()
+        fn()
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    return sorted(ms[2:])[n // 2]
+
+
+def test_a_full_cell_does_not_hold_up_the_tiled_deposit(api):
+    """2^20 electrons, half of them in one cell: while a cell was one thread's
+    work this took about a thousand times as long as a uniform plasma; summed by
+    warps and by several CTAs it is of the same order (30 times allowed)."""
+    n = 1 << 20
+    ctx = api.qed_init_tables(api.config(dt=0.1, max_particles=n))
+    y = api.Yee(64, 64, 64, 1.0, 1.0, 1.0)
+    e = _electrons(api, n, 64.0)
+    uniform = _time(lambda: api.qed_pic_deposit(ctx, e, y, 1.0))
+    for k in "xyz":
+        getattr(e, k)[: n // 2].mul_(1.0 / 64).add_(5.0)
+    clustered = _time(lambda: api.qed_pic_deposit(ctx, e, y, 1.0))
+    assert clustered < 30 * uniform, (clustered, uniform)
