@@ -82,7 +82,7 @@ static void free_ctx(qed_ctx *c) {
   if (!c) return;
   free_host_step(c);
   void *ptrs[] = {c->R64, c->F64, c->Y64, c->P64, c->Yp64, c->R32, c->F32, c->Y32,
-                  c->P32, c->Yp32, c->tile_state, c->sync, c->snap, c->pic_n, c->d_counters,
+                  c->P32, c->Yp32, c->tile_state, c->sync, c->snap, c->pic_n, c->dep_cnt, c->d_counters,
                   c->heavy_flags, c->heavy_list, c->pair_n, c->pair_sum, c->cls_chunk_cnt,
                   c->cls_chunk_off, c->cls_off, c->sub_cnt, c->sub_gf, c->rec_e,
                   c->rec_k, c->sub_meta, c->fill_meta, c->ord_n, c->compact_n, c->replay_n, c->stage, c->stage_tag,
@@ -262,6 +262,10 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   // later entries (and particles with more than SUB_REC photons) replay
   c->rec_cap = rec_entries(cfg->max_particles);
   c->replay_rate = 1.0;
+  // counters of the tiled deposit, 32 bytes each: a tile of 256 cells has at least
+  // 128 particles on average there, so max_particles / 64 allow for ragged tiles
+  c->dep_segs = cfg->max_particles / 64 > 32768 ? cfg->max_particles / 64 : 32768;
+  const size_t dep_bytes = 32 * (size_t)(c->dep_segs + 1);
   const size_t rsize = f64 ? sizeof(double) : sizeof(float);
   // staging records for the leptons the streaming pass defers (a record is
   // 16 words); past stage_cap a deferred particle is gathered from its arrays
@@ -270,6 +274,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
       cudaMalloc(&c->sync, sizeof(unsigned int) * 4) != cudaSuccess ||
       cudaMalloc(&c->snap, sizeof(int64_t) * 4) != cudaSuccess ||
       cudaMalloc(&c->pic_n, sizeof(int64_t) * 2) != cudaSuccess ||
+      cudaMalloc(&c->dep_cnt, dep_bytes) != cudaSuccess ||
       cudaMalloc(&c->d_counters, sizeof(qed_counters)) != cudaSuccess ||
       cudaMalloc(&c->heavy_flags, (size_t)c->heavy_slots + 4096) != cudaSuccess ||
       cudaMalloc(&c->heavy_list, sizeof(int) * (size_t)c->heavy_slots) != cudaSuccess ||
@@ -299,6 +304,7 @@ extern "C" int qed_init_tables(const qed_config *cfg, qed_ctx **out, qed_stream_
   if (e == cudaSuccess) e = cudaMemsetAsync(c->sync, 0, sizeof(unsigned int) * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->snap, 0, sizeof(int64_t) * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counters, 0, sizeof(qed_counters), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->dep_cnt, 0, dep_bytes, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->pair_n, 0, 2 * sizeof(unsigned int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->pair_sum, 0, sizeof(uint32_t) * (size_t)c->cls_chunks, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->compact_n, 0, COMPACT_WORDS * sizeof(unsigned int), st);

@@ -24,6 +24,8 @@ struct qed_ctx {
   int64_t max_tiles;
   int64_t *snap;       // [4] counts snapshotted at the start of a fused step
   int64_t *pic_n;      // [2] lepton counts at the start of a qed_pic_step
+  uint32_t *dep_cnt;   // tiled deposit: a sector of its own, then one per segment (zero between calls)
+  int64_t dep_segs;    // segments
   int64_t heavy_slots;   // block-tile slots of both lepton species
   uint8_t *heavy_flags;  // [heavy_slots] streaming-pass class flags
   int *heavy_list;       // [heavy_slots] ordered deferred slots

@@ -291,28 +291,24 @@ template <class Real> __device__ __forceinline__ int64_t dep_count(const DepArgs
   return n > A.cap ? A.cap : n;
 }
 
-// Segment of the records of one tile, or of one of `ways` parts of a tile: the
-// CTAs of a grid with few tiles spread their atomics over that many counters.
-// A sector each: neighbouring counters in one sector would share its queue.
-struct alignas(32) TileSeg { uint32_t cursor, end, start, pad[5]; };
-
+// Scratch of the tiled path.  A tile's records are a segment, or one of `ways`
+// segments: the particles of a grid with few tiles spread their atomics over
+// that many counters.  A counter has a sector of its own: neighbours in one
+// sector would share its queue.
+constexpr int SECTOR = 8;  // words
 struct TileArgs {
-  TileSeg *seg;       // [ntiles * ways]
-  uint32_t *total;    // records allocated
-  uint32_t *n_parts;  // parts of tiles with records
-  uint4 *part;        // [ntiles + rec_cap / DEP_PART_MIN] them: tile, first record, last + 1, batches with heavy cells
+  uint32_t *cnt;     // [segment * SECTOR] particles counted (zero between calls)
+  uint32_t *cursor;  // [segment * SECTOR] next record
+  uint32_t *meta;    // [0] records, [1] parts, [2] whether this call is tiled
+  uint4 *part;       // [ntiles + rec_cap / DEP_PART_MIN] parts of tiles: tile, first record, last + 1, batches with heavy cells
   uint32_t ntiles, ways, rec_cap;
   uint32_t most_ctas;  // CTAs of k_dep_tile that fill the chip twice
   uint32_t ntx, nty;
   int64_t min_n, max_n;  // other numbers of particles are deposited directly
 };
 
-// Direct deposit: a particle's 24 contributions as atomics (launches too small
-// for the tiled path, and its particles without a record).
-template <class Real>
-__global__ void __launch_bounds__(DEPOSIT_THREADS) k_pic_deposit(DepArgs<Real> A, TileArgs T) {
-  const int64_t n = dep_count(A);
-  if (n >= T.min_n && n <= T.max_n) return;  // the tiled path's
+// Direct deposit: a particle's 24 contributions as atomics.
+template <class Real> __device__ __forceinline__ void deposit_direct(const DepArgs<Real> &A, int64_t n) {
   unsigned bad = 0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
@@ -327,6 +323,12 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_pic_deposit(DepArgs<Real> A
     dep_direct(A, d);
   }
   if (bad) atomicOr(&A.cnt->status, (unsigned)QED_STATUS_NONFINITE);
+}
+
+// (calls too small for the tiled path by their capacity)
+template <class Real>
+__global__ void __launch_bounds__(DEPOSIT_THREADS) k_pic_deposit(DepArgs<Real> A) {
+  deposit_direct(A, dep_count(A));
 }
 
 // ---------------------------------------------------------------------------
@@ -396,12 +398,17 @@ constexpr uint32_t NO_TILE = 0xFFFFFFFFu;
 // numbers and a stride a sheet's tiles all fell to one CTA in 32.
 constexpr uint32_t DEP_PART = 8192, DEP_PART_MIN = 2048;
 
-// Particles per tile (in T.end), one atomic per distinct tile of a warp: the
+// Particles per tile, one atomic per distinct tile of a warp: the
 // atomics of particles stored by cell would otherwise queue up on the counters
 // of a few tiles.
 __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A, TileArgs T) {
   const int64_t n = dep_count(A);
-  if (n < T.min_n || n > T.max_n) return;
+  const bool tiled = n >= T.min_n && n <= T.max_n;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the launches that follow
+    T.meta[0] = T.meta[1] = 0u;
+    T.meta[2] = tiled;
+  }
+  if (!tiled) return;
   const int lane = threadIdx.x & 31;
   unsigned bad = 0;
   // warp-uniform loop
@@ -420,7 +427,7 @@ __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A,
       }
     }
     const unsigned same = __match_any_sync(0xFFFFFFFFu, t);
-    if (t != NO_TILE && lane == __ffs(same) - 1) atomicAdd(&T.seg[t].end, (uint32_t)__popc(same));
+    if (t != NO_TILE && lane == __ffs(same) - 1) atomicAdd(&T.cnt[t * SECTOR], (uint32_t)__popc(same));
   }
   if (bad) atomicOr(&A.cnt->status, (unsigned)QED_STATUS_NONFINITE);
 }
@@ -432,15 +439,16 @@ constexpr int ALLOC_THREADS = 256;
 __global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(DepArgs<float> A, TileArgs T) {
   __shared__ uint32_t sm[33], s_start[ALLOC_THREADS];
   __shared__ uint32_t s_base;
+  if (*(volatile uint32_t *)&T.meta[2] == 0u) return;
   const uint32_t t = blockIdx.x * ALLOC_THREADS + threadIdx.x, nseg = T.ntiles * T.ways;
-  const uint32_t c = t < nseg ? T.seg[t].end : 0u;
+  const uint32_t c = t < nseg ? T.cnt[t * SECTOR] : 0u;
   const uint32_t ex = block_excl_scan(c, sm);
-  if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(T.total, sm[32]) : 0u;
+  if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(&T.meta[0], sm[32]) : 0u;
   __syncthreads();
   s_start[threadIdx.x] = s_base + ex;
-  if (t < nseg) {
-    T.seg[t].start = T.seg[t].cursor = s_base + ex;
-    T.seg[t].end = s_base + ex + c;
+  if (c) {
+    T.cursor[t * SECTOR] = s_base + ex;
+    T.cnt[t * SECTOR] = 0u;
   }
   __syncthreads();
   // the tiles with records, in parts of (nearly) equal numbers
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(DepArgs<float> A, T
   const uint32_t most = fill < DEP_PART_MIN ? DEP_PART_MIN : fill > DEP_PART ? DEP_PART : fill;
   const uint32_t k = len <= most ? len > 0 : (len + most - 1) / most;
   const uint32_t at = block_excl_scan(k, sm);
-  if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(T.n_parts, sm[32]) : 0u;
+  if (threadIdx.x == 0) s_base = sm[32] ? atomicAdd(&T.meta[1], sm[32]) : 0u;
   __syncthreads();
   if (k == 1) T.part[s_base + at] = make_uint4(t / T.ways, beg, beg + len, 0u);
   for (uint32_t q = 0; k > 1 && q < k; ++q)
@@ -466,7 +474,10 @@ __global__ void __launch_bounds__(ALLOC_THREADS) k_dep_alloc(DepArgs<float> A, T
 __global__ void __launch_bounds__(DEPOSIT_THREADS, 4)
 k_dep_scatter(DepArgs<float> A, TileArgs T, DepRec *rec) {
   const int64_t n = dep_count(A);
-  if (n < T.min_n || n > T.max_n) return;
+  if (*(volatile uint32_t *)&T.meta[2] == 0u) {
+    deposit_direct(A, n);
+    return;
+  }
   const int lane = threadIdx.x & 31;
   for (int64_t b = (int64_t)blockIdx.x * DEPOSIT_THREADS + (threadIdx.x & ~31); b < n;
        b += (int64_t)gridDim.x * DEPOSIT_THREADS) {
@@ -490,7 +501,7 @@ k_dep_scatter(DepArgs<float> A, TileArgs T, DepRec *rec) {
     const unsigned same = __match_any_sync(0xFFFFFFFFu, t);
     const int leader = __ffs(same) - 1;
     uint32_t pos = 0;
-    if (t != NO_TILE && lane == leader) pos = atomicAdd(&T.seg[t].cursor, (uint32_t)__popc(same));
+    if (t != NO_TILE && lane == leader) pos = atomicAdd(&T.cursor[t * SECTOR], (uint32_t)__popc(same));
     pos = __shfl_sync(0xFFFFFFFFu, pos, leader) + __popc(same & ((1u << lane) - 1u));
     if (t != NO_TILE) {
       if (pos < T.rec_cap) put_rec(rec + pos, r);
@@ -694,11 +705,10 @@ __device__ __forceinline__ uint32_t dep_sort(const DepRec *rec, uint32_t m, Tile
 __global__ void __launch_bounds__(TILE_THREADS, 4)
 k_dep_tile(DepArgs<float> A, TileArgs T, const DepRec *rec) {
   __shared__ TileSmem s;
-  const int64_t n = dep_count(A);
-  if (n < T.min_n || n > T.max_n) return;
+  if (*(volatile uint32_t *)&T.meta[2] == 0u) return;
   const int c = threadIdx.x;
   // (little is kept over the sums: 36 of the 64 registers are theirs)
-  const volatile uint32_t *const parts = T.n_parts;
+  const volatile uint32_t *const parts = &T.meta[1];
   if (c == 0) s.heavy = 0;
   for (uint32_t part = blockIdx.x; part < *parts; part += gridDim.x) {
     dep_begin(A, T, T.part[part].x, s);
@@ -842,7 +852,10 @@ cudaError_t particle_grid(const qed_ctx *c, Kern kern, int64_t capacity, unsigne
 
 // When the tiled path is taken.  The rule is on the number of particles on the
 // device; the host sees only capacities, so where the capacity allows the
-// tiled path both are launched and the kernels of the other return at once.
+// tiled path its four kernels are launched and for fewer particles the scatter
+// pass deposits them directly, the others return at once (1000 particles, room
+// for 2^24: 24.7 us a call; 29.4 with a launch of its own for the direct deposit
+// and a clear of the counters, 13.7 by one kernel).
 // Measured, tiled / direct in us (stored by cell; random order):
 //   64^3 cells:  2^18 particles 28/22; 32/23    2^20 47/93; 65/83    2^23 372/941; 424/672
 //   128^3:       2^20 109/68; 117/79            2^22 213/297; 243/322
@@ -862,41 +875,45 @@ constexpr int64_t L2_CELLS = 6 << 20;
 // (128^3, 2^22: 470 us with 4096, 370 with 16384; uniform 288, 281)
 constexpr int64_t DEP_SEGMENTS = 16384;
 
-// The tiled path's launches, where the capacities allow it.  The scratch is the
-// step's: records in the staging area, segments in the per-entry counts (both
-// are free between steps, and calls that share a context are ordered).
-cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_yee *y, TileArgs &T, cudaStream_t st) {
+// The launches of a deposit where the capacities allow the tiled path, else
+// *done is left false.  The scratch is the step's (free between steps, and calls
+// that share a context are ordered): records in the staging area, cursors and
+// parts in the per-entry counts.
+cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_yee *y, bool *done, cudaStream_t st) {
+  TileArgs T;
   T.ntx = (y->nx + TLX - 1) / TLX;
   T.nty = (y->ny + TLY - 1) / TLY;
   const int64_t cells = (int64_t)y->nx * y->ny * y->nz;
   const int64_t ntiles = (int64_t)T.ntx * T.nty * ((y->nz + TLZ - 1) / TLZ);
   T.ways = 1;
   while (ntiles * T.ways < DEP_SEGMENTS && T.ways < 64) T.ways *= 2;
+  const int64_t nseg = ntiles * T.ways;
   T.min_n = cells > L2_CELLS ? cells / 2 : 2 * cells;
   if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
-  const int64_t max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
+  T.max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
   const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
   T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
   T.most_ctas = (uint32_t)c->num_sms * 8;
-  const int64_t scratch = 8 * (ntiles * T.ways + 1) + 4 * (ntiles + T.rec_cap / DEP_PART_MIN);
-  if (max_n < T.min_n || A.cap < T.min_n || A.cap > 0x7fffffff || scratch > c->heavy_slots) return cudaSuccess;
-  T.max_n = max_n;
+  const int64_t scratch = SECTOR * nseg + 4 * (ntiles + T.rec_cap / DEP_PART_MIN);
+  if (T.max_n < T.min_n || A.cap < T.min_n || A.cap > 0x7fffffff || nseg > c->dep_segs || scratch > c->heavy_slots)
+    return cudaSuccess;
+  *done = true;
   T.ntiles = (uint32_t)ntiles;
-  T.seg = reinterpret_cast<TileSeg *>(c->sub_cnt);
-  T.total = &T.seg[ntiles * T.ways].end;
-  T.n_parts = &T.seg[ntiles * T.ways].cursor;
-  T.part = reinterpret_cast<uint4 *>(T.seg + ntiles * T.ways + 1);
+  T.meta = c->dep_cnt;
+  T.cnt = c->dep_cnt + SECTOR;
+  T.cursor = c->sub_cnt;
+  T.part = reinterpret_cast<uint4 *>(c->sub_cnt + SECTOR * nseg);
   DepRec *rec = static_cast<DepRec *>(c->stage);
-  const uint32_t nseg = T.ntiles * T.ways;
   unsigned count_blocks = 0, blocks = 0;
-  cudaError_t e = cudaMemsetAsync(T.seg, 0, sizeof(TileSeg) * ((size_t)nseg + 1), st);
-  if (e == cudaSuccess) e = particle_grid(c, k_dep_count, A.cap, &count_blocks);
+  cudaError_t e = particle_grid(c, k_dep_count, A.cap, &count_blocks);
   if (e == cudaSuccess) e = particle_grid(c, k_dep_scatter, A.cap, &blocks);
   if (e != cudaSuccess) return e;
   k_dep_count<<<count_blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
-  k_dep_alloc<<<(nseg + ALLOC_THREADS - 1) / ALLOC_THREADS, ALLOC_THREADS, 0, st>>>(A, T);
+  k_dep_alloc<<<(unsigned)((nseg + ALLOC_THREADS - 1) / ALLOC_THREADS), ALLOC_THREADS, 0, st>>>(A, T);
   k_dep_scatter<<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T, rec);
-  const uint32_t most = (uint32_t)c->num_sms * 32, need = T.ntiles + T.rec_cap / DEP_PART_MIN;
+  // (four waves; a call without tiles waits for every CTA to leave: 24.7 us a call
+  // of 1000 particles with 16 CTAs per SM, 28.3 with 32)
+  const uint32_t most = (uint32_t)c->num_sms * 16, need = T.ntiles + T.rec_cap / DEP_PART_MIN;
   k_dep_tile<<<need < most ? need : most, TILE_THREADS, 0, st>>>(A, T, rec);
   c->launches += 4;
   return cudaGetLastError();
@@ -918,16 +935,15 @@ cudaError_t launch_deposit(qed_ctx *c, const qed_species *s, const qed_yee *y, d
   A.scale = (Real)((double)s->q * weight_unit / (y->dx * y->dy * y->dz));
   A.half_dt = (Real)(0.5 * c->cfg.dt);
   A.cnt = c->d_counters;
-  TileArgs T{};
-  T.max_n = -1;  // all numbers directly
-  unsigned blocks = 0;
-  cudaError_t e = particle_grid(c, k_pic_deposit<Real>, s->capacity, &blocks);
-  if (e != cudaSuccess) return e;
   if constexpr (sizeof(Real) == 4) {
-    e = launch_deposit_tiled(c, A, y, T, st);
-    if (e != cudaSuccess) return e;
+    bool done = false;
+    const cudaError_t e = launch_deposit_tiled(c, A, y, &done, st);
+    if (e != cudaSuccess || done) return e;
   }
-  k_pic_deposit<Real><<<blocks, DEPOSIT_THREADS, 0, st>>>(A, T);
+  unsigned blocks = 0;
+  const cudaError_t e = particle_grid(c, k_pic_deposit<Real>, s->capacity, &blocks);
+  if (e != cudaSuccess) return e;
+  k_pic_deposit<Real><<<blocks, DEPOSIT_THREADS, 0, st>>>(A);
   c->launches += 1;
   return cudaGetLastError();
 }
