@@ -250,7 +250,7 @@ __device__ __forceinline__ void spread(float *J, const DepArgs<Real> &A, Real fx
 }
 
 // Velocity times dt-independent parts of one particle's deposit: reduced
-// coordinates (cells) of its mid-step position and the currents a v.  The
+// coordinates (cells) of its mid-step position and its velocity.  The
 // products are written with explicit fused operations so that every kernel
 // that calls this rounds alike.
 template <class Real> struct DepPoint { Real f[3], j[3]; };
@@ -273,16 +273,18 @@ __device__ __forceinline__ bool dep_point(const DepArgs<Real> &A, int64_t p, Dep
   d.f[0] = (fma(-A.half_dt, vx, A.x[p]) - A.x0) * A.idx;
   d.f[1] = (fma(-A.half_dt, vy, A.y[p]) - A.y0) * A.idy;
   d.f[2] = (fma(-A.half_dt, vz, A.z[p]) - A.z0) * A.idz;
-  d.j[0] = vx; d.j[1] = vy; d.j[2] = vz;  // scaled by the caller
+  d.j[0] = vx; d.j[1] = vy; d.j[2] = vz;
   const Real lim = (Real)4.0e15;  // reduced coordinates beyond this are not finite cells
   return fabs(d.f[0]) < lim && fabs(d.f[1]) < lim && fabs(d.f[2]) < lim;  // also false for NaN
 }
 
 template <class Real>
-__device__ __forceinline__ void dep_direct(const DepArgs<Real> &A, const DepPoint<Real> &d) {
-  spread(A.jx, A, d.f[0] - (Real)0.5, d.f[1], d.f[2], d.j[0]);
-  spread(A.jy, A, d.f[0], d.f[1] - (Real)0.5, d.f[2], d.j[1]);
-  spread(A.jz, A, d.f[0], d.f[1], d.f[2] - (Real)0.5, d.j[2]);
+__device__ __forceinline__ void dep_direct(const DepArgs<Real> &A, const DepPoint<Real> &d, Real a) {
+  // (a v in place: scaled beforehand, FP64 took 16 operations a particle more,
+  // 1209 us for 1088 at 180^3 and 2^22)
+  spread(A.jx, A, d.f[0] - (Real)0.5, d.f[1], d.f[2], a * d.j[0]);
+  spread(A.jy, A, d.f[0], d.f[1] - (Real)0.5, d.f[2], a * d.j[1]);
+  spread(A.jz, A, d.f[0], d.f[1], d.f[2] - (Real)0.5, a * d.j[2]);
 }
 
 template <class Real> __device__ __forceinline__ int64_t dep_count(const DepArgs<Real> &A) {
@@ -317,10 +319,7 @@ template <class Real> __device__ __forceinline__ void deposit_direct(const DepAr
       bad = 1;
       continue;
     }
-    const Real a = A.scale * A.w[p];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) d.j[c] *= a;
-    dep_direct(A, d);
+    dep_direct(A, d, A.scale * A.w[p]);
   }
   if (bad) atomicOr(&A.cnt->status, (unsigned)QED_STATUS_NONFINITE);
 }
@@ -508,12 +507,9 @@ k_dep_scatter(DepArgs<float> A, TileArgs T, DepRec *rec) {
       else direct = true;  // no room for its record
     }
     if (direct) {
-      const float a = A.scale * A.w[p];
       DepPoint<float> d;
       dep_point(A, p, d);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) d.j[c] *= a;
-      dep_direct(A, d);
+      dep_direct(A, d, A.scale * A.w[p]);
     }
   }
 }
