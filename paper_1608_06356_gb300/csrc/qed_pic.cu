@@ -308,7 +308,9 @@ struct TileArgs {
   uint32_t ntiles, ways, rec_cap;
   uint32_t most_ctas;  // CTAs of k_dep_tile that fill the chip twice
   uint32_t ntx, nty;
-  int64_t min_n, max_n;  // other numbers of particles are deposited directly
+  // particles from min_n on are deposited by tiles if their order is scattered,
+  // from min_sorted on in any order, above max_n directly
+  int64_t min_n, min_sorted, max_n;
 };
 
 // Direct deposit: a particle's 24 contributions as atomics.
@@ -399,12 +401,33 @@ constexpr uint32_t NO_TILE = 0xFFFFFFFFu;
 // numbers and a stride a sheet's tiles all fell to one CTA in 32.
 constexpr uint32_t DEP_PART = 8192, DEP_PART_MIN = 2048;
 
+// Whether consecutive particles lie far apart, from eight samples of 32 of them
+// (the same for every CTA): in more than 16 tiles a sample.  32 particles of a
+// row of cells, one or two cells to a particle, lie in 4 to 9.
+__device__ __forceinline__ bool dep_scattered(const DepArgs<float> &A, const TileArgs &T, int64_t n) {
+  constexpr int SAMPLES = DEPOSIT_THREADS / 32;
+  __shared__ uint32_t s_tiles[SAMPLES];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  DepPoint<float> d;
+  float w[3];
+  uint32_t t = 0xFFFFFFFFu, cell;
+  const int64_t p = n / SAMPLES * wid + lane;
+  if (p < n && dep_point(A, p, d)) t = dep_tile(A, T, d, w, cell);
+  const unsigned first = __ballot_sync(0xFFFFFFFFu, lane == __ffs(__match_any_sync(0xFFFFFFFFu, t)) - 1);
+  if (lane == 0) s_tiles[wid] = __popc(first);
+  __syncthreads();
+  uint32_t tiles = 0;
+#pragma unroll
+  for (int q = 0; q < SAMPLES; ++q) tiles += s_tiles[q];
+  return tiles > 16 * SAMPLES;
+}
+
 // Particles per tile, one atomic per distinct tile of a warp: the
 // atomics of particles stored by cell would otherwise queue up on the counters
 // of a few tiles.
 __global__ void __launch_bounds__(DEPOSIT_THREADS) k_dep_count(DepArgs<float> A, TileArgs T) {
   const int64_t n = dep_count(A);
-  const bool tiled = n >= T.min_n && n <= T.max_n;
+  const bool tiled = n >= T.min_n && n <= T.max_n && (n >= T.min_sorted || dep_scattered(A, T, n));
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the launches that follow
     T.meta[0] = T.meta[1] = 0u;
     T.meta[2] = tiled;
@@ -854,20 +877,22 @@ cudaError_t particle_grid(const qed_ctx *c, Kern kern, int64_t capacity, unsigne
 // pass deposits them directly, the others return at once (1000 particles, room
 // for 2^24: 24.7 us a call; 29.4 with a launch of its own for the direct deposit
 // and a clear of the counters, 13.7 by one kernel).
-// Measured, tiled / direct in us (stored by cell; random order):
-//   64^3 cells:  2^18 particles 28/22; 32/23    2^20 47/93; 65/83    2^23 372/941; 424/672
-//   128^3:       2^20 109/68; 117/79            2^22 213/297; 243/322
-//   180^3:       2^22 355/282; 384/331          2^23 484/539; 551/654
-//   81 x 39 x 167: 2^19 (one a cell), random 70/42
-// so two particles per cell and 2^18 pay for a tile's fixed work; where J (12
-// bytes a cell) no longer fits L2 half of one, as each direct deposit of a
-// random order then fetches its lines (256^3, 2^24 random: 1340/5000).  Few
-// tiles leave the chip idle (16^3, 2^18: 188/78) and a very full cell is one
-// thread's work (32^3 by cell: 128 a cell 739/696, 256 a cell 2057/1435).
+// Measured on the device, tiled / direct in us (stored by cell; random order):
+//   32^3 cells:  2^18 particles 28/37; 32/28    3 2^17 31/66; 34/42   2^20 62/177; 58/111
+//   64^3:        3 2^17 33/32; 39/33            2^19 36/42; 44/43     2^23 407/917; 368/657
+//   128^3:       2^21 148/139; 165/157          2^22 214/284; 246/323 2^24 580/1455; 834/1268
+//   180^3:       2^22 350/275; 381/331          2^23 479/534; 550/651
+//   200^3:       2^22 420/284; 449/501          2^23 546/535; 617/898
+//   256^3:       2^23 852/556; 919/2538         2^24 1094/1026; 1349/5055
+// so two particles per cell and 3 2^17 pay for a tile's fixed work.  Where J (12
+// bytes a cell) no longer fits L2 a direct deposit in random order fetches its
+// lines each time, and half a particle per cell pays; stored by cell it does not
+// (k_dep_count looks at the order first: the 1026 above become 1040).
+// Grids of few tiles and more than 64 particles a cell are not taken.
 // FP64 contexts deposit directly: GB300 adds and multiplies doubles at a small
 // fraction of its float rate, and a tile is that work (128^3, 2^22 random: 1093 us
 // directly, 2369 by tiles; 64^3, 2^19: 161, 352).
-constexpr int64_t TILED_MIN_PARTICLES = 1 << 18, TILED_MIN_TILES = 128, TILED_MAX_PER_CELL = 64;
+constexpr int64_t TILED_MIN_PARTICLES = 3 << 17, TILED_MIN_TILES = 128, TILED_MAX_PER_CELL = 64;
 constexpr int64_t L2_CELLS = 6 << 20;
 // counters of a grid with few tiles: a ball of particles queues on few of them
 // (128^3, 2^22: 470 us with 4096, 370 with 16384; uniform 288, 281)
@@ -886,8 +911,8 @@ cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_
   T.ways = 1;
   while (ntiles * T.ways < DEP_SEGMENTS && T.ways < 64) T.ways *= 2;
   const int64_t nseg = ntiles * T.ways;
-  T.min_n = cells > L2_CELLS ? cells / 2 : 2 * cells;
-  if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
+  T.min_sorted = 2 * cells > TILED_MIN_PARTICLES ? 2 * cells : TILED_MIN_PARTICLES;
+  T.min_n = cells > L2_CELLS ? cells / 2 : T.min_sorted;
   T.max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
   const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
   T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
