@@ -185,6 +185,24 @@ extern "C" int qed_autotune(qed_ctx *c, const qed_species *e, const qed_species 
   return QED_OK;
 }
 
+// What the timed steps of this context read.  The single pass (FP32, Method I; not
+// the learned sampler with ordered appends) has no launch to size and no
+// schedule to set but the photon stage's and the learned sampler's dense pass;
+// hole filling sizes its own launches.
+static bool single_pass(const qed_ctx *c) {
+  const bool mlp = c->cfg.sampler == QED_SAMPLER_MLP && c->mlp_ready;
+  return c->cfg.precision == QED_FP32 && c->cfg.generator == QED_GEN_METHOD_I &&
+         !(mlp && c->cfg.append_order == QED_APPEND_ORDERED);
+}
+static bool group_matters(const qed_ctx *c, int grp) {
+  if (grp == QED_TUNE_PHOTON) return true;
+  if (grp == QED_TUNE_COMPACT) return single_pass(c) && c->cfg.sampler == QED_SAMPLER_MLP && c->mlp_ready;
+  return !single_pass(c);
+}
+static bool sched_matters(const qed_ctx *c, int k) {
+  return (k == QED_SCHED_EMIT_LANES || k == QED_SCHED_SCAN_DRAWS) && !single_pass(c);
+}
+
 extern "C" int qed_autotune_groups(qed_ctx *c, const qed_species *e, const qed_species *p,
                                    const qed_species *g, const qed_fields *f, int reps,
                                    qed_tuning *out, qed_stream_t stream) {
@@ -198,9 +216,17 @@ extern "C" int qed_autotune_groups(qed_ctx *c, const qed_species *e, const qed_s
   memcpy(saved_sched, c->sched, sizeof(saved_sched));
   int64_t step = 2000000;
   int rc = QED_OK;
-  double best_ms = 1e300;
+  // the step as it is: the time of every value of what the step does not read,
+  // which keeps as many CTAs per SM as fit and the default schedule
+  double best_ms = 0.0;
+  rc = time_steps(c, e, p, g, f, reps, step, a, b, st, &best_ms);
   // coordinate descent: one group at a time, the others at their current best
   for (int grp = 0; grp < QED_TUNE_GROUPS && rc == QED_OK; ++grp) {
+    if (!group_matters(c, grp)) {
+      for (int factor = 1; factor <= QED_TUNE_MAX_FACTOR; ++factor) out->ms[grp][factor - 1] = best_ms;
+      c->grid_factor[grp] = QED_TUNE_MAX_FACTOR;
+      continue;
+    }
     int best = 0;
     double best_g = 1e300;
     for (int factor = 1; factor <= QED_TUNE_MAX_FACTOR && rc == QED_OK; ++factor) {
@@ -220,6 +246,14 @@ extern "C" int qed_autotune_groups(qed_ctx *c, const qed_species *e, const qed_s
       {16, 8, 12, 20, 24, 0}, {12, 4, 8, 16, 0, 0}, {8, 2, 4, 12, 0, 0},
       {8, 1, 4, 12, 16, 0},   {32, 16, 24, 33, 0, 0}};
   for (int k = 0; k < QED_SCHED_PARAMS && rc == QED_OK; ++k) {
+    if (!sched_matters(c, k)) {
+      for (int j = 0; j < QED_SCHED_MAX_CANDIDATES && cand[k][j]; ++j) {
+        out->sched_tried[k][j] = cand[k][j];
+        out->sched_ms[k][j] = best_ms;
+      }
+      c->sched[k] = cand[k][0];
+      continue;
+    }
     int best = cand[k][0];
     double best_k = 1e300;
     for (int j = 0; j < QED_SCHED_MAX_CANDIDATES && cand[k][j] && rc == QED_OK; ++j) {
