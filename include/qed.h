@@ -332,6 +332,14 @@ int qed_last_device_status(qed_ctx *ctx, uint32_t *bits, int64_t *dropped);
  * QED_ERR_TIMEOUT) and clear it with qed_reset_counters. */
 int qed_test_wait_expiry(qed_ctx *ctx, qed_stream_t stream);
 
+/* The same check of qed_compact's waits: runs it on s with the first tile of
+ * particles taken by nobody, so that the tiles that wait for it give up at the
+ * iteration limit (a few seconds), set QED_STATUS_TIMEOUT and leave the count
+ * unchanged.  s must have dead particles in its first tile (256 particles) and
+ * hold more than two tiles; its particles are not to be used afterwards.  The
+ * context is. */
+int qed_test_compact_expiry(qed_ctx *ctx, const qed_species *s, qed_stream_t stream);
+
 /* Failure-detection check of the replays: with ordered appends, a single-pass
  * lepton step whose photon records run out redoes the leptons concerned from
  * their stored state (QED_STATUS_REPLAY).  Those replays of later calls take the

@@ -123,6 +123,7 @@ SIGNATURES = {
     "qed_reset_counters": (C.c_int, [_P, _P]),
     "qed_last_device_status": (C.c_int, [_P, C.POINTER(C.c_uint32), C.POINTER(C.c_int64)]),
     "qed_test_wait_expiry": (C.c_int, [_P, _P]),
+    "qed_test_compact_expiry": (C.c_int, [_P, C.POINTER(qed_species), _P]),
     "qed_test_replay_rate": (C.c_int, [_P, C.c_double]),
     "qed_launch_count": (C.c_int64, [_P]),
     "qed_profile_begin": (C.c_int, [_P, C.c_int]),

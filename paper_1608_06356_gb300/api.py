@@ -393,6 +393,12 @@ def qed_test_wait_expiry(ctx: Context, stream=None) -> None:
     B.check(B.lib().qed_test_wait_expiry(ctx.handle, _stream(stream)), "qed_test_wait_expiry")
 
 
+def qed_test_compact_expiry(ctx: Context, s: Species, stream=None) -> None:
+    """Stable compaction behind a tile that nobody takes (sets QED_STATUS_TIMEOUT)."""
+    B.check(B.lib().qed_test_compact_expiry(ctx.handle, C.byref(s.struct()), _stream(stream)),
+            "qed_test_compact_expiry")
+
+
 def qed_test_replay_rate(ctx: Context, factor: float) -> None:
     """Let the replays of ordered appends disagree with their step (1: off)."""
     B.check(B.lib().qed_test_replay_rate(ctx.handle, float(factor)), "qed_test_replay_rate")

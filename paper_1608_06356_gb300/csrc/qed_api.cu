@@ -581,6 +581,17 @@ extern "C" int qed_test_wait_expiry(qed_ctx *c, qed_stream_t stream) {
   return cuda_fail(cudaGetLastError(), "qed_test_wait_expiry");
 }
 
+__global__ void k_take_first_tile(unsigned int *ticket) { *ticket = 1u; }
+
+extern "C" int qed_test_compact_expiry(qed_ctx *c, const qed_species *s, qed_stream_t stream) {
+  if (!c || !species_ok(s, true)) return QED_ERR_ARG;
+  if (check_cap(c, s)) return QED_ERR_CAPACITY;
+  k_take_first_tile<<<1, 1, 0, (cudaStream_t)stream>>>(c->compact_n);
+  c->launches += 1;
+  const int rc = cuda_fail(cudaGetLastError(), "qed_test_compact_expiry");
+  return rc != QED_OK ? rc : qed_compact(c, s, stream);
+}
+
 extern "C" int qed_test_replay_rate(qed_ctx *c, double factor) {
   if (!c || !(factor >= 0.0) || !std::isfinite(factor)) return QED_ERR_ARG;
   c->replay_rate = factor;
