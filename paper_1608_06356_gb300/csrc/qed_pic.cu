@@ -45,6 +45,7 @@ struct YeeArgs {
   int nx, ny, nz;
   float idx, idy, idz;  // inverse spacings
   bool nodes32;         // the nodes start on a 32-byte boundary
+  uint32_t row0, rows;  // rows (j, k) of this launch
 };
 
 YeeArgs yee_args(const qed_yee *y) {
@@ -72,9 +73,11 @@ template <int V> struct Cells {
   __device__ __forceinline__ bool at(const YeeArgs &A) {
     const uint32_t per_row = (uint32_t)A.nx / V;
     const uint32_t t = blockIdx.x * FIELD_THREADS + threadIdx.x;
-    const uint32_t row = t / per_row;
-    if (row >= (uint32_t)A.ny * (uint32_t)A.nz) return false;
-    const int i = (int)(t - row * per_row) * V, j = (int)(row % (uint32_t)A.ny), k = (int)(row / (uint32_t)A.ny);
+    uint32_t row = t / per_row;
+    if (row >= A.rows) return false;
+    const int i = (int)(t - row * per_row) * V;
+    row += A.row0;
+    const int j = (int)(row % (uint32_t)A.ny), k = (int)(row / (uint32_t)A.ny);
     const int64_t nx = A.nx, plane = (int64_t)A.nx * A.ny, base = (int64_t)row * nx;
     c = base + i;
     l = base + (i == 0 ? A.nx - 1 : i - 1);
@@ -838,23 +841,32 @@ bool courant_ok(const qed_yee *y, double dt) {
   return dt * std::sqrt(s) < 1.0;
 }
 
-template <int V>
-void launch_advance(const YeeArgs &A, float dt, cudaStream_t st) {
-  const unsigned grid = (unsigned)(((int64_t)(A.nx / V) * A.ny * A.nz + FIELD_THREADS - 1) / FIELD_THREADS);
-  k_yee_b_half<V><<<grid, FIELD_THREADS, 0, st>>>(A, 0.5f * dt);
-  k_yee_e<V><<<grid, FIELD_THREADS, 0, st>>>(A, dt);
-  k_yee_b_half<V><<<grid, FIELD_THREADS, 0, st>>>(A, 0.5f * dt);
+// A pass of V cells a thread over all rows: one launch, or one per slab of rows
+// where the threads' numbers would not fit 32 bits (beyond 4.2e9 cells).
+template <int V, class Launch> void field_pass(qed_ctx *c, YeeArgs A, Launch launch) {
+  const int64_t rows = (int64_t)A.ny * A.nz, per_row = A.nx / V, slab = slab_rows(per_row, FIELD_THREADS);
+  for (int64_t r = 0; r < rows; r += slab) {
+    A.row0 = (uint32_t)r;
+    A.rows = (uint32_t)(rows - r < slab ? rows - r : slab);
+    launch(A, (unsigned)((A.rows * per_row + FIELD_THREADS - 1) / FIELD_THREADS));
+    c->launches += 1;
+  }
+}
+
+template <int V> void launch_advance(qed_ctx *c, const YeeArgs &A, float dt, cudaStream_t st) {
+  auto b_half = [&](const YeeArgs &a, unsigned grid) { k_yee_b_half<V><<<grid, FIELD_THREADS, 0, st>>>(a, 0.5f * dt); };
+  field_pass<V>(c, A, b_half);
+  field_pass<V>(c, A, [&](const YeeArgs &a, unsigned grid) { k_yee_e<V><<<grid, FIELD_THREADS, 0, st>>>(a, dt); });
+  field_pass<V>(c, A, b_half);
 }
 
 cudaError_t launch_fields(qed_ctx *c, const qed_yee *y, bool advance, cudaStream_t st) {
   const YeeArgs A = yee_args(y);
   if (advance) {
-    if (A.nx % 4 == 0) launch_advance<4>(A, (float)c->cfg.dt, st);
-    else launch_advance<1>(A, (float)c->cfg.dt, st);
-    c->launches += 3;
+    if (A.nx % 4 == 0) launch_advance<4>(c, A, (float)c->cfg.dt, st);
+    else launch_advance<1>(c, A, (float)c->cfg.dt, st);
   }
-  k_yee_nodes<<<(unsigned)(((int64_t)A.nx * A.ny * A.nz + FIELD_THREADS - 1) / FIELD_THREADS), FIELD_THREADS, 0, st>>>(A);
-  c->launches += 1;
+  field_pass<1>(c, A, [&](const YeeArgs &a, unsigned grid) { k_yee_nodes<<<grid, FIELD_THREADS, 0, st>>>(a); });
   return cudaGetLastError();
 }
 

@@ -1,4 +1,4 @@
-// qed_scratch.h -- sizes of the step's scratch (plain C++).
+// qed_scratch.h -- sizes of the step's scratch and of launches (plain C++).
 #ifndef QED_SCRATCH_H
 #define QED_SCRATCH_H
 
@@ -29,6 +29,12 @@ constexpr bool holds_pairs(int64_t max_particles) {
 static_assert(holds_pairs(1) && holds_pairs(16384) && holds_pairs(16385) && holds_pairs(16387) && holds_pairs(16388) &&
                   holds_pairs(131072) && holds_pairs(131073) && holds_pairs(((int64_t)1 << 30) - 4096),
               "a record for every pair");
+
+// Rows of a launch with `per_row` threads a row, CTAs of `block`: thread numbers
+// up to the last CTA's fit 32 bits.
+constexpr int64_t slab_rows(int64_t per_row, int64_t block) {
+  return (((int64_t)1 << 32) - block) / per_row;
+}
 
 }  // namespace qed
 

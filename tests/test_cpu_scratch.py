@@ -32,3 +32,26 @@ def test_pair_records_hold_every_photon(tmp_path):
     subprocess.check_call(["g++", "-std=c++17", "-I" + inc, str(src), "-o", str(exe)])
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, f"max_particles {r.stdout.strip()}"
+
+
+def test_field_slabs_number_their_threads_in_32_bits(tmp_path):
+    """Every thread number of a field pass fits 32 bits, the slabs cover all rows,
+    and grids below 4.2e9 cells take one launch (a Yee grid and its nodes are 68
+    bytes a cell: 4.3e9 cells still fit the device)."""
+    src = tmp_path / "slabs.cpp"
+    src.write_text("""
+        #include <initializer_list>
+        #include "qed_scratch.h"
+        using namespace qed;
+        int main() {
+          for (int64_t per_row : {1, 2, 3, 127, 128, 129, 1000, 1639, 16384, 65535, 65536}) {
+            const int64_t s = slab_rows(per_row, 128);
+            const int64_t threads = (s * per_row + 127) / 128 * 128;
+            if (s < 1 || threads > ((int64_t)1 << 32) || s * per_row < 4200000000ll) return 1;
+          }
+          return 0;
+        }""")
+    exe = tmp_path / "slabs"
+    inc = os.path.join(ROOT, "paper_1608_06356_gb300", "csrc")
+    subprocess.check_call(["g++", "-std=c++17", "-I" + inc, str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)]).returncode == 0
