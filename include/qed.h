@@ -65,8 +65,8 @@ enum {
   QED_STATUS_NONFINITE = 4u,/* non-finite momentum or field met (particle skipped) */
   QED_STATUS_TIMEOUT = 8u,  /* a look-back wait hit its iteration limit */
   QED_STATUS_SUBSTEPS = 16u,/* sub-step count was capped at qed_config.max_substeps */
-  QED_STATUS_REPLAY = 32u   /* a replayed emission chain found fewer photons than its
-                               counting pass (should not happen); the missing photons
+  QED_STATUS_REPLAY = 32u   /* a replayed emission chain found fewer photons than were
+                               counted for it (should not happen); the missing photons
                                were written with zero energy */
 };
 
@@ -86,10 +86,9 @@ enum { QED_FIELDS_UNIFORM = 0, QED_FIELDS_PER_PARTICLE = 1, QED_FIELDS_GRID = 2 
  *   count, then particle index, then sub-step -- so reruns give the same
  *   arrays bit for bit.
  * ANY: the same photons (ids, energies, positions, weights, fields) in an
- *   order that depends on the scheduling of the GPU's warps; the lepton step
- *   then runs in a single pass (FP32 contexts with event generator Method I;
- *   other contexts append in the ORDERED way).  Capacity overflow drops
- *   whichever appends come last. */
+ *   order that depends on the scheduling of the GPU's warps (FP32 contexts
+ *   with event generator Method I; other contexts append in the ORDERED way).
+ *   Capacity overflow drops whichever appends come last. */
 enum { QED_APPEND_ORDERED = 0, QED_APPEND_ANY = 1 };
 
 /* ---- configuration ---------------------------------------------------- */
@@ -235,10 +234,13 @@ int qed_step_fused(qed_ctx *ctx, const qed_species *e, const qed_species *p,
  * HOST memory, streamed through the GPU in chunks of `chunk` leptons: chunk
  * k is copied in, stepped and copied back while the next is copied in and
  * the previous copied out (the caller's stream steps, two streams of the
- * context copy; the host arrays should be page-locked for the copies to
- * overlap).  Particle ids key the random draws, so the leptons and the set
- * of photons are those of one qed_step_fused call on the whole species with
- * no photons present at the start.
+ * context copy).  Where the device can map the host arrays (page-locked memory
+ * from the CUDA runtime) and they start on 16-byte boundaries, one kernel per
+ * chunk and direction copies through the mapped pointers; other arrays go by a
+ * copy each (pageable ones without overlap).  Particle ids key the random
+ * draws, so the leptons and the set of photons are those of one qed_step_fused
+ * call on the whole species with no photons present at the start; the photons
+ * are appended chunk by chunk, each in the order of a step of its leptons.
  *   l_host  a lepton species whose arrays (x..pz, w, id, the per-particle
  *           fields with QED_FIELDS_PER_PARTICLE, od_p/od_r with Methods
  *           II/III, optional tag) are HOST pointers and whose d_n points to a
@@ -464,10 +466,12 @@ int qed_set_tuning(qed_ctx *ctx, const qed_tuning *t);
 /* Measurement hooks.  qed_profile_begin creates CUDA events (call it outside
  * any timed or captured region) so that each of the next max_steps calls of
  * qed_step_fused records events on its stream between its phases:
+ *   (the multi-pass lepton step; a single-pass one has its kernel in phase 0,
+ *   the ordered writes or the learned sampler's dense pass in 1, no 2 to 4)
  *   0 lepton streaming pass      1 lepton class list (3 launches)
  *   2 lepton counting pass       3 scan of the photon counts
  *   4 lepton writing pass        5 photon streaming pass
- *   6 photon list + ordered pass
+ *   6 pair scan and writing pass
  * qed_profile_end synchronises, returns the summed milliseconds of the
  * lepton stage (phases 0-4) and of the photon stage (5-6) and the number of
  * steps recorded, and releases the events; qed_profile_end_phases does the

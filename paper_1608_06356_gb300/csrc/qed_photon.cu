@@ -119,7 +119,9 @@ __global__ void __launch_bounds__(PH_THREADS, sizeof(Real) == 4 ? 4 : 2) k_photo
       uint64_t pid = 0;
       uint32_t r2 = 0;
       int64_t N = 1;
-      // (the words do not wait for the flag: few photons of a step are dead)
+      // (the words do not wait for the flag; 8.4M photons with fields, all alive,
+      // half or all dead: 204, 203 and 73 us, against 240, 247 and 96 in the stream
+      // and list that read the flag first)
       uint8_t alive = 0;
       Real x = 0, y = 0, z = 0, px = 0, py = 0, pz = 0;
       if (i < n) {
