@@ -313,7 +313,7 @@ struct TileArgs {
   uint32_t ntx, nty;
   // particles from min_n on are deposited by tiles if their order is scattered,
   // from min_sorted on in any order, above max_n directly
-  int64_t min_n, min_sorted, max_n;
+  int64_t min_n, min_sorted, max_n, cells;
 };
 
 // Direct deposit: a particle's 24 contributions as atomics.
@@ -404,9 +404,12 @@ constexpr uint32_t NO_TILE = 0xFFFFFFFFu;
 // numbers and a stride a sheet's tiles all fell to one CTA in 32.
 constexpr uint32_t DEP_PART = 8192, DEP_PART_MIN = 2048;
 
-// Whether consecutive particles lie far apart, from eight samples of 32 of them
-// (the same for every CTA): in more than 16 tiles a sample.  32 particles of a
-// row of cells, one or two cells to a particle, lie in 4 to 9.
+// Whether the particles' order is scattered enough for tiles, from eight samples
+// of 32 consecutive ones (the same for every CTA): by the tiles a sample lies in,
+// 4 cells / n + 1 of them in an order by cell, which drift adds to.  The line is
+// where both sides measured the same: 256^3 cells, one a cell 6.4 tiles (drift by
+// 0.2 cells; by none 1051 us directly, 1131 by tiles, by two cells 1519, 1161), half
+// of one 18.9 (583, 884; 909, 908); 320^3, half 14.3 (1128, 1685; 2229, 1728).
 __device__ __forceinline__ bool dep_scattered(const DepArgs<float> &A, const TileArgs &T, int64_t n) {
   constexpr int SAMPLES = DEPOSIT_THREADS / 32;
   __shared__ uint32_t s_tiles[SAMPLES];
@@ -422,7 +425,7 @@ __device__ __forceinline__ bool dep_scattered(const DepArgs<float> &A, const Til
   uint32_t tiles = 0;
 #pragma unroll
   for (int q = 0; q < SAMPLES; ++q) tiles += s_tiles[q];
-  return tiles > 16 * SAMPLES;
+  return tiles * n > SAMPLES * (10 * T.cells - 4 * n);
 }
 
 // Particles per tile, one atomic per distinct tile of a warp: the
@@ -898,8 +901,9 @@ cudaError_t particle_grid(const qed_ctx *c, Kern kern, int64_t capacity, unsigne
 //   256^3:       2^23 852/556; 919/2538         2^24 1094/1026; 1349/5055
 // so two particles per cell and 3 2^17 pay for a tile's fixed work.  Where J (12
 // bytes a cell) no longer fits L2 a direct deposit in random order fetches its
-// lines each time, and half a particle per cell pays; stored by cell it does not
-// (k_dep_count looks at the order first: the 1026 above become 1040).
+// lines each time, and half a particle per cell pays; stored by cell it takes one
+// and a half (200^3: 679/776), in between as the order goes (dep_scattered, which
+// makes the 1026 above 1040).
 // Grids of few tiles and more than 64 particles a cell are not taken.
 // FP64 contexts deposit directly: GB300 adds and multiplies doubles at a small
 // fraction of its float rate, and a tile is that work (128^3, 2^22 random: 1093 us
@@ -923,8 +927,11 @@ cudaError_t launch_deposit_tiled(qed_ctx *c, const DepArgs<float> &A, const qed_
   T.ways = 1;
   while (ntiles * T.ways < DEP_SEGMENTS && T.ways < 64) T.ways *= 2;
   const int64_t nseg = ntiles * T.ways;
-  T.min_sorted = 2 * cells > TILED_MIN_PARTICLES ? 2 * cells : TILED_MIN_PARTICLES;
-  T.min_n = cells > L2_CELLS ? cells / 2 : T.min_sorted;
+  const bool large = cells > L2_CELLS;
+  T.min_n = large ? cells / 2 : 2 * cells;
+  if (T.min_n < TILED_MIN_PARTICLES) T.min_n = TILED_MIN_PARTICLES;
+  T.min_sorted = large ? 3 * cells / 2 : T.min_n;
+  T.cells = cells;
   T.max_n = ntiles < TILED_MIN_TILES ? 0 : cells * TILED_MAX_PER_CELL;
   const int64_t cap = 2 * c->stage_cap;  // a staging record holds two of these
   T.rec_cap = (uint32_t)(cap < 0x7fffffff ? cap : 0x7fffffff);
