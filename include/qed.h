@@ -449,8 +449,10 @@ typedef struct {
  * order above), times `reps` fused steps plus qed_compact_fill of the photons
  * for every factor that fits (1..8 CTAs per SM), keeping the best before
  * tuning the next group; then each scheduling parameter in turn over a fixed
- * list of candidates.  Groups and parameters that the context's step does not
- * read are not timed: every value of them gets the time of the step as it is,
+ * list of candidates.  The population changes as it is stepped, so a value's time
+ * is that of the setting's default just before and after it scaled to the first
+ * step's.  Groups and parameters that the context's step does not read are not
+ * timed: every value of them gets the time of the step as it is,
  * and they keep 8 CTAs per SM (as many as fit) and their defaults.  The species
  * are advanced -- pass disposable copies.
  * The chosen values are kept in the context for all later launches and
