@@ -78,11 +78,14 @@ template <class Real> struct LeptonArgs {
 };
 
 
-// First slot of a thread: consecutive slices of 32 go to different CTAs, so that
-// a small species is spread over the SMs (FP64 runs at 2 FMAs per clock and SM:
-// 10^4 electrons in 40 CTAs of 256 took 26 us, over all SMs 11).
-__device__ __forceinline__ int64_t spread_slot() {
-  return ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+// First slot of a thread.  FP64: consecutive slices of 32 go to different CTAs, so
+// that a small species is spread over the SMs, which run FP64 at 2 FMAs per clock
+// (10^4 electrons in 40 CTAs of 256 took 26 us, over all SMs 11).  FP32 is bound by
+// memory, and a CTA's 256 slots stay together: the push of 4.2M electrons with
+// fields 49.7 us, 52.8 spread; 16.8M 182, 190.
+template <class Real> __device__ __forceinline__ int64_t first_slot() {
+  return sizeof(Real) == 8 ? ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31)
+                           : (int64_t)blockIdx.x * TILE + threadIdx.x;
 }
 
 // ---------------------------------------------------------------------------
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(TILE) k_lepton_push(LeptonArgs<Real> A) {
   const int64_t n0 = s_meta[0], n1 = s_meta[1];
   const Real dt = sel<Real>(A.C.dt, A.C.f_dt);
   uint32_t status = 0;
-  for (int64_t g = spread_slot(); g < n0 + n1; g += (int64_t)gridDim.x * TILE) {
+  for (int64_t g = first_slot<Real>(); g < n0 + n1; g += (int64_t)gridDim.x * TILE) {
     const int si = g < n0 ? 0 : 1;
     const Sp<Real> &S = A.sp[si];
     const int64_t i = si ? g - n0 : g;
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(TILE, sizeof(Real) == 4 ? 3 : 2) k_lepton_stre
   };
   const int64_t stride = (int64_t)gridDim.x * TILE;
   int buf = 0;
-  int64_t slot = spread_slot();
+  int64_t slot = first_slot<Real>();
   if (slot < nslots) prefetch(slot, 0);
   cp_async_commit();
   // nslots is a multiple of TILE: every lane of a warp runs the same iterations
